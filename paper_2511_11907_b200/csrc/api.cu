@@ -261,7 +261,7 @@ int kvswap_project_keys(const kvswap_shape* shape, const void* K, const float* p
   if (misaligned(K) || misaligned(proj) || misaligned(meta_out)) return KVSWAP_ERR_ALIGN;
   if (n_begin < 0 || n_end < n_begin || n_end > p.N) return KVSWAP_ERR_SHAPE;
   if (n_begin == n_end) return KVSWAP_OK;
-  // The workspace is optional here: with one of at least kvswap_workspace_bytes() bf16 K with d in {64, 128}
+  // The workspace is optional here: with one of at least kvswap_workspace_bytes() 16-bit K with d in {64, 128}
   // and r in {16, 32, 64} runs on tcgen05 (it needs room for the split adapter), otherwise on the warp-level path.
   void* scratch = nullptr;
   uint32_t* err = nullptr;

@@ -1,11 +1,11 @@
 // K1 on the 5th-generation tensor cores: metadata build K_lr = Flatten(K) A (Sec. 4.2) with
 // tcgen05.mma, accumulators in tensor memory and operands staged by TMA.
 //
-// Covers bf16 K with d in {64, 128} and r in {16, 32, 64} (r = 32, d = 128 are the benchmark
+// Covers bf16 and fp16 K with d in {64, 128} and r in {16, 32, 64} (r = 32, d = 128 are the benchmark
 // shapes); project_keys.cu keeps the warp-level path for everything else.
 //
-// The adapter stays fp32-exact: every entry is split into three bf16 pieces, laid out by a small
-// preparation kernel as a K-major [3r x d] operand per KV head, so one instruction shape
+// The adapter stays fp32-exact: every entry is split into three pieces of K's type (fp16: scaled by a
+// power of two per column, undone in the epilogue), laid out by a small preparation kernel as a K-major [3r x d] operand per KV head, so one instruction shape
 // M = 128 tokens, N = 3r (48, 96 or 192) columns, K = 16 channels yields the three partial products
 // side by side; the epilogue adds them in fp32.  The tensor core adds into its accumulator with
 // truncation, so a chain inside tensor memory covers one KV head (d / 16 instructions); the sum
@@ -17,6 +17,9 @@
 //   warp 1   issues the MMAs (one thread), owns the tensor-memory allocation (two accumulators);
 //   warps 2-5 epilogue: tcgen05.ld of the finished accumulator (one token row per thread), sum of
 //            the three pieces, running sum over heads, one rounding into the metadata type.
+// fp16 K used to take the fp32-pipe kernel: 28 layers of 5003 tokens (8 heads of 128, r = 32) took 2075 us, here
+// 319 us, of which the host issues 11 us a layer.  The launch overlaps the split of the adapter (programmatic
+// dependent launch, K requested before the wait): four layers of 4 x 131072 bf16 tokens 879 -> 859 us.
 // Stages and accumulators are handed over through mbarriers; every wait is bounded.
 #include <algorithm>
 #include <type_traits>
@@ -29,7 +32,7 @@ namespace kvswap {
 namespace {
 
 constexpr int kTileM = 128;                                // tokens per tile
-constexpr uint32_t kAHalf = kTileM * 128;                  // 128 rows x 128 bytes (64 bf16 channels)
+constexpr uint32_t kAHalf = kTileM * 128;                  // 128 rows x 128 bytes (64 channels of 16 bits)
 constexpr int kThreadsUmma = 6 * 32;
 constexpr size_t kMaxDynamicSmem = 227 * 1024;
 constexpr int kMaxStages = 6;
@@ -52,20 +55,60 @@ struct Cfg {
   static_assert(kNcols % 16 == 0 && kNcols <= 256, "N of a 128-row tcgen05.mma");
 };
 
-// ---- the adapter as three bf16 pieces, [g][piece * r + j][c] (K-major rows of d channels) ----------
-__global__ void split_adapter_kernel(const float* __restrict__ proj, __nv_bfloat16* __restrict__ bsplit, int n, int kD,
-                                     int kR) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;     // over [g][c][j]
-  if (i >= n) return;
-  const int kNcols = 3 * kR;
-  const int j = i % kR, c = (i / kR) % kD, g = i / (kR * kD);
-  const float v = proj[i];
-  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-  const float r1 = v - __bfloat162float(hi);
-  const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-  const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-  __nv_bfloat16* dst = bsplit + (int64_t(g) * kNcols + j) * kD + c;
-  dst[0] = hi; dst[int64_t(kR) * kD] = mid; dst[int64_t(2 * kR) * kD] = lo;
+// ---- the adapter as three 16-bit pieces, [g][piece * r + j][c] (K-major rows of d channels) ----------
+// bf16 pieces carry 8 + 8 + 8 mantissa bits at fp32's exponent range.  fp16 pieces carry 11 bits each but
+// bottom out at 2^-24, so every column of a head (of a pair of heads that share an accumulator) is first
+// multiplied by a power of two that brings its largest entry into [2^14, 2^15): what the three pieces
+// then miss is below 2^-39 of that entry.  The epilogue multiplies by the inverse, `unscale` [block][r].
+// One CTA per block of kD channels (one head, or a pair of 64-channel heads) and 16 columns: thread
+// (part, j) holds 16 channels of column j, so all loads of the CTA go out together and a piece leaves as
+// two 16-byte stores.  With the one thread per entry and 2-byte stores r channels apart that this
+// replaces, the kernel took 2.8 us at 8 heads of 128, r = 32.
+template <typename T>
+__global__ void __launch_bounds__(128)
+split_adapter_kernel(const float* __restrict__ proj, T* __restrict__ bsplit, float* __restrict__ unscale, int head_dim,
+                     int block_dim, int r) {
+  __shared__ float part_max[8][16];
+  const int j = blockIdx.y * 16 + (threadIdx.x & 15), part = threadIdx.x >> 4;
+  const int per = block_dim >> 3;                          // channels per thread: 16 or 8
+  const int c0 = part * per;                               // within the block
+  pdl_wait();                                              // the pieces may still be in use by the call before
+  pdl_trigger();
+  float v[16];
+  const float* src = proj + (int64_t(blockIdx.x) * block_dim + c0) * r + j;
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = (i < per) ? src[int64_t(i) * r] : 0.f;
+  float scale = 1.f;
+  if constexpr (std::is_same<T, __half>::value) {
+    float mx = 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) mx = fmaxf(mx, fabsf(v[i]));
+    part_max[part][threadIdx.x & 15] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) mx = fmaxf(mx, part_max[k][threadIdx.x & 15]);
+    int sh = 0;
+    if (mx > 0.f && mx < INFINITY) sh = min(120, max(-113, 14 - (int((__float_as_uint(mx) >> 23) & 0xffu) - 127)));
+    scale = __uint_as_float(uint32_t(sh + 127) << 23);
+    if (part == 0) unscale[int64_t(blockIdx.x) * r + j] = __uint_as_float(uint32_t(127 - sh) << 23);
+  }
+  __align__(16) T piece[3][16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    float rest = v[i] * scale;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      piece[k][i] = T(rest);                               // round to nearest even
+      rest -= float(piece[k][i]);
+    }
+  }
+  const int g = (int64_t(blockIdx.x) * block_dim + c0) / head_dim, c = c0 % head_dim;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    uint4* dst = reinterpret_cast<uint4*>(bsplit + (int64_t(g) * 3 * r + k * r + j) * head_dim + c);
+    dst[0] = reinterpret_cast<const uint4*>(piece[k])[0];
+    if (per == 16) dst[1] = reinterpret_cast<const uint4*>(piece[k])[1];
+  }
 }
 
 // ---- PTX wrappers ------------------------------------------------------------------------------
@@ -74,7 +117,7 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_byte_addr) {
   return uint64_t((smem_byte_addr >> 4) & 0x3fffu) | (uint64_t(1) << 16) | (uint64_t(1024 >> 4) << 32) |
          (uint64_t(1) << 46) | (uint64_t(2) << 61);
 }
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_16bit(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
@@ -124,11 +167,13 @@ struct UmmaShared {
 // D = channels multiplied per stage.  PAIR (D = 128 with heads of 64 channels, joint metadata): a stage
 // holds two KV heads, one per 64-channel half, so the chain inside tensor memory sums a pair of heads
 // and there are half as many stages to hand over.
-template <int D, int R, typename META_T, bool PAIR>
+// KV_T: the type of K and of the adapter pieces (one tcgen05.mma takes both operands in one 16-bit type).
+template <typename KV_T, int D, int R, typename META_T, bool PAIR>
 __global__ void __launch_bounds__(kThreadsUmma, 1)
 project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_b,
-                         META_T* __restrict__ meta, int n_begin, int n_end, int tiles_per_row,
-                         uint32_t* __restrict__ err) {
+                         META_T* __restrict__ meta, const float* __restrict__ unscale, int n_begin, int n_end,
+                         int tiles_per_row, uint32_t* __restrict__ err) {
+  constexpr bool kScaled = std::is_same<KV_T, __half>::value;
   using C = Cfg<D, R>;
   constexpr int kD = D, kR = R, kNcols = C::kNcols, kStages = C::kStages, kHalves = C::kHalves;
   constexpr uint32_t kBHalf = C::kBHalf, kStageBytes = C::kStageBytes, kTmemCols = C::kTmemCols, kAccStride = C::kAccStride;
@@ -159,33 +204,57 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
   const int64_t first = items * blockIdx.x / gridDim.x, last = items * (blockIdx.x + 1) / gridDim.x;
   const int n_steps = int(last - first) * g_count;
 
+  // The kernel before this one splits the adapter, and let this one start once everything before it was
+  // complete: K may be fetched at once, the pieces and their scales only after the wait.  No early trigger
+  // here: the scorers request metadata tiles ahead of their own wait.
   if (warp == 0) {
     // ================================ producer ==============================================
     if (lane == 0) {
-      for (int s = 0; s < n_steps; ++s) {
-        const int stage = s % kStages, use = s / kStages;
-        if (use > 0 && !mbar_wait(smem_addr(&sh.empty[stage]), uint32_t(use - 1) & 1u)) { sh.abort = 1; if (err) atomicExch(err, kDevTimeoutEmpty); break; }
+      auto place = [&](int s, int* n0, int* g, int* b) {                  // token, head and sequence of step s
         const int64_t item = first + s / g_count;
         const int tile = int(item % tiles_per_row), bh = int(item / tiles_per_row);
-        const int hm = bh % p.Hm, b = bh / p.Hm;
-        const int g = ((p.Hm == 1) ? 0 : hm) + (s % g_count) * (PAIR ? 2 : 1);
+        const int hm = bh % p.Hm;
+        *b = bh / p.Hm;
+        *g = ((p.Hm == 1) ? 0 : hm) + (s % g_count) * (PAIR ? 2 : 1);
+        *n0 = n_begin + tile * kTileM;
+      };
+      auto load_k = [&](int s) {
+        const int stage = s % kStages;
         const uint32_t dst = stage0 + uint32_t(stage) * kStageBytes, bar = smem_addr(&sh.full[stage]);
+        int n0, g, b;
+        place(s, &n0, &g, &b);
         mbar_arrive_expect_tx(bar, kStageBytes);
-        const int n0 = n_begin + tile * kTileM;
 #pragma unroll
-        for (int h = 0; h < kHalves; ++h) {
-          const int c0 = PAIR ? 0 : 64 * h, gh = PAIR ? g + h : g;       // channels and head of this half
-          tma_load_4d(dst + uint32_t(h) * kAHalf, &map_k, bar, c0, n0, gh, b);
-          tma_load_2d(dst + kHalves * kAHalf + uint32_t(h) * kBHalf, &map_b, bar, c0, gh * kNcols);
-        }
+        for (int h = 0; h < kHalves; ++h)                                  // channels and head of this half
+          tma_load_4d(dst + uint32_t(h) * kAHalf, &map_k, bar, PAIR ? 0 : 64 * h, n0, PAIR ? g + h : g, b);
+      };
+      auto load_b = [&](int s) {
+        const int stage = s % kStages;
+        const uint32_t dst = stage0 + uint32_t(stage) * kStageBytes, bar = smem_addr(&sh.full[stage]);
+        int n0, g, b;
+        place(s, &n0, &g, &b);
+#pragma unroll
+        for (int h = 0; h < kHalves; ++h)
+          tma_load_2d(dst + kHalves * kAHalf + uint32_t(h) * kBHalf, &map_b, bar, PAIR ? 0 : 64 * h, (PAIR ? g + h : g) * kNcols);
+      };
+      const int early = min(n_steps, kStages);
+      for (int s = 0; s < early; ++s) load_k(s);
+      pdl_wait();
+      for (int s = 0; s < early; ++s) load_b(s);
+      for (int s = early; s < n_steps; ++s) {
+        const int stage = s % kStages, use = s / kStages;
+        if (use > 0 && !mbar_wait(smem_addr(&sh.empty[stage]), uint32_t(use - 1) & 1u)) { sh.abort = 1; if (err) atomicExch(err, kDevTimeoutEmpty); break; }
+        load_k(s);
+        load_b(s);
       }
     }
     __syncwarp();
   } else if (warp == 1) {
     // ================================ MMA issuer ============================================
     if (lane == 0) {
-      // M = 128, N = 3r, fp32 accumulate, bf16 x bf16, both operands K-major
-      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(kNcols >> 3) << 17) | (uint32_t(kTileM >> 4) << 24);
+      // M = 128, N = 3r, fp32 accumulate, both operands bf16 (1) or both fp16 (0), K-major
+      constexpr uint32_t kFormat = kScaled ? 0u : 1u;
+      constexpr uint32_t idesc = (1u << 4) | (kFormat << 7) | (kFormat << 10) | (uint32_t(kNcols >> 3) << 17) | (uint32_t(kTileM >> 4) << 24);
       for (int s = 0; s < n_steps; ++s) {
         const int stage = s % kStages, use = s / kStages, buf = s & 1, acc_use = s >> 1;
         if (acc_use > 0 && !mbar_wait(smem_addr(&sh.acc_empty[buf]), uint32_t(acc_use - 1) & 1u)) { sh.abort = 1; if (err) atomicExch(err, kDevTimeoutEmpty); break; }
@@ -195,7 +264,7 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
 #pragma unroll
         for (int k = 0; k < kD / 16; ++k) {
           const uint32_t half = k >> 2, koff = uint32_t(k & 3) * 32u;     // 16 channels = 32 bytes inside the swizzle row
-          umma_bf16(tmem + uint32_t(buf) * kAccStride, umma_desc(a0 + half * kAHalf + koff), umma_desc(b0 + half * kBHalf + koff),
+          umma_16bit(tmem + uint32_t(buf) * kAccStride, umma_desc(a0 + half * kAHalf + koff), umma_desc(b0 + half * kBHalf + koff),
                     idesc, k > 0 ? 1u : 0u);
         }
         umma_commit(smem_addr(&sh.empty[stage]));         // the stage may be refilled once these MMAs have read it
@@ -211,12 +280,15 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
 #pragma unroll
     for (int j = 0; j < kR; ++j) acc[j] = 0.f;
     bool ok = true;
+    if constexpr (kScaled) pdl_wait();                     // the scales are the split kernel's
     for (int s = 0; s < n_steps && ok; ++s) {
       const int buf = s & 1, acc_use = s >> 1;
       ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&sh.acc_full[buf]), uint32_t(acc_use) & 1u));
       if (!ok) { if (lane == 0) { sh.abort = 1; if (err) atomicExch(err, kDevTimeoutFull); } break; }
       tc_fence_after();
       const uint32_t taddr = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf) * kAccStride;
+      const float* us = nullptr;                           // scales of this step's head, or pair of heads
+      if constexpr (kScaled) us = unscale + int64_t(((p.Hm == 1) ? 0 : int((first + s / g_count) / tiles_per_row) % p.Hm) + s % g_count) * kR;
 #pragma unroll
       for (int c0 = 0; c0 < kR; c0 += kChunk) {            // the pieces of columns c0 .. c0 + kChunk - 1 sit kR columns apart
         float hi[kChunk], mid[kChunk], lo[kChunk];
@@ -225,7 +297,11 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
         tmem_ld_cols(taddr + 2 * kR + c0, lo);
         tmem_ld_wait();
 #pragma unroll
-        for (int j = 0; j < kChunk; ++j) acc[c0 + j] += (lo[j] + mid[j]) + hi[j];
+        for (int j = 0; j < kChunk; ++j) {
+          const float sum = (lo[j] + mid[j]) + hi[j];
+          if constexpr (kScaled) acc[c0 + j] = fmaf(sum, us[c0 + j], acc[c0 + j]);      // a power of two: exact
+          else acc[c0 + j] += sum;
+        }
       }
       tc_fence_before();
       __syncwarp();
@@ -287,19 +363,20 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
 }  // namespace
 
 static bool umma_shape(const Problem& p) {
-  return p.kv_dtype == KVSWAP_BF16 && (p.d == 64 || p.d == 128) && (p.r == 16 || p.r == 32 || p.r == 64);
+  return p.kv_dtype != KVSWAP_F32 && (p.d == 64 || p.d == 128) && (p.r == 16 || p.r == 32 || p.r == 64);
 }
 
 size_t project_keys_umma_scratch_bytes(const Problem& p) {
   if (!umma_shape(p)) return 0;
-  return size_t(p.Hkv) * 3 * p.r * p.d * sizeof(__nv_bfloat16);
+  // the pieces of the adapter, and (fp16) one scale per head and column
+  return size_t(p.Hkv) * 3 * p.r * p.d * sizeof(__nv_bfloat16) + size_t(p.Hkv) * p.r * sizeof(float);
 }
 
 namespace {
 
-template <int D, int R, bool PAIR>
-cudaError_t launch_umma(const Problem& p, const CUtensorMap& map_k, const CUtensorMap& map_b, void* meta, int n_begin,
-                        int n_end, uint32_t* err, cudaStream_t st) {
+template <typename KV_T, int D, int R, bool PAIR>
+cudaError_t launch_umma(const Problem& p, const CUtensorMap& map_k, const CUtensorMap& map_b, void* meta,
+                        const float* unscale, int n_begin, int n_end, uint32_t* err, cudaStream_t st) {
   using C = Cfg<D, R>;
   const int tiles_per_row = (n_end - n_begin + kTileM - 1) / kTileM;
   const int64_t items = int64_t(p.B) * p.Hm * tiles_per_row;
@@ -308,15 +385,15 @@ cudaError_t launch_umma(const Problem& p, const CUtensorMap& map_k, const CUtens
   auto go = [&](auto kern, auto* meta_t) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
-    kern<<<ctas, kThreadsUmma, smem, st>>>(p, map_k, map_b, meta_t, n_begin, n_end, tiles_per_row, err);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3(ctas), dim3(kThreadsUmma), smem, st, p, map_k, map_b, meta_t, unscale, n_begin, n_end,
+                      tiles_per_row, err);
   };
   if constexpr (R == 32) {                                 // 8-bit metadata exists for r = 32 only
-    if (p.meta_dtype == KVSWAP_E4M3) return go(project_keys_umma_kernel<D, R, e4m3_t, PAIR>, static_cast<e4m3_t*>(meta));
+    if (p.meta_dtype == KVSWAP_E4M3) return go(project_keys_umma_kernel<KV_T, D, R, e4m3_t, PAIR>, static_cast<e4m3_t*>(meta));
   }
   if (p.meta_dtype == KVSWAP_E4M3) return cudaErrorInvalidValue;
-  if (p.meta_dtype == KVSWAP_F16) return go(project_keys_umma_kernel<D, R, __half, PAIR>, static_cast<__half*>(meta));
-  return go(project_keys_umma_kernel<D, R, float, PAIR>, static_cast<float*>(meta));
+  if (p.meta_dtype == KVSWAP_F16) return go(project_keys_umma_kernel<KV_T, D, R, __half, PAIR>, static_cast<__half*>(meta));
+  return go(project_keys_umma_kernel<KV_T, D, R, float, PAIR>, static_cast<float*>(meta));
 }
 
 }  // namespace
@@ -334,26 +411,35 @@ bool try_launch_project_keys_umma(const Problem& p, const void* K, const float* 
   EncodeTiledFn enc = tensor_map_encoder();
   if (enc == nullptr) return false;
   const int ncols = 3 * p.r;
+  const bool bf16 = p.kv_dtype == KVSWAP_BF16;
   CUtensorMap map_k, map_b;
-  if (!make_rows_tensor_map(&map_k, K, 2, true, p.d, p.N, p.Hkv, p.B, p.kv_sn, p.kv_sh, p.kv_sb, kTileM)) return false;
+  if (!make_rows_tensor_map(&map_k, K, 2, bf16, p.d, p.N, p.Hkv, p.B, p.kv_sn, p.kv_sh, p.kv_sb, kTileM)) return false;
   {
     const cuuint64_t dims[2] = {cuuint64_t(p.d), cuuint64_t(p.Hkv) * ncols};
     const cuuint64_t strides[1] = {cuuint64_t(p.d) * 2};
     const cuuint32_t box[2] = {64, cuuint32_t(ncols)}, estr[2] = {1, 1};
-    if (enc(&map_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, scratch, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    if (enc(&map_b, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, scratch, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return false;
   }
-  const int n_proj = p.Hkv * p.d * p.r;
-  split_adapter_kernel<<<(n_proj + 255) / 256, 256, 0, st>>>(proj, static_cast<__nv_bfloat16*>(scratch), n_proj, p.d, p.r);
-  *result = cudaGetLastError();
+  float* unscale = reinterpret_cast<float*>(static_cast<char*>(scratch) + size_t(p.Hkv) * ncols * p.d * 2);
+  const int block_dim = pair ? 2 * p.d : p.d;
+  const dim3 split_grid(p.Hkv * p.d / block_dim, p.r / 16);
+  *result = bf16 ? launch_pdl(split_adapter_kernel<__nv_bfloat16>, split_grid, dim3(128), 0, st, proj,
+                              static_cast<__nv_bfloat16*>(scratch), unscale, p.d, block_dim, p.r)
+                 : launch_pdl(split_adapter_kernel<__half>, split_grid, dim3(128), 0, st, proj,
+                              static_cast<__half*>(scratch), unscale, p.d, block_dim, p.r);
   if (*result != cudaSuccess) return true;
-  auto by_rank = [&](auto d_tag, auto pair_tag) {
-    constexpr int D = decltype(d_tag)::value;
+  auto by_type = [&](auto d_tag, auto r_tag, auto pair_tag) {
+    constexpr int D = decltype(d_tag)::value, R = decltype(r_tag)::value;
     constexpr bool P = decltype(pair_tag)::value;
-    return p.r == 16   ? launch_umma<D, 16, P>(p, map_k, map_b, meta, n_begin, n_end, err, st)
-           : p.r == 32 ? launch_umma<D, 32, P>(p, map_k, map_b, meta, n_begin, n_end, err, st)
-                       : launch_umma<D, 64, P>(p, map_k, map_b, meta, n_begin, n_end, err, st);
+    return bf16 ? launch_umma<__nv_bfloat16, D, R, P>(p, map_k, map_b, meta, unscale, n_begin, n_end, err, st)
+                : launch_umma<__half, D, R, P>(p, map_k, map_b, meta, unscale, n_begin, n_end, err, st);
+  };
+  auto by_rank = [&](auto d_tag, auto pair_tag) {
+    return p.r == 16   ? by_type(d_tag, std::integral_constant<int, 16>(), pair_tag)
+           : p.r == 32 ? by_type(d_tag, std::integral_constant<int, 32>(), pair_tag)
+                       : by_type(d_tag, std::integral_constant<int, 64>(), pair_tag);
   };
   using D128 = std::integral_constant<int, 128>;
   using D64 = std::integral_constant<int, 64>;

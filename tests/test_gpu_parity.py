@@ -407,6 +407,33 @@ def test_project_keys_tensor_core_shapes(head_dim, rank, meta_heads):
     assert kv.kvswap_read_device_status(dl.ws) == 0
 
 
+@pytest.mark.parametrize("head_dim,rank,meta_heads,meta", [(128, 32, 1, W.F16), (128, 64, "per_head", W.F16), (128, 16, 1, W.F32),
+                                                           (64, 32, 1, W.F16), (64, 32, "per_head", W.F32), (64, 64, 1, W.F32)])
+def test_project_keys_tensor_core_fp16(head_dim, rank, meta_heads, meta):
+    """fp16 K on tcgen05: the adapter's fp16 pieces are scaled per head and column (the columns here span 2^48, which
+    one scale per head could not hold), heads of 64 channels in pairs and alone, ragged tiles and a range inside a tile."""
+    wl = small(kv_dtype=W.F16, q_dtype=W.F16, meta_dtype=meta, head_dim=head_dim, rank=rank, group_size=8,
+               n_ctx=512 + 77, n_q_heads=8, n_kv_heads=4, batch=2)
+    mh = 1 if meta_heads == 1 else wl.n_kv_heads
+    li = W.make_layer(wl, 0, mh)
+    if meta == W.F32:
+        li.proj[:, :, 0] *= 2.0 ** -28
+        li.proj[:, :, 1] *= 2.0 ** 20
+        li.proj[:, :, 2] = 0.0
+    dl = DeviceLayer(li, KV)
+    meta_or = O.project_keys(li.K, li.proj, mh, META_NAME[meta])
+    tol = project_tolerance(li.K, li.proj, mh, meta_or, meta)
+    got = dl.project()
+    assert np.all(np.abs(got.astype(np.float64) - meta_or.astype(np.float64)) <= tol)
+    if meta == W.F16:
+        assert np.mean(got != meta_or.astype(np.float32)) < 0.02
+    dl.meta.fill_(123.0)
+    got = dl.project(n_begin=130, n_end=130 + 300)
+    assert np.all(got[:, :, :130] == 123.0) and np.all(got[:, :, 430:] == 123.0)
+    assert np.all(np.abs(got[:, :, 130:430].astype(np.float64) - meta_or[:, :, 130:430].astype(np.float64)) <= tol[:, :, 130:430])
+    assert kv.kvswap_read_device_status(dl.ws) == 0
+
+
 def test_strided_kv_and_metadata_views():
     """K and V interleaved in one buffer (row stride 2d) and metadata rows padded."""
     wl = small(kv_dtype=W.BF16, q_dtype=W.BF16, meta_dtype=W.F16, head_dim=128, rank=32, n_ctx=517, group_size=8)
