@@ -119,6 +119,9 @@ def _ptr(t) -> Optional[int]:
 def _stream(stream) -> Optional[int]:
     if stream is None:
         import torch
+        if torch.cuda.is_initialized():
+            # the handle alone: torch.cuda.current_stream() builds a Stream object, 3.4 us of an 11 us call
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
         stream = torch.cuda.current_stream()
     return getattr(stream, "cuda_stream", stream) or None
 
