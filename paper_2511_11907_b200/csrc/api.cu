@@ -83,7 +83,7 @@ static int workspace_score_pitch(const Problem& p) { return (std::max(p.NG, 1) +
 // batch and head counts alone, at a fixed place in front of everything else, so that one workspace
 // keeps them zero between calls while the context grows.
 static bool hist_capable(const Problem& p) {
-  return (p.meta_dtype == KVSWAP_F16 || p.meta_dtype == KVSWAP_E4M3) && p.r == 32 && int64_t(p.B) * p.S <= 1024;
+  return score_stream_rows(p) && int64_t(p.B) * p.S <= 1024;
 }
 
 // The scorer counts the leading digit of every group score's key and the TopK starts from those
@@ -150,7 +150,7 @@ cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q,
   }
   if (p.NG < 1) return cudaSuccess;                                       // nothing to score
   if (score_stream_supported(p)) {
-    // fp16 metadata rows of 64 bytes: the tensor-core scorer, which builds the low-rank queries itself
+    // dense metadata rows of common ranks: the tensor-core scorer, which builds the low-rank queries itself
     // where it can and counts the leading digits of its scores for the TopK that follows
     uint32_t* top_hist = counts_top_digit(p) ? reinterpret_cast<uint32_t*>(base + w.off_hist) : nullptr;
     const bool fused = score_stream_fuses_query(p);
@@ -165,7 +165,7 @@ cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q,
   }
   cudaError_t e = launch_lowrank_query(p, q, proj, uq, stream);
   if (e != cudaSuccess) return e;
-  return launch_score_pool(p, uq, meta, scores, static_cast<uint32_t*>(ws), stream);
+  return launch_score_pool(p, uq, meta, scores, stream);
 }
 
 cudaError_t select_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected,

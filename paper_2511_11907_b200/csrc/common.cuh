@@ -89,14 +89,14 @@ bool try_launch_project_keys_umma(const Problem& p, const void* K, const float* 
                                   int n_end, void* scratch, uint32_t* err, cudaStream_t st, cudaError_t* result);
 cudaError_t launch_lowrank_query(const Problem& p, const void* q, const float* proj, float* uq,
                                  cudaStream_t st);
-cudaError_t launch_score_pool(const Problem& p, const float* uq, const void* meta, float* scores,
-                              uint32_t* err, cudaStream_t st);
-// The streaming tensor-core scorer (score_stream.cu) for fp16 metadata rows of 64 bytes.  Where it
+cudaError_t launch_score_pool(const Problem& p, const float* uq, const void* meta, float* scores, cudaStream_t st);
+// The streaming tensor-core scorer (score_stream.cuh) for dense metadata rows of common ranks.  Where it
 // builds the low-rank queries itself it takes q and proj (uq unused), else -- or when q is NULL --
 // uq [B, Su, r] from launch_lowrank_query or from the kernel of launch_combine_select.  `top_hist` (may be NULL): per (sequence, scope) a histogram of the leading
 // 12 bits of the group scores' keys (4096 16-bit counters, two per word) followed, after all
 // histograms, by one ticket word per (sequence, scope).  Everything is zero on entry; the scorer
 // counts, and launch_topk_parts, which starts from the counts, leaves everything zero again.
+bool score_stream_rows(const Problem& p);        // metadata type and rank are among the scorer's
 bool score_stream_supported(const Problem& p);
 bool score_stream_fuses_query(const Problem& p);
 bool score_stream_counts_top_digit(const Problem& p);

@@ -24,7 +24,7 @@ namespace kvswap {
 constexpr int kPartThreads = 1024;
 constexpr int kPartWarps = kPartThreads / 32;
 constexpr int kPartKeys = 4 * kPartThreads;  // keys per part
-constexpr int kMaxParts = 4;
+constexpr int kMaxParts = 8;
 constexpr int kFewKeys = 32;                 // candidates that one warp ranks directly instead of by another digit
 
 // Thread t holds the populations c[0..3] of bins base .. base + 3, base = 4096 - 4 (t + 1): the
@@ -278,7 +278,7 @@ __device__ __forceinline__ void topk_parts_body(const Problem& p, const float* _
 inline int plan_topk_parts(const Problem& p) {
   if (p.NG < 1 || p.NG > kMaxParts * kPartKeys || int64_t(p.B) * p.S > 65535) return 0;
   const int need = (p.NG + kPartKeys - 1) / kPartKeys;
-  return need <= 1 ? 1 : need <= 2 ? 2 : 4;
+  return need <= 1 ? 1 : need <= 2 ? 2 : need <= 4 ? 4 : 8;
 }
 
 }  // namespace kvswap

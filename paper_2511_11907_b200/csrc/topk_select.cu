@@ -298,8 +298,8 @@ template <int D> constexpr int kCombineRows = (kPartThreads / D < 14) ? kPartThr
 //
 // The combine CTAs have nothing to do until the gather before them has finished.  With q_ahead they
 // use that time for the summed low-rank queries of the layer whose scorer is enqueued next (row sets
-// cta, cta + n_comb, ..): half of the CTA's threads run the scorer's own build_queries() and store the
-// rows where that scorer looks for them, so that it starts on its tiles as soon as this kernel ends.
+// cta, cta + n_comb, ..): they run the scorer's own build_queries() and store the rows where that scorer
+// looks for them, so that it starts on its tiles as soon as this kernel ends.
 template <int P, int D>
 __global__ void __launch_bounds__(kPartThreads)
 combine_select_kernel(Problem p, const float* __restrict__ scores, uint32_t* __restrict__ top_hist,
@@ -315,14 +315,22 @@ combine_select_kernel(Problem p, const float* __restrict__ scores, uint32_t* __r
   }
   __shared__ float w_s[kRows][kMaxSplits];
   __shared__ float norm_s[kRows][2];
-  __shared__ float qsum[kQuerySumFloats], upart[kQueryPartFloats], urow[kQueryCols * 32];
+  __shared__ float qsum[kQuerySumFloats], upart[kQueryPartFloats], urow[kQueryCols * 64];
   pdl_trigger();
-  if (q_ahead != nullptr && threadIdx.x < kQueryThreads) {
+  if (q_ahead != nullptr) {
     for (int rest = blockIdx.x; rest < n_rests; rest += n_comb) {
       const RowSet rs = row_set(p, rest, n_sub);
-      build_queries<15>(p, q_ahead, proj_ahead, rs, qsum, upart, urow);
-      store_queries(p, rs, urow, uq_ahead);
-      asm volatile("bar.sync 15, %0;" ::"n"(kQueryThreads) : "memory");       // urow is free for the next row set
+      if (p.r == 32) {
+        build_queries<15, 32, kPartWarps>(p, q_ahead, proj_ahead, rs, qsum, upart, urow);
+        store_queries<32>(p, rs, urow, uq_ahead);
+      } else if (p.r == 16) {
+        build_queries<15, 16, kPartWarps>(p, q_ahead, proj_ahead, rs, qsum, upart, urow);
+        store_queries<16>(p, rs, urow, uq_ahead);
+      } else {
+        build_queries<15, 64, kPartWarps>(p, q_ahead, proj_ahead, rs, qsum, upart, urow);
+        store_queries<64>(p, rs, urow, uq_ahead);
+      }
+      __syncthreads();                                  // urow is free for the next row set
     }
   }
   pdl_wait();
@@ -342,7 +350,10 @@ cudaError_t launch_topk_parts(const Problem& p, const float* scores, uint32_t* t
   if (P == 0) return cudaErrorInvalidValue;
   const dim3 grid(P, p.B * p.S), block(kPartThreads);
   auto go = [&](auto kern) { return launch_pdl(kern, grid, block, 0, st, p, scores, top_hist, group_idx, n_selected); };
-  return P == 1 ? go(topk_parts_kernel<1>) : P == 2 ? go(topk_parts_kernel<2>) : go(topk_parts_kernel<4>);
+  return P == 1   ? go(topk_parts_kernel<1>)
+         : P == 2 ? go(topk_parts_kernel<2>)
+         : P == 4 ? go(topk_parts_kernel<4>)
+                  : go(topk_parts_kernel<8>);
 }
 
 cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_t* top_hist, int32_t* group_idx,
@@ -364,8 +375,14 @@ cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_
     return launch_pdl(kern, grid, block, 0, st, p, scores, top_hist, group_idx, n_selected, n_probs, partial, out, lse,
                       splits, n_rows, n_comb, q_ahead, proj_ahead, uq_ahead, n_rests, n_sub);
   };
-  if (d == 128) return P == 1 ? go(combine_select_kernel<1, 128>) : P == 2 ? go(combine_select_kernel<2, 128>) : go(combine_select_kernel<4, 128>);
-  return P == 1 ? go(combine_select_kernel<1, 64>) : P == 2 ? go(combine_select_kernel<2, 64>) : go(combine_select_kernel<4, 64>);
+  auto by_parts = [&](auto d_tag) {
+    constexpr int D = decltype(d_tag)::value;
+    return P == 1   ? go(combine_select_kernel<1, D>)
+           : P == 2 ? go(combine_select_kernel<2, D>)
+           : P == 4 ? go(combine_select_kernel<4, D>)
+                    : go(combine_select_kernel<8, D>);
+  };
+  return d == 128 ? by_parts(std::integral_constant<int, 128>()) : by_parts(std::integral_constant<int, 64>());
 }
 
 }  // namespace kvswap

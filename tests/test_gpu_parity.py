@@ -434,6 +434,50 @@ def test_project_keys_tensor_core_fp16(head_dim, rank, meta_heads, meta):
     assert kv.kvswap_read_device_status(dl.ws) == 0
 
 
+STREAM = [   # K/V type, metadata type, rank, G, per-head, scope, B, H_kv, rho, N (tile edges: 4096 or 3072 bytes of rows)
+    (W.BF16, W.F16, 16, 8, False, KV, 1, 8, 4, 128 * 19 + 9),
+    (W.BF16, W.F16, 64, 8, False, KV, 2, 8, 1, 32 * 37 + 8),
+    (W.F16, W.F16, 64, 32, False, ALL, 1, 8, 2, 32 * 33 + 31),
+    (W.BF16, W.F16, 64, 2, True, KV, 2, 3, 2, 1999),
+    (W.F32, W.F32, 16, 1, False, KV, 2, 2, 4, 64 * 17 + 1),
+    (W.F32, W.F32, 32, 4, False, KV, 1, 9, 1, 32 * 40 + 4),
+    (W.F32, W.F32, 32, 16, True, KV, 1, 2, 3, 1027),
+    (W.BF16, W.F16, 32, 12, False, KV, 2, 10, 1, 48 * 21 + 13),
+    (W.BF16, W.F16, 64, 5, False, ALL, 1, 4, 2, 20 * 41 + 3),
+    (W.F16, W.F16, 16, 48, False, KV, 1, 4, 2, 48 * 25),
+    (W.F32, W.F32, 32, 24, False, KV, 1, 2, 2, 24 * 31 + 5),
+    (W.BF16, W.F16, 32, 8, True, ALL, 2, 8, 1, 48 * 30 + 17),
+    (W.F32, W.F32, 16, 3, True, ALL, 1, 2, 2, 48 * 12 + 2),
+    (W.BF16, W.F16, 16, 8, True, ALL, 1, 10, 1, 1300),
+    (W.F32, W.F32, 16, 4, True, ALL, 1, 2, 1, 240001),     # several tiles per warp: blocks of tiles, head by head
+    (W.F32, W.F32, 16, 4, False, ALL, 1, 2, 1, 131072),    # 32768 groups: eight TopK parts
+    (W.F32, W.F32, 16, 7, False, KV, 1, 2, 1, 130003),
+]
+
+
+@pytest.mark.parametrize("kv_type,meta,rank,G,per_head,scope,B,Hkv,rho,N", STREAM)
+def test_streaming_scorer_shapes(kv_type, meta, rank, G, per_head, scope, B, Hkv, rho, N):
+    """The predictor over every stored type and rank of the streaming scorer: groups that leave the registers and groups
+    that go through the warp's buffer, one term per score and one per metadata head, ragged last tiles."""
+    wl = small("stream", batch=B, n_ctx=N, n_q_heads=Hkv * rho, n_kv_heads=Hkv, rank=rank, group_size=G,
+               top_k=max(1, min(N // G // 3, 500)), kv_dtype=kv_type, q_dtype=kv_type, meta_dtype=meta,
+               calib_rows=max(512, Hkv * 64))
+    mh = Hkv if per_head else 1
+    li = W.make_layer(wl, 0, mh)
+    dl = DeviceLayer(li, scope)
+    meta_or = O.project_keys(li.K, li.proj, mh, META_NAME[meta])
+    dl.set_meta(meta_or)
+    R, absdot = oracle_score_parts(li, meta_or, scope)
+    for _ in range(2):                                       # the second call finds the counters the first one left
+        idx, nsel, Rg = dl.score_select()
+        check_scores(R, Rg[:, :, :R.shape[2]], absdot)
+        check_selection(R, idx, nsel, wl.top_k)
+        assert np.array_equal(idx, O.select(Rg[:, :, :R.shape[2]].astype(np.float64), wl.top_k))
+    idx2, nsel2, _ = dl.score_select(with_scores=False)
+    assert np.array_equal(idx, idx2) and np.array_equal(nsel, nsel2)
+    assert kv.kvswap_read_device_status(dl.ws) == 0
+
+
 def test_strided_kv_and_metadata_views():
     """K and V interleaved in one buffer (row stride 2d) and metadata rows padded."""
     wl = small(kv_dtype=W.BF16, q_dtype=W.BF16, meta_dtype=W.F16, head_dim=128, rank=32, n_ctx=517, group_size=8)
