@@ -109,7 +109,7 @@ void plan_workspace(const Problem& p, Workspace* w) {
   w->uq_bytes = align256(sizeof(float) * size_t(p.B) * p.Su * p.r);
   w->off_uq = off;       off += 2 * w->uq_bytes;
   w->off_scores = off;   off += align256(sizeof(float) * size_t(p.B) * p.S * workspace_score_pitch(p));
-  w->off_partial = off;  off += align256(sizeof(float) * size_t(p.B) * p.Hq * w->splits * (p.d + 2));
+  w->off_partial = off;  off += align256(sizeof(float) * size_t(p.B) * p.Hq * std::max(w->splits, w->splits_room) * (p.d + 2));
   w->off_softmax = off;  off += align256(sizeof(float) * size_t(p.B) * p.Hq * (size_t(p.r) + 2 * size_t(score_softmax_chunks(p))));
   w->off_adapter = off;  off += align256(project_keys_umma_scratch_bytes(p) + 1024);   // 1 KiB: tensor-map base alignment
   w->total = off;
@@ -201,6 +201,9 @@ bool select_with_combine_launch(const Problem& p_in, const Workspace& w, int32_t
 cudaError_t score_select_launch(const Problem& p, const Workspace& w, const void* q, const float* proj,
                                 const void* meta, int32_t* group_idx, int32_t* n_selected, float* group_scores_opt,
                                 void* ws, cudaStream_t stream) {
+  if (score_select_cluster_pays_alone(p))
+    return launch_score_select_cluster(p, q, proj, meta, group_scores_opt, group_idx, n_selected,
+                                       static_cast<uint32_t*>(ws), stream);
   cudaError_t e = score_launch(p, w, q, proj, meta, group_scores_opt, ws, stream);
   if (e == cudaSuccess) e = select_launch(p, w, group_idx, n_selected, group_scores_opt, ws, stream);
   return e;

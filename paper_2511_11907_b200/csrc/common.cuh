@@ -50,8 +50,10 @@ struct Workspace {
   size_t off_adapter;  // bf16 [H_kv, 3 r, d]       adapter split into three bf16 pieces (project_keys on tcgen05)
   size_t total;
   int splits;          // split-K factor of sparse_decode for this shape
+  int splits_room;     // splits the partials are planned for (whatever the flags of a call)
   int heads_per_cta;   // query heads sharing one K/V pass in sparse_decode
   int depth;           // shared-memory stages per compute warp in sparse_decode
+  bool merge_in_cluster;   // sparse_decode on its own: the splits of a list form a cluster that merges them (no combine pass)
 };
 
 int resolve(const kvswap_shape* s, Problem* p);            // validation; returns kvswap_status
@@ -103,6 +105,14 @@ bool score_stream_counts_top_digit(const Problem& p);
 cudaError_t launch_score_stream(const Problem& p, const void* q, const float* proj, const float* uq,
                                 const void* meta, float* scores, uint32_t* top_hist, uint32_t* err,
                                 cudaStream_t st);
+// Scorer and TopK of a short context in one launch of clusters (score_select_cluster.cuh).  `scores`: NULL or the
+// caller's [B, S, NG].  Uses no workspace.
+struct ClusterGrid { int clusters, ctas; bool whole_sm; };          // whole_sm: one of its CTAs fills an SM's shared memory
+bool score_select_cluster_grid(const Problem& p, ClusterGrid* g);   // false: the shape does not take it
+bool score_select_cluster_supported(const Problem& p);
+bool score_select_cluster_pays_alone(const Problem& p);
+cudaError_t launch_score_select_cluster(const Problem& p, const void* q, const float* proj, const void* meta, float* scores,
+                                        int32_t* group_idx, int32_t* n_selected, uint32_t* err, cudaStream_t st);
 cudaError_t launch_topk_select(const Problem& p, const float* scores, int32_t* group_idx,
                                int32_t* n_selected, cudaStream_t st);
 bool topk_parts_supported(const Problem& p);   // false: row too long for launch_topk_parts

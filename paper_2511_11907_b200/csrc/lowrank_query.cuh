@@ -38,6 +38,44 @@ __device__ __forceinline__ RowSet row_set(const Problem& p, int rest, int n_sub)
   return RowSet{bh / hm_count, bh % hm_count, rest % n_sub};
 }
 
+// The terms that feed the rows of a row set: term t adds to row t (or 0) and reads KV head head0 + t.
+struct QueryTerms { int n_terms, head0; bool row_per_term; };
+__device__ __forceinline__ QueryTerms query_terms(const Problem& p, RowSet rs) {
+  const bool joint = p.Hm == 1;
+  const bool all_heads = joint && p.scope == KVSWAP_SCOPE_ALL_HEADS;
+  const bool multi = multi_term(p);
+  return QueryTerms{(all_heads || multi) ? p.Hkv : joint ? min(kQueryCols, p.S - rs.sub * kQueryCols) : 1,
+                    (all_heads || multi) ? 0 : joint ? rs.sub * kQueryCols : rs.hm, (joint && !all_heads) || multi};
+}
+// log2 of the 32-channel pieces of a head: 4, 2 or 1
+__device__ __forceinline__ int query_chunk_shift(const Problem& p) { return (p.d == 128) ? 2 : (p.d == 64) ? 1 : 0; }
+
+// Sum over a KV head's query heads of channel c: the loads of four heads go out together.
+__device__ __forceinline__ float query_sum(const Problem& p, const void* q, int b, int head, int c) {
+  const int64_t at = (int64_t(b) * p.Hq + int64_t(head) * p.rho) * p.d + c;
+  float s = 0.f;
+  for (int h0 = 0; h0 < p.rho; h0 += 4) {
+    float v[4];
+#pragma unroll
+    for (int hh = 0; hh < 4; ++hh) v[hh] = (h0 + hh < p.rho) ? load_q(q, p.q_dtype, at + int64_t(h0 + hh) * p.d) : 0.f;
+    s += (v[0] + v[1]) + (v[2] + v[3]);
+  }
+  return s;
+}
+
+// Entry (row, j) of the summed queries of up to eight terms from the partial products upart[item][32] of
+// column block j / 32, added in a fixed order; s: the sum over the terms before these.
+__device__ __forceinline__ float query_entry(const float* upart, int row, int j, int nt, int ch_shift, bool row_per_term, float s) {
+  const int chunks = 1 << ch_shift;
+  if (row_per_term) {                                                  // the items of term `row`
+    if (row < nt)
+      for (int ch = 0; ch < chunks; ++ch) s += upart[((row << ch_shift) + ch) * 32 + (j & 31)];
+  } else if (row == 0) {
+    for (int it = 0; it < (nt << ch_shift); ++it) s += upart[it * 32 + (j & 31)];
+  }
+  return s;
+}
+
 // Summed low-rank queries of one row set into urow[8][R], R = p.r = 16, 32 or 64 (rows beyond the set's
 // scopes are zero).  The KV heads that feed the rows are taken eight at a time, 32 columns at a time.  An
 // item is 32 channels of one head: a warp multiplies the head's summed query by the adapter rows (coalesced
@@ -58,14 +96,8 @@ __device__ void build_queries(const Problem& p, const void* q, const float* __re
   constexpr int kLoads = (R == 16) ? 16 : 32;                             // adapter reads per item
   constexpr int kPasses = (R + 31) / 32;                                  // blocks of 32 columns
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool joint = p.Hm == 1;
-  const bool all_heads = joint && p.scope == KVSWAP_SCOPE_ALL_HEADS;
-  const bool multi = multi_term(p);
-  // term t of the row set: (row it adds to, KV head it reads)
-  const int n_terms = (all_heads || multi) ? p.Hkv : joint ? min(kQueryCols, p.S - rs.sub * kQueryCols) : 1;
-  const int head0 = (all_heads || multi) ? 0 : joint ? rs.sub * kQueryCols : rs.hm;      // head of term t: head0 + t
-  const bool row_per_term = (joint && !all_heads) || multi;               // row of term t: t, else 0
-  const int ch_shift = (p.d == 128) ? 2 : (p.d == 64) ? 1 : 0;            // 32-channel pieces of a head: 4, 2 or 1
+  const QueryTerms qt = query_terms(p, rs);
+  const int n_terms = qt.n_terms, head0 = qt.head0, ch_shift = query_chunk_shift(p);
   const int chunks = 1 << ch_shift;
   const int d_shift = ch_shift + 5;
   // channel and column of load cc of an item: R = 16 takes channels 2 cc and 2 cc + 1 at once
@@ -92,15 +124,7 @@ __device__ void build_queries(const Problem& p, const void* q, const float* __re
       if (pass == 0) {
         for (int i = tid; i < (nt << d_shift); i += 32 * NW) {
           const int tt = i >> d_shift, c = i & (p.d - 1);
-          const int64_t at = (int64_t(rs.b) * p.Hq + int64_t(head0 + t0 + tt) * p.rho) * p.d + c;
-          float s = 0.f;
-          for (int h0 = 0; h0 < p.rho; h0 += 4) {                      // the loads of four heads go out together
-            float v[4];
-#pragma unroll
-            for (int hh = 0; hh < 4; ++hh) v[hh] = (h0 + hh < p.rho) ? load_q(q, p.q_dtype, at + int64_t(h0 + hh) * p.d) : 0.f;
-            s += (v[0] + v[1]) + (v[2] + v[3]);
-          }
-          qsum[tt * 128 + c] = s;
+          qsum[tt * 128 + c] = query_sum(p, q, rs.b, head0 + t0 + tt, c);
         }
         sync();
       }
@@ -119,14 +143,7 @@ __device__ void build_queries(const Problem& p, const void* q, const float* __re
       if (tid < kQueryCols * 32) {
         const int row = tid >> 5, j = tid & 31, at = row * R + pass * 32 + j;
         if (pass * 32 + j < R) {
-          float s = (t0 == 0) ? 0.f : urow[at];
-          if (row_per_term) {                                          // the items of term `row`
-            if (row < nt)
-              for (int ch = 0; ch < chunks; ++ch) s += upart[((row << ch_shift) + ch) * 32 + j];
-          } else if (row == 0) {
-            for (int it = 0; it < n_items; ++it) s += upart[it * 32 + j];
-          }
-          urow[at] = s;
+          urow[at] = query_entry(upart, row, j, nt, ch_shift, qt.row_per_term, (t0 == 0) ? 0.f : urow[at]);
         }
       }
       sync();

@@ -9,11 +9,9 @@
 // kDepth tiles in flight per warp; the first tiles are requested before the dependency wait, since nothing
 // the library runs during decoding writes metadata.
 //
-// The accumulator leaves lane (g, t) the scores of scope g for tokens 2t and 2t+1 of eight.  With G a power
-// of two up to 32 (template GS = log2 G) a group's maximum is a max over two registers and at most two
-// shuffles, and a finished group score leaves the registers at once.  Every other G that fits a tile
-// (GS = -1) goes through a small shared-memory buffer of the warp, [scope][token], from which lane (g, t)
-// takes the groups t, t + 4, .. of scope g; so do scores that sum a term on every metadata head (per-head
+// With G a power of two up to 32 (template GS = log2 G) a finished group score leaves the registers at
+// once.  Every other G that fits a tile (GS = -1) goes through a small shared-memory buffer of the warp,
+// [scope][token]; so do scores that sum a term on every metadata head (per-head
 // metadata under the all-heads scope): there a warp runs through the heads of up to kMultiTiles tiles,
 // adding each head's products to the buffer, before it takes the maxima.
 //
@@ -49,19 +47,7 @@ constexpr int kScoreDepth = 2;
 constexpr int kScoreCols = kQueryCols;                    // scores per metadata row and instruction
 constexpr int kHistWords = kScoreCols * kKeyTopBins / 2;  // two 16-bit counters per word
 constexpr int kMaxSets = 4;                               // row sets one CTA may touch when it builds the queries itself
-constexpr int kGenericRows = 48;                          // GS = -1: token rows per tile, at most
-constexpr int kGenericPitch = 56;                         // floats between scopes of the warp's buffer (bank spread)
 constexpr int kMultiTiles = 8;                            // tiles whose scores a warp sums over the heads together
-
-// Rows of one stage.  4 KB where a finished score leaves the registers (the hand-over of a stage costs the
-// same whatever its size: 4 KB x 2 stages measured 1.3 us per layer faster than 2 KB x 4 at B = 4,
-// N = 131072); GS = -1 takes 3 KB, which leaves room for the warps' score buffers.
-template <int META, int R, int GS>
-struct ScoreStage {
-  static constexpr int kBytes = GS >= 0 ? 4096 : 3072;
-  static constexpr int kFit = kBytes / MetaRows<META, R>::kRowBytes;
-  static constexpr int kRows = GS >= 0 ? kFit : (kFit < kGenericRows ? kFit : kGenericRows);
-};
 
 template <int META, int R, int GS>
 struct ScoreSmem {
@@ -195,7 +181,6 @@ score_stream_kernel(Problem p, StreamArgs a) {
   uint32_t* my_hist = nullptr;                      // its global histogram
   int my_col = -1;                                  // its column of the shared-memory histogram, or -1
   bool scope_ok = false;                            // the lane's scope exists
-  float run = -INFINITY;                            // running maximum of a 16- or 32-row group
   float* const sc = sm->sc + (GS >= 0 ? 0 : warp * kCols * kGenericPitch);
   int stage = 0;
   uint32_t phase = 0;
@@ -259,85 +244,29 @@ score_stream_kernel(Problem p, StreamArgs a) {
     if (!__all_sync(kFull, mbar_wait(smem_addr(&sm->full[warp * kDepth + stage]), phase))) { timed_out = true; break; }
     const int rows = min(tile_rows, rows_total - tile * tile_rows);   // a multiple of G: groups never straddle tiles
     const uint32_t base = ring + uint32_t(stage) * kStageBytes + score_lane_offset<META, R>(lane);
-    if constexpr (GS >= 0) {
-      constexpr int g_shift = GS;
-      const int ngt = rows >> g_shift;              // groups in this tile
-      float* dst = my_row + ((tile * tile_rows) >> g_shift);         // first group of the tile in this lane's row
-      float mine[(kStageRows + 31) / 32] = {};      // G = 8: the groups of reads qt, qt + 4, .. are this lane's to publish
-#pragma unroll
-      for (int it = 0; it < kStageRows / 8; ++it) {
-        if (it * 8 < rows) {
-          float x0, x1;
-          score_rows8<META, R>(base + uint32_t(it) * 8u * kRowBytes, query, &x0, &x1);
-          if constexpr (GS == 0) {                                   // tokens 2t and 2t+1 of this read are groups
-            if (scope_ok && it * 8 + 2 * qt < rows) publish(dst + it * 8 + 2 * qt, x0 * query.inv);
-            if (scope_ok && it * 8 + 2 * qt + 1 < rows) publish(dst + it * 8 + 2 * qt + 1, x1 * query.inv);
-          } else {
-            float m = fmaxf(x0, x1);
-            if constexpr (GS >= 2) m = fmaxf(m, __shfl_xor_sync(kFull, m, 1));
-            if constexpr (GS >= 3) m = fmaxf(m, __shfl_xor_sync(kFull, m, 2));
-            // (a ragged last tile holds a whole number of groups, but not of 8-row reads when G < 8)
-            if constexpr (GS == 1) { if (scope_ok && it * 4 + qt < ngt) publish(dst + it * 4 + qt, m * query.inv); }
-            else if constexpr (GS == 2) {
-              if (scope_ok && (qt & 1) == 0 && it * 2 + (qt >> 1) < ngt) publish(dst + it * 2 + (qt >> 1), m * query.inv);
-            }
-            else if constexpr (GS == 3) { if (qt == (it & 3)) mine[it >> 2] = m; }
-            else {                                                 // G = 16 or 32: 2 or 4 reads per group
-              run = fmaxf(run, m);
-              if (((it + 1) & ((1 << (GS - 3)) - 1)) == 0) {
-                const int gi = it >> (GS - 3);
-                if (scope_ok && qt == (gi & 3)) publish(dst + gi, run * query.inv);
-                run = -INFINITY;
-              }
-            }
-          }
-        }
+    if (!multi) {
+      float* dst = my_row + (GS >= 0 ? (tile * tile_rows) >> GS : tile * (tile_rows / p.G));   // first group of the tile
+      score_tile_groups<META, R, GS, kStageRows>(base, rows, lane, query, p.G, scope_ok, sc,
+                                                 [&](int gi, float x) { publish(dst + gi, x); });
+    } else if constexpr (GS < 0) {
+      // the one scope's token scores of the whole block of tiles, summed over the terms
+      float* s = sc + c.in * tile_rows;
+      for (int it = 0; it * 8 < rows; ++it) {
+        float x0, x1;
+        score_rows8<META, R>(base + uint32_t(it) * 8u * kRowBytes, query, &x0, &x1);
+        const int i = it * 8 + 2 * qt;                           // (a tile's rows need not be whole reads)
+        if (rq == 0 && i < rows) s[i] = (c.term == 0 ? 0.f : s[i]) + x0 * query.inv;
+        if (rq == 0 && i + 1 < rows) s[i + 1] = (c.term == 0 ? 0.f : s[i + 1]) + x1 * query.inv;
       }
-      if constexpr (GS == 3) {
-#pragma unroll
-        for (int h = 0; h < (kStageRows + 31) / 32; ++h)
-          if (scope_ok && (4 * h + qt) * 8 < rows) publish(dst + 4 * h + qt, mine[h] * query.inv);
-      }
-    } else {
-      // token scores into the warp's buffer: [scope][token of the tile], or with several terms the one scope's
-      // tokens of the whole block, summed over the terms
-      if (!multi) {
-#pragma unroll 2
-        for (int it = 0; it * 8 < rows; ++it) {
-          float x0, x1;
-          score_rows8<META, R>(base + uint32_t(it) * 8u * kRowBytes, query, &x0, &x1);
-          *reinterpret_cast<float2*>(sc + rq * kGenericPitch + it * 8 + 2 * qt) = make_float2(x0 * query.inv, x1 * query.inv);
-        }
+      if (c.term == n_terms - 1 && c.in == c.block - 1) {         // the block's sums are complete
         __syncwarp();
-        const int ngt = rows / p.G;
-        float* dst = my_row + tile * (tile_rows / p.G);
-        if (scope_ok) {
-          for (int gi = qt; gi < ngt; gi += 4) {
-            const float* s = sc + rq * kGenericPitch + gi * p.G;
-            float m = s[0];
-            for (int i = 1; i < p.G; ++i) m = fmaxf(m, s[i]);
-            publish(dst + gi, m);
-          }
-        }
-      } else {
-        float* s = sc + c.in * tile_rows;
-        for (int it = 0; it * 8 < rows; ++it) {
-          float x0, x1;
-          score_rows8<META, R>(base + uint32_t(it) * 8u * kRowBytes, query, &x0, &x1);
-          const int i = it * 8 + 2 * qt;                           // (a tile's rows need not be whole reads)
-          if (rq == 0 && i < rows) s[i] = (c.term == 0 ? 0.f : s[i]) + x0 * query.inv;
-          if (rq == 0 && i + 1 < rows) s[i + 1] = (c.term == 0 ? 0.f : s[i + 1]) + x1 * query.inv;
-        }
-        if (c.term == n_terms - 1 && c.in == c.block - 1) {         // the block's sums are complete
-          __syncwarp();
-          const int n_groups = (min((c.tile + c.block) * tile_rows, rows_total) - c.tile * tile_rows) / p.G;
-          float* dst = my_row + c.tile * (tile_rows / p.G);
-          for (int gi = lane; gi < n_groups; gi += 32) {
-            const float* t = sc + gi * p.G;
-            float m = t[0];
-            for (int i = 1; i < p.G; ++i) m = fmaxf(m, t[i]);
-            publish(dst + gi, m);
-          }
+        const int n_groups = (min((c.tile + c.block) * tile_rows, rows_total) - c.tile * tile_rows) / p.G;
+        float* dst = my_row + c.tile * (tile_rows / p.G);
+        for (int gi = lane; gi < n_groups; gi += 32) {
+          const float* t = sc + gi * p.G;
+          float m = t[0];
+          for (int i = 1; i < p.G; ++i) m = fmaxf(m, t[i]);
+          publish(dst + gi, m);
         }
       }
     }

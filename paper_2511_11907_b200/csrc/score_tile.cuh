@@ -179,4 +179,85 @@ __device__ __forceinline__ void score_rows8(uint32_t addr, const ScoreQuery<META
   *x1 = d[1] + d[3];
 }
 
+// ReduceMax over the groups of one staged tile of `rows` rows (a multiple of G); `base` = stage +
+// score_lane_offset().  Every finished group goes to publish(group within the tile, score) in exactly one lane,
+// the lane of its scope (lane / 4), if `scope_ok`.  GS = log2 G: the maximum is a max over two registers and at
+// most two shuffles.  GS = -1: any G, through the warp's buffer `sc` [8 scopes][kGenericPitch].
+constexpr int kGenericRows = 48;                          // GS = -1: token rows per tile, at most
+constexpr int kGenericPitch = 56;                         // floats between scopes of the buffer (bank spread)
+
+template <int META, int R, int GS, int STAGE_ROWS, typename Publish>
+__device__ __forceinline__ void score_tile_groups(uint32_t base, int rows, int lane, const ScoreQuery<META, R>& query,
+                                                  int G, bool scope_ok, float* sc, const Publish& publish) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  constexpr int kRowBytes = MetaRows<META, R>::kRowBytes;
+  const int rq = lane >> 2, qt = lane & 3;
+  if constexpr (GS >= 0) {
+    const int ngt = rows >> GS;                       // groups in this tile
+    float mine[(STAGE_ROWS + 31) / 32] = {};          // G = 8: the groups of reads qt, qt + 4, .. are this lane's to publish
+    float run = -INFINITY;                            // running maximum of a 16- or 32-row group
+#pragma unroll
+    for (int it = 0; it < STAGE_ROWS / 8; ++it) {
+      if (it * 8 < rows) {
+        float x0, x1;
+        score_rows8<META, R>(base + uint32_t(it) * 8u * kRowBytes, query, &x0, &x1);
+        if constexpr (GS == 0) {                                   // tokens 2t and 2t+1 of this read are groups
+          if (scope_ok && it * 8 + 2 * qt < rows) publish(it * 8 + 2 * qt, x0 * query.inv);
+          if (scope_ok && it * 8 + 2 * qt + 1 < rows) publish(it * 8 + 2 * qt + 1, x1 * query.inv);
+        } else {
+          float m = fmaxf(x0, x1);
+          if constexpr (GS >= 2) m = fmaxf(m, __shfl_xor_sync(kAll, m, 1));
+          if constexpr (GS >= 3) m = fmaxf(m, __shfl_xor_sync(kAll, m, 2));
+          // (a ragged last tile holds a whole number of groups, but not of 8-row reads when G < 8)
+          if constexpr (GS == 1) { if (scope_ok && it * 4 + qt < ngt) publish(it * 4 + qt, m * query.inv); }
+          else if constexpr (GS == 2) {
+            if (scope_ok && (qt & 1) == 0 && it * 2 + (qt >> 1) < ngt) publish(it * 2 + (qt >> 1), m * query.inv);
+          }
+          else if constexpr (GS == 3) { if (qt == (it & 3)) mine[it >> 2] = m; }
+          else {                                                   // G = 16 or 32: 2 or 4 reads per group
+            run = fmaxf(run, m);
+            if (((it + 1) & ((1 << (GS - 3)) - 1)) == 0) {
+              const int gi = it >> (GS - 3);
+              if (scope_ok && qt == (gi & 3)) publish(gi, run * query.inv);
+              run = -INFINITY;
+            }
+          }
+        }
+      }
+    }
+    if constexpr (GS == 3) {
+#pragma unroll
+      for (int h = 0; h < (STAGE_ROWS + 31) / 32; ++h)
+        if (scope_ok && (4 * h + qt) * 8 < rows) publish(4 * h + qt, mine[h] * query.inv);
+    }
+  } else {
+#pragma unroll 2
+    for (int it = 0; it * 8 < rows; ++it) {
+      float x0, x1;
+      score_rows8<META, R>(base + uint32_t(it) * 8u * kRowBytes, query, &x0, &x1);
+      *reinterpret_cast<float2*>(sc + rq * kGenericPitch + it * 8 + 2 * qt) = make_float2(x0 * query.inv, x1 * query.inv);
+    }
+    __syncwarp();
+    const int ngt = rows / G;
+    if (scope_ok) {
+      for (int gi = qt; gi < ngt; gi += 4) {
+        const float* s = sc + rq * kGenericPitch + gi * G;
+        float m = s[0];
+        for (int i = 1; i < G; ++i) m = fmaxf(m, s[i]);
+        publish(gi, m);
+      }
+    }
+  }
+}
+
+// Rows of one stage: 4 KB where a finished score leaves the registers (the hand-over of a stage costs the
+// same whatever its size: 4 KB x 2 stages measured 1.3 us per layer faster than 2 KB x 4 at B = 4,
+// N = 131072); GS = -1 takes 3 KB, which leaves room for the warps' score buffers.
+template <int META, int R, int GS>
+struct ScoreStage {
+  static constexpr int kBytes = GS >= 0 ? 4096 : 3072;
+  static constexpr int kFit = kBytes / MetaRows<META, R>::kRowBytes;
+  static constexpr int kRows = GS >= 0 ? kFit : (kFit < kGenericRows ? kFit : kGenericRows);
+};
+
 }  // namespace kvswap

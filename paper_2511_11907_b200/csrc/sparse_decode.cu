@@ -26,6 +26,7 @@
 #include <cstdint>
 
 #include "async_copy.cuh"
+#include "cluster.cuh"
 #include "combine.cuh"
 #include "common.cuh"
 
@@ -405,12 +406,16 @@ struct TokenSource {
   __device__ __forceinline__ int group_of(int v) const { return g_shift >= 0 ? (v >> g_shift) : (v / G); }
 };
 
-template <typename KV_T, typename Q_T, int D, int RH, typename Engine>
+// MERGE: the splits of a list are the CTAs of one cluster, which merges them itself (`partial` is not used).  A
+// variant of its own: with a branch at run time instead the other kernel took 0.4 us longer (25.6 against 26.0 us
+// at B = 4, 8 x 8192 tokens attended).
+template <typename KV_T, typename Q_T, int D, int RH, typename Engine, bool MERGE>
 __global__ void __launch_bounds__(kThreads, 2)
 sparse_decode_splitk_kernel(Problem p, const Q_T* __restrict__ q, const KV_T* __restrict__ K,
                             const KV_T* __restrict__ V, const int32_t* __restrict__ group_idx,
                             const int32_t* __restrict__ n_selected, float* __restrict__ partial,
-                            int splits, int depth, int g_shift, uint32_t* __restrict__ err) {
+                            float* __restrict__ out, float* __restrict__ lse, int splits, int depth, int g_shift,
+                            uint32_t* __restrict__ err) {
   constexpr uint32_t ROWB = D * sizeof(KV_T);                  // bytes of one K or V row
   constexpr uint32_t HALFB = kTok * ROWB;                      // K (or V) part of a stage
   constexpr uint32_t STAGEB = 2 * HALFB;
@@ -558,6 +563,9 @@ sparse_decode_splitk_kernel(Problem p, const Q_T* __restrict__ q, const KV_T* __
   eng.store(sm_m + warp * 8, sm_l + warp * 8, sm_acc + warp * RH * D);
   __syncthreads();
   if (settled && !wait_early) pdl_wait();
+  // partial [RH][D + 2] = (m, l, acc[D]) of this split: to the caller's scratch for the combine pass, or, when
+  // the splits of a list are the CTAs of one cluster, to shared memory for the merge below
+  float* const sm_part = sm_acc + kWarps * RH * D;
   for (int i = threadIdx.x; i < RH * D; i += kThreads) {
     const int hh = i / D, c = i % D;
     float mx = -INFINITY;
@@ -572,9 +580,54 @@ sparse_decode_splitk_kernel(Problem p, const Q_T* __restrict__ q, const KV_T* __
         a = fmaf(sm_acc[(k * RH + hh) * D + c], w, a);
       }
     }
-    float* dst = partial + ((int64_t(b) * p.Hq + h0 + hh) * splits + split) * (D + 2);
+    float* dst = MERGE ? sm_part + hh * (D + 2) : partial + ((int64_t(b) * p.Hq + h0 + hh) * splits + split) * (D + 2);
     if (c == 0) { dst[0] = mx; dst[1] = lsum; }
     dst[2 + c] = a;
+  }
+  if constexpr (MERGE) {
+
+  // ---- merge of the splits through the cluster's shared memory: every CTA writes a share of the outputs, with
+  // the weights and the order of combine_row() (combine.cuh): the same bits --------------------------------------
+  cluster_arrive();
+  cluster_wait();                                  // every split's partial is in place
+  float* const w_s = sm_m;                         // [RH][kMaxClusterCtas] weights of the splits, then [RH][2] (1 / sum, lse)
+  float* const norm_s = w_s + RH * kMaxClusterCtas;
+  static_assert(RH * (kMaxClusterCtas + 2) <= 2 * kWarps * 8 + kWarps * RH * D, "fits before sm_part");
+  const uint32_t part_addr = smem_addr(sm_part);
+  if (warp < RH) {
+    const bool have = lane < splits;
+    const uint32_t src_addr = cluster_map(part_addr, uint32_t(have ? lane : 0)) + uint32_t(warp) * (D + 2) * 4u;
+    const float m_s = have ? cluster_load(src_addr) : -INFINITY, l_s = have ? cluster_load(src_addr + 4u) : 0.f;
+    float mx = m_s;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, off));
+    const float w = (have && mx > -INFINITY) ? exp2f(m_s - mx) : 0.f;
+    float lsum = fmaf(l_s, w, 0.f);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) lsum += __shfl_xor_sync(kFull, lsum, off);
+    if (have) w_s[warp * kMaxClusterCtas + lane] = w;
+    if (lane == 0) {
+      norm_s[warp * 2] = (lsum > 0.f) ? 1.f / lsum : 0.f;
+      norm_s[warp * 2 + 1] = (lsum > 0.f) ? (mx + log2f(lsum)) * kLn2 : -INFINITY;
+    }
+  }
+  __syncthreads();
+  const int share = (RH * D + splits - 1) / splits;
+  for (int i = split * share + threadIdx.x; i < min(RH * D, (split + 1) * share); i += kThreads) {
+    const int hh = i / D, c = i % D;
+    const uint32_t src_addr = part_addr + uint32_t(hh * (D + 2) + 2 + c) * 4u;
+    float v[kMaxClusterCtas];
+#pragma unroll
+    for (int s = 0; s < kMaxClusterCtas; ++s) v[s] = (s < splits) ? cluster_load(cluster_map(src_addr, uint32_t(s))) : 0.f;
+    float a = 0.f;
+#pragma unroll
+    for (int s = 0; s < kMaxClusterCtas; ++s) if (s < splits) a = fmaf(v[s], w_s[hh * kMaxClusterCtas + s], a);
+    const int64_t row = int64_t(b) * p.Hq + h0 + hh;
+    out[row * D + c] = a * norm_s[hh * 2];
+    if (lse != nullptr && c == 0) lse[row] = norm_s[hh * 2 + 1];
+  }
+  cluster_arrive();
+  cluster_wait();                                  // no CTA leaves while a peer may still read its partial
   }
 }
 
@@ -607,12 +660,22 @@ cudaError_t launch_one(const Problem& p, const Workspace& w, const void* q, cons
   constexpr bool kMma = sizeof(KV_T) == 2 && std::is_same<KV_T, Q_T>::value;
   using Engine = typename std::conditional<kMma, MmaEngine<KV_T, KV_T, D, RH>, AluEngine<KV_T, Q_T, D, (RH <= 4 ? RH : 4)>>::type;
   if (!kMma && RH > 4) return cudaErrorInvalidValue;             // never planned: see plan_sparse_decode
-  auto kern = sparse_decode_splitk_kernel<KV_T, Q_T, D, RH, Engine>;
+  const dim3 grid(w.splits, p.Hkv * (p.rho / RH), p.B);
+  const Q_T* qt = static_cast<const Q_T*>(q);
+  const KV_T* Kt = static_cast<const KV_T*>(K);
+  const KV_T* Vt = static_cast<const KV_T*>(V);
+  if (combine && w.merge_in_cluster) {
+    auto kern = sparse_decode_splitk_kernel<KV_T, Q_T, D, RH, Engine, true>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    return launch_pdl_cluster(kern, w.splits, grid, dim3(kThreads), smem, st, p, qt, Kt, Vt, group_idx, n_selected,
+                              static_cast<float*>(nullptr), out, lse, w.splits, depth, g_shift, err);
+  }
+  auto kern = sparse_decode_splitk_kernel<KV_T, Q_T, D, RH, Engine, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  e = launch_pdl(kern, dim3(w.splits, p.Hkv * (p.rho / RH), p.B), dim3(kThreads), smem, st, p,
-                 static_cast<const Q_T*>(q), static_cast<const KV_T*>(K), static_cast<const KV_T*>(V), group_idx,
-                 n_selected, partial, w.splits, depth, g_shift, err);
+  e = launch_pdl(kern, grid, dim3(kThreads), smem, st, p, qt, Kt, Vt, group_idx, n_selected, partial, out, lse, w.splits,
+                 depth, g_shift, err);
   if (e != cudaSuccess || !combine) return e;
   return launch_pdl(combine_kernel<D>, dim3(p.B * p.Hq), dim3(D), 0, st, static_cast<const float*>(partial), out,
                     lse, w.splits);
@@ -667,14 +730,44 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
   // Cost of a split factor s, in chunk times of the slowest CTA: waves * (chunks per CTA + the
   // fixed part of a CTA -- first index fetch, first rows, merge -- worth about 14 chunks), with
   // 2 CTAs per SM resident; at least two chunks per warp and split.
-  const int64_t slots = int64_t(kNumSMs) * 2;
-  const int64_t max_splits = std::min<int64_t>(256, std::max<int64_t>(1, n_chunks / (2 * kWarps)));
-  int64_t best = 1, best_cost = INT64_MAX;
-  for (int64_t s = 1; s <= max_splits; ++s) {
-    const int64_t waves = (problems * s + slots - 1) / slots;
-    if (waves > 2 && s > 1) break;
-    const int64_t cost = waves * ((n_chunks + s - 1) / s + 14);
-    if (cost < best_cost) { best_cost = cost; best = s; }
+  auto split_cost = [&](int64_t s, int64_t slots) {
+    return (problems * s + slots - 1) / slots * ((n_chunks + s - 1) / s + 14);
+  };
+  auto best_splits = [&](int64_t slots, int64_t limit) {
+    const int64_t max_splits = std::min<int64_t>(limit, std::max<int64_t>(1, n_chunks / (2 * kWarps)));
+    int64_t best = 1;
+    for (int64_t s = 2; s <= max_splits && problems * s <= 2 * slots; ++s)
+      if (split_cost(s, slots) < split_cost(best, slots)) best = s;
+    return best;
+  };
+  const int64_t slots = 2 * kNumSMs;
+  int64_t best = best_splits(slots, 256);
+  w->merge_in_cluster = false;
+  w->splits_room = int(best);
+  ClusterGrid predictor;
+  if (score_select_cluster_grid(p, &predictor)) {
+    // A short context, whose predictor is one launch of clusters: here the splits of a list form a cluster of at
+    // most 8 that merges them, which saves the combine launch and lets attention and predictor run side by
+    // side.  The largest cluster is taken whose lists all fit beside the next layer's predictor (a GPC has some
+    // 36 slots for these CTAs, and a cluster stays in one GPC).  At B = 4, N = 4096, M = 128: clusters of 6
+    // 11.8 us per layer, of 8 (256 CTAs, which do not fit) 15.3, the chain of three kernels 13.6.
+    constexpr int kGpcs = 8, kGpcSlots = 35;
+    const int64_t most = std::min<int64_t>(8, std::max<int64_t>(1, n_chunks / (2 * kWarps)));
+    int64_t m = 0;
+    for (int64_t s = most; s >= 1 && m == 0; --s) {
+      int64_t fit = 0;
+      for (int gpc = 0; gpc < kGpcs; ++gpc) {
+        const int held = (predictor.clusters + gpc) / kGpcs * predictor.ctas * (predictor.whole_sm ? 2 : 1);
+        fit += std::max(0, kGpcSlots - held) / s;
+      }
+      if (problems <= fit && problems * s <= 200) m = s;
+    }
+    if (m < 2 && most >= 2 && problems * 2 <= 264) m = 2;      // pairs find room anywhere
+    // What fewer splits cost must stay below what the two launches cost (about 16 chunk times).
+    if (m > 0 && split_cost(m, slots) - split_cost(best, slots) <= 16) {
+      best = m;
+      w->merge_in_cluster = true;
+    }
   }
   w->splits = int(best);
   const size_t row = size_t(p.d) * (p.kv_dtype == KVSWAP_F32 ? 4 : 2);

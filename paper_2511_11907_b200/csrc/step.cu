@@ -251,6 +251,36 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
       if (next && probed(l + 1)) ev(probe_opt->ev_mid);
       return KVSWAP_OK;
     };
+    // Short contexts: the predictor of a layer is one launch of clusters and so is its attention (the splits
+    // merge in the cluster), and the two run side by side:
+    //   predict(0) | predict(1) attention(0) | predict(2) attention(1) | ..
+    // predict(l + 1) waits for attention(l - 1) and only then lets attention(l) start, which finds the selection
+    // of predict(l) complete: attention(l - 1) waited for it before it wrote its results.  Two launches a layer
+    // instead of three, and neither waits for the other: 36 layers of B = 1, N = 16384, 8 KV heads, M = 256 through
+    // host memory 539 -> 430 us; at B = 1, N = 4096 a layer takes 8.5 us against 12.9.
+    if (score_select_cluster_supported(p) && w.merge_in_cluster) {
+      auto predict = [&](int l) -> int {
+        if (probed(l)) ev(probe_opt->ev_begin);
+        const cudaError_t e = launch_score_select_cluster(
+            p_settled, static_cast<const char*>(q) + size_t(l) * q_bytes, layers->proj[l], layers->meta[l], nullptr,
+            group_idx + size_t(l) * idx_elems, n_selected + size_t(l) * nsel_elems, static_cast<uint32_t*>(ws), stream);
+        if (probed(l)) ev(probe_opt->ev_mid);
+        return e == cudaSuccess ? KVSWAP_OK : KVSWAP_ERR_CUDA;
+      };
+      int status = predict(0);
+      for (int l = 0; l < L && status == KVSWAP_OK; ++l) {
+        if (l + 1 < L) status = predict(l + 1);
+        if (status != KVSWAP_OK) break;
+        // (the last layer's attention follows an attention directly: its selection is complete when that one is)
+        const cudaError_t e = launch_sparse_decode(
+            l + 1 < L ? p_settled : p, w, static_cast<const char*>(q) + size_t(l) * q_bytes, layers->K[l], layers->V[l],
+            group_idx + size_t(l) * idx_elems, n_selected + size_t(l) * nsel_elems, nullptr, out + size_t(l) * out_elems,
+            lse_opt ? lse_opt + size_t(l) * p.B * p.Hq : nullptr, static_cast<uint32_t*>(ws), stream);
+        if (probed(l)) ev(probe_opt->ev_end);
+        if (e != cudaSuccess) status = KVSWAP_ERR_CUDA;
+      }
+      return status;
+    }
     int status = score(0);
     if (status == KVSWAP_OK) status = select(0);
     for (int l = 0; l < L && status == KVSWAP_OK; ++l) {

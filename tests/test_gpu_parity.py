@@ -455,10 +455,18 @@ STREAM = [   # K/V type, metadata type, rank, G, per-head, scope, B, H_kv, rho, 
 ]
 
 
+@pytest.mark.parametrize("wide", [False, True])
 @pytest.mark.parametrize("kv_type,meta,rank,G,per_head,scope,B,Hkv,rho,N", STREAM)
-def test_streaming_scorer_shapes(kv_type, meta, rank, G, per_head, scope, B, Hkv, rho, N):
-    """The predictor over every stored type and rank of the streaming scorer: groups that leave the registers and groups
-    that go through the warp's buffer, one term per score and one per metadata head, ragged last tiles."""
+def test_streaming_scorer_shapes(kv_type, meta, rank, G, per_head, scope, B, Hkv, rho, N, wide):
+    """The predictor over every stored type and rank of the tensor-core scorers: groups that leave the registers and groups
+    that go through the warp's buffer, one term per score and one per metadata head, ragged last tiles.  The short
+    contexts are scored and selected by one cluster per sequence; `wide`, so many sequences that the clusters would
+    not fit side by side, sends the same rows to the streaming kernel."""
+    if wide:
+        if N > 10000:
+            pytest.skip("streamed already")
+        ns = 1 if scope == ALL or per_head else min(8, Hkv)
+        B, N = 300 // (Hkv if per_head and scope == KV else 1) // ns + 1, min(N, 640 + N % 64)
     wl = small("stream", batch=B, n_ctx=N, n_q_heads=Hkv * rho, n_kv_heads=Hkv, rank=rank, group_size=G,
                top_k=max(1, min(N // G // 3, 500)), kv_dtype=kv_type, q_dtype=kv_type, meta_dtype=meta,
                calib_rows=max(512, Hkv * 64))
@@ -476,6 +484,23 @@ def test_streaming_scorer_shapes(kv_type, meta, rank, G, per_head, scope, B, Hkv
     idx2, nsel2, _ = dl.score_select(with_scores=False)
     assert np.array_equal(idx, idx2) and np.array_equal(nsel, nsel2)
     assert kv.kvswap_read_device_status(dl.ws) == 0
+
+
+@pytest.mark.parametrize("kind", ["equal", "two_values", "outlier", "tiny_spread"])
+@pytest.mark.parametrize("NG,M", [(1030, 400), (4096, 1), (700, 699)])
+def test_select_of_degenerate_scores(kind, NG, M):
+    """The cluster's select counts scores in bins of equal width over their range: scores that all fall into one bin
+    (equal ones, a far outlier) or have hardly any range; always exactly the top M, lower index first."""
+    wl = small("degenerate", batch=1, n_ctx=NG, group_size=1, top_k=M, n_q_heads=2, n_kv_heads=2)
+    li = W.make_layer(wl, 0, 1)
+    dl = DeviceLayer(li, KV)
+    rng = np.random.default_rng(NG + M)
+    meta = np.zeros((1, 1, NG, wl.rank), dtype=np.float32)
+    meta[..., 0] = {"equal": np.ones(NG), "two_values": rng.integers(0, 2, NG), "tiny_spread": 1 + rng.integers(0, 9, NG) * 2.0 ** -23,
+                    "outlier": np.where(np.arange(NG) == NG // 2, 1e30, rng.standard_normal(NG))}[kind]
+    dl.set_meta(meta)
+    idx, nsel, Rg = dl.score_select()
+    assert np.all(nsel == M) and np.array_equal(idx, O.select(Rg.astype(np.float64), M))
 
 
 def test_strided_kv_and_metadata_views():
