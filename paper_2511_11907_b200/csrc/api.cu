@@ -89,11 +89,12 @@ static bool hist_capable(const Problem& p) {
 // The scorer counts the leading digit of every group score's key and the TopK starts from those
 // counts (several CTAs per problem) where both kernels have that path.
 static bool counts_top_digit(const Problem& p) {
-  return !(p.flags & KVSWAP_SCORE_SOFTMAX) && hist_capable(p) && score_stream_counts_top_digit(p) && topk_parts_supported(p);
+  const bool counts = (p.flags & KVSWAP_SCORE_SOFTMAX) ? score_softmax_tc_counts(p) : score_stream_counts_top_digit(p);
+  return counts && hist_capable(p) && topk_parts_supported(p);
 }
 
 bool select_merges_with_combine(const Problem& p) {
-  return p.NG > 0 && score_stream_supported(p) && counts_top_digit(p);
+  return p.NG > 0 && counts_top_digit(p);
 }
 
 bool query_ahead_supported(const Problem& p) {
@@ -146,7 +147,9 @@ cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q,
   p.score_pitch = group_scores_opt ? p.NG : workspace_score_pitch(p);     // a caller's buffer is dense [B, S, NG]
   if (p.flags & KVSWAP_SCORE_SOFTMAX) {
     float* u_heads = reinterpret_cast<float*>(base + w.off_softmax);
-    return launch_score_softmax(p, q, proj, meta, u_heads, u_heads + size_t(p.B) * p.Hq * p.r, scores, stream);
+    uint32_t* top_hist = counts_top_digit(p) ? reinterpret_cast<uint32_t*>(base + w.off_hist) : nullptr;
+    return launch_score_softmax(p, q, proj, meta, u_heads, u_heads + size_t(p.B) * p.Hq * p.r, scores, top_hist,
+                                static_cast<uint32_t*>(ws), stream);
   }
   if (p.NG < 1) return cudaSuccess;                                       // nothing to score
   if (score_stream_supported(p)) {
@@ -174,7 +177,7 @@ cudaError_t select_launch(const Problem& p_in, const Workspace& w, int32_t* grou
   float* scores = group_scores_opt ? group_scores_opt : reinterpret_cast<float*>(base + w.off_scores);
   Problem p = p_in;
   p.score_pitch = group_scores_opt ? p.NG : workspace_score_pitch(p);
-  if (p.NG > 0 && score_stream_supported(p) && counts_top_digit(p))
+  if (p.NG > 0 && counts_top_digit(p))
     return launch_topk_parts(p, scores, reinterpret_cast<uint32_t*>(base + w.off_hist), group_idx, n_selected, stream);
   return launch_topk_select(p, scores, group_idx, n_selected, stream);
 }

@@ -75,7 +75,11 @@ cudaError_t launch_flush_rows(const Problem& p, const void* const* K_fast, const
 int score_softmax_chunks(const Problem& p);
 bool score_softmax_supported(const Problem& p);
 cudaError_t launch_score_softmax(const Problem& p, const void* q, const float* proj, const void* meta, float* u,
-                                 float* stats, float* scores, cudaStream_t st);
+                                 float* stats, float* scores, uint32_t* top_hist, uint32_t* err, cudaStream_t st);
+bool score_softmax_tc_supported(const Problem& p);
+bool score_softmax_tc_counts(const Problem& p);   // it counts leading digits into top_hist as the streaming scorer does
+cudaError_t launch_score_softmax_tc(const Problem& p, const void* meta, const float* u, float* stats, float* scores,
+                                    uint32_t* top_hist, uint32_t* err, cudaStream_t st);
 // Reuse buffer (reuse_buffer.cu).
 bool reuse_supported(const Problem& p, int n_slots, int max_groups);
 size_t reuse_state_words(const Problem& p, int n_slots, int max_groups);

@@ -122,3 +122,23 @@ def _tc(**kw):
 ], ids=lambda x: x if isinstance(x, str) else None)
 def test_softmax_variant_tensor_core_shapes(name, wl, scope):
     _check(wl, 1, scope)
+
+
+@pytest.mark.parametrize("mh,scope,kw", [
+    (1, KV, dict(rank=16, n_ctx=48 * 33 + 9)),
+    (1, KV, dict(rank=64, group_size=32, n_ctx=32 * 41 + 31, n_q_heads=64, n_kv_heads=8)),     # a group longer than the usual stage
+    (1, ALL, dict(rank=64, n_ctx=24 * 50 + 8)),
+    (1, KV, dict(rank=16, meta_dtype=W.F32, kv_dtype=W.F32, q_dtype=W.F32, n_q_heads=6, n_kv_heads=2, n_ctx=1999)),
+    (1, ALL, dict(rank=32, meta_dtype=W.F32, n_q_heads=40, n_kv_heads=10, group_size=5)),
+    (0, KV, dict(n_q_heads=24, n_kv_heads=8, n_ctx=1801)),
+    (0, KV, dict(n_q_heads=24, n_kv_heads=2, group_size=4, rank=64)),                            # 12 heads per sum: two blocks
+    (0, ALL, dict(n_q_heads=16, n_kv_heads=4, group_size=12, n_ctx=12 * 170 + 3)),
+    (0, ALL, dict(n_q_heads=24, n_kv_heads=2, rank=16, batch=1, n_ctx=90003, top_k=300)),        # blocks of tiles, head by head
+    (1, KV, dict(n_q_heads=20, n_kv_heads=10, n_ctx=70005, batch=1, top_k=500)),                 # two scope blocks, several tiles per warp
+    (1, KV, dict(group_size=64, n_ctx=64 * 30 + 5)),                                             # groups longer than a tile
+    (0, ALL, dict(group_size=50, n_ctx=50 * 41, n_kv_heads=2)),
+    (1, KV, dict(batch=160, n_ctx=200, top_k=5)),                                                # more row sets than SMs
+])
+def test_softmax_variant_rows_scopes_and_groups(mh, scope, kw):
+    wl = _tc(**kw)
+    _check(wl, 1 if mh else wl.n_kv_heads, scope)
