@@ -9,6 +9,8 @@
 //                             already isolates a few hundred candidates and later passes touch
 //                             only those; stops as soon as a digit bin is taken whole.
 //   topk_select_kernel        longer rows: keys in shared memory (or re-read), 8-bit digits.
+#include <algorithm>
+
 #include "async_copy.cuh"
 #include "combine.cuh"
 #include "lowrank_query.cuh"
@@ -362,17 +364,26 @@ cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_
                                   cudaStream_t st) {
   const int P = plan_topk_parts(p);
   if (P == 0 || (d != 64 && d != 128) || splits > kMaxSplits) return cudaErrorInvalidValue;
+  // Query sets of the launch: the scorer's row sets, except that the KV heads of per-head metadata are taken eight at a
+  // time like the scopes of joint metadata (a row's sum is the same; one head at a time used 4 of the CTA's 32 warps:
+  // 20.6 us per launch at B = 4, 8 heads).  With fewer combine CTAs than sets, CTAs for queries alone are added.
   int n_rests = 0, n_sub = 1;
+  Problem pq = p;
   if (q_ahead != nullptr) {
     if (!score_stream_fuses_query(p) || proj_ahead == nullptr || uq_ahead == nullptr) return cudaErrorInvalidValue;
     score_stream_row_sets(p, &n_rests, &n_sub);
+    if (p.Hm != 1 && p.scope == KVSWAP_SCOPE_KV_HEAD) {
+      pq.Hm = 1;
+      n_sub = (p.Hkv + kQueryCols - 1) / kQueryCols;
+      n_rests = p.B * n_sub;
+    }
   }
   const int n_probs = p.B * p.S;
   const int rows_per_cta = (d == 128) ? kCombineRows<128> : kCombineRows<64>;
-  const int n_comb = (n_rows + rows_per_cta - 1) / rows_per_cta;
+  const int n_comb = std::max((n_rows + rows_per_cta - 1) / rows_per_cta, std::min(n_rests, 32));
   const dim3 grid(n_comb + P * n_probs), block(kPartThreads);
   auto go = [&](auto kern) {
-    return launch_pdl(kern, grid, block, 0, st, p, scores, top_hist, group_idx, n_selected, n_probs, partial, out, lse,
+    return launch_pdl(kern, grid, block, 0, st, pq, scores, top_hist, group_idx, n_selected, n_probs, partial, out, lse,
                       splits, n_rows, n_comb, q_ahead, proj_ahead, uq_ahead, n_rests, n_sub);
   };
   auto by_parts = [&](auto d_tag) {
