@@ -314,61 +314,106 @@ bool try_launch_mma(const Problem& p, const void* K, const float* proj, void* me
   return true;
 }
 
-// A handful of tokens (one flushed group, for every layer): one CTA per (token, sequence, metadata
-// head, layer).  Eight slices of the contraction index x 32 output columns; every thread keeps up
-// to eight columns (r <= 256); the slices are summed through shared memory in a fixed order.
+// A handful of tokens (one flushed group, for every layer): one CTA per (eight tokens, sequence, metadata head,
+// layer).  The rows of K are staged in shared memory, [channel][token]; a warp takes a sixteenth of every head's
+// channels and reads each adapter row once for all eight tokens (a lane holds columns lane, lane + 32, ..); the
+// warps' sums are added through shared memory in a fixed order.  Bound by the adapter's trip from L2: a CTA per
+// token, which this replaces, read it eight times as often and took 54 us for 12 layers of 8 sequences (8 heads of
+// 128, r = 32, G = 8), this one 11.
 constexpr int kGroupTokens = 64;              // token ranges up to this length take this kernel
+constexpr int kGroupTile = 8;                 // tokens per CTA
+constexpr int kGroupWarps = 16;
 
-template <typename KV_T, typename META_T>
-__global__ void __launch_bounds__(256)
-project_group_kernel(Problem p, const ProjectTable tab, int n_begin, int n_tokens) {
-  __shared__ float part_sum[8][256];
-  const int layer = blockIdx.x / n_tokens, n = n_begin + blockIdx.x % n_tokens;
+template <typename KV_T, typename META_T, int RC>   // RC = ceil(r / 32) columns per lane
+__global__ void __launch_bounds__(kGroupWarps * 32)
+project_group_kernel(Problem p, const ProjectTable tab, int n_begin, int n_tokens, int tiles) {
+  extern __shared__ __align__(16) float k_s[];       // [heads of the sum * d][kGroupTile]
+  __shared__ float part_sum[kGroupWarps][kGroupTile][32];
+  const int layer = blockIdx.x / tiles, t0 = (blockIdx.x % tiles) * kGroupTile;
+  const int nt = min(kGroupTile, n_tokens - t0), n0 = n_begin + t0;
   const int b = blockIdx.y, head_out = blockIdx.z;
   const KV_T* __restrict__ K = static_cast<const KV_T*>(tab.K[layer]);
   const float* __restrict__ proj = tab.proj[layer];
   META_T* __restrict__ meta = static_cast<META_T*>(tab.meta[layer]);
   const int g_first = (p.Hm == 1) ? 0 : head_out;
   const int g_count = (p.Hm == 1) ? p.Hkv : 1;
-  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
-  float acc[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kPer = Elt<KV_T>::kPer16B;
+  const int row_vecs = p.d / kPer;
+  for (int i = threadIdx.x; i < g_count * kGroupTile * row_vecs; i += kGroupWarps * 32) {
+    const int t = i % kGroupTile, v = (i / kGroupTile) % row_vecs, g = i / (kGroupTile * row_vecs);
+    float f[kPer] = {};
+    if (t < nt)
+      widen16B(*reinterpret_cast<const uint4*>(K + int64_t(b) * p.kv_sb + int64_t(g_first + g) * p.kv_sh +
+                                               int64_t(n0 + t) * p.kv_sn + v * kPer), f, KV_T());
 #pragma unroll
-  for (int j = 0; j < 8; ++j) acc[j] = 0.f;
-  const int per_part = p.d / 8;                                  // d is 64 or 128
-  for (int gi = 0; gi < g_count; ++gi) {
-    const int g = g_first + gi;
-    const KV_T* row = K + int64_t(b) * p.kv_sb + int64_t(g) * p.kv_sh + int64_t(n) * p.kv_sn;
-    const float* Pg = proj + int64_t(g) * p.d * p.r;
-    for (int c = part * per_part; c < (part + 1) * per_part; ++c) {
-      const float k = float(row[c]);
+    for (int e = 0; e < kPer; ++e) k_s[(g * p.d + v * kPer + e) * kGroupTile + t] = f[e];
+  }
+  __syncthreads();
+  float acc[kGroupTile][RC];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
+  for (int t = 0; t < kGroupTile; ++t)
+#pragma unroll
+    for (int j = 0; j < RC; ++j) acc[t][j] = 0.f;
+  const int per_warp = p.d / kGroupWarps;                        // 8 or 4 channels of every head
+  for (int g = 0; g < g_count; ++g) {
+    const float* Pg = proj + (int64_t(g_first + g) * p.d + warp * per_warp) * p.r;
+    const float* kg = k_s + (g * p.d + warp * per_warp) * kGroupTile;
+#pragma unroll 4
+    for (int c = 0; c < per_warp; ++c) {
+      const float4 ka = *reinterpret_cast<const float4*>(kg + c * kGroupTile);
+      const float4 kb = *reinterpret_cast<const float4*>(kg + c * kGroupTile + 4);
+      const float k[kGroupTile] = {ka.x, ka.y, ka.z, ka.w, kb.x, kb.y, kb.z, kb.w};
+#pragma unroll
+      for (int j = 0; j < RC; ++j) {
         const int col = lane + 32 * j;
-        if (col < p.r) acc[j] = fmaf(k, Pg[int64_t(c) * p.r + col], acc[j]);
+        const float a = (col < p.r) ? Pg[int64_t(c) * p.r + col] : 0.f;
+#pragma unroll
+        for (int t = 0; t < kGroupTile; ++t) acc[t][j] = fmaf(k[t], a, acc[t][j]);
       }
     }
   }
 #pragma unroll
-  for (int j = 0; j < 8; ++j) part_sum[part][lane + 32 * j] = acc[j];
-  __syncthreads();
-  for (int col = threadIdx.x; col < p.r; col += blockDim.x) {
-    float s = 0.f;
+  for (int j = 0; j < RC; ++j) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) s += part_sum[k][col];
-    META_T* out = meta + int64_t(b) * p.meta_sb + int64_t(head_out) * p.meta_sh + int64_t(n) * p.meta_sn + col;
-    if constexpr (sizeof(META_T) == 1) out->bits = uint8_t(to_e4m3x2(s * meta_store_scale(p), 0.f) & 0xffu);
-    else if constexpr (sizeof(META_T) == 2) *out = __float2half_rn(s);
-    else *out = s;
+    for (int t = 0; t < kGroupTile; ++t) part_sum[warp][t][lane] = acc[t][j];
+    __syncthreads();
+    const int t = threadIdx.x >> 5, col = lane + 32 * j;         // warp t sums token t
+    if (t < nt && col < p.r) {
+      float s = 0.f;
+#pragma unroll
+      for (int w = 0; w < kGroupWarps; ++w) s += part_sum[w][t][lane];
+      META_T* out = meta + int64_t(b) * p.meta_sb + int64_t(head_out) * p.meta_sh + int64_t(n0 + t) * p.meta_sn + col;
+      if constexpr (sizeof(META_T) == 1) out->bits = uint8_t(to_e4m3x2(s * meta_store_scale(p), 0.f) & 0xffu);
+      else if constexpr (sizeof(META_T) == 2) *out = __float2half_rn(s);
+      else *out = s;
+    }
+    __syncthreads();
   }
 }
+
+template <typename KV_T, typename META_T, int RC>
+cudaError_t launch_group(const Problem& p, const ProjectTable& tab, int n_layers, int n_begin, int n_tokens, cudaStream_t st) {
+  const int tiles = (n_tokens + kGroupTile - 1) / kGroupTile;
+  const size_t smem = size_t(p.Hm == 1 ? p.Hkv : 1) * p.d * kGroupTile * sizeof(float);
+  auto kern = project_group_kernel<KV_T, META_T, RC>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (e != cudaSuccess) return e;
+  kern<<<dim3(tiles * n_layers, p.B, p.Hm), kGroupWarps * 32, smem, st>>>(p, tab, n_begin, n_tokens, tiles);
+  return cudaGetLastError();
+}
+constexpr size_t kGroupMaxSmem = 200 * 1024;  // staged rows; a joint adapter over more heads takes the tiled kernel
 
 template <typename KV_T, typename META_T>
 cudaError_t dispatch_rc(const Problem& p, const ProjectTable& tab, int n_layers, int n_begin, int n_end,
                         cudaStream_t st) {
-  if (n_end - n_begin <= kGroupTokens) {
-    const int n_tokens = n_end - n_begin;
-    project_group_kernel<KV_T, META_T><<<dim3(n_tokens * n_layers, p.B, p.Hm), 256, 0, st>>>(p, tab, n_begin, n_tokens);
-    return cudaGetLastError();
+  const size_t staged = size_t(p.Hm == 1 ? p.Hkv : 1) * p.d * kGroupTile * sizeof(float);
+  if (n_end - n_begin <= kGroupTokens && staged <= kGroupMaxSmem) {
+    const int n = n_end - n_begin;
+    if (p.r <= 32) return launch_group<KV_T, META_T, 1>(p, tab, n_layers, n_begin, n, st);
+    if (p.r <= 64) return launch_group<KV_T, META_T, 2>(p, tab, n_layers, n_begin, n, st);
+    if (p.r <= 128) return launch_group<KV_T, META_T, 4>(p, tab, n_layers, n_begin, n, st);
+    return launch_group<KV_T, META_T, 8>(p, tab, n_layers, n_begin, n, st);
   }
   const int tiles = (n_end - n_begin + kTok - 1) / kTok;
   dim3 grid(tiles * n_layers, p.B, p.Hm);
