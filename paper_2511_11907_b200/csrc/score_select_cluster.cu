@@ -20,10 +20,10 @@ bool plan(const Problem& p, Plan* pl) {
   int g_shift = -1;
   for (int s = 0; s <= 5; ++s) if ((1 << s) == p.G) g_shift = s;
   if (g_shift < 0 && p.meta_dtype == KVSWAP_E4M3) return false;
-  const int fit = (g_shift >= 0 ? 4096 : 3072) / (p.r * elem);
+  const int fit = score_stage_rows(g_shift < 0, p.r * elem);
   pl->g_shift = g_shift;
-  pl->tile_rows = g_shift >= 0 ? fit : std::min(fit, kGenericRows) / p.G * p.G;
-  if (pl->tile_rows < 1) return false;
+  pl->tile_rows = g_shift >= 0 ? fit : fit / p.G * p.G;
+  if (pl->tile_rows < p.G) return false;                 // a group does not fit a stage
   pl->tiles = int((int64_t(p.NG) * p.G + pl->tile_rows - 1) / pl->tile_rows);
   const int ns = (p.Hm == 1) ? std::min(kQueryCols, p.S) : 1;
   pl->n_sub = (p.Hm == 1) ? (p.S + kQueryCols - 1) / kQueryCols : 1;
@@ -80,8 +80,9 @@ cudaError_t launch_score_select_cluster(const Problem& p, const void* q, const f
                          : launch_score_select_rows<KVSWAP_F16, 64>(p, a, pl.g_shift, pl.cluster, pl.n_rests, st);
     case KVSWAP_E4M3: return launch_score_select_rows<KVSWAP_E4M3, 32>(p, a, pl.g_shift, pl.cluster, pl.n_rests, st);
     default:
-      return p.r == 16 ? launch_score_select_rows<KVSWAP_F32, 16>(p, a, pl.g_shift, pl.cluster, pl.n_rests, st)
-                       : launch_score_select_rows<KVSWAP_F32, 32>(p, a, pl.g_shift, pl.cluster, pl.n_rests, st);
+      return p.r == 16   ? launch_score_select_rows<KVSWAP_F32, 16>(p, a, pl.g_shift, pl.cluster, pl.n_rests, st)
+             : p.r == 32 ? launch_score_select_rows<KVSWAP_F32, 32>(p, a, pl.g_shift, pl.cluster, pl.n_rests, st)
+                         : launch_score_select_rows<KVSWAP_F32, 64>(p, a, pl.g_shift, pl.cluster, pl.n_rests, st);
   }
 }
 

@@ -51,7 +51,7 @@ struct ClusterSmem {
   float urow[kQueryCols * R];
   uint32_t key_min, key_max;                              // of the scope this CTA selects for
   unsigned long long full[kClusterWarps * 2];
-  float sc[GS >= 0 ? 4 : kClusterWarps * kQueryCols * kGenericPitch];
+  float sc[GS >= 0 ? 4 : kClusterWarps * kQueryCols * generic_pitch(ScoreStage<META, R, GS>::kRows)];
 };
 
 template <int META, int R, int GS>
@@ -149,7 +149,7 @@ score_select_cluster_kernel(Problem p, ClusterArgs a) {
   const uint32_t dst_keys = cluster_map(smem_addr(keys), owner);
   uint32_t key_min = 0xffffffffu, key_max = 0u;
   float* const out_row = a.scores ? a.scores + (int64_t(rs.b) * p.S + s0 + (scope_ok ? rq : 0)) * p.NG : nullptr;
-  float* const sc = sm->sc + (GS >= 0 ? 0 : warp * kQueryCols * kGenericPitch);
+  float* const sc = sm->sc + (GS >= 0 ? 0 : warp * kQueryCols * generic_pitch(kStageRows));
   bool timed_out = false;
   int stage = 0;
   uint32_t phase = 0;
@@ -216,6 +216,7 @@ template <> cudaError_t launch_score_select_rows<KVSWAP_F16, 64>(const Problem&,
 template <> cudaError_t launch_score_select_rows<KVSWAP_E4M3, 32>(const Problem&, const ClusterArgs&, int, int, int, cudaStream_t);
 template <> cudaError_t launch_score_select_rows<KVSWAP_F32, 16>(const Problem&, const ClusterArgs&, int, int, int, cudaStream_t);
 template <> cudaError_t launch_score_select_rows<KVSWAP_F32, 32>(const Problem&, const ClusterArgs&, int, int, int, cudaStream_t);
+template <> cudaError_t launch_score_select_rows<KVSWAP_F32, 64>(const Problem&, const ClusterArgs&, int, int, int, cudaStream_t);
 
 constexpr int kClusterMaxKeys = 16384;                  // keys of one scope in the selecting CTA's shared memory
 

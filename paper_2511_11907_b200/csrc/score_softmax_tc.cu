@@ -16,7 +16,8 @@ auto by_rows(const Problem& p, F&& f) {
     return f(std::integral_constant<int, KVSWAP_F16>(), std::integral_constant<int, 64>());
   }
   if (p.r == 16) return f(std::integral_constant<int, KVSWAP_F32>(), std::integral_constant<int, 16>());
-  return f(std::integral_constant<int, KVSWAP_F32>(), std::integral_constant<int, 32>());
+  if (p.r == 32) return f(std::integral_constant<int, KVSWAP_F32>(), std::integral_constant<int, 32>());
+  return f(std::integral_constant<int, KVSWAP_F32>(), std::integral_constant<int, 64>());
 }
 
 // Launch plans of the statistics (pool = false) and the pooling kernel; false: the shape is not taken.

@@ -1,5 +1,5 @@
 // Softmax variant of the scorer on the tensor cores (KVSWAP_SCORE_SOFTMAX; what it computes: score_softmax.cu)
-// for metadata rows that are dense in memory, fp16 of rank 16, 32 or 64 or fp32 of rank 16 or 32.
+// for metadata rows that are dense in memory, fp16 or fp32 of rank 16, 32 or 64.
 //
 //   softmax_tc_stats_kernel  per head the running maximum and sum of 2^(logit - max) over a share of the tokens
 //   softmax_tc_pool_kernel   the logits again (the rows now come from L2), weights, sum over the heads of a scope,

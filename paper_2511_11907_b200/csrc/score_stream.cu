@@ -26,9 +26,9 @@ bool plan(const Problem& p, Plan* pl) {
   if (multi_term(p)) g_shift = -1;
   // E4M3 metadata is offered for groups of a power of two and one term per score only
   if (g_shift < 0 && p.meta_dtype == KVSWAP_E4M3) return false;
-  const int fit = (g_shift >= 0 ? 4096 : 3072) / (p.r * elem);
-  const int tile_rows = g_shift >= 0 ? fit : std::min(fit, kGenericRows) / p.G * p.G;
-  if (tile_rows < 1) return false;                        // a group does not fit a stage
+  const int fit = score_stage_rows(g_shift < 0, p.r * elem);
+  const int tile_rows = g_shift >= 0 ? fit : fit / p.G * p.G;
+  if (tile_rows < p.G) return false;                      // a group does not fit a stage
   const int64_t rows_total = int64_t(p.NG) * p.G;
   const int64_t tiles_per_row = (rows_total + tile_rows - 1) / tile_rows;
   const int n_sub = (p.Hm == 1) ? (p.S + kScoreCols - 1) / kScoreCols : 1;
@@ -68,7 +68,7 @@ bool score_stream_rows(const Problem& p) {
   switch (p.meta_dtype) {
     case KVSWAP_F16: return p.r == 16 || p.r == 32 || p.r == 64;
     case KVSWAP_E4M3: return p.r == 32;
-    default: return p.r == 16 || p.r == 32;
+    default: return p.r == 16 || p.r == 32 || p.r == 64;
   }
 }
 bool score_stream_supported(const Problem& p) { Plan pl; return plan(p, &pl); }
@@ -104,8 +104,9 @@ cudaError_t launch_score_stream(const Problem& p, const void* q, const float* pr
                          : launch_score_stream_rows<KVSWAP_F16, 64>(p, a, pl.g_shift, pl.fused, pl.ctas, st);
     case KVSWAP_E4M3: return launch_score_stream_rows<KVSWAP_E4M3, 32>(p, a, pl.g_shift, pl.fused, pl.ctas, st);
     default:
-      return p.r == 16 ? launch_score_stream_rows<KVSWAP_F32, 16>(p, a, pl.g_shift, pl.fused, pl.ctas, st)
-                       : launch_score_stream_rows<KVSWAP_F32, 32>(p, a, pl.g_shift, pl.fused, pl.ctas, st);
+      return p.r == 16   ? launch_score_stream_rows<KVSWAP_F32, 16>(p, a, pl.g_shift, pl.fused, pl.ctas, st)
+             : p.r == 32 ? launch_score_stream_rows<KVSWAP_F32, 32>(p, a, pl.g_shift, pl.fused, pl.ctas, st)
+                         : launch_score_stream_rows<KVSWAP_F32, 64>(p, a, pl.g_shift, pl.fused, pl.ctas, st);
   }
 }
 

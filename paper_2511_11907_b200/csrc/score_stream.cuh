@@ -1,6 +1,6 @@
 // K2, streaming tensor-core scorer: low-rank query (Eq. 1), token scoring, head aggregation and group
 // ReduceMax (Sec. 4.3) for metadata rows that are dense in memory: fp16 of rank 16, 32 or 64, E4M3 of rank
-// 32, fp32 of rank 16 or 32.  The arithmetic of a block of rows is in score_tile.cuh.
+// 32, fp32 of rank 16, 32 or 64 (there with groups of up to 16).  The arithmetic of a block of rows is in score_tile.cuh.
 //
 // One persistent CTA per SM, 16 warps.  Work item = (sequence b, metadata head hm, block of 8 scopes, tile
 // of up to 4 KB of rows); items are numbered with the tile fastest, a "row set" is the items of one
@@ -57,7 +57,7 @@ struct ScoreSmem {
   float qsum[kQuerySumFloats];                            // scratch of build_queries
   float upart[kQueryPartFloats];
   float urow[kMaxSets][kScoreCols * R];                   // summed low-rank queries per row set of the CTA
-  float sc[GS >= 0 ? 4 : kScoreWarps * kScoreCols * kGenericPitch];
+  float sc[GS >= 0 ? 4 : kScoreWarps * kScoreCols * generic_pitch(ScoreStage<META, R, GS>::kRows)];
 };
 
 struct StreamArgs {
@@ -181,7 +181,7 @@ score_stream_kernel(Problem p, StreamArgs a) {
   uint32_t* my_hist = nullptr;                      // its global histogram
   int my_col = -1;                                  // its column of the shared-memory histogram, or -1
   bool scope_ok = false;                            // the lane's scope exists
-  float* const sc = sm->sc + (GS >= 0 ? 0 : warp * kCols * kGenericPitch);
+  float* const sc = sm->sc + (GS >= 0 ? 0 : warp * kCols * generic_pitch(kStageRows));
   int stage = 0;
   uint32_t phase = 0;
   bool timed_out = false;
@@ -316,6 +316,7 @@ template <> cudaError_t launch_score_stream_rows<KVSWAP_F16, 64>(const Problem&,
 template <> cudaError_t launch_score_stream_rows<KVSWAP_E4M3, 32>(const Problem&, const StreamArgs&, int, bool, int, cudaStream_t);
 template <> cudaError_t launch_score_stream_rows<KVSWAP_F32, 16>(const Problem&, const StreamArgs&, int, bool, int, cudaStream_t);
 template <> cudaError_t launch_score_stream_rows<KVSWAP_F32, 32>(const Problem&, const StreamArgs&, int, bool, int, cudaStream_t);
+template <> cudaError_t launch_score_stream_rows<KVSWAP_F32, 64>(const Problem&, const StreamArgs&, int, bool, int, cudaStream_t);
 
 template <int META, int R, int GS>
 cudaError_t launch_score_stream_gs(const Problem& p, const StreamArgs& a, bool fused, int ctas, cudaStream_t st) {

@@ -1,6 +1,6 @@
 // Scores of eight metadata rows at a time on the tensor cores: the per-warp arithmetic of the streaming
 // scorer (Eq. 1 and the head sum of Sec. 4.3), for metadata rows of R = 16, 32 or 64 entries in fp16,
-// E4M3 (R = 32) or fp32 (R = 16, 32).
+// E4M3 (R = 32) or fp32.
 //
 // With joint metadata one row feeds up to 8 scores (the per-KV-head scopes): an [rows x R].[R x 8]
 // contraction, which the fp32 pipes cannot sustain at HBM rate; it runs on mma.sync m16n8k16 with fp32
@@ -31,7 +31,7 @@ template <int META, int R>
 struct MetaRows {
   static constexpr int kElem = META == KVSWAP_F32 ? 4 : META == KVSWAP_F16 ? 2 : 1;
   static constexpr int kRowBytes = R * kElem;
-  static_assert(kRowBytes == 32 || kRowBytes == 64 || kRowBytes == 128, "rows the tile reads are laid out for");
+  static_assert(kRowBytes == 32 || kRowBytes == 64 || kRowBytes == 128 || kRowBytes == 256, "rows the tile reads are laid out for");
 };
 
 __device__ __forceinline__ void mma16816_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
@@ -121,12 +121,13 @@ struct ScoreQuery {
 
 // Byte offset inside an 8-row block at which a lane starts reading (score_rows8 adds the rest).  Rows of 128
 // bytes are read in two 16-byte pieces, the odd rows' in the other order, so that the eight lanes of a
-// shared-memory phase fall into eight different bank groups.
+// shared-memory phase fall into eight different bank groups; rows of 256 in four, the odd rows' halves swapped.
 template <int META, int R>
 __device__ __forceinline__ uint32_t score_lane_offset(int lane) {
   constexpr int kRowBytes = MetaRows<META, R>::kRowBytes;
   if constexpr (kRowBytes <= 64) return uint32_t(lane) * (kRowBytes / 4);
-  else return uint32_t(lane >> 2) * 128u + uint32_t(lane & 3) * 32u + uint32_t((lane >> 2) & 1) * 16u;
+  else if constexpr (kRowBytes == 128) return uint32_t(lane >> 2) * 128u + uint32_t(lane & 3) * 32u + uint32_t((lane >> 2) & 1) * 16u;
+  else return uint32_t(lane >> 2) * 256u + uint32_t(lane & 3) * 64u + uint32_t((lane >> 2) & 1) * 32u;
 }
 
 // Unscaled scores of scope g for tokens 2t and 2t + 1 of the 8-row block; `addr` = block + score_lane_offset().
@@ -138,6 +139,15 @@ __device__ __forceinline__ void score_rows8(uint32_t addr, const ScoreQuery<META
     asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(raw[0]), "=r"(raw[1]) : "r"(addr));
   } else if constexpr (kRowBytes == 64) {
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(raw[0]), "=r"(raw[1]), "=r"(raw[2]), "=r"(raw[3]) : "r"(addr));
+  } else if constexpr (kRowBytes == 256) {
+    uint32_t x[16];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(x[4 * i]), "=r"(x[4 * i + 1]), "=r"(x[4 * i + 2]), "=r"(x[4 * i + 3])
+                   : "r"(addr ^ uint32_t(i * 16)));
+    const bool swapped = (addr & 32u) != 0u;         // blocks are 128-byte aligned
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { raw[i] = swapped ? x[8 + i] : x[i]; raw[8 + i] = swapped ? x[i] : x[8 + i]; }
   } else {
     uint32_t x[4], y[4];
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(addr));
@@ -182,9 +192,9 @@ __device__ __forceinline__ void score_rows8(uint32_t addr, const ScoreQuery<META
 // ReduceMax over the groups of one staged tile of `rows` rows (a multiple of G); `base` = stage +
 // score_lane_offset().  Every finished group goes to publish(group within the tile, score) in exactly one lane,
 // the lane of its scope (lane / 4), if `scope_ok`.  GS = log2 G: the maximum is a max over two registers and at
-// most two shuffles.  GS = -1: any G, through the warp's buffer `sc` [8 scopes][kGenericPitch].
+// most two shuffles.  GS = -1: any G, through the warp's buffer `sc` [8 scopes][generic_pitch(STAGE_ROWS)].
 constexpr int kGenericRows = 48;                          // GS = -1: token rows per tile, at most
-constexpr int kGenericPitch = 56;                         // floats between scopes of the buffer (bank spread)
+__host__ __device__ constexpr int generic_pitch(int rows) { return rows % 32 == 24 ? rows + 16 : rows + 8; }   // floats between scopes (bank spread)
 
 template <int META, int R, int GS, int STAGE_ROWS, typename Publish>
 __device__ __forceinline__ void score_tile_groups(uint32_t base, int rows, int lane, const ScoreQuery<META, R>& query,
@@ -235,13 +245,13 @@ __device__ __forceinline__ void score_tile_groups(uint32_t base, int rows, int l
     for (int it = 0; it * 8 < rows; ++it) {
       float x0, x1;
       score_rows8<META, R>(base + uint32_t(it) * 8u * kRowBytes, query, &x0, &x1);
-      *reinterpret_cast<float2*>(sc + rq * kGenericPitch + it * 8 + 2 * qt) = make_float2(x0 * query.inv, x1 * query.inv);
+      *reinterpret_cast<float2*>(sc + rq * generic_pitch(STAGE_ROWS) + it * 8 + 2 * qt) = make_float2(x0 * query.inv, x1 * query.inv);
     }
     __syncwarp();
     const int ngt = rows / G;
     if (scope_ok) {
       for (int gi = qt; gi < ngt; gi += 4) {
-        const float* s = sc + rq * kGenericPitch + gi * G;
+        const float* s = sc + rq * generic_pitch(STAGE_ROWS) + gi * G;
         float m = s[0];
         for (int i = 1; i < G; ++i) m = fmaxf(m, s[i]);
         publish(gi, m);
@@ -252,12 +262,18 @@ __device__ __forceinline__ void score_tile_groups(uint32_t base, int rows, int l
 
 // Rows of one stage: 4 KB where a finished score leaves the registers (the hand-over of a stage costs the
 // same whatever its size: 4 KB x 2 stages measured 1.3 us per layer faster than 2 KB x 4 at B = 4,
-// N = 131072); GS = -1 takes 3 KB, which leaves room for the warps' score buffers.
+// N = 131072); GS = -1 takes 3 KB, which leaves room for the warps' score buffers.  A stage is read eight rows at
+// a time, whole: it holds a multiple of eight, which for rows of 256 bytes takes 4 KB.
+__host__ __device__ constexpr int score_stage_bytes(bool generic, int row_bytes) { return generic && row_bytes <= 128 ? 3072 : 4096; }
+__host__ __device__ constexpr int score_stage_rows(bool generic, int row_bytes) {
+  const int fit = score_stage_bytes(generic, row_bytes) / row_bytes;
+  return generic && fit > kGenericRows ? kGenericRows : fit;
+}
 template <int META, int R, int GS>
 struct ScoreStage {
-  static constexpr int kBytes = GS >= 0 ? 4096 : 3072;
-  static constexpr int kFit = kBytes / MetaRows<META, R>::kRowBytes;
-  static constexpr int kRows = GS >= 0 ? kFit : (kFit < kGenericRows ? kFit : kGenericRows);
+  static constexpr int kBytes = score_stage_bytes(GS < 0, MetaRows<META, R>::kRowBytes);
+  static constexpr int kRows = score_stage_rows(GS < 0, MetaRows<META, R>::kRowBytes);
+  static_assert(kRows % 8 == 0, "whole reads");
 };
 
 }  // namespace kvswap

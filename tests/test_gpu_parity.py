@@ -452,6 +452,10 @@ STREAM = [   # K/V type, metadata type, rank, G, per-head, scope, B, H_kv, rho, 
     (W.F32, W.F32, 16, 4, True, ALL, 1, 2, 1, 240001),     # several tiles per warp: blocks of tiles, head by head
     (W.F32, W.F32, 16, 4, False, ALL, 1, 2, 1, 131072),    # 32768 groups: eight TopK parts
     (W.F32, W.F32, 16, 7, False, KV, 1, 2, 1, 130003),
+    (W.F32, W.F32, 64, 8, False, KV, 1, 8, 1, 16 * 45 + 9),
+    (W.F32, W.F32, 64, 12, True, KV, 2, 2, 2, 12 * 70 + 5),
+    (W.F32, W.F32, 64, 4, True, ALL, 1, 4, 1, 12 * 60 + 7),
+    (W.F32, W.F32, 64, 32, False, KV, 1, 2, 2, 999),       # a group that does not fit a stage
 ]
 
 
@@ -501,6 +505,23 @@ def test_select_of_degenerate_scores(kind, NG, M):
     dl.set_meta(meta)
     idx, nsel, Rg = dl.score_select()
     assert np.all(nsel == M) and np.array_equal(idx, O.select(Rg.astype(np.float64), M))
+
+
+@pytest.mark.parametrize("kv_type,meta,head_dim,rank,meta_heads,n", [(W.BF16, W.F16, 128, 32, 1, 8), (W.F16, W.F16, 64, 64, 4, 13),
+                                                                   (W.F32, W.F32, 64, 16, 1, 1), (W.F32, W.F32, 128, 100, 4, 33),
+                                                                   (W.BF16, W.F32, 128, 200, 1, 64)])
+def test_project_keys_of_a_few_tokens(kv_type, meta, head_dim, rank, meta_heads, n):
+    """Short token ranges (a flushed group): eight tokens per CTA, ragged, up to eight columns per lane."""
+    wl = small(kv_dtype=kv_type, q_dtype=kv_type, meta_dtype=meta, head_dim=head_dim, rank=min(rank, head_dim) if meta_heads > 1 else rank,
+               group_size=8, n_ctx=150, n_q_heads=8, n_kv_heads=4, batch=2)
+    li = W.make_layer(wl, 0, meta_heads)
+    dl = DeviceLayer(li, KV)
+    meta_or = O.project_keys(li.K, li.proj, meta_heads, META_NAME[meta])
+    tol = project_tolerance(li.K, li.proj, meta_heads, meta_or, meta)
+    dl.meta.fill_(123.0)
+    got = dl.project(n_begin=70, n_end=70 + n)
+    assert np.all(got[:, :, :70] == 123.0) and np.all(got[:, :, 70 + n:] == 123.0)
+    assert np.all(np.abs(got[:, :, 70:70 + n].astype(np.float64) - meta_or[:, :, 70:70 + n].astype(np.float64)) <= tol[:, :, 70:70 + n])
 
 
 def test_strided_kv_and_metadata_views():

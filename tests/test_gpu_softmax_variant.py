@@ -130,6 +130,7 @@ def test_softmax_variant_tensor_core_shapes(name, wl, scope):
     (1, ALL, dict(rank=64, n_ctx=24 * 50 + 8)),
     (1, KV, dict(rank=16, meta_dtype=W.F32, kv_dtype=W.F32, q_dtype=W.F32, n_q_heads=6, n_kv_heads=2, n_ctx=1999)),
     (1, ALL, dict(rank=32, meta_dtype=W.F32, n_q_heads=40, n_kv_heads=10, group_size=5)),
+    (1, KV, dict(rank=64, meta_dtype=W.F32, n_q_heads=12, n_kv_heads=4, group_size=16, n_ctx=1505)),
     (0, KV, dict(n_q_heads=24, n_kv_heads=8, n_ctx=1801)),
     (0, KV, dict(n_q_heads=24, n_kv_heads=2, group_size=4, rank=64)),                            # 12 heads per sum: two blocks
     (0, ALL, dict(n_q_heads=16, n_kv_heads=4, group_size=12, n_ctx=12 * 170 + 3)),
