@@ -266,10 +266,10 @@ int kvswap_sparse_decode_static(const kvswap_shape* shape, const void* q, const 
 /*
  * Per-layer tensors of a model with L layers that all share one kvswap_shape.  Each member is a
  * HOST array of L DEVICE pointers: K[l], V[l] are [B, H_kv, N, d]; meta[l] is [B, H_m, N, r];
- * proj[l] is [H_kv, d, r] fp32.  max_lookahead bounds how many layers the predictor stream of
- * kvswap_decode_step_tiered may run ahead of its attention: 1 = layer l is predicted while layer
- * l-1 is attended (what a model allows, whose layer-l prediction needs the input of layer l-1);
- * 0 = no limit.  kvswap_decode_step always predicts exactly one layer ahead and ignores the value.
+ * proj[l] is [H_kv, d, r] fp32.  max_lookahead bounds how many layers the predictor may run ahead of the
+ * attention: 1 = layer l is predicted while layer l-1 is attended (what a model allows, whose layer-l
+ * prediction needs the input of layer l-1); 0 = no limit.  Both steps predict exactly one layer ahead,
+ * which satisfies every bound.
  * Negative values are KVSWAP_ERR_SHAPE.
  */
 typedef struct {
@@ -376,10 +376,10 @@ int kvswap_decode_step(const kvswap_shape* shape, const kvswap_layers* layers, c
 /*
  * The decode step over a tiered cache (Sec. 4.4.2, Sec. 4.4.3): the full K/V of every layer lives
  * in a slow tier, each layer has a reuse buffer (kvswap_reuse_* above) in device memory, and the
- * step's attention reads only reuse stores.  Per layer the internal predictor stream runs
- * score/select, kvswap_reuse_lookup and kvswap_reuse_fill, so a layer's misses are fetched while
- * the layers before it are attended on `cuda_stream`; the attention is kvswap_sparse_decode over
- * the layer's reuse store with the slot list.  Arrays of L per-layer pointers are HOST arrays.
+ * step's attention reads only reuse stores.  Per layer score/select runs on `cuda_stream`, one layer
+ * ahead; kvswap_reuse_lookup and kvswap_reuse_fill follow it on an internal stream, so a layer's misses
+ * are fetched while the layer before it is attended on `cuda_stream`; the attention is
+ * kvswap_sparse_decode over the layer's reuse store with the slot list.  Arrays of L per-layer pointers are HOST arrays.
  *   K_slow, V_slow    [L] slow-tier stores, laid out by shape's kv strides (GPU-readable memory)
  *   K_reuse, V_reuse  [L] reuse stores [B, H_kv, (n_slots + 1) G, d]; the caller keeps the
  *                     N mod G newest tokens in rows [n_slots G, n_slots G + N mod G)

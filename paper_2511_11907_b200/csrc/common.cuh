@@ -90,6 +90,10 @@ cudaError_t launch_reuse_lookup(const Problem& p, int n_slots, int max_groups, c
 cudaError_t launch_reuse_fill(const Problem& p, int n_slots, const void* K_slow, const void* V_slow, void* K_reuse,
                               void* V_reuse, const int32_t* miss_group, const int32_t* miss_slot, const int32_t* n_miss,
                               cudaStream_t st);
+cudaError_t launch_reuse_fetch(const Problem& p, int n_slots, int max_groups, const int32_t* group_idx,
+                               const int32_t* n_selected, int32_t* state, const void* K_slow, const void* V_slow,
+                               void* K_reuse, void* V_reuse, int32_t* slot_idx, int32_t* miss_group, int32_t* miss_slot,
+                               int32_t* n_miss, cudaStream_t st);   // lookup, then fill, in one launch
 size_t project_keys_umma_scratch_bytes(const Problem& p);
 bool try_launch_project_keys_umma(const Problem& p, const void* K, const float* proj, void* meta, int n_begin,
                                   int n_end, void* scratch, uint32_t* err, cudaStream_t st, cudaError_t* result);

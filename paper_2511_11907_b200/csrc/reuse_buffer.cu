@@ -10,6 +10,7 @@
 //                         (one block scan each); the k-th miss takes the k-th such slot.
 //   reuse_fill_kernel     one CTA per missed group: copies its G rows of K and V from the slow
 //                         tier (any device-accessible memory, e.g. pinned host memory) into the slot.
+//   reuse_fetch_kernel    both in one launch, for the tiered step.
 //
 // State of one buffer set (caller-owned device memory, one per layer), int32 words:
 //   head[B*S] | slot_group[B*S*C] | group_slot[B*S*max_groups]
@@ -18,6 +19,7 @@
 #include <algorithm>
 
 #include "async_copy.cuh"
+#include "cluster.cuh"
 #include "common.cuh"
 
 namespace kvswap {
@@ -53,23 +55,35 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* warp_tot, int* t
   return incl - v + (warp > 0 ? warp_tot[warp - 1] : 0);
 }
 
-__global__ void __launch_bounds__(kThreads)
-reuse_lookup_kernel(int M, int NG, int C, int max_groups, const int32_t* __restrict__ group_idx,
-                    const int32_t* __restrict__ n_selected, int32_t* __restrict__ head_all,
-                    int32_t* __restrict__ slot_group_all, int32_t* __restrict__ group_slot_all,
-                    int32_t* __restrict__ slot_idx, int32_t* __restrict__ miss_group, int32_t* __restrict__ miss_slot,
-                    int32_t* __restrict__ n_miss_out) {
-  extern __shared__ unsigned char smem[];
+// Lists and tables of a lookup (see the file comment); all indexed by problem.
+struct LookupArgs {
+  int M, NG, C, max_groups;
+  const int32_t* group_idx;
+  const int32_t* n_selected;
+  int32_t* head;
+  int32_t* slot_group;
+  int32_t* group_slot;
+  int32_t* slot_idx;
+  int32_t* miss_group;
+  int32_t* miss_slot;
+  int32_t* n_miss;
+};
+
+// Lookup of problem `prob` by the kThreads threads of a CTA; smem: busy flags [C], then victims [M].  Returns the
+// number of misses.
+__device__ __forceinline__ int reuse_lookup_body(const LookupArgs& a, int prob, unsigned char* smem) {
+  const int M = a.M, NG = a.NG, C = a.C, max_groups = a.max_groups;
+  int32_t* const miss_group = a.miss_group;
+  int32_t* const miss_slot = a.miss_slot;
   unsigned char* busy = smem;                                    // [C]
   int32_t* victim = reinterpret_cast<int32_t*>(smem + ((C + 15) & ~15));   // [M]
   __shared__ int warp_tot[32];
 
-  const int prob = blockIdx.x;
-  const int32_t* idx = group_idx + int64_t(prob) * M;
-  int32_t* slot_group = slot_group_all + int64_t(prob) * C;
-  int32_t* group_slot = group_slot_all + int64_t(prob) * max_groups;
-  const int head = head_all[prob];
-  const int n_sel = max(0, min(n_selected[prob], M));
+  const int32_t* idx = a.group_idx + int64_t(prob) * M;
+  int32_t* slot_group = a.slot_group + int64_t(prob) * C;
+  int32_t* group_slot = a.group_slot + int64_t(prob) * max_groups;
+  const int head = a.head[prob];
+  const int n_sel = max(0, min(a.n_selected[prob], M));
 
   for (int c = threadIdx.x; c < C; c += kThreads) busy[c] = 0;
   __syncthreads();
@@ -157,7 +171,7 @@ reuse_lookup_kernel(int M, int NG, int C, int max_groups, const int32_t* __restr
     if (e < per && i < M) {
       int s = slot[e];
       if (grp[e] >= 0 && s < 0) s = group_slot[grp[e]];        // a repeated entry: the slot its first entry loaded
-      slot_idx[int64_t(prob) * M + i] = s;
+      a.slot_idx[int64_t(prob) * M + i] = s;
     }
   }
   for (int k = n_miss + threadIdx.x; k < M; k += kThreads) {
@@ -165,39 +179,92 @@ reuse_lookup_kernel(int M, int NG, int C, int max_groups, const int32_t* __restr
     miss_slot[int64_t(prob) * M + k] = -1;
   }
   if (threadIdx.x == 0) {
-    n_miss_out[prob] = n_miss;
-    if (n_miss > 0) { int h = victim[n_miss - 1] + 1; head_all[prob] = (h >= C) ? 0 : h; }
+    a.n_miss[prob] = n_miss;
+    if (n_miss > 0) { int h = victim[n_miss - 1] + 1; a.head[prob] = (h >= C) ? 0 : h; }
   }
+  return n_miss;
 }
 
-// One CTA per (miss ordinal, sequence x scope).  Rows are copied in 16-byte pieces.
-__global__ void __launch_bounds__(256)
-reuse_fill_kernel(Problem p, int M, int C, const unsigned char* __restrict__ K_slow,
-                  const unsigned char* __restrict__ V_slow, unsigned char* __restrict__ K_reuse,
-                  unsigned char* __restrict__ V_reuse, const int32_t* __restrict__ miss_group,
-                  const int32_t* __restrict__ miss_slot, const int32_t* __restrict__ n_miss, int elem_bytes) {
-  const int prob = blockIdx.y, k = blockIdx.x;
-  if (k >= n_miss[prob]) return;
-  const int j = miss_group[int64_t(prob) * M + k], slot = miss_slot[int64_t(prob) * M + k];
-  if (j < 0 || slot < 0) return;
+__global__ void __launch_bounds__(kThreads)
+reuse_lookup_kernel(LookupArgs a) {
+  extern __shared__ unsigned char smem[];
+  reuse_lookup_body(a, blockIdx.x, smem);
+}
+
+// Where a fill copies from and to.
+struct FillArgs {
+  int C, elem_bytes;
+  const unsigned char* K_slow;
+  const unsigned char* V_slow;
+  unsigned char* K_reuse;
+  unsigned char* V_reuse;
+};
+
+// The rows of misses first, first + step, .. < n_miss of problem `prob`, in 16-byte pieces, by `threads` threads;
+// kAhead pieces per thread are in flight.
+template <int kAhead>
+__device__ __forceinline__ void reuse_fill_body(const Problem& p, const FillArgs& f, const int32_t* miss_group,
+                                                const int32_t* miss_slot, int M, int prob, int n_miss, int first, int step,
+                                                int threads) {
   const int b = prob / p.S, s = prob % p.S;
   const int g_first = (p.scope == KVSWAP_SCOPE_KV_HEAD) ? s : 0;
   const int g_count = (p.scope == KVSWAP_SCOPE_KV_HEAD) ? 1 : p.Hkv;
-  const int pieces = p.d * elem_bytes / 16;                      // per row
-  const int64_t R = int64_t(C + 1) * p.G;                        // rows per head of the reuse store
-  const int total = 2 * g_count * p.G * pieces;
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    const int piece = t % pieces;
-    const int row = (t / pieces) % p.G;
-    const int gi = (t / (pieces * p.G)) % g_count;
-    const bool is_v = t >= g_count * p.G * pieces;
-    const int g = g_first + gi;
-    const int64_t src = (int64_t(b) * p.kv_sb + int64_t(g) * p.kv_sh + (int64_t(j) * p.G + row) * p.kv_sn) * elem_bytes +
-                        piece * 16;
-    const int64_t dst = ((int64_t(b) * p.Hkv + g) * R + int64_t(slot) * p.G + row) * p.d * elem_bytes + piece * 16;
-    const uint4 v = *reinterpret_cast<const uint4*>((is_v ? V_slow : K_slow) + src);
-    *reinterpret_cast<uint4*>((is_v ? V_reuse : K_reuse) + dst) = v;
+  const int pieces = p.d * f.elem_bytes / 16;                    // per row
+  const int64_t R = int64_t(f.C + 1) * p.G;                      // rows per head of the reuse store
+  const int per_miss = 2 * g_count * p.G * pieces;
+  const int mine = (n_miss > first) ? (n_miss - first + step - 1) / step : 0;
+  for (int64_t t0 = threadIdx.x; t0 < int64_t(mine) * per_miss; t0 += int64_t(threads) * kAhead) {
+    uint4 v[kAhead];
+    unsigned char* to[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int64_t t = t0 + int64_t(u) * threads;
+      to[u] = nullptr;
+      if (t < int64_t(mine) * per_miss) {
+        const int k = first + int(t / per_miss) * step, e = int(t % per_miss);
+        const int j = __ldcg(miss_group + int64_t(prob) * M + k), slot = __ldcg(miss_slot + int64_t(prob) * M + k);
+        const int piece = e % pieces, row = (e / pieces) % p.G, gi = (e / (pieces * p.G)) % g_count;
+        const bool is_v = e >= g_count * p.G * pieces;
+        const int g = g_first + gi;
+        if (j >= 0 && slot >= 0) {
+          const int64_t src = (int64_t(b) * p.kv_sb + int64_t(g) * p.kv_sh + (int64_t(j) * p.G + row) * p.kv_sn) * f.elem_bytes +
+                              piece * 16;
+          to[u] = (is_v ? f.V_reuse : f.K_reuse) +
+                  ((int64_t(b) * p.Hkv + g) * R + int64_t(slot) * p.G + row) * p.d * f.elem_bytes + piece * 16;
+          v[u] = *reinterpret_cast<const uint4*>((is_v ? f.V_slow : f.K_slow) + src);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) if (to[u] != nullptr) *reinterpret_cast<uint4*>(to[u]) = v[u];
   }
+}
+
+// Lookup and fill of a step in one launch: a cluster per problem, whose first CTA looks the selection up and which
+// then copies the missed groups together.  The copy needs some 150 KB in flight to fill the slow tier's link (50 GB/s
+// from pinned host memory), so a few CTAs do, and the rest of the GPU is free for the predictor of the next layer:
+// a CTA per miss, 2048 of them, kept it out.
+constexpr int kFetchAhead = 4;
+
+__global__ void __launch_bounds__(kThreads)
+reuse_fetch_kernel(Problem p, LookupArgs a, FillArgs f) {
+  extern __shared__ unsigned char smem[];
+  const int rank = int(cluster_rank()), n_ctas = int(cluster_size()), prob = blockIdx.x / n_ctas;
+  pdl_wait();
+  if (rank == 0) reuse_lookup_body(a, prob, smem);
+  cluster_arrive();
+  cluster_wait();                                                // the miss list is written
+  const int n_miss = __ldcg(a.n_miss + prob);
+  reuse_fill_body<kFetchAhead>(p, f, a.miss_group, a.miss_slot, a.M, prob, n_miss, rank, n_ctas, kThreads);
+}
+
+// One CTA per (miss ordinal, sequence x scope).
+__global__ void __launch_bounds__(256)
+reuse_fill_kernel(Problem p, int M, FillArgs f, const int32_t* __restrict__ miss_group, const int32_t* __restrict__ miss_slot,
+                  const int32_t* __restrict__ n_miss) {
+  const int prob = blockIdx.y, k = blockIdx.x;
+  if (k >= n_miss[prob]) return;
+  reuse_fill_body<1>(p, f, miss_group, miss_slot, M, prob, k + 1, k, 1, 256);
 }
 
 __global__ void reuse_init_kernel(int32_t* state, int64_t n_head, int64_t n_total) {
@@ -223,32 +290,60 @@ cudaError_t launch_reuse_init(const Problem& p, int n_slots, int max_groups, int
   return cudaGetLastError();
 }
 
+namespace {
+
+LookupArgs lookup_args(const Problem& p, int n_slots, int max_groups, const int32_t* group_idx, const int32_t* n_selected,
+                       int32_t* state, int32_t* slot_idx, int32_t* miss_group, int32_t* miss_slot, int32_t* n_miss) {
+  const int64_t probs = int64_t(p.B) * p.S;
+  return LookupArgs{p.M, std::min(p.NG, max_groups), n_slots, max_groups, group_idx, n_selected, state, state + probs,
+                    state + probs + probs * n_slots, slot_idx, miss_group, miss_slot, n_miss};
+}
+FillArgs fill_args(const Problem& p, int n_slots, const void* K_slow, const void* V_slow, void* K_reuse, void* V_reuse) {
+  return FillArgs{n_slots, (p.kv_dtype == KVSWAP_F32) ? 4 : 2, static_cast<const unsigned char*>(K_slow),
+                  static_cast<const unsigned char*>(V_slow), static_cast<unsigned char*>(K_reuse),
+                  static_cast<unsigned char*>(V_reuse)};
+}
+template <typename K>
+cudaError_t lookup_smem(K kern, const Problem& p, int n_slots, size_t* smem) {
+  *smem = size_t((n_slots + 15) & ~15) + sizeof(int32_t) * size_t(p.M);
+  return *smem > 40 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(*smem)) : cudaSuccess;
+}
+
+}  // namespace
+
 cudaError_t launch_reuse_lookup(const Problem& p, int n_slots, int max_groups, const int32_t* group_idx,
                                 const int32_t* n_selected, int32_t* state, int32_t* slot_idx, int32_t* miss_group,
                                 int32_t* miss_slot, int32_t* n_miss, cudaStream_t st) {
-  const int64_t probs = int64_t(p.B) * p.S;
-  int32_t* head = state;
-  int32_t* slot_group = head + probs;
-  int32_t* group_slot = slot_group + probs * n_slots;
-  const size_t smem = size_t((n_slots + 15) & ~15) + sizeof(int32_t) * size_t(p.M);
-  if (smem > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(reuse_lookup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-  }
-  reuse_lookup_kernel<<<int(probs), kThreads, smem, st>>>(p.M, std::min(p.NG, max_groups), n_slots, max_groups, group_idx,
-                                                          n_selected, head, slot_group, group_slot, slot_idx, miss_group,
-                                                          miss_slot, n_miss);
+  size_t smem = 0;
+  cudaError_t e = lookup_smem(reuse_lookup_kernel, p, n_slots, &smem);
+  if (e != cudaSuccess) return e;
+  reuse_lookup_kernel<<<p.B * p.S, kThreads, smem, st>>>(
+      lookup_args(p, n_slots, max_groups, group_idx, n_selected, state, slot_idx, miss_group, miss_slot, n_miss));
   return cudaGetLastError();
 }
 
 cudaError_t launch_reuse_fill(const Problem& p, int n_slots, const void* K_slow, const void* V_slow, void* K_reuse,
                               void* V_reuse, const int32_t* miss_group, const int32_t* miss_slot, const int32_t* n_miss,
                               cudaStream_t st) {
-  const int e = (p.kv_dtype == KVSWAP_F32) ? 4 : 2;
-  reuse_fill_kernel<<<dim3(p.M, p.B * p.S), 256, 0, st>>>(
-      p, p.M, n_slots, static_cast<const unsigned char*>(K_slow), static_cast<const unsigned char*>(V_slow),
-      static_cast<unsigned char*>(K_reuse), static_cast<unsigned char*>(V_reuse), miss_group, miss_slot, n_miss, e);
+  reuse_fill_kernel<<<dim3(p.M, p.B * p.S), 256, 0, st>>>(p, p.M, fill_args(p, n_slots, K_slow, V_slow, K_reuse, V_reuse),
+                                                          miss_group, miss_slot, n_miss);
   return cudaGetLastError();
+}
+
+cudaError_t launch_reuse_fetch(const Problem& p, int n_slots, int max_groups, const int32_t* group_idx,
+                               const int32_t* n_selected, int32_t* state, const void* K_slow, const void* V_slow,
+                               void* K_reuse, void* V_reuse, int32_t* slot_idx, int32_t* miss_group, int32_t* miss_slot,
+                               int32_t* n_miss, cudaStream_t st) {
+  size_t smem = 0;
+  cudaError_t e = lookup_smem(reuse_fetch_kernel, p, n_slots, &smem);
+  if (e != cudaSuccess) return e;
+  const int probs = p.B * p.S;
+  int cluster = 1;
+  while (cluster < 8 && probs * cluster < 16) cluster *= 2;
+  return launch_pdl_cluster(reuse_fetch_kernel, cluster, dim3(probs * cluster), dim3(kThreads), smem, st, p,
+                            lookup_args(p, n_slots, max_groups, group_idx, n_selected, state, slot_idx, miss_group, miss_slot,
+                                        n_miss),
+                            fill_args(p, n_slots, K_slow, V_slow, K_reuse, V_reuse));
 }
 
 }  // namespace kvswap

@@ -1,6 +1,6 @@
 // C-ABI entry points that serve all layers of a model in one call: the decode step over
 // HBM-resident stores (one stream, each layer predicted one layer ahead of its attention), the
-// decode step over reuse buffers in front of a slow tier (the predictor on a stream of its own)
+// decode step over reuse buffers in front of a slow tier (its copies on a stream of their own)
 // and the append steps.  The tiered step keeps one internal stream and a set of events per device;
 // nothing else here keeps state.
 #include <algorithm>
@@ -67,17 +67,16 @@ static kvswap_shape reuse_store_shape(const kvswap_shape& s, int32_t n_slots) {
   return r;
 }
 
-// Per-device resources of kvswap_decode_step's two-stream schedule: a stream for the predictor and
-// two events per layer.  Created on first use, kept for the life of the process.
+// Per-device resources of the tiered step: a stream for the slow tier's copies and two events per layer.  Created
+// on first use, kept for the life of the process.
 namespace {
 struct StepResources {
-  cudaStream_t predictor = nullptr;
-  cudaEvent_t fork = nullptr;
+  cudaStream_t fetch[2] = {nullptr, nullptr};   // layers take turns
+  cudaEvent_t join = nullptr;
   std::vector<cudaEvent_t> selected;     // selected[l]: layer l's selection is written
-  std::vector<cudaEvent_t> attended;     // attended[l]: layer l's attention output is written
+  std::vector<cudaEvent_t> fetched;      // fetched[l]: layer l's selected groups are in its reuse store
 };
 constexpr int kMaxDevices = 64;
-constexpr int kHostLead = 3;           // layers by which the host enqueues the predictor ahead of the attention
 std::mutex g_step_mutex;
 StepResources g_step[kMaxDevices];
 
@@ -98,23 +97,24 @@ cudaError_t step_resources(int n_layers, StepResources** out) {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   StepResources& r = g_step[dev];
-  if (r.predictor == nullptr) {
-    e = cudaStreamCreateWithFlags(&r.predictor, cudaStreamNonBlocking);
-    if (e != cudaSuccess) { r.predictor = nullptr; return e; }
+  for (cudaStream_t& f : r.fetch) {
+    if (f != nullptr) continue;
+    e = cudaStreamCreateWithFlags(&f, cudaStreamNonBlocking);
+    if (e != cudaSuccess) { f = nullptr; return e; }
   }
-  if (r.fork == nullptr) {
-    e = cudaEventCreateWithFlags(&r.fork, cudaEventDisableTiming);
-    if (e != cudaSuccess) { r.fork = nullptr; return e; }
+  if (r.join == nullptr) {
+    e = cudaEventCreateWithFlags(&r.join, cudaEventDisableTiming);
+    if (e != cudaSuccess) { r.join = nullptr; return e; }
   }
   if ((e = grow(&r.selected, n_layers)) != cudaSuccess) return e;
-  if ((e = grow(&r.attended, n_layers)) != cudaSuccess) return e;
+  if ((e = grow(&r.fetched, n_layers)) != cudaSuccess) return e;
   *out = &r;
   return cudaSuccess;
 }
 }  // namespace
 
 // One decode step over all layers; with `tiers` the attention is served from per-layer reuse buffers
-// that the predictor stream keeps filled from the slow tier.
+// that a fetch stream keeps filled from the slow tier.
 static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* layers, const kvswap_tiers* tiers,
                             const void* q, float* out, float* lse_opt, int32_t* group_idx, int32_t* n_selected,
                             void* ws, size_t ws_bytes, const kvswap_probe* probe_opt, void* cuda_stream) {
@@ -290,25 +290,15 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
     return status;
   }
 
-  // Tiered schedule: a layer's groups are predicted ahead of
-  // its attention, concurrently with the layers before it.  The predictor therefore runs on a
-  // stream of its own, ahead of the attention on the caller's stream by at most `look` layers
-  // (any number when the caller sets no limit):
-  //   predictor stream:  ... wait attended[l-1-look];  score/select(l);  record selected[l]  ...
-  //   caller's stream:   ... wait selected[l];         attention(l);     record attended[l]  ...
-  // With look = 1, predictor(l) overlaps attention(l-1) only: nothing runs further ahead than a
-  // model whose layer-(l-1) input (from which the paper forms the approximate query) exists
-  // once layer l-2 is done could run.  With look >= 2 the caller's stream waits for two layers'
-  // selections at a time, so that every second attention follows the previous one without a
-  // stream-level wait in between and, its inputs being settled, starts fetching while that one
-  // is still finishing.  Everything on the predictor stream is ordered after the work already
-  // in the caller's stream (fork event) and joins it again through the last selection event.
-  const bool bounded = layers->max_lookahead > 0 && layers->max_lookahead < L;
-  const int look = bounded ? layers->max_lookahead : L;
-  const int join = look >= 2 ? 2 : 1;          // layers of attention per wait on the predictor
-  // q is an input of the step (the fork event orders both streams after whatever produced it) and
-  // each selection is awaited through its event before the attention that reads it is launched:
-  // the inputs of both the predictor and the attention are settled.
+  // Tiered schedule.  The caller's stream predicts and attends, one layer ahead as in kvswap_decode_step; the slow
+  // tier's link is kept busy from a stream of its own:
+  //   caller's stream:  predict(0) | predict(1) wait fetched[0] attend(0) | predict(2) wait fetched[1] attend(1) | ..
+  //   fetch streams:    wait selected[l];  lookup and fill(l);  record fetched[l]        (two, layers take turns: the
+  //                     lookup of a layer runs while the layer before it is still copied)
+  // A layer's misses cross the link while the layer before it is attended and the next one predicted.  (With lookup
+  // and fill behind each other on the predictor's stream the link idled during every prediction: 1580 us for four
+  // steps of four layers, B = 1, N = 16384, M = 256, 8 KV heads of 128, of which the link needs 1184; now 1427.)
+  // q is an input of the step and a slot list is awaited through its event: the inputs are settled.
   kvswap_shape shape_settled = shape_attn;
   shape_settled.flags |= KVSWAP_INPUTS_SETTLED;
   Problem p_settled = p;
@@ -316,71 +306,38 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
   std::lock_guard<std::mutex> lock(g_step_mutex);
   StepResources* res = nullptr;
   if (step_resources(L, &res) != cudaSuccess) return KVSWAP_ERR_CUDA;
-  cudaStream_t pred = res->predictor;
-  if (cudaEventRecord(res->fork, stream) != cudaSuccess || cudaStreamWaitEvent(pred, res->fork, 0) != cudaSuccess)
-    return KVSWAP_ERR_CUDA;
 
-  auto enqueue_predictor = [&](int l) -> int {
-    if (bounded && l > look && cudaStreamWaitEvent(pred, res->attended[l - 1 - look], 0) != cudaSuccess)
-      return KVSWAP_ERR_CUDA;
-    const bool probed = probe_opt != nullptr && probe_opt->layer == l;
-    if (probed && probe_opt->ev_begin) cudaEventRecord(static_cast<cudaEvent_t>(probe_opt->ev_begin), pred);
+  auto predict_and_fetch = [&](int l) -> int {
     const void* ql = static_cast<const char*>(q) + size_t(l) * q_bytes;
-    if (score_select_launch(p_settled, w, ql, layers->proj[l], layers->meta[l], group_idx + size_t(l) * idx_elems,
-                            n_selected + size_t(l) * nsel_elems, nullptr, ws, pred) != cudaSuccess)
+    int32_t* idx_l = group_idx + size_t(l) * idx_elems;
+    int32_t* nsel_l = n_selected + size_t(l) * nsel_elems;
+    if (score_select_launch(p_settled, w, ql, layers->proj[l], layers->meta[l], idx_l, nsel_l, nullptr, ws, stream) != cudaSuccess ||
+        cudaEventRecord(res->selected[l], stream) != cudaSuccess ||
+        cudaStreamWaitEvent(res->fetch[l & 1], res->selected[l], 0) != cudaSuccess ||
+        launch_reuse_fetch(p, tiers->n_slots, tiers->max_groups, idx_l, nsel_l, static_cast<int32_t*>(tiers->state[l]),
+                           tiers->K_slow[l], tiers->V_slow[l], tiers->K_reuse[l], tiers->V_reuse[l],
+                           tiers->slot_idx + size_t(l) * idx_elems, tiers->miss_group + size_t(l) * idx_elems,
+                           tiers->miss_slot + size_t(l) * idx_elems, tiers->n_miss + size_t(l) * nsel_elems,
+                           res->fetch[l & 1]) != cudaSuccess ||
+        cudaEventRecord(res->fetched[l], res->fetch[l & 1]) != cudaSuccess)
       return KVSWAP_ERR_CUDA;
-    if (tiers != nullptr) {
-      // Hits keep their slots, misses are fetched from the slow tier -- still on the predictor
-      // stream, so the fetch for this layer overlaps the attention of the layers before it.
-      int32_t* slot_l = tiers->slot_idx + size_t(l) * idx_elems;
-      int32_t* mg_l = tiers->miss_group + size_t(l) * idx_elems;
-      int32_t* ms_l = tiers->miss_slot + size_t(l) * idx_elems;
-      int32_t* nm_l = tiers->n_miss + size_t(l) * nsel_elems;
-      if (launch_reuse_lookup(p, tiers->n_slots, tiers->max_groups, group_idx + size_t(l) * idx_elems,
-                              n_selected + size_t(l) * nsel_elems, static_cast<int32_t*>(tiers->state[l]), slot_l, mg_l,
-                              ms_l, nm_l, pred) != cudaSuccess ||
-          launch_reuse_fill(p, tiers->n_slots, tiers->K_slow[l], tiers->V_slow[l], tiers->K_reuse[l],
-                            tiers->V_reuse[l], mg_l, ms_l, nm_l, pred) != cudaSuccess)
-        return KVSWAP_ERR_CUDA;
-    }
-    if (probed && probe_opt->ev_mid) cudaEventRecord(static_cast<cudaEvent_t>(probe_opt->ev_mid), pred);
-    if (cudaEventRecord(res->selected[l], pred) != cudaSuccess) return KVSWAP_ERR_CUDA;
     return KVSWAP_OK;
   };
-  auto enqueue_attention = [&](int l) -> int {
-    if (l % join == 0 &&
-        cudaStreamWaitEvent(stream, res->selected[std::min(L - 1, l + join - 1)], 0) != cudaSuccess)
-      return KVSWAP_ERR_CUDA;
-    const bool probed = probe_opt != nullptr && probe_opt->layer == l;
-    const void* ql = static_cast<const char*>(q) + size_t(l) * q_bytes;
-    const void* Kl = tiers ? tiers->K_reuse[l] : layers->K[l];
-    const void* Vl = tiers ? tiers->V_reuse[l] : layers->V[l];
-    const int32_t* list_l = (tiers ? tiers->slot_idx : group_idx) + size_t(l) * idx_elems;
-    const int r = kvswap_sparse_decode(&shape_settled, ql, Kl, Vl, list_l, n_selected + size_t(l) * nsel_elems,
-                                       out + size_t(l) * out_elems,
-                                       lse_opt ? lse_opt + size_t(l) * p.B * p.Hq : nullptr, ws_attn, ws_attn_bytes,
-                                       cuda_stream);
-    if (probed && probe_opt->ev_end) cudaEventRecord(static_cast<cudaEvent_t>(probe_opt->ev_end), stream);
-    if (bounded && r == KVSWAP_OK && cudaEventRecord(res->attended[l], stream) != cudaSuccess)
-      return KVSWAP_ERR_CUDA;
-    return r;
-  };
-
-  // Host order: a predictor is handed to its stream before the wait on its selection is enqueued
-  // (join - 1 layers ahead at least), up to kHostLead layers ahead of the attention that consumes
-  // it, and never before the attention whose event it waits on (look - join + 1 at most).
-  const int lead = std::max(join - 1, std::min(look - join + 1, kHostLead));
-  int status = KVSWAP_OK;
-  int next_pred = 0;
+  int status = predict_and_fetch(0);
   for (int l = 0; l < L && status == KVSWAP_OK; ++l) {
-    while (status == KVSWAP_OK && next_pred < L && next_pred <= l - l % join + lead)
-      status = enqueue_predictor(next_pred++);
-    if (status == KVSWAP_OK) status = enqueue_attention(l);
+    if (l + 1 < L) status = predict_and_fetch(l + 1);
+    if (status != KVSWAP_OK) break;
+    if (cudaStreamWaitEvent(stream, res->fetched[l], 0) != cudaSuccess) { status = KVSWAP_ERR_CUDA; break; }
+    status = kvswap_sparse_decode(&shape_settled, static_cast<const char*>(q) + size_t(l) * q_bytes, tiers->K_reuse[l],
+                                  tiers->V_reuse[l], tiers->slot_idx + size_t(l) * idx_elems,
+                                  n_selected + size_t(l) * nsel_elems, out + size_t(l) * out_elems,
+                                  lse_opt ? lse_opt + size_t(l) * p.B * p.Hq : nullptr, ws_attn, ws_attn_bytes, cuda_stream);
   }
   if (status != KVSWAP_OK) {
-    // a launch failed: join whatever the predictor stream was given after its last awaited event
-    if (cudaEventRecord(res->fork, pred) != cudaSuccess || cudaStreamWaitEvent(stream, res->fork, 0) != cudaSuccess)
-      return KVSWAP_ERR_CUDA;
+    // a launch failed: join whatever the fetch streams were given after their last awaited events
+    for (cudaStream_t f : res->fetch)
+      if (cudaEventRecord(res->join, f) != cudaSuccess || cudaStreamWaitEvent(stream, res->join, 0) != cudaSuccess)
+        return KVSWAP_ERR_CUDA;
   }
   return status;
 }
