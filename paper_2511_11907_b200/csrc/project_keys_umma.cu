@@ -26,7 +26,9 @@
 
 #include "async_copy.cuh"
 #include "common.cuh"
+#include "project_keys_short.cuh"
 #include "tensor_map.cuh"
+#include "umma.cuh"
 
 namespace kvswap {
 namespace {
@@ -111,50 +113,6 @@ split_adapter_kernel(const float* __restrict__ proj, T* __restrict__ bsplit, flo
   }
 }
 
-// ---- PTX wrappers ------------------------------------------------------------------------------
-// K-major operand tile with 128-byte swizzle: rows of 128 bytes, groups of 8 rows 1024 bytes apart.
-__device__ __forceinline__ uint64_t umma_desc(uint32_t smem_byte_addr) {
-  return uint64_t((smem_byte_addr >> 4) & 0x3fffu) | (uint64_t(1) << 16) | (uint64_t(1024 >> 4) << 32) |
-         (uint64_t(1) << 46) | (uint64_t(2) << 61);
-}
-__device__ __forceinline__ void umma_16bit(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[32]) { tmem_ld32(taddr, v); }
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[16]) { tmem_ld16(taddr, v); }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
 struct UmmaShared {
   unsigned long long full[kMaxStages];     // stage loaded (TMA bytes)
   unsigned long long empty[kMaxStages];    // stage consumed (MMA commit)
@@ -190,8 +148,7 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
     mbar_init_fence();
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&sh.tmem_base)), "r"(kTmemCols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    tmem_alloc(smem_addr(&sh.tmem_base), kTmemCols);
   }
   tc_fence_before();
   __syncthreads();
@@ -252,9 +209,7 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
   } else if (warp == 1) {
     // ================================ MMA issuer ============================================
     if (lane == 0) {
-      // M = 128, N = 3r, fp32 accumulate, both operands bf16 (1) or both fp16 (0), K-major
-      constexpr uint32_t kFormat = kScaled ? 0u : 1u;
-      constexpr uint32_t idesc = (1u << 4) | (kFormat << 7) | (kFormat << 10) | (uint32_t(kNcols >> 3) << 17) | (uint32_t(kTileM >> 4) << 24);
+      constexpr uint32_t idesc = umma_idesc(kScaled, kNcols);
       for (int s = 0; s < n_steps; ++s) {
         const int stage = s % kStages, use = s / kStages, buf = s & 1, acc_use = s >> 1;
         if (acc_use > 0 && !mbar_wait(smem_addr(&sh.acc_empty[buf]), uint32_t(acc_use - 1) & 1u)) { sh.abort = 1; if (err) atomicExch(err, kDevTimeoutEmpty); break; }
@@ -356,7 +311,7 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    tmem_free(tmem, kTmemCols);
   }
 }
 
@@ -401,19 +356,24 @@ cudaError_t launch_umma(const Problem& p, const CUtensorMap& map_k, const CUtens
 // Returns true (and sets *result) when this path took the problem.
 bool try_launch_project_keys_umma(const Problem& p, const void* K, const float* proj, void* meta, int n_begin,
                                   int n_end, void* scratch, uint32_t* err, cudaStream_t st, cudaError_t* result) {
-  if (scratch == nullptr || project_keys_umma_scratch_bytes(p) == 0) return false;
-  if (p.meta_dtype == KVSWAP_E4M3 && p.r != 32) return false;
-  // Heads of 64 channels are multiplied in pairs where one metadata row sums all heads; alone they
-  // leave each stage half as much to do, and at r = 16 the warp-level kernel is the faster one.
-  const bool pair = p.d == 64 && p.Hm == 1 && p.Hkv % 2 == 0;
-  if (p.d == 64 && !pair && p.r == 16) return false;
+  if (!umma_shape(p) || (p.meta_dtype == KVSWAP_E4M3 && p.r != 32)) return false;
   if (p.kv_sn != p.d && (p.kv_sn * 2) % 16 != 0) return false;
   EncodeTiledFn enc = tensor_map_encoder();
   if (enc == nullptr) return false;
+  ShortPlan sp;
+  const bool is_short = plan_project_keys_short(p, n_begin, n_end, &sp);        // needs no scratch
+  // Heads of 64 channels are multiplied in pairs where one metadata row sums all heads; alone they
+  // leave each stage half as much to do, and at r = 16 the warp-level kernel is the faster one.
+  const bool pair = p.d == 64 && p.Hm == 1 && p.Hkv % 2 == 0;
+  if (!is_short && (scratch == nullptr || (p.d == 64 && !pair && p.r == 16))) return false;
   const int ncols = 3 * p.r;
   const bool bf16 = p.kv_dtype == KVSWAP_BF16;
   CUtensorMap map_k, map_b;
   if (!make_rows_tensor_map(&map_k, K, 2, bf16, p.d, p.N, p.Hkv, p.B, p.kv_sn, p.kv_sh, p.kv_sb, kTileM)) return false;
+  if (is_short) {
+    *result = launch_project_keys_short(p, sp, map_k, proj, meta, n_begin, n_end, err, st);
+    return true;
+  }
   {
     const cuuint64_t dims[2] = {cuuint64_t(p.d), cuuint64_t(p.Hkv) * ncols};
     const cuuint64_t strides[1] = {cuuint64_t(p.d) * 2};

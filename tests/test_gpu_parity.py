@@ -524,6 +524,26 @@ def test_project_keys_of_a_few_tokens(kv_type, meta, head_dim, rank, meta_heads,
     assert np.all(np.abs(got[:, :, 70:70 + n].astype(np.float64) - meta_or[:, :, 70:70 + n].astype(np.float64)) <= tol[:, :, 70:70 + n])
 
 
+@pytest.mark.parametrize("kv_type,meta,head_dim,rank,Hkv,mh,B,N", [
+    (W.BF16, W.F16, 128, 32, 8, 1, 1, 5003), (W.F16, W.F16, 128, 32, 8, 8, 1, 3001), (W.F16, W.F32, 64, 64, 4, 1, 2, 1300),
+    (W.BF16, W.F32, 128, 16, 3, 1, 1, 2000), (W.BF16, W.F16, 64, 16, 3, 3, 2, 700), (W.F16, W.F16, 128, 64, 2, 1, 1, 257),
+    (W.BF16, W.F16, 128, 32, 8, 1, 3, 4800), (W.F16, W.F16, 64, 32, 8, 1, 4, 7200), (W.F16, W.F16, 128, 64, 4, 4, 3, 3300)])
+def test_project_keys_short_and_persistent(kv_type, meta, head_dim, rank, Hkv, mh, B, N):
+    """Prompts whose (tile, head) pairs all get a CTA (one head or several per CTA, one to eight CTAs per tile) and, in
+    the last three, more of them than fit at once: those take the persistent kernel."""
+    wl = small(kv_dtype=kv_type, q_dtype=kv_type, meta_dtype=meta, head_dim=head_dim, rank=rank, group_size=8, n_ctx=N,
+               n_q_heads=Hkv, n_kv_heads=Hkv, batch=B, calib_rows=max(512, Hkv * head_dim))
+    li = W.make_layer(wl, 0, mh)
+    dl = DeviceLayer(li, KV)
+    meta_or = O.project_keys(li.K, li.proj, mh, META_NAME[meta])
+    tol = project_tolerance(li.K, li.proj, mh, meta_or, meta)
+    for _ in range(2):                                       # back to back: the second call finds the first one's operands
+        kv.kvswap_project_keys(dl.shape, dl.K, dl.proj, dl.meta, 0, N, dl.ws)
+    got = dl.project(n_begin=0, n_end=N)
+    assert np.all(np.abs(got.astype(np.float64) - meta_or.astype(np.float64)) <= tol)
+    assert kv.kvswap_read_device_status(dl.ws) == 0
+
+
 def test_strided_kv_and_metadata_views():
     """K and V interleaved in one buffer (row stride 2d) and metadata rows padded."""
     wl = small(kv_dtype=W.BF16, q_dtype=W.BF16, meta_dtype=W.F16, head_dim=128, rank=32, n_ctx=517, group_size=8)
