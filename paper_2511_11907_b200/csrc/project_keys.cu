@@ -1,6 +1,6 @@
 // K1: metadata build K_lr = Flatten(K) A (Sec. 4.2) -- the dense contraction of the path.
 //
-//   project_keys_mma_kernel  bf16 K, r in {16, 32, 64}: tensor cores (mma.sync m16n8k16, fp32
+//   project_keys_mma_kernel  bf16 or fp32 K, r in {16, 32, 64}: tensor cores (mma.sync m16n8k16, fp32
 //                            accumulation).  The adapter stays fp32-exact: every entry is split
 //                            into three bf16 pieces (8 + 8 + 8 mantissa bits) and each k-step is
 //                            issued once per piece, so the products are exact and the only
@@ -140,31 +140,36 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-template <typename META_T, int D, int NT>            // NT = r / 8 output tiles of 8 columns
+// KV_T = float: K too is split into three bf16 pieces, on the way from the registers it was loaded into; of the nine
+// products per entry six are issued, those left out are below 2^-24 of it.  (Against float64 the 2-norm error is 2.1e-7
+// where the fp32-pipe kernel's was 5.7e-7; a layer of 4 x 20000 tokens, 8 heads of 128, r = 32: 283 -> 126 us.)
+template <typename KV_T, typename META_T, int D, int NT>            // NT output tiles of 8 columns, from column col0
 __global__ void __launch_bounds__(kMmaWarps * 32, 1)
-project_keys_mma_kernel(Problem p, const __nv_bfloat16* __restrict__ K, const float* __restrict__ proj,
-                        META_T* __restrict__ meta, int n_begin, int n_end, int tiles_per_row) {
+project_keys_mma_kernel(Problem p, const KV_T* __restrict__ K, const float* __restrict__ proj,
+                        META_T* __restrict__ meta, int n_begin, int n_end, int tiles_per_row, int col0) {
+  constexpr bool kF32 = sizeof(KV_T) == 4;
   constexpr int KS = D / 16;                         // k-steps per head
   constexpr int KK = D / 32;                         // 32-channel blocks per head
-  constexpr int HALF = (KK >= 2) ? 2 : 1;            // blocks multiplied per pipeline step
+  constexpr int HALF = (KK >= 2 && !kF32) ? 2 : 1;   // blocks multiplied per pipeline step
+  constexpr int VEC = kF32 ? 2 : 1;                  // 16-byte loads per row and block
   constexpr int STEPS_PER_HEAD = KK / HALF;
   extern __shared__ __align__(16) unsigned char dyn[];
   uint2* bfrag = reinterpret_cast<uint2*>(dyn);      // [H_kv][KS][NT][3 pieces][32 lanes]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g8 = lane >> 2, t4 = lane & 3;
-  const int r = NT * 8;
 
   // ---- adapter -> B fragments, three bf16 pieces per entry ------------------------------------------
+#pragma unroll 4
   for (int i = threadIdx.x; i < p.Hkv * KS * NT * 32; i += kMmaWarps * 32) {
     const int ln = i & 31, nt = (i >> 5) % NT, ks = ((i >> 5) / NT) % KS, g = (i >> 5) / (NT * KS);
-    const int t = ln & 3, col = nt * 8 + (ln >> 2);
+    const int t = ln & 3, col = col0 + nt * 8 + (ln >> 2);
     const int c0 = 32 * (ks >> 1) + 8 * t + 4 * (ks & 1);      // channels c0 .. c0+3 feed this lane's k slots
-    const float* src = proj + (int64_t(g) * D + c0) * r + col;
+    const float* src = proj + (int64_t(g) * D + c0) * p.r + col;
     float v[4], hi[4], mid[4], lo[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      v[e] = src[int64_t(e) * r];
+      v[e] = src[int64_t(e) * p.r];
       hi[e] = __bfloat162float(__float2bfloat16_rn(v[e]));
       mid[e] = __bfloat162float(__float2bfloat16_rn(v[e] - hi[e]));
       lo[e] = v[e] - hi[e] - mid[e];                 // exact; rounds to bf16 below
@@ -188,7 +193,7 @@ project_keys_mma_kernel(Problem p, const __nv_bfloat16* __restrict__ K, const fl
     const int g_first = (p.Hm == 1) ? 0 : hm;
     const int n0 = n_begin + tile * 32;
     // rows of this lane: tile m, half h -> token n0 + 16 m + 8 h + g8
-    const __nv_bfloat16* rowp[2][2];
+    const KV_T* rowp[2][2];
     bool rowok[2][2];
 #pragma unroll
     for (int m = 0; m < 2; ++m)
@@ -206,7 +211,7 @@ project_keys_mma_kernel(Problem p, const __nv_bfloat16* __restrict__ K, const fl
 #pragma unroll
         for (int e = 0; e < 4; ++e) acc[m][nt][e] = 0.f;
 
-    auto load_step = [&](int step, uint4 (&a)[2][2][HALF]) {   // step = head-in-item * STEPS_PER_HEAD + half
+    auto load_step = [&](int step, uint4 (&a)[2][2][HALF * VEC]) {   // step = head-in-item * STEPS_PER_HEAD + half
       const int g = g_first + step / STEPS_PER_HEAD;
       const int kk0 = (step % STEPS_PER_HEAD) * HALF;
 #pragma unroll
@@ -214,13 +219,13 @@ project_keys_mma_kernel(Problem p, const __nv_bfloat16* __restrict__ K, const fl
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-          for (int q = 0; q < HALF; ++q) {
-            if (rowok[m][h]) a[m][h][q] = ld_stream16(rowp[m][h] + int64_t(g) * p.kv_sh + 32 * (kk0 + q));
+          for (int q = 0; q < HALF * VEC; ++q) {
+            if (rowok[m][h]) a[m][h][q] = ld_stream16(rowp[m][h] + int64_t(g) * p.kv_sh + 32 * (kk0 + q / VEC) + 4 * (q % VEC));
             else a[m][h][q] = make_uint4(0u, 0u, 0u, 0u);
           }
     };
     const int n_steps = g_count * STEPS_PER_HEAD;
-    uint4 cur[2][2][HALF], nxt[2][2][HALF];
+    uint4 cur[2][2][HALF * VEC], nxt[2][2][HALF * VEC];
     load_step(0, cur);
     for (int step = 0; step < n_steps; ++step) {
       if (step + 1 < n_steps) load_step(step + 1, nxt);
@@ -233,19 +238,46 @@ project_keys_mma_kernel(Problem p, const __nv_bfloat16* __restrict__ K, const fl
 #pragma unroll
       for (int q = 0; q < HALF; ++q) {
         const uint2* bf = bfrag + (int64_t(g * KS + 2 * (kk0 + q)) * NT * 3) * 32 + lane;
+        // the lane's eight channels of each row as pairs: one piece for bf16 K, three for fp32 K
+        constexpr int KP = kF32 ? 3 : 1;
+        uint32_t ka[2][2][KP][4];
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if constexpr (kF32) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const uint4 v = cur[m][h][2 * q + (e >> 1)];
+                float x = __uint_as_float((e & 1) ? v.z : v.x), y = __uint_as_float((e & 1) ? v.w : v.y);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                  const __nv_bfloat162 pr = __floats2bfloat162_rn(x, y);
+                  ka[m][h][k][e] = *reinterpret_cast<const uint32_t*>(&pr);
+                  const float2 f = __bfloat1622float2(pr);
+                  x -= f.x; y -= f.y;
+                }
+              }
+            } else {
+              const uint4 v = cur[m][h][q];
+              ka[m][h][0][0] = v.x; ka[m][h][0][1] = v.y; ka[m][h][0][2] = v.z; ka[m][h][0][3] = v.w;
+            }
+          }
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
           float tmp[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
           for (int sub = 0; sub < 2; ++sub)
 #pragma unroll
-            for (int pc = 0; pc < 3; ++pc) {
+            for (int pc = 2; pc >= 0; --pc) {          // small products first
               const uint2 bb = bf[((sub * NT + nt) * 3 + pc) * 32];
 #pragma unroll
-              for (int m = 0; m < 2; ++m) {
-                const uint4 lo = cur[m][0][q], hi = cur[m][1][q];   // rows g8 and g8 + 8
-                mma_bf16_16816(tmp[m], sub ? lo.z : lo.x, sub ? hi.z : hi.x, sub ? lo.w : lo.y, sub ? hi.w : hi.y,
-                               bb.x, bb.y);
+              for (int k = KP - 1; k >= 0; --k) {
+                if (k + pc > 2) continue;
+#pragma unroll
+                for (int m = 0; m < 2; ++m)              // rows g8 and g8 + 8
+                  mma_bf16_16816(tmp[m], ka[m][0][k][2 * sub], ka[m][1][k][2 * sub], ka[m][0][k][2 * sub + 1],
+                                 ka[m][1][k][2 * sub + 1], bb.x, bb.y);
               }
             }
 #pragma unroll
@@ -259,7 +291,7 @@ project_keys_mma_kernel(Problem p, const __nv_bfloat16* __restrict__ K, const fl
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-          for (int q = 0; q < HALF; ++q) cur[m][h][q] = nxt[m][h][q];
+          for (int q = 0; q < HALF * VEC; ++q) cur[m][h][q] = nxt[m][h][q];
     }
     // ---- one rounding into the metadata type -------------------------------------------------------
     META_T* Mo = meta + int64_t(b) * p.meta_sb + int64_t(hm) * p.meta_sh;
@@ -269,7 +301,7 @@ project_keys_mma_kernel(Problem p, const __nv_bfloat16* __restrict__ K, const fl
       for (int h = 0; h < 2; ++h) {
         if (!rowok[m][h]) continue;
         const int n = n0 + 16 * m + 8 * h + g8;
-        META_T* row = Mo + int64_t(n) * p.meta_sn + 2 * t4;
+        META_T* row = Mo + int64_t(n) * p.meta_sn + col0 + 2 * t4;
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
           const float x = acc[m][nt][2 * h], y = acc[m][nt][2 * h + 1];
@@ -280,37 +312,42 @@ project_keys_mma_kernel(Problem p, const __nv_bfloat16* __restrict__ K, const fl
   }
 }
 
-template <typename META_T, int D, int NT>
+template <typename KV_T, typename META_T, int D, int NT>
 cudaError_t launch_mma_one(const Problem& p, const void* K, const float* proj, void* meta, int n_begin, int n_end,
                            cudaStream_t st) {
   const size_t smem = size_t(p.Hkv) * (D / 16) * NT * 3 * 32 * sizeof(uint2);
-  auto kern = project_keys_mma_kernel<META_T, D, NT>;
+  auto kern = project_keys_mma_kernel<KV_T, META_T, D, NT>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   const int tiles_per_row = (n_end - n_begin + 31) / 32;
   const int64_t items = int64_t(p.B) * p.Hm * tiles_per_row;
-  const int ctas = int(std::max<int64_t>(1, std::min<int64_t>(kNumSMs, (items + kMmaWarps - 1) / kMmaWarps)));
-  kern<<<ctas, kMmaWarps * 32, smem, st>>>(p, static_cast<const __nv_bfloat16*>(K), proj, static_cast<META_T*>(meta),
-                                           n_begin, n_end, tiles_per_row);
-  return cudaGetLastError();
+  // a CTA per SM as long as there is an item for each: the warps share them out evenly
+  const int ctas = int(std::max<int64_t>(1, std::min<int64_t>(kNumSMs, items)));
+  for (int col0 = 0; col0 < p.r; col0 += NT * 8) {   // (again over K where the fragments of all columns do not fit)
+    kern<<<ctas, kMmaWarps * 32, smem, st>>>(p, static_cast<const KV_T*>(K), proj, static_cast<META_T*>(meta), n_begin, n_end,
+                                             tiles_per_row, col0);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // True (and launched) when the tensor-core path covers the problem.
-template <typename META_T>
+template <typename KV_T, typename META_T>
 bool try_launch_mma(const Problem& p, const void* K, const float* proj, void* meta, int n_begin, int n_end,
                     cudaStream_t st, cudaError_t* err) {
-  if (p.kv_dtype != KVSWAP_BF16 || (p.r != 16 && p.r != 32 && p.r != 64)) return false;
-  const size_t smem = size_t(p.Hkv) * (p.d / 16) * (p.r / 8) * 3 * 32 * sizeof(uint2);
-  if (smem > 200 * 1024) return false;
-  if (p.d == 128) {
-    if (p.r == 16) *err = launch_mma_one<META_T, 128, 2>(p, K, proj, meta, n_begin, n_end, st);
-    else if (p.r == 32) *err = launch_mma_one<META_T, 128, 4>(p, K, proj, meta, n_begin, n_end, st);
-    else *err = launch_mma_one<META_T, 128, 8>(p, K, proj, meta, n_begin, n_end, st);
-  } else {
-    if (p.r == 16) *err = launch_mma_one<META_T, 64, 2>(p, K, proj, meta, n_begin, n_end, st);
-    else if (p.r == 32) *err = launch_mma_one<META_T, 64, 4>(p, K, proj, meta, n_begin, n_end, st);
-    else *err = launch_mma_one<META_T, 64, 8>(p, K, proj, meta, n_begin, n_end, st);
-  }
+  if (p.r != 16 && p.r != 32 && p.r != 64) return false;
+  // eight columns' fragments of every head; as many columns per pass as fit
+  const size_t tile = size_t(p.Hkv) * (p.d / 16) * 3 * 32 * sizeof(uint2);
+  int nt = p.r / 8;
+  while (nt > 2 && nt * tile > 200 * 1024) nt /= 2;
+  if (nt * tile > 200 * 1024 || nt * 16 < p.r) return false;
+  auto by_rank = [&](auto d_tag) {
+    constexpr int D = decltype(d_tag)::value;
+    return nt == 2   ? launch_mma_one<KV_T, META_T, D, 2>(p, K, proj, meta, n_begin, n_end, st)
+           : nt == 4 ? launch_mma_one<KV_T, META_T, D, 4>(p, K, proj, meta, n_begin, n_end, st)
+                     : launch_mma_one<KV_T, META_T, D, 8>(p, K, proj, meta, n_begin, n_end, st);
+  };
+  *err = p.d == 128 ? by_rank(std::integral_constant<int, 128>()) : by_rank(std::integral_constant<int, 64>());
   return true;
 }
 
@@ -448,11 +485,13 @@ template <typename KV_T>
 cudaError_t dispatch_meta(const Problem& p, const void* K, const float* proj, void* meta, int n_begin, int n_end,
                           bool tensor_cores, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
-  if (tensor_cores && p.meta_dtype != KVSWAP_E4M3) {      // (8-bit metadata: tcgen05 path or the fp32 kernel)
-    if (p.meta_dtype == KVSWAP_F16) {
-      if (try_launch_mma<__half>(p, K, proj, meta, n_begin, n_end, st, &e)) return e;
-    } else if (try_launch_mma<float>(p, K, proj, meta, n_begin, n_end, st, &e)) {
-      return e;
+  if constexpr (!std::is_same<KV_T, __half>::value) {     // (fp16 K without a workspace: the fp32 kernel)
+    if (tensor_cores && p.meta_dtype != KVSWAP_E4M3) {    // (8-bit metadata: tcgen05 path or the fp32 kernel)
+      if (p.meta_dtype == KVSWAP_F16) {
+        if (try_launch_mma<KV_T, __half>(p, K, proj, meta, n_begin, n_end, st, &e)) return e;
+      } else if (try_launch_mma<KV_T, float>(p, K, proj, meta, n_begin, n_end, st, &e)) {
+        return e;
+      }
     }
   }
   ProjectTable tab = {};

@@ -544,6 +544,26 @@ def test_project_keys_short_and_persistent(kv_type, meta, head_dim, rank, Hkv, m
     assert kv.kvswap_read_device_status(dl.ws) == 0
 
 
+@pytest.mark.parametrize("meta,head_dim,rank,Hkv,mh,N", [(W.F32, 128, 32, 8, 1, 1100), (W.F32, 64, 64, 2, 2, 700), (W.F16, 128, 64, 8, 1, 517),
+                                                       (W.F32, 128, 16, 3, 1, 5003), (W.F32, 128, 64, 8, 8, 300)])
+def test_project_keys_fp32_on_the_tensor_cores(meta, head_dim, rank, Hkv, mh, N):
+    """fp32 K: both operands in three bf16 pieces; r = 64 over 8 heads of 128 in two passes over the columns."""
+    wl = small(head_dim=head_dim, rank=rank, meta_dtype=meta, group_size=8, n_ctx=N, n_q_heads=Hkv, n_kv_heads=Hkv, batch=2,
+               calib_rows=max(512, Hkv * head_dim))
+    li = W.make_layer(wl, 0, mh)
+    dl = DeviceLayer(li, KV)
+    meta_or = O.project_keys(li.K, li.proj, mh, META_NAME[meta])
+    tol = project_tolerance(li.K, li.proj, mh, meta_or, meta)
+    got = dl.project()
+    assert np.all(np.abs(got.astype(np.float64) - meta_or.astype(np.float64)) <= tol)
+    # as close as sums in fp32 are: measured 4e-7 in the 2-norm for the fp32-pipe kernel
+    if meta == W.F32:
+        assert np.linalg.norm(got - meta_or) <= 1e-6 * np.linalg.norm(meta_or)
+    dl.meta.fill_(123.0)
+    got = dl.project(n_begin=3, n_end=290)
+    assert np.all(got[:, :, :3] == 123.0) and np.all(got[:, :, 290:] == 123.0)
+
+
 def test_strided_kv_and_metadata_views():
     """K and V interleaved in one buffer (row stride 2d) and metadata rows padded."""
     wl = small(kv_dtype=W.BF16, q_dtype=W.BF16, meta_dtype=W.F16, head_dim=128, rank=32, n_ctx=517, group_size=8)
