@@ -54,10 +54,11 @@ struct ScoreSmem {
   unsigned char tiles[kScoreWarps * kScoreDepth * ScoreStage<META, R, GS>::kBytes];      // 128 KB of stages, or 96
   uint32_t hist[kHistWords];                              // 64 KB
   unsigned long long full[kScoreWarps * kScoreDepth];
-  float qsum[kQuerySumFloats];                            // scratch of build_queries
-  float upart[kQueryPartFloats];
   float urow[kMaxSets][kScoreCols * R];                   // summed low-rank queries per row set of the CTA
-  float sc[GS >= 0 ? 4 : kScoreWarps * kScoreCols * generic_pitch(ScoreStage<META, R, GS>::kRows)];
+  static constexpr int kScratch = kQuerySumFloats + kQueryPartFloats;
+  // scratch of build_queries (qsum, then upart), afterwards the warps' score buffers
+  static constexpr int kBuffers = GS >= 0 ? 0 : kScoreWarps * kScoreCols * generic_pitch(ScoreStage<META, R, GS>::kRows);
+  float sc[kBuffers > kScratch ? kBuffers : kScratch];
 };
 
 struct StreamArgs {
@@ -168,7 +169,7 @@ score_stream_kernel(Problem p, StreamArgs a) {
   if (!settled) pdl_wait();
   if constexpr (FUSED) {
     for (int s = 0; s < n_sets; ++s)
-      build_queries<0, R>(p, a.q, a.proj, row_set(p, rest0 + s, a.n_sub), sm->qsum, sm->upart, sm->urow[s]);
+      build_queries<0, R>(p, a.q, a.proj, row_set(p, rest0 + s, a.n_sub), sm->sc, sm->sc + kQuerySumFloats, sm->urow[s]);
   }
   if (settled) pdl_wait();
   pdl_trigger();

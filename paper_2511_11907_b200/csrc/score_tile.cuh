@@ -263,8 +263,8 @@ __device__ __forceinline__ void score_tile_groups(uint32_t base, int rows, int l
 // Rows of one stage: 4 KB where a finished score leaves the registers (the hand-over of a stage costs the
 // same whatever its size: 4 KB x 2 stages measured 1.3 us per layer faster than 2 KB x 4 at B = 4,
 // N = 131072); GS = -1 takes 3 KB, which leaves room for the warps' score buffers.  A stage is read eight rows at
-// a time, whole: it holds a multiple of eight, which for rows of 256 bytes takes 4 KB.
-__host__ __device__ constexpr int score_stage_bytes(bool generic, int row_bytes) { return generic && row_bytes <= 128 ? 3072 : 4096; }
+// a time, whole: it holds a multiple of eight, which for rows of 256 bytes takes 4 KB; so do 32 rows of 128 bytes.
+__host__ __device__ constexpr int score_stage_bytes(bool generic, int row_bytes) { return generic && row_bytes < 128 ? 3072 : 4096; }
 __host__ __device__ constexpr int score_stage_rows(bool generic, int row_bytes) {
   const int fit = score_stage_bytes(generic, row_bytes) / row_bytes;
   return generic && fit > kGenericRows ? kGenericRows : fit;

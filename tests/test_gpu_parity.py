@@ -456,6 +456,8 @@ STREAM = [   # K/V type, metadata type, rank, G, per-head, scope, B, H_kv, rho, 
     (W.F32, W.F32, 64, 12, True, KV, 2, 2, 2, 12 * 70 + 5),
     (W.F32, W.F32, 64, 4, True, ALL, 1, 4, 1, 12 * 60 + 7),
     (W.F32, W.F32, 64, 32, False, KV, 1, 2, 2, 999),       # a group that does not fit a stage
+    (W.BF16, W.F16, 64, 32, True, ALL, 2, 8, 1, 32 * 61 + 7),
+    (W.F32, W.F32, 32, 31, False, KV, 1, 2, 2, 31 * 40 + 3),
 ]
 
 
