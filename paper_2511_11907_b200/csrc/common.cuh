@@ -36,7 +36,10 @@ struct Problem {
 // kFlagInputsTwoBack, on the TopK enqueued behind such a gather: its scores and counts were complete
 // before the gather's wait returned, i.e. before any of its own CTAs started, and nothing it writes is
 // touched by the gather: it does not wait at all.
+// kFlagWaitLate, on it too: everything it writes over or may be read by was finished before any of its CTAs started, so
+// the dependency wait comes last, for those that wait on this kernel.
 constexpr int kFlagWaitEarly = 1 << 16;
+constexpr int kFlagWaitLate = 1 << 18;
 constexpr int kFlagInputsTwoBack = 1 << 17;
 
 // Partition of the caller's workspace (byte offsets, each 256-byte aligned).
@@ -53,6 +56,7 @@ struct Workspace {
   int splits_room;     // splits the partials are planned for (whatever the flags of a call)
   int heads_per_cta;   // query heads sharing one K/V pass in sparse_decode
   int depth;           // shared-memory stages per compute warp in sparse_decode
+  bool beside;         // a decode step runs the gather beside the next layer's one-launch predictor (splits planned for what that leaves)
   bool merge_in_cluster;   // sparse_decode on its own: the splits of a list form a cluster that merges them (no combine pass)
 };
 

@@ -440,6 +440,7 @@ sparse_decode_splitk_kernel(Problem p, const Q_T* __restrict__ q, const KV_T* __
   // which the previous launch's combine may still be reading) have to wait for it.
   const bool settled = (p.flags & KVSWAP_INPUTS_SETTLED) != 0;
   const bool wait_early = settled && (p.flags & kFlagWaitEarly) != 0;
+  const bool wait_late = settled && (p.flags & kFlagWaitLate) != 0;
   if (!settled) pdl_wait();
   if (!wait_early) pdl_trigger();
 
@@ -562,7 +563,7 @@ sparse_decode_splitk_kernel(Problem p, const Q_T* __restrict__ q, const KV_T* __
   float* sm_acc = sm_l + kWarps * 8;                                // [kWarps][RH][D]
   eng.store(sm_m + warp * 8, sm_l + warp * 8, sm_acc + warp * RH * D);
   __syncthreads();
-  if (settled && !wait_early) pdl_wait();
+  if (settled && !wait_early && !wait_late) pdl_wait();
   // partial [RH][D + 2] = (m, l, acc[D]) of this split: to the caller's scratch for the combine pass, or, when
   // the splits of a list are the CTAs of one cluster, to shared memory for the merge below
   float* const sm_part = sm_acc + kWarps * RH * D;
@@ -629,6 +630,7 @@ sparse_decode_splitk_kernel(Problem p, const Q_T* __restrict__ q, const KV_T* __
   cluster_arrive();
   cluster_wait();                                  // no CTA leaves while a peer may still read its partial
   }
+  if (wait_late) pdl_wait();
 }
 
 // K5: merge the split partials of one (sequence, head): one CTA of D threads per row (combine.cuh).
@@ -742,7 +744,7 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
   };
   const int64_t slots = 2 * kNumSMs;
   int64_t best = best_splits(slots, 256);
-  w->merge_in_cluster = false;
+  w->merge_in_cluster = w->beside = false;
   w->splits_room = int(best);
   ClusterGrid predictor;
   if (score_select_cluster_grid(p, &predictor)) {
@@ -764,9 +766,19 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
     }
     if (m < 2 && most >= 2 && problems * 2 <= 264) m = 2;      // pairs find room anywhere
     // What fewer splits cost must stay below what the two launches cost (about 16 chunk times).
+    const int held = predictor.clusters * predictor.ctas * (predictor.whole_sm ? 2 : 1);
     if (m > 0 && split_cost(m, slots) - split_cost(best, slots) <= 16) {
       best = m;
       w->merge_in_cluster = true;
+    } else if (held <= slots / 2) {
+      // Too long a list for that, but the gather still runs beside the predictor, in the slots it leaves, unless that
+      // makes it much longer: 12.3 against 15.7 us per layer at B = 2, N = 18546, 4 KV heads, 4608 tokens attended;
+      // with twice the chunks per CTA (B = 8, N = 16384, 8 heads, 2048 tokens) 28.5 against 27.6.
+      const int64_t s = best_splits(slots - held, 256);
+      if (split_cost(s, slots - held) - split_cost(best, slots) <= 16) {
+        best = s;
+        w->beside = true;
+      }
     }
   }
   w->splits = int(best);

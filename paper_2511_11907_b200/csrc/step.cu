@@ -258,7 +258,8 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
     // of predict(l) complete: attention(l - 1) waited for it before it wrote its results.  Two launches a layer
     // instead of three, and neither waits for the other: 36 layers of B = 1, N = 16384, 8 KV heads, M = 256 through
     // host memory 539 -> 430 us; at B = 1, N = 4096 a layer takes 8.5 us against 12.9.
-    if (score_select_cluster_supported(p) && w.merge_in_cluster) {
+    // Where the splits do not merge in clusters a combine follows each gather.
+    if (score_select_cluster_supported(p) && (w.merge_in_cluster || w.beside)) {
       auto predict = [&](int l) -> int {
         if (probed(l)) ev(probe_opt->ev_begin);
         const cudaError_t e = launch_score_select_cluster(
@@ -267,14 +268,18 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
         if (probed(l)) ev(probe_opt->ev_mid);
         return e == cudaSuccess ? KVSWAP_OK : KVSWAP_ERR_CUDA;
       };
+      // predict(l + 1) had waited for all that came before it when attention(l) was let in: that one waits last.
+      Problem p_late = p_settled;
+      p_late.flags |= kFlagWaitLate;
+      float* partial = w.merge_in_cluster ? nullptr : reinterpret_cast<float*>(static_cast<char*>(ws) + w.off_partial);
       int status = predict(0);
       for (int l = 0; l < L && status == KVSWAP_OK; ++l) {
         if (l + 1 < L) status = predict(l + 1);
         if (status != KVSWAP_OK) break;
         // (the last layer's attention follows an attention directly: its selection is complete when that one is)
         const cudaError_t e = launch_sparse_decode(
-            l + 1 < L ? p_settled : p, w, static_cast<const char*>(q) + size_t(l) * q_bytes, layers->K[l], layers->V[l],
-            group_idx + size_t(l) * idx_elems, n_selected + size_t(l) * nsel_elems, nullptr, out + size_t(l) * out_elems,
+            l + 1 < L ? p_late : p, w, static_cast<const char*>(q) + size_t(l) * q_bytes, layers->K[l], layers->V[l],
+            group_idx + size_t(l) * idx_elems, n_selected + size_t(l) * nsel_elems, partial, out + size_t(l) * out_elems,
             lse_opt ? lse_opt + size_t(l) * p.B * p.Hq : nullptr, static_cast<uint32_t*>(ws), stream);
         if (probed(l)) ev(probe_opt->ev_end);
         if (e != cudaSuccess) status = KVSWAP_ERR_CUDA;

@@ -105,14 +105,15 @@ def test_decode_step_head_dim_64(meta_heads):
     _run_case(wl, meta_heads, W.SCOPE_KV_HEAD)
 
 
-@pytest.mark.parametrize("n_ctx", [16384 + 5, 70000 + 5])    # one launch of clusters per predictor; scorer and TopK
+# one launch of clusters per predictor, its attention merging in clusters; the same with a combine; scorer and TopK
+@pytest.mark.parametrize("n_ctx,top_k", [(16384 + 5, 96), (16384 + 5, 700), (70000 + 5, 96)])
 @pytest.mark.parametrize("meta_heads", ["joint", "per_head"])
-def test_decode_steps_back_to_back_with_alternating_queries(meta_heads, n_ctx):
+def test_decode_steps_back_to_back_with_alternating_queries(meta_heads, n_ctx, top_k):
     """Steps enqueued without a pause, alternating between two query sets: inside a step the TopK of a
     layer does not wait for the gather before it, the scorer reads queries that the launch before it
     formed, and consecutive steps reuse the same workspace buffers -- every step must still give what
     the per-layer calls give for its queries."""
-    wl = W.CONFIGS[5].reduced("cfg5-soak", layers=6, batch=2, n_ctx=n_ctx, top_k=96, calib_rows=1024, walk_steps=2)
+    wl = W.CONFIGS[5].reduced("cfg5-soak", layers=6, batch=2, n_ctx=n_ctx, top_k=top_k, calib_rows=1024, walk_steps=2)
     dw = DW.build(wl, 1 if meta_heads == "joint" else wl.n_kv_heads, W.SCOPE_KV_HEAD, reserve_bytes=1 << 30)
     ws = rt.alloc_workspace(dw.shape)
     for l in range(wl.layers):
