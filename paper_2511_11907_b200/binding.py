@@ -1,4 +1,4 @@
-"""ctypes binding of libkvswap.so: argument marshalling only.
+"""Binding of libkvswap.so: argument marshalling only, through ctypes or, for the per-layer calls, natively.
 
 Every function has the name and argument order of its C entry point (include/kvswap.h).
 Tensors are torch CUDA tensors; the binding passes ``data_ptr()`` and the current CUDA stream
@@ -131,18 +131,42 @@ def _check(status: int, where: str) -> None:
         raise KVSwapError(status, where)
 
 
+def _entry_points():
+    """What the extension module needs for the per-layer calls; raises as load() does."""
+    import torch
+    lib = load()
+    addr = [ctypes.cast(f, ctypes.c_void_p).value for f in (lib.kvswap_project_keys, lib.kvswap_score_select,
+                                                            lib.kvswap_sparse_decode)]
+    return (*addr, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+
+
+# The per-layer calls, marshalled natively (csrc/pycalls.cpp); tensors or None, stream=None is torch's current one:
+#   kvswap_project_keys(shape, K, proj, meta_out, n_begin, n_end, ws, stream=None)
+#   kvswap_score_select(shape, q, proj, meta, group_idx, n_selected, group_scores_opt, ws, stream=None)
+#   kvswap_sparse_decode(shape, q, K, V, group_idx, n_selected, out, lse_opt, ws, stream=None)
+_NATIVE = ("kvswap_project_keys", "kvswap_score_select", "kvswap_sparse_decode")
+
+
+def __getattr__(name):
+    """Takes the per-layer calls from the extension module on their first use (it may be built after this import)."""
+    if name not in _NATIVE:
+        raise AttributeError(f"module {__name__!r} has no attribute {name!r}")
+    try:
+        from . import _calls
+    except ImportError as e:
+        raise RuntimeError("the binding's extension module is not built: build it with "
+                           "`python -m paper_2511_11907_b200.build`") from e
+    _calls.setup(_entry_points, KVSwapError)
+    globals().update({n: getattr(_calls, n) for n in _NATIVE})
+    return globals()[name]
+
+
 def kvswap_workspace_bytes(shape: kvswap_shape) -> int:
     return int(load().kvswap_workspace_bytes(ctypes.byref(shape)))
 
 
 def kvswap_validate_shape(shape: kvswap_shape) -> int:
     return int(load().kvswap_validate_shape(ctypes.byref(shape)))
-
-
-def kvswap_project_keys(shape, K, proj, meta_out, n_begin, n_end, ws, stream=None) -> None:
-    _check(load().kvswap_project_keys(ctypes.byref(shape), _ptr(K), _ptr(proj), _ptr(meta_out), int(n_begin),
-                                      int(n_end), _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(),
-                                      _stream(stream)), "kvswap_project_keys")
 
 
 def kvswap_append_kv(shape: kvswap_shape, k_new, v_new, K, V, proj, meta, stream=None) -> bool:
@@ -187,20 +211,6 @@ def reuse_attention_shape(shape: kvswap_shape, n_slots: int) -> kvswap_shape:
     other.n_ctx = n_slots * G + shape.n_ctx % G
     other.kv_stride_b, other.kv_stride_h, other.kv_stride_n = Hkv * R * d, R * d, d
     return other
-
-
-def kvswap_score_select(shape, q, proj, meta, group_idx, n_selected, group_scores_opt, ws, stream=None) -> None:
-    _check(load().kvswap_score_select(ctypes.byref(shape), _ptr(q), _ptr(proj), _ptr(meta), _ptr(group_idx),
-                                      _ptr(n_selected), _ptr(group_scores_opt), _ptr(ws),
-                                      0 if ws is None else ws.numel() * ws.element_size(), _stream(stream)),
-           "kvswap_score_select")
-
-
-def kvswap_sparse_decode(shape, q, K, V, group_idx, n_selected, out, lse_opt, ws, stream=None) -> None:
-    _check(load().kvswap_sparse_decode(ctypes.byref(shape), _ptr(q), _ptr(K), _ptr(V), _ptr(group_idx),
-                                       _ptr(n_selected), _ptr(out), _ptr(lse_opt), _ptr(ws),
-                                       0 if ws is None else ws.numel() * ws.element_size(), _stream(stream)),
-           "kvswap_sparse_decode")
 
 
 def kvswap_workspace_init(ws, stream=None) -> None:

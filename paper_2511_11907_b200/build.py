@@ -1,7 +1,8 @@
 """Builds libkvswap.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
 
 Usage:  python -m paper_2511_11907_b200.build [--force]
-Objects go to ``_build/`` at the repository root; the shared library lands next to this file.
+Objects go to ``_build/`` at the repository root; the shared library and the binding's extension module land next to
+this file.
 """
 from __future__ import annotations
 
@@ -10,6 +11,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -17,6 +19,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJ_DIR = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libkvswap.so")
+CALLS = os.path.join(PKG, "_calls.so")      # the binding's per-layer calls (csrc/pycalls.cpp), an extension module
 
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
               "-Xcompiler", "-fPIC", "--use_fast_math=false", "-I", INCLUDE, "-I", CSRC]
@@ -40,7 +43,7 @@ def _deps_mtime() -> float:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every .cu under csrc/ and link libkvswap.so; returns its path."""
-    if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _deps_mtime():
+    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= _deps_mtime() for f in (LIB, CALLS)):
         return LIB
     os.makedirs(OBJ_DIR, exist_ok=True)
     nvcc = _nvcc()
@@ -64,6 +67,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", INCLUDE, "-I", sysconfig.get_paths()["include"],
+           os.path.join(CSRC, "pycalls.cpp"), "-o", CALLS]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"g++ failed on pycalls.cpp:\n{res.stdout}\n{res.stderr}")
     return LIB
 
 
