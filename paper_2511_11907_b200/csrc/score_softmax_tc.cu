@@ -28,12 +28,24 @@ bool plan(const Problem& p, bool pool, bool counts, SoftmaxArgs* a, int* n_sets)
   const int64_t rows_total = int64_t(p.NG) * p.G;
   a->atomic = p.G > fit && (p.G > kSoftmaxMaxRows || p.G * row_bytes > 4096);
   a->tile_rows = !pool || a->atomic ? fit : p.G > fit ? p.G : fit / p.G * p.G;
+  const bool scoped = p.Hm == 1 && p.scope == KVSWAP_SCOPE_KV_HEAD;
+  a->n_sub = scoped ? (p.S + kSoftmaxScopes - 1) / kSoftmaxScopes : 1;
+  const int64_t sets = int64_t(p.B) * (pool ? scored_heads(p) * a->n_sub : p.Hm);
+  if (sets > (1 << 20)) return false;
+  // Where a warp gets few tiles, shorter ones even the warps out: a tile costs its rows and some eight rows' worth of
+  // hand-over.  (B = 4, N = 40001: three tiles of 24 rows instead of two of 48 in the longest share.)
+  if (p.G <= a->tile_rows && !a->atomic) {
+    const int64_t warps = std::max<int64_t>(1, kNumSMs / sets) * kSoftmaxWarps;
+    int best = a->tile_rows;
+    auto cost = [&](int rows) { return ((rows_total + rows - 1) / rows + warps - 1) / warps * (rows + 8); };
+    const int step = pool ? p.G : 8;
+    for (int rows = a->tile_rows - step; rows >= 16; rows -= step) if (cost(rows) < cost(best)) best = rows;
+    a->tile_rows = best;
+  }
   if ((rows_total + a->tile_rows - 1) / a->tile_rows > (1 << 28)) return false;
   a->tiles = int((rows_total + a->tile_rows - 1) / a->tile_rows);
   a->stage_bytes = (a->tile_rows + 7) / 8 * 8 * row_bytes;
   a->pitch = (a->tile_rows + 7) / 8 * 8 + 8;
-  const bool scoped = p.Hm == 1 && p.scope == KVSWAP_SCOPE_KV_HEAD;
-  a->n_sub = scoped ? (p.S + kSoftmaxScopes - 1) / kSoftmaxScopes : 1;
   a->p_shift = 3;
   if (!pool) {
     a->units = 1;
@@ -48,8 +60,6 @@ bool plan(const Problem& p, bool pool, bool counts, SoftmaxArgs* a, int* n_sets)
     a->units = scoped ? std::min(kSoftmaxScopes, p.S) : multi_term(p) ? p.Hkv : 1;
   }
   a->n_blocks = a->units * a->kb;
-  const int64_t sets = int64_t(p.B) * (pool ? scored_heads(p) * a->n_sub : p.Hm);
-  if (sets > (1 << 20)) return false;
   *n_sets = int(sets);
   a->ctas_per_set = int(std::max<int64_t>(1, std::min<int64_t>({kNumSMs / sets, (a->tiles + kSoftmaxWarps - 1) / kSoftmaxWarps,
                                                                 int64_t(score_softmax_chunks(p))})));
