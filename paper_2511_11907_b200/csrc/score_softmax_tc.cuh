@@ -279,7 +279,7 @@ softmax_tc_pool_kernel(Problem p, SoftmaxArgs a) {
   };
   for (int k = 0; k < a.depth && k < my_stages; ++k) fill(k);
   if (a.top_hist != nullptr)
-    for (int i = threadIdx.x; i < kCounters / 4; i += kSoftmaxThreads) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = threadIdx.x; i < ns * (kKeyTopBins / 8); i += kSoftmaxThreads) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
   pdl_wait();
   pdl_trigger();
 
@@ -424,11 +424,10 @@ softmax_tc_pool_kernel(Problem p, SoftmaxArgs a) {
   // ---- the CTA's counts join the global histograms ---------------------------------------------------------------------
   if (a.top_hist != nullptr) {
     __syncthreads();
-    for (int i = threadIdx.x; i < kCounters / 4; i += kSoftmaxThreads) {
+    for (int i = threadIdx.x; i < ns * (kKeyTopBins / 8); i += kSoftmaxThreads) {
       const uint4 v = reinterpret_cast<const uint4*>(hist)[i];
       if ((v.x | v.y | v.z | v.w) == 0u) continue;
       const int col = (i * 8) / kKeyTopBins;                       // 8 counters per vector
-      if (col >= ns) continue;
       unsigned long long* H = reinterpret_cast<unsigned long long*>(
           a.top_hist + (int64_t(rs.b) * p.S + s0 + col) * (kKeyTopBins / 2) + ((i * 4) % (kKeyTopBins / 2)));
       const unsigned long long lo = (unsigned long long)v.x | ((unsigned long long)v.y << 32);
