@@ -257,7 +257,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
     // predict(l + 1) waits for attention(l - 1) and only then lets attention(l) start, which finds the selection
     // of predict(l) complete: attention(l - 1) waited for it before it wrote its results.  Two launches a layer
     // instead of three, and neither waits for the other: 36 layers of B = 1, N = 16384, 8 KV heads, M = 256 through
-    // host memory 539 -> 430 us; at B = 1, N = 4096 a layer takes 8.5 us against 12.9.
+    // host memory 539 -> 425 us; at B = 1, N = 4096 a layer takes 8.5 us against 12.9.
     // Where the splits do not merge in clusters a combine follows each gather.
     if (score_select_cluster_supported(p) && (w.merge_in_cluster || w.beside)) {
       auto predict = [&](int l) -> int {
