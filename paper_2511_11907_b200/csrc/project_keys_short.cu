@@ -81,7 +81,9 @@ project_keys_short_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, 
   if (tid == kIssuer) {
     for (int s = 0; s < hpc; ++s) { mbar_init(smem_addr(&full[s]), 1); mbar_init(smem_addr(&done[s]), 1); }
     mbar_init_fence();
-    pdl_wait();                                                        // K may be the previous kernel's output
+  }
+  pdl_wait();                                                          // K and the adapter may be the previous kernel's output
+  if (tid == kIssuer) {
     for (int s = 0; s < hpc; ++s) {
       const uint32_t dst = stage0 + uint32_t(s) * C::kHeadBytes, bar = smem_addr(&full[s]);
       mbar_arrive_expect_tx(bar, C::kHalves * C::kAHalf);
@@ -93,8 +95,7 @@ project_keys_short_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, 
   if (warp == kIssuer / 32) { __syncwarp(); tmem_alloc(smem_addr(&tmem_base), tmem_cols); }
 
   // ---- the adapter's pieces, straight into the operand layout ----------------------------------------------------------
-  // Task = (column j, eight channels); the loads of a head go out together.  (The adapter is never an output of work
-  // in the stream.)  fp16 pieces are scaled per column as split_adapter_kernel does it.
+  // Task = (column j, eight channels); the loads of a head go out together.  fp16 pieces are scaled per column as split_adapter_kernel does it.
   constexpr int kTasks = R * (D / 8), kPer = (kTasks + kThreads - 1) / kThreads;
   for (int s = 0; s < hpc; ++s) {
     const float* src = proj + int64_t(blk0 + s) * D * R;
@@ -209,8 +210,7 @@ project_keys_short_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, 
   if (n_ctas > 1) { cluster_arrive(); cluster_wait(); }                // every CTA's sums are in place
 
   // ---- this CTA's share of the rows: sum over the cluster in rank order, one rounding ------------------------------------------
-  // (No trigger: the scorers request metadata tiles ahead of their own wait.)
-  pdl_wait();
+  // (No trigger: a scorer whose inputs are settled requests metadata tiles ahead of its own wait.)
   const int share = kRows / n_ctas, r0 = rank * share;
   for (int e = tid; e < share * (R / 4); e += kThreads) {
     const int row = r0 + e / (R / 4), c4 = e % (R / 4);

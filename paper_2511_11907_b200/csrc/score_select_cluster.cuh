@@ -78,6 +78,9 @@ score_select_cluster_kernel(Problem p, ClusterArgs a) {
     mbar_init_fence();
   }
   __syncwarp();
+  // Without KVSWAP_INPUTS_SETTLED any input -- query, adapter, metadata -- may be the previous kernel's output.
+  const bool settled = (p.flags & KVSWAP_INPUTS_SETTLED) != 0;
+  if (!settled) { pdl_wait(); pdl_trigger(); }
 
   // ---- this warp's contiguous share of the tiles; the first ones are requested at once -------------------------
   const int tile_rows = GS >= 0 ? kStageRows : a.tile_rows;
@@ -100,8 +103,8 @@ score_select_cluster_kernel(Problem p, ClusterArgs a) {
   for (int k = 0; k < a.depth && k < my_tiles; ++k) fill(k, k);
 
   // ---- this warp's pieces of the queries: item = (32 columns, KV head, 32 channels) ---------------------------
-  // The adapter is never written during decoding, so its rows are requested ahead of the wait.  The products
-  // are added in the order of build_queries (lowrank_query.cuh): the same bits.
+  // The adapter's rows are requested ahead of the cluster barrier.  The products are added in the order of
+  // build_queries (lowrank_query.cuh): the same bits.
   constexpr int kPasses = (R + 31) / 32, kLoads = (R == 16) ? 16 : 32;
   const QueryTerms terms = query_terms(p, rs);
   const int ch_shift = query_chunk_shift(p), n_items = terms.n_terms << ch_shift;
@@ -117,9 +120,6 @@ score_select_cluster_kernel(Problem p, ClusterArgs a) {
   int item = rank + n_ctas * warp;
   if (item < n_items * kPasses) request(item);
   for (int i = threadIdx.x; i < kKeyTopBins; i += kClusterThreads) sm->select.hist[i] = 0;
-  // Without KVSWAP_INPUTS_SETTLED the query may be the previous kernel's output: wait first.
-  const bool settled = (p.flags & KVSWAP_INPUTS_SETTLED) != 0;
-  if (!settled) { pdl_wait(); pdl_trigger(); }
   cluster_wait();                                       // every CTA of the cluster has started
   for (; item < n_items * kPasses; item += n_ctas * kClusterWarps) {
     const int it = item % n_items, pass = item / n_items;

@@ -7,7 +7,8 @@
 //
 // Both walk the tiles as the streaming scorer does (score_stream.cuh): 16 warps per CTA, each with its own
 // contiguous share of tiles and its own ring of stages filled by bulk asynchronous copies (bounded waits), the first
-// ones requested ahead of the dependency wait.  A CTA belongs to one row set.  The logits of eight heads and
+// ones requested ahead of the dependency wait: the query kernel in front of both lets its successor start only after its
+// own wait, when all that came before it, the metadata's producer included, was complete.  A CTA belongs to one row set.  The logits of eight heads and
 // eight tokens are one call of score_rows8() (score_tile.cuh: products exact, one rounding per accumulation);
 // the row operands of all heads of the set, "blocks" of eight, lie ready as fragments in shared memory, so the
 // number of heads is not limited by registers.

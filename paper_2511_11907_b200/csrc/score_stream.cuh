@@ -6,8 +6,7 @@
 // of up to 4 KB of rows); items are numbered with the tile fastest, a "row set" is the items of one
 // (b, hm, scope block).  Every warp takes an equal contiguous share of tiles and pulls them into its own
 // ring of shared-memory stages with bulk asynchronous copies (cp.async.bulk + mbarrier, bounded waits),
-// kDepth tiles in flight per warp; the first tiles are requested before the dependency wait, since nothing
-// the library runs during decoding writes metadata.
+// kDepth tiles in flight per warp; where the inputs are settled the first tiles are requested before the dependency wait.
 //
 // With G a power of two up to 32 (template GS = log2 G) a finished group score leaves the registers at
 // once.  Every other G that fits a tile (GS = -1) goes through a small shared-memory buffer of the warp,
@@ -158,20 +157,21 @@ score_stream_kernel(Problem p, StreamArgs a) {
     }
     advance(f);
   };
-  // The metadata is never written by a kernel that runs during decoding: request the first tiles now.
-  for (int k = 0; k < kDepth && k < my_stages; ++k) fill(k);
 
-  // ---- dependency wait and the summed low-rank queries ---------------------------------------------------
-  // Without KVSWAP_INPUTS_SETTLED the query may be the previous kernel's output: wait first.  With it,
-  // only this kernel's writes (scores and histograms, which the previous call's TopK may still read)
-  // have to wait, so the queries are built while that kernel finishes.
-  const bool settled = FUSED && (p.flags & KVSWAP_INPUTS_SETTLED) != 0;
-  if (!settled) pdl_wait();
+  // ---- dependency wait, first tiles and the summed low-rank queries --------------------------------------
+  // Without KVSWAP_INPUTS_SETTLED any input may be the previous kernel's output: wait first.  With it, only this
+  // kernel's writes (scores and histograms, which the previous call's TopK may still read) have to wait, so the
+  // queries are built while that kernel finishes.  Queries found in memory (not FUSED) are the previous kernel's in
+  // either case, but that kernel let this one start when all before it was complete, or the metadata is settled:
+  // its first tiles go out ahead of the wait.
+  const bool settled = (p.flags & KVSWAP_INPUTS_SETTLED) != 0;
+  if (FUSED && !settled) pdl_wait();
+  for (int k = 0; k < kDepth && k < my_stages; ++k) fill(k);
   if constexpr (FUSED) {
     for (int s = 0; s < n_sets; ++s)
       build_queries<0, R>(p, a.q, a.proj, row_set(p, rest0 + s, a.n_sub), sm->sc, sm->sc + kQuerySumFloats, sm->urow[s]);
   }
-  if (settled) pdl_wait();
+  if (!FUSED || settled) pdl_wait();
   pdl_trigger();
   if constexpr (!FUSED) __syncthreads();             // the histogram is cleared (the fused path has synchronised)
 
