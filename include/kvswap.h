@@ -90,7 +90,9 @@ typedef enum { KVSWAP_SCOPE_KV_HEAD = 0, KVSWAP_SCOPE_ALL_HEADS = 1 } kvswap_sco
  *       writes them, or a full dependency (an event wait, a copy, a host synchronisation) lies
  *       in between.  The first kernel of the call then starts while the previous kernel of the
  *       stream is still finishing (programmatic dependent launch) and only waits for it before
- *       writing its own results.  Without the flag it waits first.  Results are the same.
+ *       writing its own results.  Without the flag it waits first.  Results are the same.  A step over
+ *       all layers takes it as the same promise about the step's inputs: without it the step's first
+ *       kernel waits.
  *   KVSWAP_SCORE_SOFTMAX   a variant of the predictor (kvswap_score_select, and the steps built on
  *       it): each query head's low-rank scores pass through a softmax over the tokens of the
  *       context's complete groups, scaled by 1/sqrt(d), BEFORE the sum over heads -- the scores

@@ -183,8 +183,9 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
     // leaves the other room on an SM, so they run one after the other, and what the order hides is
     // the latency-bound part: the TopK of layer l + 1 is not needed before attention l + 1, and the
     // gather of layer l starts fetching while the scorer of layer l + 1 drains.
-    // Settled inputs: q is an input of the step; a selection is complete before the scorer that
-    // precedes its attention passes its own dependency wait.
+    // Settled inputs: the first layer's predictor waits for whatever wrote the step's inputs (unless the caller
+    // has promised that they are settled), so they are complete before any later kernel of the step starts; a selection
+    // is complete before the scorer that precedes its attention passes its own dependency wait.
     Problem p_settled = p;
     p_settled.flags |= KVSWAP_INPUTS_SETTLED;
     kvswap_shape shape_settled = *shape;
@@ -201,7 +202,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
     auto score = [&](int l) -> int {
       if (probed(l)) ev(probe_opt->ev_begin);
       const void* ql = static_cast<const char*>(q) + size_t(l) * q_bytes;
-      return score_launch(p_settled, w, ql, layers->proj[l], layers->meta[l], nullptr, ws, stream,
+      return score_launch(l == 0 ? p : p_settled, w, ql, layers->proj[l], layers->meta[l], nullptr, ws, stream,
                           formed_for == l ? (l & 1) : -1) == cudaSuccess
                  ? KVSWAP_OK : KVSWAP_ERR_CUDA;
     };
@@ -263,7 +264,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
       auto predict = [&](int l) -> int {
         if (probed(l)) ev(probe_opt->ev_begin);
         const cudaError_t e = launch_score_select_cluster(
-            p_settled, static_cast<const char*>(q) + size_t(l) * q_bytes, layers->proj[l], layers->meta[l], nullptr,
+            l == 0 ? p : p_settled, static_cast<const char*>(q) + size_t(l) * q_bytes, layers->proj[l], layers->meta[l], nullptr,
             group_idx + size_t(l) * idx_elems, n_selected + size_t(l) * nsel_elems, static_cast<uint32_t*>(ws), stream);
         if (probed(l)) ev(probe_opt->ev_mid);
         return e == cudaSuccess ? KVSWAP_OK : KVSWAP_ERR_CUDA;
@@ -303,7 +304,8 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
   // A layer's misses cross the link while the layer before it is attended and the next one predicted.  (With lookup
   // and fill behind each other on the predictor's stream the link idled during every prediction: 1580 us for four
   // steps of four layers, B = 1, N = 16384, M = 256, 8 KV heads of 128, of which the link needs 1184; now 1427.)
-  // q is an input of the step and a slot list is awaited through its event: the inputs are settled.
+  // The first layer's predictor waits for the step's inputs (unless the caller has promised that they are settled), and
+  // a slot list is awaited through its event: the inputs of the others are settled.
   kvswap_shape shape_settled = shape_attn;
   shape_settled.flags |= KVSWAP_INPUTS_SETTLED;
   Problem p_settled = p;
@@ -316,7 +318,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
     const void* ql = static_cast<const char*>(q) + size_t(l) * q_bytes;
     int32_t* idx_l = group_idx + size_t(l) * idx_elems;
     int32_t* nsel_l = n_selected + size_t(l) * nsel_elems;
-    if (score_select_launch(p_settled, w, ql, layers->proj[l], layers->meta[l], idx_l, nsel_l, nullptr, ws, stream) != cudaSuccess ||
+    if (score_select_launch(l == 0 ? p : p_settled, w, ql, layers->proj[l], layers->meta[l], idx_l, nsel_l, nullptr, ws, stream) != cudaSuccess ||
         cudaEventRecord(res->selected[l], stream) != cudaSuccess ||
         cudaStreamWaitEvent(res->fetch[l & 1], res->selected[l], 0) != cudaSuccess ||
         launch_reuse_fetch(p, tiers->n_slots, tiers->max_groups, idx_l, nsel_l, static_cast<int32_t*>(tiers->state[l]),

@@ -101,3 +101,34 @@ def test_project_keys_behind_the_producer_of_the_adapter(N, per_head, dtype):
     K, proj = _randn(1, H, N, d, dtype=t, seed=7), _randn(H, d, r, seed=8)
     meta, ws = torch.empty((1, hm, N, r), device="cuda"), rt.alloc_workspace(shape)
     _check(proj, lambda: kv.kvswap_project_keys(shape, K, proj, meta, 0, N, ws), [meta])
+
+
+# 2 layers of one sequence, 32 heads of 128 in fp32
+@pytest.mark.parametrize("what", ["query", "adapter", "metadata"])
+@pytest.mark.parametrize("N,G,r", [(2048, 8, 32), (32768, 1, 16), (4096, 8, 128)])
+@pytest.mark.parametrize("kind", ["step", "tiered"])
+def test_step_behind_the_producer_of_an_input(what, N, G, r, kind):
+    L, H, d, M = 2, 8, 128, 64
+    shape, _, _, _, _, _, _ = _select_args(N, G, r=r, top_k=M)
+    q = _randn(L, 1, 4 * H, d, seed=9)
+    proj = [_randn(H, d, r, seed=10 + l) * 0.1 for l in range(L)]
+    meta = [_randn(1, 1, N, r, seed=20 + l) for l in range(L)]
+    K, V = ([_randn(1, H, N, d, seed=30 + 10 * i + l) for l in range(L)] for i in range(2))
+    out = torch.empty((L, 1, 4 * H, d), device="cuda")
+    idx, nsel = torch.empty((L, 1, H, M), dtype=torch.int32, device="cuda"), torch.empty((L, 1, H), dtype=torch.int32, device="cuda")
+    target = {"query": q, "adapter": proj[0], "metadata": meta[0]}[what]
+    if kind == "step":
+        layers, ws = kv.make_layers(K, V, meta, proj, 0), rt.alloc_workspace(shape)
+        _check(target, lambda: kv.kvswap_decode_step(shape, layers, q, out, None, idx, nsel, ws), [out, idx, nsel])
+        return
+    slots, groups = 2 * M, N // G
+    kr, vr = ([torch.zeros((1, H, (slots + 1) * G, d), device="cuda") for _ in range(L)] for _ in range(2))
+    state = [torch.empty(kv.kvswap_reuse_state_bytes(shape, slots, groups) // 4, dtype=torch.int32, device="cuda") for _ in range(L)]
+    lists, n_miss = [torch.empty_like(idx) for _ in range(3)], torch.empty_like(nsel)
+    layers = kv.make_layers(kr, vr, meta, proj, 0)
+    tiers = kv.make_tiers(slots, groups, K, V, kr, vr, state, *lists, n_miss)
+    ws = torch.empty(kv.kvswap_tiered_workspace_bytes(shape, slots), dtype=torch.uint8, device="cuda")
+    kv.kvswap_workspace_init(ws)
+    for s in state:
+        kv.kvswap_reuse_init(shape, slots, groups, s)
+    _check(target, lambda: kv.kvswap_decode_step_tiered(shape, layers, tiers, q, out, None, idx, nsel, ws), [idx, nsel])
