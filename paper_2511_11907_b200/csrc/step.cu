@@ -188,6 +188,8 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
     // is complete before the scorer that precedes its attention passes its own dependency wait.
     Problem p_settled = p;
     p_settled.flags |= KVSWAP_INPUTS_SETTLED;
+    Problem p_wait = p;                             // the last attention: its selection may be the launch before it
+    p_wait.flags &= ~KVSWAP_INPUTS_SETTLED;
     kvswap_shape shape_settled = *shape;
     shape_settled.flags |= KVSWAP_INPUTS_SETTLED;
     auto ev = [&](void* e) { if (e != nullptr) cudaEventRecord(static_cast<cudaEvent_t>(e), stream); };
@@ -228,7 +230,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
       // wrote, need not wait for the gather.
       Problem p_early = p_settled;
       p_early.flags |= kFlagWaitEarly;
-      const Problem& pa = !next ? p : merges ? p_early : p_settled;
+      const Problem& pa = !next ? p_wait : merges ? p_early : p_settled;
       if (launch_sparse_decode(pa, w, ql, layers->K[l], layers->V[l], idx_l, nsel_l, partial, out_l, lse_l,
                                static_cast<uint32_t*>(ws), stream, /*combine=*/false) != cudaSuccess)
         return KVSWAP_ERR_CUDA;
@@ -279,7 +281,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
         if (status != KVSWAP_OK) break;
         // (the last layer's attention follows an attention directly: its selection is complete when that one is)
         const cudaError_t e = launch_sparse_decode(
-            l + 1 < L ? p_late : p, w, static_cast<const char*>(q) + size_t(l) * q_bytes, layers->K[l], layers->V[l],
+            l + 1 < L ? p_late : p_wait, w, static_cast<const char*>(q) + size_t(l) * q_bytes, layers->K[l], layers->V[l],
             group_idx + size_t(l) * idx_elems, n_selected + size_t(l) * nsel_elems, partial, out + size_t(l) * out_elems,
             lse_opt ? lse_opt + size_t(l) * p.B * p.Hq : nullptr, static_cast<uint32_t*>(ws), stream);
         if (probed(l)) ev(probe_opt->ev_end);

@@ -132,3 +132,32 @@ def test_step_behind_the_producer_of_an_input(what, N, G, r, kind):
     for s in state:
         kv.kvswap_reuse_init(shape, slots, groups, s)
     _check(target, lambda: kv.kvswap_decode_step_tiered(shape, layers, tiers, q, out, None, idx, nsel, ws), [idx, nsel])
+
+
+@pytest.mark.parametrize("layers_n", [1, 2, 3])
+@pytest.mark.parametrize("N,M", [(2048, 64), (16384, 700), (70000, 96)])
+def test_step_whose_inputs_are_settled_still_orders_its_own_kernels(layers_n, N, M):
+    """KVSWAP_INPUTS_SETTLED on a step is about the step's inputs: the selections its attention reads are not among them."""
+    L, H, d, r, G = layers_n, 8, 128, 32, 8
+    shape = kv.make_shape(batch=1, n_ctx=N, n_q_heads=4 * H, n_kv_heads=H, head_dim=d, rank=r, meta_heads=1, group_size=G,
+                          top_k=M, kv_dtype=kv.KVSWAP_BF16, meta_dtype=kv.KVSWAP_F16, q_dtype=kv.KVSWAP_BF16)
+    bf = torch.bfloat16
+    q = [_randn(L, 1, 4 * H, d, dtype=bf, seed=40 + i) for i in range(2)]
+    K, V = ([_randn(1, H, N, d, dtype=bf, seed=50 + 10 * i + l) for l in range(L)] for i in range(2))
+    meta = [_randn(1, 1, N, r, dtype=torch.float16, seed=70 + l) for l in range(L)]
+    proj = [_randn(H, d, r, seed=80 + l) for l in range(L)]
+    layers, ws = kv.make_layers(K, V, meta, proj, 0), rt.alloc_workspace(shape)
+    out = torch.empty((L, 1, 4 * H, d), device="cuda")
+    idx, nsel = torch.empty((L, 1, H, M), dtype=torch.int32, device="cuda"), torch.empty((L, 1, H), dtype=torch.int32, device="cuda")
+    want = []
+    for i in range(2):
+        kv.kvswap_decode_step(shape, layers, q[i], out, None, idx, nsel, ws)
+        want.append((out.clone(), idx.clone()))
+    torch.cuda.synchronize()
+    flagged = shape.with_flags(kv.KVSWAP_INPUTS_SETTLED)
+    bad = torch.zeros((), dtype=torch.int64, device="cuda")
+    for i in range(40):
+        kv.kvswap_decode_step(flagged, layers, q[i % 2], out, None, idx, nsel, ws)
+        bad += (~torch.isfinite(out)).any() | (out != want[i % 2][0]).any() | (idx != want[i % 2][1]).any()
+    torch.cuda.synchronize()
+    assert int(bad) == 0 and kv.kvswap_read_device_status(ws) == 0
