@@ -110,7 +110,7 @@ void plan_workspace(const Problem& p, Workspace* w) {
   w->uq_bytes = align256(sizeof(float) * size_t(p.B) * p.Su * p.r);
   w->off_uq = off;       off += 2 * w->uq_bytes;
   w->off_scores = off;   off += align256(sizeof(float) * size_t(p.B) * p.S * workspace_score_pitch(p));
-  w->off_partial = off;  off += align256(sizeof(float) * size_t(p.B) * p.Hq * std::max(w->splits, w->splits_room) * (p.d + 2));
+  w->off_partial = off;  off += align256(sizeof(float) * size_t(p.B) * p.Hq * w->splits_room * (p.d + 2));
   w->off_softmax = off;  off += align256(sizeof(float) * size_t(p.B) * p.Hq * (size_t(p.r) + 2 * size_t(score_softmax_chunks(p))));
   w->off_adapter = off;  off += align256(project_keys_umma_scratch_bytes(p) + 1024);   // 1 KiB: tensor-map base alignment
   w->total = off;

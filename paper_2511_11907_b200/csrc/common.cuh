@@ -53,7 +53,7 @@ struct Workspace {
   size_t off_adapter;  // bf16 [H_kv, 3 r, d]       adapter split into three bf16 pieces (project_keys on tcgen05)
   size_t total;
   int splits;          // split-K factor of sparse_decode for this shape
-  int splits_room;     // splits the partials are planned for (whatever the flags of a call)
+  int splits_room;     // splits the partials are planned for: no fewer than `splits` of any context length and flags
   int heads_per_cta;   // query heads sharing one K/V pass in sparse_decode
   int depth;           // shared-memory stages per compute warp in sparse_decode
   bool beside;         // a decode step runs the gather beside the next layer's one-launch predictor (splits planned for what that leaves)

@@ -745,7 +745,10 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
   const int64_t slots = 2 * kNumSMs;
   int64_t best = best_splits(slots, 256);
   w->merge_in_cluster = w->beside = false;
-  w->splits_room = int(best);
+  // No plan of these heads, types and M has more splits than this, whatever the rows past the last group, the
+  // flags or the context length: one workspace serves a context as it grows.
+  const int64_t most_chunks = (int64_t(p.M) * p.G + p.G - 1 + kTok - 1) / kTok;
+  w->splits_room = int(std::max<int64_t>(1, std::min<int64_t>({256, most_chunks / (2 * kWarps), 2 * slots / problems})));
   ClusterGrid predictor;
   if (score_select_cluster_grid(p, &predictor)) {
     // A short context, whose predictor is one launch of clusters: here the splits of a list form a cluster of at

@@ -221,6 +221,36 @@ def test_workspace_grows_with_the_problem(lib):
     assert big > small
 
 
+def test_a_workspace_for_the_longest_context_serves_every_shorter_one(lib):
+    """The bytes a shape needs never fall as its context grows, token by token through a group and from the short-context
+    schedules to the long ones, nor with more groups to select, and do not depend on the flags."""
+    import random
+    rng = random.Random(5)
+    # a partly filled group needed fewer bytes here than the empty one before it
+    a = dict(batch=2, n_q_heads=16, n_kv_heads=4, head_dim=128, rank=32, meta_heads=4, group_size=16, top_k=592,
+             kv_dtype=W.BF16, meta_dtype=W.F16, q_dtype=W.BF16)
+    shapes = [(a, 64992)]
+    for _ in range(400):
+        H, t, G = rng.choice([1, 2, 4, 8]), rng.choice([W.F32, W.BF16, W.F16]), rng.choice([1, 4, 8, 12, 16, 64])
+        shapes.append((dict(batch=rng.choice([1, 2, 3, 8, 16]), n_q_heads=H * rng.choice([1, 2, 3, 4, 8]), n_kv_heads=H,
+                            head_dim=rng.choice([64, 128]), rank=rng.choice([16, 32, 64, 128]), meta_heads=rng.choice([1, H]),
+                            group_size=G, top_k=max(1, int(2 ** rng.uniform(8, 14)) // G), kv_dtype=t,
+                            meta_dtype=W.F32 if t == W.F32 else W.F16, q_dtype=rng.choice([W.F32, t]),
+                            scope=rng.choice([W.SCOPE_KV_HEAD, W.SCOPE_ALL_HEADS])), int(2 ** rng.uniform(8, 17))))
+    for a, n in shapes:
+        G = a["group_size"]
+        need = lambda n_ctx, **kw: kv.kvswap_workspace_bytes(good_shape(**dict(a, n_ctx=n_ctx, **kw)))
+        lengths = sorted({max(1, n * k // 16) for k in range(1, 17)} | {n + k for k in range(2 * G + 1)})
+        sizes = [need(x) for x in lengths]
+        assert sizes[0] > 0 and sizes == sorted(sizes), (a, n)
+        assert need(n) == need(n, flags=kv.KVSWAP_SCORE_SOFTMAX) == need(n, flags=kv.KVSWAP_INPUTS_SETTLED)
+        more = [need(n, top_k=a["top_k"] * k // 8 + 1) for k in range(9)]
+        assert more == sorted(more), (a, n)
+        slots = 2 * a["top_k"]
+        tiered = [kv.kvswap_tiered_workspace_bytes(good_shape(**dict(a, n_ctx=x)), slots) for x in lengths]
+        assert tiered == sorted(tiered), (a, n)
+
+
 def test_device_status_entry_points_validate_their_arguments(lib):
     assert lib.kvswap_workspace_init(None, 1024, None) == 1            # NULL workspace
     assert lib.kvswap_workspace_init(ctypes.c_void_p(4096), 16, None) == 5   # shorter than the header
