@@ -46,10 +46,10 @@
  *  - Errors are returned, never raised: no call aborts or traps.
  *  - `ws` is caller-provided scratch of at least kvswap_workspace_bytes(shape) bytes, cleared once
  *    with kvswap_workspace_init before its first use.  The predictor keeps a region at its head
- *    (sized by B, H_kv, the scope, the metadata type and r alone) zero from call to call; the rest is
- *    undefined between calls.  One workspace may serve shapes that differ in n_ctx, top_k and
- *    flags; clear it again before using it for another batch size, head count, rank or scope, and after
- *    a call that returned KVSWAP_ERR_CUDA.  Calls that run concurrently on different streams need
+ *    (sized by B, H_kv and the scope alone) zero from call to call; the rest is
+ *    undefined between calls.  One workspace may serve shapes that differ in anything else, n_ctx, top_k,
+ *    flags, rank and types among them; clear it again before using it for another batch size, head count or
+ *    scope, and after a call that returned KVSWAP_ERR_CUDA.  Calls that run concurrently on different streams need
  *    different workspaces.
  */
 #ifndef KVSWAP_H_

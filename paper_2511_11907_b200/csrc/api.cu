@@ -79,18 +79,16 @@ int resolve(const kvswap_shape* s, Problem* p) {
 // that the top-k kernel can load them as vectors whatever NG is.
 static int workspace_score_pitch(const Problem& p) { return (std::max(p.NG, 1) + 31) / 32 * 32; }
 
-// Room for the leading-digit histograms (score_stream.cu, topk_select.cu) is planned from the
-// batch and head counts alone, at a fixed place in front of everything else, so that one workspace
-// keeps them zero between calls while the context grows.
-static bool hist_capable(const Problem& p) {
-  return score_stream_rows(p) && int64_t(p.B) * p.S <= 1024;
-}
+// Room for the leading-digit histograms (score_stream.cuh, topk_select.cu) is planned from the
+// batch and head counts and the scope alone, also for ranks and types whose calls never count, at a fixed place
+// in front of everything else: one workspace keeps them zero between calls whatever else changes.
+static bool hist_room(const Problem& p) { return int64_t(p.B) * p.S <= 1024; }
 
 // The scorer counts the leading digit of every group score's key and the TopK starts from those
 // counts (several CTAs per problem) where both kernels have that path.
 static bool counts_top_digit(const Problem& p) {
   const bool counts = (p.flags & KVSWAP_SCORE_SOFTMAX) ? score_softmax_tc_counts(p) : score_stream_counts_top_digit(p);
-  return counts && hist_capable(p) && topk_parts_supported(p);
+  return counts && hist_room(p) && topk_parts_supported(p);
 }
 
 bool select_merges_with_combine(const Problem& p) {
@@ -106,7 +104,7 @@ void plan_workspace(const Problem& p, Workspace* w) {
   plan_sparse_decode(p, w);
 
   size_t off = 256;  // first 256 bytes reserved
-  w->off_hist = off;     off += hist_capable(p) ? align256(size_t(p.B) * p.S * (sizeof(uint16_t) * kKeyTopBins + sizeof(uint32_t))) : 0;
+  w->off_hist = off;     off += hist_room(p) ? align256(size_t(p.B) * p.S * (sizeof(uint16_t) * kKeyTopBins + sizeof(uint32_t))) : 0;
   w->uq_bytes = align256(sizeof(float) * size_t(p.B) * p.Su * p.r);
   w->off_uq = off;       off += 2 * w->uq_bytes;
   w->off_scores = off;   off += align256(sizeof(float) * size_t(p.B) * p.S * workspace_score_pitch(p));

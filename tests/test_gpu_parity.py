@@ -622,3 +622,33 @@ def test_device_status_word_round_trip():
     assert "wait" in kv.status_string(10)
     kv.kvswap_workspace_init(ws)
     assert kv.kvswap_read_device_status(ws) == 0
+
+
+def test_one_workspace_serves_ranks_types_and_flags_in_turn():
+    """Without clearing it in between: calls that count digits in the region at its head, and calls of ranks and types
+    that never do, leave that region as the others expect it."""
+    B, H, d, N, G, M = 2, 8, 128, 40000, 8, 200
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    kinds = [(32, W.F16, 0), (128, W.F16, 0), (32, W.F16, kv.KVSWAP_SCORE_SOFTMAX), (64, W.F32, 0), (32, W.E4M3, 0), (24, W.F32, 0),
+             (16, W.F16, 0), (128, W.F32, kv.KVSWAP_SCORE_SOFTMAX)]
+    calls = []
+    for r, meta_type, flags in kinds:
+        shape = kv.make_shape(batch=B, n_ctx=N, n_q_heads=4 * H, n_kv_heads=H, head_dim=d, rank=r, meta_heads=1, group_size=G,
+                              top_k=M, kv_dtype=W.BF16, meta_dtype=meta_type, q_dtype=W.BF16, flags=flags)
+        q = torch.randn((B, 4 * H, d), generator=g, device="cuda").bfloat16()
+        proj = torch.randn((H, d, r), generator=g, device="cuda") * 0.1
+        meta = torch.randn((B, 1, N, r), generator=g, device="cuda").to(rt._TORCH_DTYPE[meta_type])
+        idx, nsel = rt.alloc_selection(shape)
+        ws = rt.alloc_workspace(shape)
+        kv.kvswap_score_select(shape, q, proj, meta, idx, nsel, None, ws)
+        calls.append((shape, q, proj, meta, idx, nsel))
+    ws = torch.empty(max(kv.kvswap_workspace_bytes(c[0]) for c in calls), dtype=torch.uint8, device="cuda")
+    kv.kvswap_workspace_init(ws)
+    for a in range(len(calls)):
+        for b in range(len(calls)):
+            for shape, q, proj, meta, want, _ in (calls[a], calls[b]):
+                idx, nsel = rt.alloc_selection(shape)
+                kv.kvswap_score_select(shape, q, proj, meta, idx, nsel, None, ws)
+                assert torch.equal(idx, want), (kinds[a], kinds[b])
+    assert kv.kvswap_read_device_status(ws) == 0
