@@ -9,7 +9,23 @@ namespace {
 
 struct Plan {
   int g_shift, tile_rows, tiles, n_sub, n_rests, cluster, depth;
+  bool whole_sm;                                         // a CTA's shared memory leaves no room for a second one
 };
+
+size_t cta_smem(const Problem& p, bool power_of_two, int depth) {
+  auto by_group = [&](auto m, auto r) {
+    constexpr int META = decltype(m)::value, R = decltype(r)::value;
+    return power_of_two ? score_select_smem<META, R, 0>(depth, p.NG) : score_select_smem<META, R, -1>(depth, p.NG);
+  };
+  using F16 = std::integral_constant<int, KVSWAP_F16>;
+  using F32 = std::integral_constant<int, KVSWAP_F32>;
+  using R16 = std::integral_constant<int, 16>;
+  using R32 = std::integral_constant<int, 32>;
+  using R64 = std::integral_constant<int, 64>;
+  if (p.meta_dtype == KVSWAP_E4M3) return score_select_smem<KVSWAP_E4M3, 32, 0>(depth, p.NG);
+  if (p.meta_dtype == KVSWAP_F16) return p.r == 16 ? by_group(F16(), R16()) : p.r == 32 ? by_group(F16(), R32()) : by_group(F16(), R64());
+  return p.r == 16 ? by_group(F32(), R16()) : p.r == 32 ? by_group(F32(), R32()) : by_group(F32(), R64());
+}
 
 bool plan(const Problem& p, Plan* pl) {
   if (p.NG < 1 || p.NG > kClusterMaxKeys || (p.flags & KVSWAP_SCORE_SOFTMAX) || !score_stream_rows(p) || p.meta_sn != p.r ||
@@ -36,12 +52,16 @@ bool plan(const Problem& p, Plan* pl) {
   while (c < ns) c *= 2;
   while (c < (n_rests <= 2 ? 16 : 8) && pl->tiles > c * kClusterWarps && n_rests * 2 * c <= 120) c *= 2;
   pl->cluster = c;
-  // A second stage per warp makes a CTA fill an SM's shared memory; only where there are SMs to spare.
+  // A second stage per warp makes a CTA fill an SM's shared memory; only where there are SMs to spare.  So do many
+  // keys (fp16 rows of rank 32: 6784).  All clusters have to be resident at once: two CTAs per SM, or, with a CTA's
+  // shared memory above half of an SM's, two clusters of 8 per GPC.  (At B = 18, 8 heads, N = 8192, G = 1, rank 32, which
+  // do not fit so, predictor and attention 42.0 us in clusters, 29.5 with the two kernels.)
   const int64_t ctas = n_rests * c;
-  pl->depth = pl->tiles > c * kClusterWarps && ctas <= 100 ? 2 : 1;
+  pl->depth = pl->tiles > c * kClusterWarps && ctas <= 100 && cta_smem(p, g_shift >= 0, 2) <= 227 * 1024 ? 2 : 1;
+  pl->whole_sm = cta_smem(p, g_shift >= 0, pl->depth) > 113 * 1024;
   // Beyond two tiles per warp the streaming kernels on all SMs are the faster: at B = 4, N = 32768 (r = 32, G = 8,
   // four tiles per warp) 14.5 us of both against 12 to 18 for clusters, at B = 1, N = 65536 13.4 against 16.
-  return ctas <= 264 && pl->tiles <= 2 * c * kClusterWarps;
+  return ctas <= (pl->whole_sm ? 132 : 264) && pl->tiles <= 2 * c * kClusterWarps;
 }
 
 }  // namespace
@@ -50,7 +70,7 @@ bool score_select_cluster_supported(const Problem& p) { Plan pl; return plan(p, 
 bool score_select_cluster_grid(const Problem& p, ClusterGrid* g) {
   Plan pl;
   if (!plan(p, &pl)) return false;
-  *g = ClusterGrid{pl.n_rests, pl.cluster, pl.depth > 1};
+  *g = ClusterGrid{pl.n_rests, pl.cluster, pl.whole_sm};
   return true;
 }
 

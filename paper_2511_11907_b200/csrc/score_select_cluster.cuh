@@ -220,15 +220,18 @@ template <> cudaError_t launch_score_select_rows<KVSWAP_F32, 64>(const Problem&,
 
 constexpr int kClusterMaxKeys = 16384;                  // keys of one scope in the selecting CTA's shared memory
 
+// Shared memory of a CTA with `depth` stages per warp and NG keys; GS counts only as a power of two (>= 0) or not.
 template <int META, int R, int GS>
-cudaError_t launch_score_select_gs(const Problem& p, const ClusterArgs& a, int cluster, int n_rests, cudaStream_t st) {
+constexpr size_t score_select_smem(int depth, int NG) {
   constexpr size_t kFixed = (sizeof(ClusterSmem<META, R, GS>) + 127) & ~size_t(127);
   constexpr size_t kStages = size_t(kClusterWarps) * ScoreStage<META, R, GS>::kBytes;
   static_assert(kFixed + kStages + 4 * kClusterMaxKeys <= 227 * 1024, "at least one stage per warp fits");
-  ClusterArgs args = a;
-  const size_t room = 227 * 1024 - kFixed - 4 * size_t(p.NG + 3);
-  args.depth = (a.depth >= 2 && 2 * kStages <= room) ? 2 : 1;
-  const size_t smem = kFixed + args.depth * kStages + 4 * size_t((p.NG + 3) & ~3);
+  return kFixed + size_t(depth) * kStages + 4 * size_t((NG + 3) & ~3);
+}
+
+template <int META, int R, int GS>
+cudaError_t launch_score_select_gs(const Problem& p, const ClusterArgs& args, int cluster, int n_rests, cudaStream_t st) {
+  const size_t smem = score_select_smem<META, R, GS>(args.depth, p.NG);
   auto kern = score_select_cluster_kernel<META, R, GS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
