@@ -74,12 +74,12 @@ bool score_select_cluster_grid(const Problem& p, ClusterGrid* g) {
   return true;
 }
 
-// On its own, not beside an attention, a cluster that selects for one scope only (per-head metadata) pays while
-// every warp has one tile: at B = 1, 8 heads, N = 16384 (two) 10.2 us against 9.5 of the two kernels, at
-// N = 4096 7.0 against 9.2.
+// On its own, not beside an attention, a cluster that selects for fewer than eight scopes pays while every warp has one
+// tile: per-head metadata at B = 1, 8 heads, N = 16384 (two tiles) 10.2 us against 9.5 of the two kernels, at N = 4096
+// 7.0 against 9.2; joint metadata of 4 heads at B = 1, N = 25000 (two tiles) 11.2 against 10.7.
 bool score_select_cluster_pays_alone(const Problem& p) {
   Plan pl;
-  return plan(p, &pl) && (p.Hm == 1 || pl.tiles <= pl.cluster * kClusterWarps);
+  return plan(p, &pl) && ((p.Hm == 1 && p.S >= kQueryCols) || pl.tiles <= pl.cluster * kClusterWarps);
 }
 
 cudaError_t launch_score_select_cluster(const Problem& p, const void* q, const float* proj, const void* meta, float* scores,

@@ -218,7 +218,11 @@ template <> cudaError_t launch_score_select_rows<KVSWAP_F32, 16>(const Problem&,
 template <> cudaError_t launch_score_select_rows<KVSWAP_F32, 32>(const Problem&, const ClusterArgs&, int, int, int, cudaStream_t);
 template <> cudaError_t launch_score_select_rows<KVSWAP_F32, 64>(const Problem&, const ClusterArgs&, int, int, int, cudaStream_t);
 
-constexpr int kClusterMaxKeys = 16384;                  // keys of one scope in the selecting CTA's shared memory
+// Keys of one scope in the selecting CTA's shared memory.  With more, one CTA takes longer to select from them than the
+// TopK in parts: scorer and select at B = 1, 8 heads, r = 32, G = 1 14.0 us against 14.9 of the two kernels for 6000
+// groups, 15.3 against 14.9 for 8192, 22.5 against 16.5 for 16384; at B = 16 19.8 against 24.4, 30.9 against 20.0 and
+// 48.1 against 38.7.
+constexpr int kClusterMaxKeys = 6144;
 
 // Shared memory of a CTA with `depth` stages per warp and NG keys; GS counts only as a power of two (>= 0) or not.
 template <int META, int R, int GS>
