@@ -386,6 +386,7 @@ int kvswap_sparse_decode(const kvswap_shape* shape, const void* q, const void* K
   plan_workspace(p, &w);
   if (ws_bytes < w.total) return KVSWAP_ERR_WORKSPACE;
   float* partial = reinterpret_cast<float*>(static_cast<char*>(ws) + w.off_partial);
+  w.merge_in_cluster = w.merge_alone;
   cudaError_t e = launch_sparse_decode(p, w, q, K, V, group_idx, n_selected, partial, out, lse_opt,
                                        static_cast<uint32_t*>(ws), static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? KVSWAP_OK : KVSWAP_ERR_CUDA;

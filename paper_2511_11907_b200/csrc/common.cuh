@@ -57,7 +57,8 @@ struct Workspace {
   int heads_per_cta;   // query heads sharing one K/V pass in sparse_decode
   int depth;           // shared-memory stages per compute warp in sparse_decode
   bool beside;         // a decode step runs the gather beside the next layer's one-launch predictor (splits planned for what that leaves)
-  bool merge_in_cluster;   // sparse_decode on its own: the splits of a list form a cluster that merges them (no combine pass)
+  bool merge_in_cluster;   // the splits of a list form a cluster that merges them (no combine pass; the same bits)
+  bool merge_alone;    // ... also when sparse_decode is called on its own
 };
 
 int resolve(const kvswap_shape* s, Problem* p);            // validation; returns kvswap_status

@@ -670,6 +670,10 @@ cudaError_t launch_one(const Problem& p, const Workspace& w, const void* q, cons
     auto kern = sparse_decode_splitk_kernel<KV_T, Q_T, D, RH, Engine, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
+    if (w.splits > 8) {                            // more than the portable size
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
     return launch_pdl_cluster(kern, w.splits, grid, dim3(kThreads), smem, st, p, qt, Kt, Vt, group_idx, n_selected,
                               static_cast<float*>(nullptr), out, lse, w.splits, depth, g_shift, err);
   }
@@ -744,39 +748,35 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
   };
   const int64_t slots = 2 * kNumSMs;
   int64_t best = best_splits(slots, 256);
-  w->merge_in_cluster = w->beside = false;
+  w->merge_in_cluster = w->merge_alone = w->beside = false;
   // No plan of these heads, types and M has more splits than this, whatever the rows past the last group, the
   // flags or the context length: one workspace serves a context as it grows.
   const int64_t most_chunks = (int64_t(p.M) * p.G + p.G - 1 + kTok - 1) / kTok;
   w->splits_room = int(std::max<int64_t>(1, std::min<int64_t>({256, most_chunks / (2 * kWarps), 2 * slots / problems})));
   ClusterGrid predictor;
   if (score_select_cluster_grid(p, &predictor)) {
-    // A short context, whose predictor is one launch of clusters: here the splits of a list form a cluster of at
-    // most 8 that merges them, which saves the combine launch and lets attention and predictor run side by
-    // side.  The largest cluster is taken whose lists all fit beside the next layer's predictor (a GPC has some
-    // 36 slots for these CTAs, and a cluster stays in one GPC).  At B = 4, N = 4096, M = 128: clusters of 6
-    // 11.8 us per layer, of 8 (256 CTAs, which do not fit) 15.3, the chain of three kernels 13.6.
+    // A short context, whose predictor is one launch of clusters: in a decode step the attention runs beside the next
+    // layer's predictor.  The step's results are those of the calls bit for bit, so both have one split factor, in
+    // general the one a call on its own is fastest with.  The step merges the splits in a cluster, which saves the combine
+    // launch, where the clusters of all lists fit beside the predictor (a GPC has some 36 slots for these CTAs, and a
+    // cluster stays in one GPC), else by a combine kernel.  With the factor cut down to what fits in clusters instead, a
+    // call was up to 2.1 us slower (5.7 -> 7.8 us at B = 2, 2 heads, N = 12765, 2040 tokens attended: 8 splits for 16),
+    // and the step gained little: clusters of 16 there take 8.8 us a layer, of 8 9.9; at B = 4, 8 heads, N = 4096, 1024
+    // tokens 8 splits and a combine 13.7, clusters of 6 12.9.
     constexpr int kGpcs = 8, kGpcSlots = 35;
-    const int64_t most = std::min<int64_t>(8, std::max<int64_t>(1, n_chunks / (2 * kWarps)));
-    int64_t m = 0;
-    for (int64_t s = most; s >= 1 && m == 0; --s) {
-      int64_t fit = 0;
-      for (int gpc = 0; gpc < kGpcs; ++gpc) {
-        const int held = (predictor.clusters + gpc) / kGpcs * predictor.ctas * (predictor.whole_sm ? 2 : 1);
-        fit += std::max(0, kGpcSlots - held) / s;
-      }
-      if (problems <= fit && problems * s <= 200) m = s;
-    }
-    if (m < 2 && most >= 2 && problems * 2 <= 264) m = 2;      // pairs find room anywhere
-    // What fewer splits cost must stay below what the two launches cost (about 16 chunk times).
-    const int held = predictor.clusters * predictor.ctas * (predictor.whole_sm ? 2 : 1);
-    if (m > 0 && split_cost(m, slots) - split_cost(best, slots) <= 16) {
-      best = m;
-      w->merge_in_cluster = true;
-    } else if (held <= slots / 2) {
-      // Too long a list for that, but the gather still runs beside the predictor, in the slots it leaves, unless that
-      // makes it much longer: 12.3 against 15.7 us per layer at B = 2, N = 18546, 4 KV heads, 4608 tokens attended;
-      // with twice the chunks per CTA (B = 8, N = 16384, 8 heads, 2048 tokens) 28.5 against 27.6.
+    const int cta_slots = predictor.whole_sm ? 2 : 1, held = predictor.clusters * predictor.ctas * cta_slots;
+    int64_t fit = 0;                               // clusters of `best` CTAs
+    for (int gpc = 0; gpc < kGpcs; ++gpc)
+      fit += std::max(0, kGpcSlots - (predictor.clusters + gpc) / kGpcs * predictor.ctas * cta_slots) / best;
+    if (best <= kMaxClusterCtas && ((problems <= fit && problems * best <= 200) || (best == 2 && problems * 2 <= 264))) {
+      w->merge_in_cluster = true;                  // (pairs find room anywhere)
+    } else if (!score_select_cluster_pays_alone(p)) {
+      w->beside = true;                            // (a caller of the two calls has gained nothing to give away)
+    } else if (held <= (rh > 4 ? slots / 4 : slots / 2)) {
+      // Fewer splits, in the slots that the predictor leaves, where that costs a call at most 5 %: 12.3 against 15.7 us
+      // per layer at B = 2, N = 18546, 4 KV heads, 4608 tokens attended; with twice the chunks per CTA (B = 8,
+      // N = 16384, 8 heads, 2048 tokens) 28.5 against 27.6.  Gathers of more than four heads per CTA are held up by
+      // predictors of many CTAs: B = 6, 2 KV heads of 8, N = 8093, per-head metadata 16.9 us beside, 15.7 behind.
       const int64_t s = best_splits(slots - held, 256);
       if (split_cost(s, slots - held) - split_cost(best, slots) <= 16) {
         best = s;
@@ -784,6 +784,10 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
       }
     }
   }
+  // On its own, a call saves a launch by merging in clusters, which counts where the host sets the pace (calls on a small
+  // fp32 layer 16.2 us against 18.6); clusters of more than 8 take longer than gather and combine even so
+  // (B = 1, N = 16384, 8 heads, 2048 tokens attended: 8.3 us against 6.5).
+  w->merge_alone = w->merge_in_cluster && best <= 8;
   w->splits = int(best);
   const size_t row = size_t(p.d) * (p.kv_dtype == KVSWAP_F32 ? 4 : 2);
   const size_t stage = 2 * kTok * row;

@@ -75,6 +75,7 @@ extern "C" int kvswap_sparse_decode_static(const kvswap_shape* shape, const void
     return KVSWAP_ERR_ALIGN;
   void* scratch = nullptr;
   if (scratch_address(&scratch) != cudaSuccess) return KVSWAP_ERR_CUDA;
+  w.merge_in_cluster = w.merge_alone;
   cudaError_t e = launch_sparse_decode(p, w, q, K, V, group_idx, n_selected,
                                        reinterpret_cast<float*>(static_cast<char*>(scratch) + 256), out, lse_opt,
                                        static_cast<uint32_t*>(scratch), static_cast<cudaStream_t>(cuda_stream));

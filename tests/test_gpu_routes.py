@@ -1,17 +1,84 @@
-"""Calls on both sides of the lines between the kernels that the library chooses from, each checked to have taken the one
-it should, against the oracle."""
+"""Decode steps and calls on every schedule the library chooses from, each checked to have taken it: a step gives
+exactly what the per-layer calls give, and a predictor what the oracle gives, on both sides of the lines between them."""
 import dataclasses
 
 import pytest
+import torch
 
 from paper_2511_11907_b200 import binding as kv
+from paper_2511_11907_b200 import device_workload as DW
+from paper_2511_11907_b200 import runtime as rt
 from paper_2511_11907_b200 import workloads as W
 from launches import launched
+from test_gpu_decode_step import _run_case
 from test_gpu_parity import run_layer_parity
 
 pytestmark = pytest.mark.gpu
 
 KV = W.SCOPE_KV_HEAD
+
+# kernels of a step of several layers
+CLUSTERS = {"score_select_cluster_kernel", "sparse_decode_splitk_kernel"}      # the splits merge in clusters
+BESIDE = CLUSTERS | {"combine_kernel"}
+
+
+def _wl(**kw):
+    base = dict(layers=4, batch=2, n_ctx=20011, top_k=40, calib_rows=1024)
+    base.update(kw)
+    if base.get("kv_dtype") == W.F32:
+        base.update(meta_dtype=W.F32, q_dtype=W.F32)
+    return dataclasses.replace(W.CONFIGS[5], name="routes", walk_steps=1, **base)
+
+
+def _step_route(wl, meta_heads, scope, flags=0):
+    dw = DW.build(wl, meta_heads, scope, walk_steps=1, reserve_bytes=1 << 30)
+    shape = dw.shape.with_flags(flags)
+    ws = rt.alloc_workspace(shape)
+    for m in dw.meta:
+        m.zero_()
+    out = torch.empty((wl.layers, wl.batch, wl.n_q_heads, wl.head_dim), device="cuda")
+    idx = torch.empty((wl.layers, wl.batch, shape.n_scopes, wl.top_k), dtype=torch.int32, device="cuda")
+    nsel = torch.empty((wl.layers, wl.batch, shape.n_scopes), dtype=torch.int32, device="cuda")
+    layers = dw.layer_tables()
+    return launched(lambda: kv.kvswap_decode_step(shape, layers, dw.q_walk[0], out, None, idx, nsel, ws))
+
+
+# Predictor and attention side by side: lists of one split, of up to 8 and of up to 16 (more than a portable cluster)
+# merged in clusters, and longer ones by a combine kernel.
+@pytest.mark.parametrize("meta_heads,kw,route", [
+    ("joint", dict(batch=1, n_ctx=2048, top_k=8), CLUSTERS),                   # 1 split
+    ("joint", dict(batch=1, n_ctx=4100, top_k=40), CLUSTERS),                  # 2
+    ("per_head", dict(batch=1, n_ctx=4100, top_k=60), CLUSTERS),               # 3
+    ("joint", dict(batch=2, n_ctx=4100, top_k=128), CLUSTERS),                 # 8
+    ("joint", dict(batch=1, n_ctx=16384, top_k=150), CLUSTERS),                # 9
+    ("joint", dict(batch=1, n_ctx=16384, top_k=256), CLUSTERS),                # 16
+    ("joint", dict(batch=1, n_ctx=4096, top_k=256, kv_dtype=W.F32), CLUSTERS),
+    ("joint", dict(batch=1, n_ctx=16384, top_k=290), BESIDE),                  # 18
+    ("joint", dict(batch=4, n_ctx=8003, top_k=400), BESIDE),
+    ("per_head", dict(batch=1, n_ctx=16384, top_k=400), BESIDE),
+])
+def test_step_side_by_side(meta_heads, kw, route):
+    wl = _wl(**kw)
+    names = _step_route(wl, 1 if meta_heads == "joint" else wl.n_kv_heads, KV)
+    assert set(names) == route
+    assert len(names) == wl.layers * len(route)
+    _run_case(wl, meta_heads, KV)
+
+
+@pytest.mark.parametrize("batch,n_ctx,top_k,combine", [(1, 2048, 8, False), (2, 4100, 128, False), (1, 16384, 150, True), (1, 16384, 256, True)])
+def test_attention_on_its_own(batch, n_ctx, top_k, combine):
+    """A call merges up to 8 splits in clusters, where the step does, and more with a combine kernel."""
+    wl = _wl(batch=batch, n_ctx=n_ctx, top_k=top_k)
+    shape = rt.shape_for(wl, 1, KV)
+    K = torch.zeros((batch, 8, n_ctx, 128), dtype=torch.bfloat16, device="cuda")
+    q = torch.zeros((batch, 32, 128), dtype=torch.bfloat16, device="cuda")
+    idx, nsel = rt.alloc_selection(shape)
+    idx.copy_(torch.arange(top_k, dtype=torch.int32, device="cuda").expand_as(idx))
+    nsel.fill_(top_k)
+    (out, lse), ws = rt.alloc_output(shape), rt.alloc_workspace(shape)
+    want = ["sparse_decode_splitk_kernel"] + (["combine_kernel"] if combine else [])
+    assert launched(lambda: kv.kvswap_sparse_decode(shape, q, K, K, idx, nsel, out, lse, ws)) == want
+    assert launched(lambda: kv.kvswap_sparse_decode_static(shape, q, K, K, idx, nsel, out, lse)) == want
 
 
 # The line at 6144 groups between the launch of clusters and the streaming scorer, on both sides of it, and the line
