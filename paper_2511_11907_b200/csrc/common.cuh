@@ -213,6 +213,17 @@ __device__ __forceinline__ float meta_store_scale(const Problem& p) {
   return __uint_as_float(uint32_t(127 - p.meta_exp) << 23);
 }
 
+// Three bf16 pieces of a pair of fp32 values (x in the low half of each word) whose sum is the value: round to nearest
+// even, saturating, so that a value beyond the largest bf16 (3.39e38) leaves a remainder and not an infinity.
+__device__ __forceinline__ void split3_bf16(float x, float y, uint32_t (&w)[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(w[k]) : "f"(y), "f"(x));
+    x -= __uint_as_float(w[k] << 16);
+    y -= __uint_as_float(w[k] & 0xffff0000u);
+  }
+}
+
 // 16-byte read-only global load that does not allocate in L1 (streamed once).
 __device__ __forceinline__ uint4 ld_stream16(const void* p) {
   uint4 v;

@@ -135,11 +135,6 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint3
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
-
 // KV_T = float: K too is split into three bf16 pieces, on the way from the registers it was loaded into; of the nine
 // products per entry six are issued, those left out are below 2^-24 of it.  (Against float64 the 2-norm error is 2.1e-7
 // where the fp32-pipe kernel's was 5.7e-7; a layer of 4 x 20000 tokens, 8 heads of 128, r = 32: 283 -> 126 us.)
@@ -166,18 +161,12 @@ project_keys_mma_kernel(Problem p, const KV_T* __restrict__ K, const float* __re
     const int t = ln & 3, col = col0 + nt * 8 + (ln >> 2);
     const int c0 = 32 * (ks >> 1) + 8 * t + 4 * (ks & 1);      // channels c0 .. c0+3 feed this lane's k slots
     const float* src = proj + (int64_t(g) * D + c0) * p.r + col;
-    float v[4], hi[4], mid[4], lo[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      v[e] = src[int64_t(e) * p.r];
-      hi[e] = __bfloat162float(__float2bfloat16_rn(v[e]));
-      mid[e] = __bfloat162float(__float2bfloat16_rn(v[e] - hi[e]));
-      lo[e] = v[e] - hi[e] - mid[e];                 // exact; rounds to bf16 below
-    }
+    uint32_t w01[3], w23[3];
+    split3_bf16(src[0], src[p.r], w01);
+    split3_bf16(src[2 * int64_t(p.r)], src[3 * int64_t(p.r)], w23);
     uint2* dst = bfrag + (int64_t(i >> 5) * 3) * 32 + ln;
-    dst[0] = make_uint2(pack_bf16(hi[0], hi[1]), pack_bf16(hi[2], hi[3]));
-    dst[32] = make_uint2(pack_bf16(mid[0], mid[1]), pack_bf16(mid[2], mid[3]));
-    dst[64] = make_uint2(pack_bf16(lo[0], lo[1]), pack_bf16(lo[2], lo[3]));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dst[32 * k] = make_uint2(w01[k], w23[k]);
   }
   __syncthreads();
 
@@ -249,14 +238,10 @@ project_keys_mma_kernel(Problem p, const KV_T* __restrict__ K, const float* __re
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
                 const uint4 v = cur[m][h][2 * q + (e >> 1)];
-                float x = __uint_as_float((e & 1) ? v.z : v.x), y = __uint_as_float((e & 1) ? v.w : v.y);
+                uint32_t w[3];
+                split3_bf16(__uint_as_float((e & 1) ? v.z : v.x), __uint_as_float((e & 1) ? v.w : v.y), w);
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                  const __nv_bfloat162 pr = __floats2bfloat162_rn(x, y);
-                  ka[m][h][k][e] = *reinterpret_cast<const uint32_t*>(&pr);
-                  const float2 f = __bfloat1622float2(pr);
-                  x -= f.x; y -= f.y;
-                }
+                for (int k = 0; k < 3; ++k) ka[m][h][k][e] = w[k];
               }
             } else {
               const uint4 v = cur[m][h][q];

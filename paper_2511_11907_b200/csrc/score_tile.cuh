@@ -52,16 +52,6 @@ __device__ __forceinline__ void mma16816_bf16(float (&d)[4], uint32_t a0, uint32
 __device__ __forceinline__ uint32_t pack_half2(__half lo, __half hi) {
   return uint32_t(__half_as_ushort(lo)) | (uint32_t(__half_as_ushort(hi)) << 16);
 }
-// Three bf16 pieces of a pair of values (x in the low half of each word).
-__device__ __forceinline__ void split3_bf16(float x, float y, uint32_t (&w)[3]) {
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-    w[k] = *reinterpret_cast<const uint32_t*>(&h);
-    const float2 f = __bfloat1622float2(h);
-    x -= f.x; y -= f.y;
-  }
-}
 
 // The row operand of one warp: lane (g, t) supplies entries t R/4 .. of the query of scope g.
 template <int META, int R>

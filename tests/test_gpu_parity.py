@@ -652,3 +652,39 @@ def test_one_workspace_serves_ranks_types_and_flags_in_turn():
                 kv.kvswap_score_select(shape, q, proj, meta, idx, nsel, None, ws)
                 assert torch.equal(idx, want), (kinds[a], kinds[b])
     assert kv.kvswap_read_device_status(ws) == 0
+
+
+def test_fp32_values_beyond_the_largest_bf16_are_finite_inputs():
+    """fp32 metadata and keys take the tensor cores in bf16 pieces; values between the largest bf16 (3.39e38) and the
+    largest fp32 split like any other.  Sums of 32 and of 512 products in fp32: 2e-6 of the sum of magnitudes covers them."""
+    big = torch.finfo(torch.float32).max
+    H, d, r, N, G = 4, 128, 32, 2048, 8
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+    for n in (N, 40000):                                                  # launch of clusters, streaming scorer
+        shape = kv.make_shape(batch=1, n_ctx=n, n_q_heads=H, n_kv_heads=H, head_dim=d, rank=r, meta_heads=1, group_size=G,
+                              top_k=20, kv_dtype=W.F32, meta_dtype=W.F32, q_dtype=W.F32)
+        q = torch.randn((1, H, d), generator=g, device="cuda") * 1e-3
+        proj = torch.randn((H, d, r), generator=g, device="cuda") * 1e-3
+        meta = torch.randn((1, 1, n, r), generator=g, device="cuda")
+        meta[0, 0, 5::97, 3], meta[0, 0, 11::89, 7], meta[0, 0, 13::83, 30] = big, -big, 3.3962e38
+        idx, nsel = rt.alloc_selection(shape)
+        R = torch.empty((1, H, n // G), device="cuda")
+        kv.kvswap_score_select(shape, q, proj, meta, idx, nsel, R, rt.alloc_workspace(shape))
+        u = torch.einsum("hd,hdr->hr", q[0].double(), proj.double())
+        T = u @ meta[0, 0].double().T
+        want = T[:, :n // G * G].view(H, -1, G).max(2).values
+        bound = (u.abs() @ meta[0, 0].abs().double().T)[:, :n // G * G].view(H, -1, G).max(2).values
+        assert torch.isfinite(R).all()
+        assert ((R[0].double() - want).abs() <= 2e-6 * bound).all()
+        assert np.array_equal(idx.cpu().numpy()[0], O.select(R.cpu().numpy().astype(np.float64), 20)[0])
+    K = torch.randn((1, H, N, d), generator=g, device="cuda")
+    K[0, 1, 3::57, 9], K[0, 2, 8::61, 100], K[0, 0, 5::71, 0] = big, -big, -3.3962e38
+    out = torch.empty((1, 1, N, r), device="cuda")
+    kshape = kv.make_shape(batch=1, n_ctx=N, n_q_heads=H, n_kv_heads=H, head_dim=d, rank=r, meta_heads=1, group_size=G, top_k=20,
+                           kv_dtype=W.F32, meta_dtype=W.F32, q_dtype=W.F32)
+    kv.kvswap_project_keys(kshape, K, proj, out, 0, N, None)
+    want = torch.einsum("hnd,hdr->nr", K[0].double(), proj.double())
+    bound = torch.einsum("hnd,hdr->nr", K[0].double().abs(), proj.double().abs())
+    assert torch.isfinite(out).all()
+    assert ((out[0, 0].double() - want).abs() <= 2e-6 * bound).all()
