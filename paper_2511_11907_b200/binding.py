@@ -1,4 +1,5 @@
-"""Binding of libkvswap.so: argument marshalling only, through ctypes or, for the per-layer calls, natively.
+"""Binding of libkvswap.so: argument marshalling only, through ctypes; for the per-layer calls natively where the
+extension module is built for this interpreter (csrc/pycalls.cpp: 3.7 us a call against 5.3).
 
 Every function has the name and argument order of its C entry point (include/kvswap.h).
 Tensors are torch CUDA tensors; the binding passes ``data_ptr()`` and the current CUDA stream
@@ -140,25 +141,40 @@ def _entry_points():
     return (*addr, torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
 
 
-# The per-layer calls, marshalled natively (csrc/pycalls.cpp); tensors or None, stream=None is torch's current one:
-#   kvswap_project_keys(shape, K, proj, meta_out, n_begin, n_end, ws, stream=None)
-#   kvswap_score_select(shape, q, proj, meta, group_idx, n_selected, group_scores_opt, ws, stream=None)
-#   kvswap_sparse_decode(shape, q, K, V, group_idx, n_selected, out, lse_opt, ws, stream=None)
-_NATIVE = ("kvswap_project_keys", "kvswap_score_select", "kvswap_sparse_decode")
+def kvswap_project_keys(shape, K, proj, meta_out, n_begin, n_end, ws, stream=None) -> None:
+    """K_lr = Flatten(K) A for tokens n_begin <= n < n_end; ws may be None."""
+    _check(load().kvswap_project_keys(ctypes.byref(shape), _ptr(K), _ptr(proj), _ptr(meta_out), int(n_begin),
+                                      int(n_end), _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(),
+                                      _stream(stream)), "kvswap_project_keys")
 
 
-def __getattr__(name):
-    """Takes the per-layer calls from the extension module on their first use (it may be built after this import)."""
-    if name not in _NATIVE:
-        raise AttributeError(f"module {__name__!r} has no attribute {name!r}")
+def kvswap_score_select(shape, q, proj, meta, group_idx, n_selected, group_scores_opt, ws, stream=None) -> None:
+    """Low-rank scores, group maxima and the indices of the top_k groups; group_scores_opt may be None."""
+    _check(load().kvswap_score_select(ctypes.byref(shape), _ptr(q), _ptr(proj), _ptr(meta), _ptr(group_idx),
+                                      _ptr(n_selected), _ptr(group_scores_opt), _ptr(ws),
+                                      0 if ws is None else ws.numel() * ws.element_size(), _stream(stream)),
+           "kvswap_score_select")
+
+
+def kvswap_sparse_decode(shape, q, K, V, group_idx, n_selected, out, lse_opt, ws, stream=None) -> None:
+    """Attention over the selected groups and the rolling-buffer tail; lse_opt may be None."""
+    _check(load().kvswap_sparse_decode(ctypes.byref(shape), _ptr(q), _ptr(K), _ptr(V), _ptr(group_idx),
+                                       _ptr(n_selected), _ptr(out), _ptr(lse_opt), _ptr(ws),
+                                       0 if ws is None else ws.numel() * ws.element_size(), _stream(stream)),
+           "kvswap_sparse_decode")
+
+
+def _native_calls() -> None:
+    """Puts the extension module's per-layer calls in the place of the three above; without one they stay."""
     try:
         from . import _calls
-    except ImportError as e:
-        raise RuntimeError("the binding's extension module is not built: build it with "
-                           "`python -m paper_2511_11907_b200.build`") from e
+    except ImportError:
+        return
     _calls.setup(_entry_points, KVSwapError)
-    globals().update({n: getattr(_calls, n) for n in _NATIVE})
-    return globals()[name]
+    globals().update({n: getattr(_calls, n) for n in ("kvswap_project_keys", "kvswap_score_select", "kvswap_sparse_decode")})
+
+
+_native_calls()
 
 
 def kvswap_workspace_bytes(shape: kvswap_shape) -> int:

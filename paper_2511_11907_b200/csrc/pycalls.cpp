@@ -1,7 +1,7 @@
 // The per-layer calls of the Python binding, marshalled natively: kvswap_project_keys, kvswap_score_select and
-// kvswap_sparse_decode take tensors and pass their addresses on, as binding.py's ctypes versions do.  A model that runs its own
-// layers between the calls issues two of them per layer, and through ctypes a call cost 1.6 us of marshalling on top of
-// 3.7 us of library and launch.
+// kvswap_sparse_decode take tensors and pass their addresses on, as binding.py's ctypes versions do, in whose place they
+// are put.  A model that runs its own layers between the calls issues two of them per layer, and through ctypes a call
+// cost 1.6 us of marshalling on top of 3.7 us of library and launch.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 

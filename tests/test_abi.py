@@ -208,6 +208,50 @@ def test_8bit_metadata_shapes_are_validated(lib):
     assert kv.kvswap_validate_shape(ok.with_flags(1 << 16)) == 2           # unknown flag bit
 
 
+def test_the_extension_module_is_named_for_its_interpreter():
+    import importlib.machinery
+    name = os.path.basename(kvbuild.CALLS)
+    assert name.startswith("_calls.") and name[len("_calls"):] == importlib.machinery.EXTENSION_SUFFIXES[0] != ".so"
+
+
+@pytest.mark.parametrize("missing", ["Python.h", "g++"])
+def test_the_library_builds_without_what_the_extension_module_needs(monkeypatch, tmp_path, missing):
+    ran = []
+
+    class Done:
+        returncode, stdout, stderr = 0, "", ""
+
+    monkeypatch.setattr(kvbuild.subprocess, "run", lambda cmd, **kw: ran.append(cmd[0]) or Done())
+    which = kvbuild.shutil.which
+    if missing == "g++":
+        monkeypatch.setattr(kvbuild.shutil, "which", lambda exe: None if exe == "g++" else which(exe))
+    else:
+        monkeypatch.setattr(kvbuild.sysconfig, "get_paths", lambda: {"include": str(tmp_path)})
+    assert kvbuild.build(force=True) == kvbuild.LIB
+    assert ran and all("nvcc" in exe for exe in ran)
+
+
+def test_the_per_layer_calls_work_without_the_extension_module(lib, tmp_path):
+    """In a process that cannot import it (here: a copy of the package without it) the ctypes versions answer."""
+    import shutil
+    import subprocess
+    import sys
+    pkg = tmp_path / "paper_2511_11907_b200"
+    pkg.mkdir()
+    for f in ("__init__.py", "binding.py", "workloads.py"):
+        shutil.copy(os.path.join(ROOT, "paper_2511_11907_b200", f), pkg / f)
+    os.symlink(kv.LIB_PATH, pkg / "libkvswap.so")
+    code = ("from paper_2511_11907_b200 import binding as kv\n"
+            "s = kv.make_shape(batch=2, n_ctx=1024, n_q_heads=8, n_kv_heads=2, head_dim=64, rank=16, meta_heads=1, group_size=4,\n"
+            "                  top_k=32, kv_dtype=0, meta_dtype=0, q_dtype=0)\n"
+            "for call, n in ((kv.kvswap_project_keys, 3), (kv.kvswap_score_select, 6), (kv.kvswap_sparse_decode, 7)):\n"
+            "    args = [None] * n + ([0, 8] if n == 3 else [])\n"
+            "    try: call(s, *args, None, stream=0)\n"
+            "    except kv.KVSwapError as e: assert e.status == 1, e\n"
+            "    else: raise AssertionError('no error')\n")
+    subprocess.run([sys.executable, "-c", code], cwd=tmp_path, check=True, timeout=120)
+
+
 def test_status_strings_and_version(lib):
     seen = {kv.status_string(i) for i in range(11)}
     assert len(seen) == 11 and "ok" in seen
