@@ -170,7 +170,7 @@ def _native_calls() -> None:
         from . import _calls
     except ImportError:
         return
-    _calls.setup(_entry_points, KVSwapError)
+    _calls.setup(_entry_points, KVSwapError, kvswap_shape)
     globals().update({n: getattr(_calls, n) for n in ("kvswap_project_keys", "kvswap_score_select", "kvswap_sparse_decode")})
 
 

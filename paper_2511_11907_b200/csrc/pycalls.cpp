@@ -16,12 +16,13 @@ using DecodeFn = int (*)(const kvswap_shape*, const void*, const void*, const vo
 
 PyObject* g_resolve = nullptr;       // binding's callable: loads the library, returns what the calls need
 PyObject* g_error = nullptr;         // KVSwapError
+PyObject* g_shape = nullptr;         // kvswap_shape
 PyObject* g_device = nullptr;        // () -> current device
 PyObject* g_raw_stream = nullptr;    // (device) -> cudaStream_t of the current stream
 ProjectFn g_project = nullptr;
 SelectFn g_select = nullptr;
 DecodeFn g_decode = nullptr;
-PyObject *s_data_ptr, *s_numel, *s_element_size, *s_cuda_stream;
+PyObject *s_data_ptr, *s_numel, *s_element_size, *s_cuda_stream, *s_value;
 
 bool ready() {
   if (g_decode != nullptr) return true;
@@ -65,9 +66,9 @@ bool size_of(PyObject* t, size_t* n) {
   return true;
 }
 
-// A torch stream, a handle, or None: torch's current stream.
+// A torch stream, a handle (an int or a ctypes.c_void_p), or None: torch's current stream.
 bool stream_of(PyObject* s, void** p) {
-  unsigned long long v = 0;
+  *p = nullptr;
   PyObject* h;
   if (s == Py_None) {
     PyObject* dev = PyObject_CallNoArgs(g_device);
@@ -76,9 +77,12 @@ bool stream_of(PyObject* s, void** p) {
     Py_DECREF(dev);
   } else if (PyLong_Check(s)) {
     h = Py_NewRef(s);
-  } else {
-    h = PyObject_GetAttr(s, s_cuda_stream);
+  } else if ((h = PyObject_GetAttr(s, s_cuda_stream)) == nullptr && PyErr_ExceptionMatches(PyExc_AttributeError)) {
+    PyErr_Clear();
+    h = PyObject_GetAttr(s, s_value);
   }
+  if (h == Py_None) { Py_DECREF(h); return true; }                  // the default stream
+  unsigned long long v = 0;
   if (!as_u64(h, &v)) return false;
   *p = reinterpret_cast<void*>(v);
   return true;
@@ -117,9 +121,12 @@ bool arguments(const char* fn, const char* const* names, int n, PyObject* const*
 struct Shape {                        // the bytes of the ctypes structure
   Py_buffer view = {};
   bool get(PyObject* o) {
+    const int is_shape = PyObject_IsInstance(o, g_shape);
+    if (is_shape < 0) return false;
+    if (is_shape == 0) { PyErr_Format(PyExc_TypeError, "shape: expected a kvswap_shape, got %.100s", Py_TYPE(o)->tp_name); return false; }
     if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) != 0) return false;
     if (view.len == Py_ssize_t(sizeof(kvswap_shape))) return true;
-    PyErr_SetString(PyExc_TypeError, "shape: a kvswap_shape is expected");
+    PyErr_SetString(PyExc_TypeError, "shape: a kvswap_shape of another size");
     return false;
   }
   const kvswap_shape* ptr() const { return static_cast<const kvswap_shape*>(view.buf); }
@@ -187,12 +194,14 @@ PyObject* sparse_decode(PyObject*, PyObject* const* args, Py_ssize_t n_pos, PyOb
   return done(status, "kvswap_sparse_decode");
 }
 
-// setup(resolve, error): resolve() -> (addresses of the three entry points, current-device and raw-stream callables).
+// setup(resolve, error, shape): resolve() -> (addresses of the three entry points, current-device and raw-stream
+// callables); the classes KVSwapError and kvswap_shape.
 PyObject* setup(PyObject*, PyObject* args) {
-  PyObject *r, *e;
-  if (!PyArg_ParseTuple(args, "OO", &r, &e)) return nullptr;
+  PyObject *r, *e, *s;
+  if (!PyArg_ParseTuple(args, "OOO", &r, &e, &s)) return nullptr;
   g_resolve = Py_NewRef(r);
   g_error = Py_NewRef(e);
+  g_shape = Py_NewRef(s);
   Py_RETURN_NONE;
 }
 
@@ -211,5 +220,6 @@ PyMODINIT_FUNC PyInit__calls() {
   s_numel = PyUnicode_InternFromString("numel");
   s_element_size = PyUnicode_InternFromString("element_size");
   s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+  s_value = PyUnicode_InternFromString("value");
   return PyModule_Create(&kModule);
 }

@@ -252,6 +252,38 @@ def test_the_per_layer_calls_work_without_the_extension_module(lib, tmp_path):
     subprocess.run([sys.executable, "-c", code], cwd=tmp_path, check=True, timeout=120)
 
 
+def _per_layer_calls():
+    """(call, arguments after the shape): NULL pointers, which the library refuses before it touches a GPU."""
+    return [(kv.kvswap_project_keys, [None] * 3 + [0, 8, None]), (kv.kvswap_score_select, [None] * 7),
+            (kv.kvswap_sparse_decode, [None] * 8)]
+
+
+def test_the_per_layer_calls_take_a_shape_and_nothing_else(lib):
+    s = good_shape()
+    for call, args in _per_layer_calls():
+        with pytest.raises(kv.KVSwapError) as e:
+            call(s, *args, stream=0)
+        assert e.value.status == 1
+        for other in (bytes(s), bytearray(bytes(s)), (ctypes.c_char * ctypes.sizeof(s)).from_buffer_copy(s), None, 7, [0] * 104):
+            with pytest.raises(TypeError):
+                call(other, *args, stream=0)
+
+
+def test_the_per_layer_calls_take_every_kind_of_stream_handle(lib):
+    class Stream:
+        def __init__(self, handle):
+            self.cuda_stream = handle
+
+    for call, args in _per_layer_calls():
+        for stream in (0, ctypes.c_void_p(0), ctypes.c_void_p(None), ctypes.c_void_p(4096), Stream(0), Stream(4096), Stream(None)):
+            with pytest.raises(kv.KVSwapError) as e:
+                call(good_shape(), *args, stream=stream)
+            assert e.value.status == 1                     # reached the library
+        for stream in ("0", 1.5, object()):
+            with pytest.raises((TypeError, AttributeError)):
+                call(good_shape(), *args, stream=stream)
+
+
 def test_status_strings_and_version(lib):
     seen = {kv.status_string(i) for i in range(11)}
     assert len(seen) == 11 and "ok" in seen
