@@ -207,9 +207,12 @@ PyObject* setup(PyObject*, PyObject* args) {
 
 PyMethodDef kMethods[] = {
     {"setup", setup, METH_VARARGS, nullptr},
-    {"kvswap_project_keys", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(project_keys)), METH_FASTCALL | METH_KEYWORDS, nullptr},
-    {"kvswap_score_select", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(score_select)), METH_FASTCALL | METH_KEYWORDS, nullptr},
-    {"kvswap_sparse_decode", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(sparse_decode)), METH_FASTCALL | METH_KEYWORDS, nullptr},
+    {"kvswap_project_keys", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(project_keys)), METH_FASTCALL | METH_KEYWORDS,
+     "kvswap_project_keys(shape, K, proj, meta_out, n_begin, n_end, ws, stream=None)\n--\n\nK_lr = Flatten(K) A for tokens n_begin <= n < n_end; ws may be None."},
+    {"kvswap_score_select", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(score_select)), METH_FASTCALL | METH_KEYWORDS,
+     "kvswap_score_select(shape, q, proj, meta, group_idx, n_selected, group_scores_opt, ws, stream=None)\n--\n\nLow-rank scores, group maxima and the indices of the top_k groups; group_scores_opt may be None."},
+    {"kvswap_sparse_decode", reinterpret_cast<PyCFunction>(reinterpret_cast<void*>(sparse_decode)), METH_FASTCALL | METH_KEYWORDS,
+     "kvswap_sparse_decode(shape, q, K, V, group_idx, n_selected, out, lse_opt, ws, stream=None)\n--\n\nAttention over the selected groups and the rolling-buffer tail; lse_opt may be None."},
     {nullptr, nullptr, 0, nullptr}};
 PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, kMethods, nullptr, nullptr, nullptr, nullptr};
 

@@ -269,6 +269,18 @@ def test_the_per_layer_calls_take_a_shape_and_nothing_else(lib):
                 call(other, *args, stream=0)
 
 
+def test_the_per_layer_calls_have_signatures_and_docstrings(lib):
+    import ast
+    import inspect
+    tree = ast.parse(inspect.getsource(kv))                # those of the ctypes versions that they stand for
+    written = {f.name: f for f in tree.body if isinstance(f, ast.FunctionDef)}
+    for call, args in _per_layer_calls():
+        sig = inspect.signature(call)
+        assert list(sig.parameters) == [a.arg for a in written[call.__name__].args.args]
+        assert sig.parameters["stream"].default is None and len(sig.parameters) == len(args) + 2
+        assert call.__doc__ == ast.get_docstring(written[call.__name__])
+
+
 def test_the_per_layer_calls_take_every_kind_of_stream_handle(lib):
     class Stream:
         def __init__(self, handle):
