@@ -1,7 +1,7 @@
-"""kvswap_decode_step (all layers of one decode step in one call: each layer scored one layer ahead
-of its attention, its TopK merged with the previous layer's split-K combine, the low-rank queries
-of the layer after it formed in the same launch) gives exactly what the per-layer calls give.  The
-per-layer calls themselves are checked against the oracle in test_gpu_parity.py."""
+"""kvswap_decode_step (all layers of one decode step in one call, each layer predicted one layer ahead of its
+attention) gives exactly what the per-layer calls give.  Most shapes here are short enough for the schedule that
+runs predictor and attention side by side; test_gpu_routes.py has the others and checks which schedule a shape takes.
+The per-layer calls themselves are checked against the oracle in test_gpu_parity.py."""
 import pytest
 import torch
 
@@ -23,19 +23,20 @@ def _step_buffers(dw):
     return out, lse, idx, nsel
 
 
-def _run_case(wl, meta_heads, scope, lookahead=0):
+def _run_case(wl, meta_heads, scope, lookahead=0, flags=0):
     dw = DW.build(wl, 1 if meta_heads == "joint" else wl.n_kv_heads, scope, walk_steps=1, reserve_bytes=1 << 30)
     assert dw.layers_resident == wl.layers
-    ws = rt.alloc_workspace(dw.shape)
+    shape = dw.shape.with_flags(flags)
+    ws = rt.alloc_workspace(shape)
     for l in range(wl.layers):
-        kv.kvswap_project_keys(dw.shape, dw.K[l], dw.proj[l], dw.meta[l], 0, wl.n_ctx, ws)
+        kv.kvswap_project_keys(shape, dw.K[l], dw.proj[l], dw.meta[l], 0, wl.n_ctx, ws)
     q = dw.q_walk[0]
 
     # layer by layer through the three public calls
     out_a, lse_a, idx_a, nsel_a = _step_buffers(dw)
     for l in range(wl.layers):
-        kv.kvswap_score_select(dw.shape, q[l], dw.proj[l], dw.meta[l], idx_a[l], nsel_a[l], None, ws)
-        kv.kvswap_sparse_decode(dw.shape, q[l], dw.K[l], dw.V[l], idx_a[l], nsel_a[l], out_a[l], lse_a[l], ws)
+        kv.kvswap_score_select(shape, q[l], dw.proj[l], dw.meta[l], idx_a[l], nsel_a[l], None, ws)
+        kv.kvswap_sparse_decode(shape, q[l], dw.K[l], dw.V[l], idx_a[l], nsel_a[l], out_a[l], lse_a[l], ws)
     torch.cuda.synchronize()
     assert kv.kvswap_read_device_status(ws) == 0
 
@@ -43,7 +44,7 @@ def _run_case(wl, meta_heads, scope, lookahead=0):
     ws.fill_(0xFF)
     kv.kvswap_workspace_init(ws)
     out_b, lse_b, idx_b, nsel_b = _step_buffers(dw)
-    kv.kvswap_decode_step(dw.shape, dw.layer_tables(lookahead), q, out_b, lse_b, idx_b, nsel_b, ws)
+    kv.kvswap_decode_step(shape, dw.layer_tables(lookahead), q, out_b, lse_b, idx_b, nsel_b, ws)
     torch.cuda.synchronize()
     assert kv.kvswap_read_device_status(ws) == 0
     assert torch.equal(nsel_a, nsel_b)
@@ -57,14 +58,14 @@ def _run_case(wl, meta_heads, scope, lookahead=0):
     q_host = q.cpu().pin_memory()
     out_host = torch.full(out_c.shape, float("nan"), dtype=torch.float32).pin_memory()
     q_dev = torch.zeros_like(q)
-    kv.kvswap_decode_step_host(dw.shape, dw.layer_tables(lookahead), q_host, out_host, q_dev, out_c, idx_c, nsel_c, ws)
+    kv.kvswap_decode_step_host(shape, dw.layer_tables(lookahead), q_host, out_host, q_dev, out_c, idx_c, nsel_c, ws)
     torch.cuda.synchronize()
     assert torch.equal(idx_a, idx_c)
     assert torch.equal(out_a.cpu(), out_host)
 
     # repeated steps
     for _ in range(3):
-        kv.kvswap_decode_step(dw.shape, dw.layer_tables(lookahead), q, out_b, lse_b, idx_b, nsel_b, ws)
+        kv.kvswap_decode_step(shape, dw.layer_tables(lookahead), q, out_b, lse_b, idx_b, nsel_b, ws)
     torch.cuda.synchronize()
     assert torch.equal(idx_a, idx_b) and torch.equal(out_a, out_b)
     assert kv.kvswap_read_device_status(ws) == 0
@@ -91,7 +92,7 @@ def test_decode_step_equals_layer_by_layer_calls(meta_heads, scope):
 
 @pytest.mark.parametrize("lookahead", [1, 2, 5, 1000])
 def test_decode_step_over_many_layers(lookahead):
-    """70 thin layers: the two streams hand over 140 times within one step."""
+    """70 thin layers: predictor and attention hand over 140 times within one step."""
     wl = W.CONFIGS[3].reduced("cfg3-deep", layers=70, batch=1, n_ctx=1024 + 3, top_k=16, calib_rows=1024,
                               n_q_heads=8, n_kv_heads=2)
     _run_case(wl, "joint", W.SCOPE_KV_HEAD, lookahead)
@@ -99,8 +100,7 @@ def test_decode_step_over_many_layers(lookahead):
 
 @pytest.mark.parametrize("meta_heads", ["joint", "per_head"])
 def test_decode_step_head_dim_64(meta_heads):
-    """d = 64: the merged combine + TopK launch merges 14 rows of partials per CTA, and the low-rank
-    queries formed a layer ahead take two 32-channel pieces per head."""
+    """d = 64: two 32-channel pieces per head in the low-rank queries, half the row in the attention's stages."""
     wl = W.CONFIGS[4].reduced("cfg4-d64", layers=4, batch=3, n_ctx=4096 + 19, top_k=40, calib_rows=1024, head_dim=64)
     _run_case(wl, meta_heads, W.SCOPE_KV_HEAD)
 
@@ -147,16 +147,14 @@ def test_decode_steps_back_to_back_with_alternating_queries(meta_heads, n_ctx, t
 
 
 def test_decode_step_fp32_wide_rank_per_head():
-    """fp32 everywhere, rank 128 per-head metadata, batch 64 (generic kernels on both streams)."""
+    """fp32 everywhere, rank 128 per-head metadata, batch 64 (the general kernels)."""
     wl = W.CONFIGS[1].reduced("cfg1-wide", layers=6, batch=64, n_ctx=512, rank=128, head_dim=128, n_q_heads=32,
                               n_kv_heads=8, top_k=8, calib_rows=1536)
     _run_case(wl, "per_head", W.SCOPE_KV_HEAD)
 
 
 def test_decode_step_can_be_captured_in_a_cuda_graph():
-    """After a warm-up call (which creates the internal stream and events) the step records into a
-    CUDA graph -- the internal stream forks from and joins the capturing stream -- and replays give
-    the results of the stream-ordered call."""
+    """The step records into a CUDA graph and replays give the results of the stream-ordered call."""
     wl = W.CONFIGS[3].reduced("cfg3-graph", layers=4, batch=2, n_ctx=4096 + 5, top_k=32, calib_rows=1024)
     dw = DW.build(wl, 1, W.SCOPE_KV_HEAD, walk_steps=1, reserve_bytes=1 << 30)
     ws = rt.alloc_workspace(dw.shape)

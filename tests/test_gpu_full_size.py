@@ -80,9 +80,9 @@ def test_full_size_layer_sampled_sequence(cfg, meta_heads):
 
 @pytest.mark.parametrize("cfg,lookahead", [(5, 0), (5, 1), (4, 0)])
 def test_full_size_decode_step_equals_the_per_layer_calls(cfg, lookahead):
-    """The call the benchmark times, at its shapes (six layers of the configuration): predictor and
-    attention on two streams, settled launches, waits joined per two layers -- and exactly the
-    results of the per-layer calls, which the test above ties to the oracle."""
+    """The call the benchmark times, at its shapes (six layers of the configuration): one stream, each layer
+    scored ahead of the attention before it, combine and TopK merged -- and exactly the results of
+    the per-layer calls, which the test above ties to the oracle."""
     L = 6
     wl = W.CONFIGS[cfg].reduced(f"cfg{cfg}-six-layers", layers=L, walk_steps=2)
     dw = DW.build(wl, 1, W.SCOPE_KV_HEAD)

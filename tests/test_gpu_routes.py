@@ -15,9 +15,10 @@ from test_gpu_parity import run_layer_parity
 
 pytestmark = pytest.mark.gpu
 
-KV = W.SCOPE_KV_HEAD
+KV, ALL = W.SCOPE_KV_HEAD, W.SCOPE_ALL_HEADS
 
 # kernels of a step of several layers
+CHAIN = {"score_stream_kernel", "topk_parts_kernel", "sparse_decode_splitk_kernel", "combine_select_kernel", "combine_kernel"}
 CLUSTERS = {"score_select_cluster_kernel", "sparse_decode_splitk_kernel"}      # the splits merge in clusters
 BESIDE = CLUSTERS | {"combine_kernel"}
 
@@ -41,6 +42,48 @@ def _step_route(wl, meta_heads, scope, flags=0):
     nsel = torch.empty((wl.layers, wl.batch, shape.n_scopes), dtype=torch.int32, device="cuda")
     layers = dw.layer_tables()
     return launched(lambda: kv.kvswap_decode_step(shape, layers, dw.q_walk[0], out, None, idx, nsel, ws))
+
+
+# The merged combine + TopK launch, which also forms the queries of the layer after next: 14 rows of partials per CTA at
+# d = 64, every rank and type it takes, KV heads of per-head metadata eight at a time, several terms per score, lists
+# of 2, 4 and 8 parts, more sequences than the launch of clusters takes.
+@pytest.mark.parametrize("meta_heads,scope,kw", [
+    ("joint", KV, dict(head_dim=64, batch=3, n_ctx=20019)),
+    ("per_head", KV, dict(head_dim=64, n_ctx=18003)),
+    ("joint", KV, dict(rank=16, batch=3, n_ctx=34003)),
+    ("per_head", KV, dict(rank=16, head_dim=64, n_ctx=20003)),
+    ("joint", KV, dict(rank=64, batch=3, n_ctx=9005)),
+    ("joint", ALL, dict(rank=64, n_ctx=20005)),
+    ("joint", KV, dict(kv_dtype=W.F32, batch=3, n_ctx=9001)),
+    ("per_head", KV, dict(kv_dtype=W.F32, rank=16, n_ctx=9001)),
+    ("joint", KV, dict(kv_dtype=W.F32, rank=64, group_size=4, batch=3, n_ctx=5001)),
+    ("per_head", KV, dict(n_q_heads=24, n_kv_heads=12, n_ctx=9007)),
+    ("joint", KV, dict(n_q_heads=24, n_kv_heads=12, n_ctx=17007)),
+    ("per_head", ALL, dict(n_ctx=4099)),
+    ("per_head", ALL, dict(head_dim=64, rank=16, n_ctx=9003)),
+    ("joint", KV, dict(batch=40, n_ctx=1003)),
+    ("joint", KV, dict(batch=1, n_ctx=50003)),                                 # 2 parts
+    ("joint", KV, dict(batch=1, group_size=4, n_ctx=50003)),                   # 4 parts
+    ("joint", KV, dict(batch=1, group_size=4, n_ctx=70003)),                   # 8 parts
+    ("per_head", KV, dict(batch=1, group_size=4, head_dim=64, n_ctx=70003)),
+])
+def test_step_with_the_merged_combine_and_select(meta_heads, scope, kw):
+    wl = _wl(**kw)
+    assert set(_step_route(wl, 1 if meta_heads == "joint" else wl.n_kv_heads, scope)) == CHAIN
+    _run_case(wl, meta_heads, scope)
+
+
+@pytest.mark.parametrize("meta_heads,scope,kw", [
+    ("joint", KV, dict(n_ctx=4101)),
+    ("joint", KV, dict(head_dim=64, rank=16, n_q_heads=16, n_kv_heads=4, n_ctx=40001)),
+    ("per_head", ALL, dict(n_ctx=4099)),
+    ("per_head", KV, dict(kv_dtype=W.F32, rank=64, n_ctx=3001)),
+])
+def test_step_with_the_softmax_scorer(meta_heads, scope, kw):
+    wl = _wl(**kw)
+    route = (CHAIN - {"score_stream_kernel"}) | {"lowrank_query_heads_kernel", "softmax_tc_stats_kernel", "softmax_tc_pool_kernel"}
+    assert set(_step_route(wl, 1 if meta_heads == "joint" else wl.n_kv_heads, scope, kv.KVSWAP_SCORE_SOFTMAX)) == route
+    _run_case(wl, meta_heads, scope, flags=kv.KVSWAP_SCORE_SOFTMAX)
 
 
 # Predictor and attention side by side: lists of one split, of up to 8 and of up to 16 (more than a portable cluster)

@@ -97,7 +97,7 @@ def test_softmax_variant_in_the_decode_step():
 
 
 def _tc(**kw):
-    """A workload on the tensor-core path of the variant: joint fp16 metadata, r = 32, H_q <= 32."""
+    """A workload on the tensor-core kernels of the variant, of the kind most common there: joint fp16 metadata, r = 32."""
     base = dict(layers=1, batch=2, n_ctx=8 * 150 + 5, n_q_heads=8, n_kv_heads=2, head_dim=128, rank=32, group_size=8,
                 top_k=20, kv_dtype=W.BF16, meta_dtype=W.F16, q_dtype=W.BF16, calib_rows=512)
     base.update(kw)
