@@ -35,7 +35,7 @@
  * General conventions
  *  - Every pointer is a DEVICE pointer owned by the caller unless its comment says "host".
  *    The library never allocates, frees or keeps device memory (kvswap_decode_step_tiered creates
- *    one stream and a set of events per device on its first call), and never synchronises: work is
+ *    two streams and a set of events per device on its first call), and never synchronises: work is
  *    enqueued on `cuda_stream` (a cudaStream_t passed as void*, NULL = default stream) and the
  *    returned status covers host-side validation and launch errors only.
  *  - Tensors are row-major with a dense last dimension; K, V and the metadata take explicit
@@ -98,8 +98,8 @@ typedef enum { KVSWAP_SCOPE_KV_HEAD = 0, KVSWAP_SCOPE_ALL_HEADS = 1 } kvswap_sco
  *       context's complete groups, scaled by 1/sqrt(d), BEFORE the sum over heads -- the scores
  *       of Sec. 4.3 read as attention weights rather than logits (for one head the selection is
  *       the same; across heads a sharply peaked head then outweighs a flat one).  Group scores
- *       lie in [0, heads per scope].  Two passes over the metadata (tensor cores for joint
- *       fp16 metadata with r = 32 and H_q <= 32, general fp32 kernels otherwise).
+ *       lie in [0, heads per scope].  Two passes over the metadata (tensor cores for dense fp16 or
+ *       fp32 rows with r in {16, 32, 64}, general fp32 kernels otherwise).
  *       KVSWAP_ERR_UNSUPPORTED if H_q * (r + 2) floats exceed 160 KB.
  *   KVSWAP_META_EXP(e)     bits 8..15: a power of two for 8-bit metadata (meta_dtype = KVSWAP_E4M3),
  *       -64 <= e <= 63, 0 for every other metadata type.  The paper leaves the precision of the
@@ -380,7 +380,7 @@ int kvswap_decode_step(const kvswap_shape* shape, const kvswap_layers* layers, c
  * The decode step over a tiered cache (Sec. 4.4.2, Sec. 4.4.3): the full K/V of every layer lives
  * in a slow tier, each layer has a reuse buffer (kvswap_reuse_* above) in device memory, and the
  * step's attention reads only reuse stores.  Per layer score/select runs on `cuda_stream`, one layer
- * ahead; kvswap_reuse_lookup and kvswap_reuse_fill follow it on an internal stream, so a layer's misses
+ * ahead; kvswap_reuse_lookup and kvswap_reuse_fill follow it on two internal streams in turn, so a layer's misses
  * are fetched while the layer before it is attended on `cuda_stream`; the attention is
  * kvswap_sparse_decode over the layer's reuse store with the slot list.  Arrays of L per-layer pointers are HOST arrays.
  *   K_slow, V_slow    [L] slow-tier stores, laid out by shape's kv strides (GPU-readable memory)

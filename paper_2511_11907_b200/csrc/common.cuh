@@ -50,7 +50,7 @@ struct Workspace {
   size_t off_hist;     // uint16 [B, S, 4096] + uint32 [B, S]  leading-digit histograms of the group scores' keys and tickets, zero between calls
   size_t off_partial;  // float [B, Hq, splits, d + 2]  split-K partials (m, l, acc[d])
   size_t off_softmax;  // float [B, Hq, r] per-head low-rank queries + [B, Hq, chunks, 2] softmax statistics (scorer variant)
-  size_t off_adapter;  // bf16 [H_kv, 3 r, d]       adapter split into three bf16 pieces (project_keys on tcgen05)
+  size_t off_adapter;  // bf16 or fp16 [H_kv, 3 r, d]  adapter split into three pieces of K's type (project_keys on tcgen05), then float [H_kv, r]: fp16, its scales
   size_t total;
   int splits;          // split-K factor of sparse_decode for this shape
   int splits_room;     // splits the partials are planned for: no fewer than `splits` of any context length and flags

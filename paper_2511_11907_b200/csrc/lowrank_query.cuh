@@ -1,6 +1,6 @@
 // Summed low-rank queries (Eq. 1, the query side): u = sum over heads h of q_h A_g(h), one row per
 // selection scope.  The device code is shared by the streaming scorer, which builds the queries of
-// its own row sets (score_stream.cu), and by the kernel that builds them one layer ahead beside the
+// its own row sets (score_stream.cuh), and by the kernel that builds them one layer ahead beside the
 // split-K combine (topk_select.cu): both therefore produce the same bits.
 #pragma once
 

@@ -340,8 +340,8 @@ bool try_launch_mma(const Problem& p, const void* K, const float* proj, void* me
 // layer).  The rows of K are staged in shared memory, [channel][token]; a warp takes a sixteenth of every head's
 // channels and reads each adapter row once for all eight tokens (a lane holds columns lane, lane + 32, ..); the
 // warps' sums are added through shared memory in a fixed order.  Bound by the adapter's trip from L2: a CTA per
-// token, which this replaces, read it eight times as often and took 54 us for 12 layers of 8 sequences (8 heads of
-// 128, r = 32, G = 8), this one 14.
+// token, which this replaces, read it eight times as often and took 60 us for 12 layers of 8 sequences (8 heads of
+// 128, r = 32, G = 8), this one 9.
 constexpr int kGroupTokens = 64;              // token ranges up to this length take this kernel
 constexpr int kGroupTile = 8;                 // tokens per CTA
 constexpr int kGroupWarps = 16;

@@ -17,8 +17,8 @@
 //   warp 1   issues the MMAs (one thread), owns the tensor-memory allocation (two accumulators);
 //   warps 2-5 epilogue: tcgen05.ld of the finished accumulator (one token row per thread), sum of
 //            the three pieces, running sum over heads, one rounding into the metadata type.
-// fp16 K used to take the fp32-pipe kernel: 28 layers of 5003 tokens (8 heads of 128, r = 32) took 2075 us, here
-// 319 us, of which the host issues 11 us a layer.  The launch overlaps the split of the adapter (programmatic
+// fp16 K used to take the fp32-pipe kernel: a layer of 4 x 32768 tokens (8 heads of 128, r = 32) took 402 us, here
+// 57 us, bf16 52 us.  (Prompts of a few thousand tokens: project_keys_short.cu.)  The launch overlaps the split of the adapter (programmatic
 // dependent launch, K requested before the wait): four layers of 4 x 131072 bf16 tokens 879 -> 859 us.
 // Stages and accumulators are handed over through mbarriers; every wait is bounded.
 #include <algorithm>

@@ -10,8 +10,8 @@
 // The cluster also shares the build of the low-rank queries: a warp takes a 32-channel piece of one head and
 // sends its partial products to every CTA, so each adapter row is read once per cluster instead of once per CTA.
 // Bound by latency: launch, the queries, one round of loads, two cluster barriers, the select's phases.  A call
-// at 8 KV heads, r = 32, G = 8: 7.0 us against 11.8 of the two kernels at B = 1, N = 4096, 8.9 against 12.0 at
-// N = 16384, 8.5 against 13.7 at B = 16, N = 4096.
+// at 8 KV heads, r = 32, G = 8: 7.8 us against 11.6 of the two kernels at B = 1, N = 4096, 9.8 against 12.1 at
+// N = 16384, 9.5 against 13.7 at B = 16, N = 4096; 0.8 of it is the wait ahead of the first request.
 //
 // CTA = 16 warps.  Tiles are dealt to the cluster's warps in contiguous shares, each pulled through the warp's
 // own ring of `depth` stages with bulk asynchronous copies (bounded waits).

@@ -1,7 +1,7 @@
 // C-ABI entry points that serve all layers of a model in one call: the decode step over
 // HBM-resident stores (one stream, each layer predicted one layer ahead of its attention), the
-// decode step over reuse buffers in front of a slow tier (its copies on a stream of their own)
-// and the append steps.  The tiered step keeps one internal stream and a set of events per device;
+// decode step over reuse buffers in front of a slow tier (its copies on two streams of their own)
+// and the append steps.  The tiered step keeps those two streams and a set of events per device;
 // nothing else here keeps state.
 #include <algorithm>
 #include <mutex>
@@ -67,7 +67,7 @@ static kvswap_shape reuse_store_shape(const kvswap_shape& s, int32_t n_slots) {
   return r;
 }
 
-// Per-device resources of the tiered step: a stream for the slow tier's copies and two events per layer.  Created
+// Per-device resources of the tiered step: two streams for the slow tier's copies and two events per layer.  Created
 // on first use, kept for the life of the process.
 namespace {
 struct StepResources {
@@ -114,7 +114,7 @@ cudaError_t step_resources(int n_layers, StepResources** out) {
 }  // namespace
 
 // One decode step over all layers; with `tiers` the attention is served from per-layer reuse buffers
-// that a fetch stream keeps filled from the slow tier.
+// that the fetch streams keep filled from the slow tier.
 static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* layers, const kvswap_tiers* tiers,
                             const void* q, float* out, float* lse_opt, int32_t* group_idx, int32_t* n_selected,
                             void* ws, size_t ws_bytes, const kvswap_probe* probe_opt, void* cuda_stream) {
@@ -299,7 +299,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
   }
 
   // Tiered schedule.  The caller's stream predicts and attends, one layer ahead as in kvswap_decode_step; the slow
-  // tier's link is kept busy from a stream of its own:
+  // tier's link is kept busy from two streams of its own:
   //   caller's stream:  predict(0) | predict(1) wait fetched[0] attend(0) | predict(2) wait fetched[1] attend(1) | ..
   //   fetch streams:    wait selected[l];  lookup and fill(l);  record fetched[l]        (two, layers take turns: the
   //                     lookup of a layer runs while the layer before it is still copied)
