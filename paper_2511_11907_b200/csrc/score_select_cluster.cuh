@@ -10,8 +10,8 @@
 // The cluster also shares the build of the low-rank queries: a warp takes a 32-channel piece of one head and
 // sends its partial products to every CTA, so each adapter row is read once per cluster instead of once per CTA.
 // Bound by latency: launch, the queries, one round of loads, two cluster barriers, the select's phases.  A call
-// at 8 KV heads, r = 32, G = 8: 7.8 us against 11.6 of the two kernels at B = 1, N = 4096, 9.8 against 12.1 at
-// N = 16384, 9.5 against 13.7 at B = 16, N = 4096; 0.8 of it is the wait ahead of the first request.
+// at 8 KV heads, r = 32, G = 8: 7.5 us against 11.6 of the two kernels at B = 1, N = 4096, 9.6 against 12.1 at
+// N = 16384, 9.3 against 13.7 at B = 16, N = 4096; 0.5 of it is the wait ahead of the first request.
 //
 // CTA = 16 warps.  Tiles are dealt to the cluster's warps in contiguous shares, each pulled through the warp's
 // own ring of `depth` stages with bulk asynchronous copies (bounded waits).
@@ -77,6 +77,7 @@ score_select_cluster_kernel(Problem p, ClusterArgs a) {
     for (int s = 0; s < a.depth; ++s) mbar_init(smem_addr(&sm->full[warp * 2 + s]), 1);
     mbar_init_fence();
   }
+  for (int i = threadIdx.x; i < kKeyTopBins; i += kClusterThreads) sm->select.hist[i] = 0;
   __syncwarp();
   // Without KVSWAP_INPUTS_SETTLED any input -- query, adapter, metadata -- may be the previous kernel's output.
   const bool settled = (p.flags & KVSWAP_INPUTS_SETTLED) != 0;
@@ -119,7 +120,6 @@ score_select_cluster_kernel(Problem p, ClusterArgs a) {
   };
   int item = rank + n_ctas * warp;
   if (item < n_items * kPasses) request(item);
-  for (int i = threadIdx.x; i < kKeyTopBins; i += kClusterThreads) sm->select.hist[i] = 0;
   cluster_wait();                                       // every CTA of the cluster has started
   for (; item < n_items * kPasses; item += n_ctas * kClusterWarps) {
     const int it = item % n_items, pass = item / n_items;

@@ -770,17 +770,20 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
       fit += std::max(0, kGpcSlots - (predictor.clusters + gpc) / kGpcs * predictor.ctas * cta_slots) / best;
     if (best <= kMaxClusterCtas && ((problems <= fit && problems * best <= 200) || (best == 2 && problems * 2 <= 264))) {
       w->merge_in_cluster = true;                  // (pairs find room anywhere)
-    } else if (!score_select_cluster_pays_alone(p)) {
-      w->beside = true;                            // (a caller of the two calls has gained nothing to give away)
-    } else if (held <= (rh > 4 ? slots / 4 : slots / 2)) {
+    } else {
       // Fewer splits, in the slots that the predictor leaves, where that costs a call at most 5 %: 12.3 against 15.7 us
       // per layer at B = 2, N = 18546, 4 KV heads, 4608 tokens attended; with twice the chunks per CTA (B = 8,
       // N = 16384, 8 heads, 2048 tokens) 28.5 against 27.6.  Gathers of more than four heads per CTA are held up by
       // predictors of many CTAs: B = 6, 2 KV heads of 8, N = 8093, per-head metadata 16.9 us beside, 15.7 behind.
-      const int64_t s = best_splits(slots - held, 256);
-      if (split_cost(s, slots - held) - split_cost(best, slots) <= 16) {
+      // Where the predictor does not pay alone, a caller of the two calls has gained nothing to give away: there only
+      // half of that, else the call's own factor.
+      const bool pays = score_select_cluster_pays_alone(p);
+      const int64_t s = held <= (rh > 4 ? slots / 4 : slots / 2) ? best_splits(slots - held, 256) : 0;
+      if (s > 0 && split_cost(s, slots - held) - split_cost(best, slots) <= (pays ? 16 : 8)) {
         best = s;
         w->beside = true;
+      } else {
+        w->beside = !pays;
       }
     }
   }

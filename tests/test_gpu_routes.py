@@ -125,7 +125,7 @@ def test_attention_on_its_own(batch, n_ctx, top_k, combine):
 
 
 # The line at 6144 groups between the launch of clusters and the streaming scorer, on both sides of it, and the line
-# at one tile per warp for fewer than eight scopes.
+# at one tile per warp for one sequence of fewer than eight scopes.
 @pytest.mark.parametrize("kw,name", [
     (dict(group_size=1, n_ctx=6144), "score_select_cluster_kernel"),
     (dict(group_size=1, n_ctx=6145), "score_stream_kernel"),
@@ -134,6 +134,7 @@ def test_attention_on_its_own(batch, n_ctx, top_k, combine):
     (dict(group_size=3, n_ctx=3 * 6145), "score_stream_kernel"),
     (dict(group_size=4, n_ctx=4 * 4096, n_kv_heads=2, n_q_heads=4), "score_select_cluster_kernel"),
     (dict(group_size=4, n_ctx=4 * 4112, n_kv_heads=2, n_q_heads=4), "score_stream_kernel"),
+    (dict(group_size=4, n_ctx=4 * 4112, n_kv_heads=2, n_q_heads=4, batch=2), "score_select_cluster_kernel"),
     (dict(group_size=1, n_ctx=5000, batch=20, rank=64, n_q_heads=8), "score_select_cluster_kernel"),     # two CTAs per SM
     (dict(group_size=1, n_ctx=6000, batch=20, rank=64, n_q_heads=8), "score_stream_kernel"),             # keys leave room for one
 ])
