@@ -74,15 +74,13 @@ bool score_select_cluster_grid(const Problem& p, ClusterGrid* g) {
   return true;
 }
 
-// On its own, not beside an attention, a cluster pays while every warp has one tile: per-head metadata at B = 1, 8 heads,
-// N = 4096 7.0 us against 9.2 of the two kernels.  With two tiles it does where eight scopes are selected for, or for joint
-// metadata of several sequences, whose queries the streaming scorer's CTAs form more than once (B = 2, 4 heads,
-// N = 20000 9.8 us against 13.4); not for per-head metadata (B = 1, 8 heads, N = 16384 10.2 us against 9.5) nor
-// for one sequence of fewer heads (4, N = 25000 11.2 us against 10.6).
+// On its own, not beside an attention, a cluster that selects for one scope of per-head metadata pays while every warp
+// has one tile: at B = 1, 8 heads, N = 16384 (two) 10.2 us against 9.5 of the two kernels, at N = 4096 7.0 against
+// 9.2.  With joint metadata it pays throughout, or nearly: one sequence of 4 heads at N = 25000 11.2 us against 10.6, but
+// two at N = 20000 9.8 against 13.4, and fp32 rows of rank 64 at N = 5690, one scope, 10.0 against 13.1.
 bool score_select_cluster_pays_alone(const Problem& p) {
   Plan pl;
-  return plan(p, &pl) &&
-         ((p.Hm == 1 && (p.S >= kQueryCols || pl.n_rests > 1)) || pl.tiles <= pl.cluster * kClusterWarps);
+  return plan(p, &pl) && (p.Hm == 1 || pl.tiles <= pl.cluster * kClusterWarps);
 }
 
 cudaError_t launch_score_select_cluster(const Problem& p, const void* q, const float* proj, const void* meta, float* scores,

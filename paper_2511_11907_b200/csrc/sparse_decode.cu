@@ -748,6 +748,10 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
   };
   const int64_t slots = 2 * kNumSMs;
   int64_t best = best_splits(slots, 256);
+  const size_t row = size_t(p.d) * (p.kv_dtype == KVSWAP_F32 ? 4 : 2);
+  const size_t stage = 2 * kTok * row;
+  w->depth = int(std::max<size_t>(2, std::min<size_t>(kMaxDepth, (100u << 10) / (kWarps * stage))));
+  const size_t gather_smem = kControlBytes + 128 + size_t(kWarps) * w->depth * stage;
   w->merge_in_cluster = w->merge_alone = w->beside = false;
   // No plan of these heads, types and M has more splits than this, whatever the rows past the last group, the
   // flags or the context length: one workspace serves a context as it grows.
@@ -763,12 +767,17 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
     // call was up to 2.1 us slower (5.7 -> 7.8 us at B = 2, 2 heads, N = 12765, 2040 tokens attended: 8 splits for 16),
     // and the step gained little: clusters of 16 there take 8.8 us a layer, of 8 9.9; at B = 4, 8 heads, N = 4096, 1024
     // tokens 8 splits and a combine 13.7, clusters of 6 12.9.
-    constexpr int kGpcs = 8, kGpcSlots = 35;
+    constexpr int kGpcs = 8;
     const int cta_slots = predictor.whole_sm ? 2 : 1, held = predictor.clusters * predictor.ctas * cta_slots;
+    // fp32 rows of 128: a CTA's stages take more than half of an SM's shared memory (with two counted per SM, clusters of 11
+    // at B = 1, 8 heads, N = 5690, r = 64 took 18.8 us a layer, a combine kernel 11.6)
+    const bool one_per_sm = gather_smem > 113 * 1024;
+    const int gpc_slots = one_per_sm ? 17 : 35, held_each = one_per_sm ? 1 : cta_slots;
     int64_t fit = 0;                               // clusters of `best` CTAs
     for (int gpc = 0; gpc < kGpcs; ++gpc)
-      fit += std::max(0, kGpcSlots - (predictor.clusters + gpc) / kGpcs * predictor.ctas * cta_slots) / best;
-    if (best <= kMaxClusterCtas && ((problems <= fit && problems * best <= 200) || (best == 2 && problems * 2 <= 264))) {
+      fit += std::max(0, gpc_slots - (predictor.clusters + gpc) / kGpcs * predictor.ctas * held_each) / best;
+    const int64_t ctas = problems * best * (one_per_sm ? 2 : 1);
+    if (best <= kMaxClusterCtas && ((problems <= fit && ctas <= 200) || (best == 2 && ctas <= 264))) {
       w->merge_in_cluster = true;                  // (pairs find room anywhere)
     } else {
       // Fewer splits, in the slots that the predictor leaves, where that costs a call at most 5 %: 12.3 against 15.7 us
@@ -792,9 +801,6 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
   // (B = 1, N = 16384, 8 heads, 2048 tokens attended: 8.3 us against 6.5).
   w->merge_alone = w->merge_in_cluster && best <= 8;
   w->splits = int(best);
-  const size_t row = size_t(p.d) * (p.kv_dtype == KVSWAP_F32 ? 4 : 2);
-  const size_t stage = 2 * kTok * row;
-  w->depth = int(std::max<size_t>(2, std::min<size_t>(kMaxDepth, (100u << 10) / (kWarps * stage))));
 }
 
 // The combine pass alone, for a gather that was enqueued with combine = false.

@@ -95,7 +95,9 @@ def test_step_with_the_softmax_scorer(meta_heads, scope, kw):
     ("joint", dict(batch=2, n_ctx=4100, top_k=128), CLUSTERS),                 # 8
     ("joint", dict(batch=1, n_ctx=16384, top_k=150), CLUSTERS),                # 9
     ("joint", dict(batch=1, n_ctx=16384, top_k=256), CLUSTERS),                # 16
-    ("joint", dict(batch=1, n_ctx=4096, top_k=256, kv_dtype=W.F32), CLUSTERS),
+    ("joint", dict(batch=1, n_ctx=4096, top_k=256, kv_dtype=W.F32, head_dim=64), CLUSTERS),
+    ("joint", dict(batch=1, n_ctx=4096, top_k=256, kv_dtype=W.F32), BESIDE),   # 16, but one CTA per SM
+    ("joint", dict(batch=1, n_ctx=4096, top_k=80, kv_dtype=W.F32), CLUSTERS),
     ("joint", dict(batch=1, n_ctx=16384, top_k=290), BESIDE),                  # 18
     ("joint", dict(batch=4, n_ctx=8003, top_k=400), BESIDE),
     ("per_head", dict(batch=1, n_ctx=16384, top_k=400), BESIDE),
@@ -124,17 +126,16 @@ def test_attention_on_its_own(batch, n_ctx, top_k, combine):
     assert launched(lambda: kv.kvswap_sparse_decode_static(shape, q, K, K, idx, nsel, out, lse)) == want
 
 
-# The line at 6144 groups between the launch of clusters and the streaming scorer, on both sides of it, and the line
-# at one tile per warp for one sequence of fewer than eight scopes.
+# The lines between the launch of clusters and the streaming scorer, on both sides: 6144 groups, two tiles per warp.
 @pytest.mark.parametrize("kw,name", [
     (dict(group_size=1, n_ctx=6144), "score_select_cluster_kernel"),
     (dict(group_size=1, n_ctx=6145), "score_stream_kernel"),
     (dict(group_size=1, n_ctx=6144, rank=64), "score_select_cluster_kernel"),
     (dict(group_size=3, n_ctx=3 * 6144 + 2), "score_select_cluster_kernel"),
     (dict(group_size=3, n_ctx=3 * 6145), "score_stream_kernel"),
-    (dict(group_size=4, n_ctx=4 * 4096, n_kv_heads=2, n_q_heads=4), "score_select_cluster_kernel"),
-    (dict(group_size=4, n_ctx=4 * 4112, n_kv_heads=2, n_q_heads=4), "score_stream_kernel"),
-    (dict(group_size=4, n_ctx=4 * 4112, n_kv_heads=2, n_q_heads=4, batch=2), "score_select_cluster_kernel"),
+    (dict(group_size=4, n_ctx=4 * 4112, n_kv_heads=2, n_q_heads=4), "score_select_cluster_kernel"),      # two tiles per warp
+    (dict(group_size=8, n_ctx=8 * 4096), "score_select_cluster_kernel"),
+    (dict(group_size=8, n_ctx=8 * 4097), "score_stream_kernel"),                                         # three
     (dict(group_size=1, n_ctx=5000, batch=20, rank=64, n_q_heads=8), "score_select_cluster_kernel"),     # two CTAs per SM
     (dict(group_size=1, n_ctx=6000, batch=20, rank=64, n_q_heads=8), "score_stream_kernel"),             # keys leave room for one
 ])
