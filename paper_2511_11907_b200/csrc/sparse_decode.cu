@@ -770,7 +770,7 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
     constexpr int kGpcs = 8;
     const int cta_slots = predictor.whole_sm ? 2 : 1, held = predictor.clusters * predictor.ctas * cta_slots;
     // fp32 rows of 128: a CTA's stages take more than half of an SM's shared memory (with two counted per SM, clusters of 11
-    // at B = 1, 8 heads, N = 5690, r = 64 took 18.8 us a layer, a combine kernel 11.6)
+    // at B = 1, 8 heads, N = 5690, r = 64, all-heads scope took 18.8 us a layer, a combine kernel 12.3)
     const bool one_per_sm = gather_smem > 113 * 1024;
     const int gpc_slots = one_per_sm ? 17 : 35, held_each = one_per_sm ? 1 : cta_slots;
     int64_t fit = 0;                               // clusters of `best` CTAs
@@ -778,7 +778,9 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
       fit += std::max(0, gpc_slots - (predictor.clusters + gpc) / kGpcs * predictor.ctas * held_each) / best;
     const int64_t ctas = problems * best * (one_per_sm ? 2 : 1);
     if (best <= kMaxClusterCtas && ((problems <= fit && ctas <= 200) || (best == 2 && ctas <= 264))) {
-      w->merge_in_cluster = true;                  // (pairs find room anywhere)
+      // (256 CTAs in clusters of 8 at B = 4, N = 4096 did not all find room: 15.3 us a layer, 192 in clusters of 6 11.8;
+      // pairs find room anywhere)
+      w->merge_in_cluster = true;
     } else {
       // Fewer splits, in the slots that the predictor leaves, where that costs a call at most 5 %: 12.3 against 15.7 us
       // per layer at B = 2, N = 18546, 4 KV heads, 4608 tokens attended; with twice the chunks per CTA (B = 8,

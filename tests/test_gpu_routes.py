@@ -97,6 +97,7 @@ def test_step_with_the_softmax_scorer(meta_heads, scope, kw):
     ("joint", dict(batch=1, n_ctx=16384, top_k=256), CLUSTERS),                # 16
     ("joint", dict(batch=1, n_ctx=4096, top_k=256, kv_dtype=W.F32, head_dim=64), CLUSTERS),
     ("joint", dict(batch=1, n_ctx=4096, top_k=256, kv_dtype=W.F32), BESIDE),   # 16, but one CTA per SM
+    ("joint", dict(batch=1, n_ctx=4096, top_k=256, kv_dtype=W.F32, n_q_heads=16, n_kv_heads=4), CLUSTERS),     # 16 SMs per list
     ("joint", dict(batch=1, n_ctx=4096, top_k=80, kv_dtype=W.F32), CLUSTERS),
     ("joint", dict(batch=1, n_ctx=16384, top_k=290), BESIDE),                  # 18
     ("joint", dict(batch=4, n_ctx=8003, top_k=400), BESIDE),
