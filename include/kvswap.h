@@ -272,7 +272,8 @@ int kvswap_sparse_decode_static(const kvswap_shape* shape, const void* q, const 
  * proj[l] is [H_kv, d, r] fp32.  max_lookahead bounds how many layers the predictor may run ahead of the
  * attention: 1 = layer l is predicted while layer l-1 is attended (what a model allows, whose layer-l
  * prediction needs the input of layer l-1); 0 = no limit.  Both steps predict exactly one layer ahead,
- * which satisfies every bound.
+ * which satisfies every bound.  (Layer l is scored once the K/V of layer l-2 have been attended; where gathers are
+ * long, the split partials of that attention are merged while layer l is scored.)
  * Negative values are KVSWAP_ERR_SHAPE.
  */
 typedef struct {

@@ -5,6 +5,7 @@
 
 #include "api_internal.cuh"
 #include "async_copy.cuh"
+#include "combine.cuh"
 #include "common.cuh"
 #include "topk_keys.cuh"
 
@@ -137,7 +138,7 @@ int check_score_select(const kvswap_shape* shape, const void* q, const float* pr
 // group scores (and, where that path exists, the leading-digit histograms) in the workspace or the
 // caller's buffer, and the TopK over them.  A step may put other work between the two.
 cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q, const float* proj, const void* meta,
-                         float* group_scores_opt, void* ws, cudaStream_t stream, int uq_ahead) {
+                         float* group_scores_opt, void* ws, cudaStream_t stream, int uq_ahead, bool beside) {
   char* base = static_cast<char*>(ws);
   float* uq = reinterpret_cast<float*>(base + w.off_uq + (uq_ahead > 0 ? w.uq_bytes : 0));
   float* scores = group_scores_opt ? group_scores_opt : reinterpret_cast<float*>(base + w.off_scores);
@@ -145,7 +146,7 @@ cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q,
   p.score_pitch = group_scores_opt ? p.NG : workspace_score_pitch(p);     // a caller's buffer is dense [B, S, NG]
   if (p.flags & KVSWAP_SCORE_SOFTMAX) {
     float* u_heads = reinterpret_cast<float*>(base + w.off_softmax);
-    uint32_t* top_hist = counts_top_digit(p) ? reinterpret_cast<uint32_t*>(base + w.off_hist) : nullptr;
+    uint32_t* top_hist = counts_top_digit(p) && !beside ? reinterpret_cast<uint32_t*>(base + w.off_hist) : nullptr;
     return launch_score_softmax(p, q, proj, meta, u_heads, u_heads + size_t(p.B) * p.Hq * p.r, scores, top_hist,
                                 static_cast<uint32_t*>(ws), stream);
   }
@@ -153,7 +154,7 @@ cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q,
   if (score_stream_supported(p)) {
     // dense metadata rows of common ranks: the tensor-core scorer, which builds the low-rank queries itself
     // where it can and counts the leading digits of its scores for the TopK that follows
-    uint32_t* top_hist = counts_top_digit(p) ? reinterpret_cast<uint32_t*>(base + w.off_hist) : nullptr;
+    uint32_t* top_hist = counts_top_digit(p) && !beside ? reinterpret_cast<uint32_t*>(base + w.off_hist) : nullptr;
     const bool fused = score_stream_fuses_query(p);
     if (uq_ahead >= 0) {                                                  // the queries are in the workspace already
       if (!fused) return cudaErrorInvalidValue;
@@ -167,6 +168,16 @@ cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q,
   cudaError_t e = launch_lowrank_query(p, q, proj, uq, stream);
   if (e != cudaSuccess) return e;
   return launch_score_pool(p, uq, meta, scores, stream);
+}
+
+cudaError_t select_beside_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected, void* ws,
+                                 const CombineJob& job, cudaStream_t stream, const void* q_ahead, const float* proj_ahead,
+                                 int uq_ahead) {
+  Problem p = p_in;
+  p.score_pitch = workspace_score_pitch(p);
+  char* base = static_cast<char*>(ws);
+  return launch_select_beside(p, reinterpret_cast<float*>(base + w.off_scores), group_idx, n_selected, job, q_ahead, proj_ahead,
+                              reinterpret_cast<float*>(base + w.off_uq + (uq_ahead > 0 ? w.uq_bytes : 0)), stream);
 }
 
 cudaError_t select_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected,
@@ -184,8 +195,7 @@ cudaError_t select_launch(const Problem& p_in, const Workspace& w, int32_t* grou
 // (launch_sparse_decode with combine = false, any shape) has been enqueued before: one launch.  False
 // when the select of this shape has no such kernel (the caller then launches the two separately).
 bool select_with_combine_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected,
-                                void* ws, const float* partial, float* out, float* lse, int splits, int n_rows, int d,
-                                cudaStream_t stream, cudaError_t* result, const void* q_ahead,
+                                void* ws, const CombineJob& job, int d, cudaStream_t stream, cudaError_t* result, const void* q_ahead,
                                 const float* proj_ahead, int uq_ahead) {
   Problem p = p_in;
   p.score_pitch = workspace_score_pitch(p);
@@ -194,8 +204,7 @@ bool select_with_combine_launch(const Problem& p_in, const Workspace& w, int32_t
   float* uq = reinterpret_cast<float*>(base + w.off_uq + (uq_ahead > 0 ? w.uq_bytes : 0));
   const bool ahead = q_ahead != nullptr && uq_ahead >= 0 && score_stream_fuses_query(p);
   *result = launch_combine_select(p, reinterpret_cast<float*>(base + w.off_scores),
-                                  reinterpret_cast<uint32_t*>(base + w.off_hist), group_idx, n_selected, partial, out, lse,
-                                  splits, n_rows, d, ahead ? q_ahead : nullptr, proj_ahead, uq, stream);
+                                  reinterpret_cast<uint32_t*>(base + w.off_hist), group_idx, n_selected, job, d, ahead ? q_ahead : nullptr, proj_ahead, uq, stream);
   return true;
 }
 

@@ -19,7 +19,11 @@ int check_score_select(const kvswap_shape* shape, const void* q, const float* pr
 // uq_ahead = 0 or 1: the summed low-rank queries are already in that one of the workspace's two query
 // buffers (select_with_combine_launch put them there), and q is not read; -1: the scorer forms them.
 cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q, const float* proj, const void* meta,
-                         float* group_scores_opt, void* ws, cudaStream_t stream, int uq_ahead = -1);
+                         float* group_scores_opt, void* ws, cudaStream_t stream, int uq_ahead = -1, bool beside = false);
+// The TopK for a scorer launched with beside = true (it does not count leading digits): launch_select_beside.
+cudaError_t select_beside_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected, void* ws,
+                                 const CombineJob& job, cudaStream_t stream, const void* q_ahead, const float* proj_ahead,
+                                 int uq_ahead);
 cudaError_t select_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected,
                           float* group_scores_opt, void* ws, cudaStream_t stream);
 // select_launch merged with the combine pass of a split-K gather enqueued before it (one launch);
@@ -27,8 +31,7 @@ cudaError_t select_launch(const Problem& p_in, const Workspace& w, int32_t* grou
 // low-rank queries of the layer with that q and proj_ahead into query buffer uq_ahead (0 or 1) of the
 // workspace, where this shape's scorer can take them from (query_ahead_supported).
 bool select_with_combine_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected,
-                                void* ws, const float* partial, float* out, float* lse, int splits, int n_rows, int d,
-                                cudaStream_t stream, cudaError_t* result, const void* q_ahead = nullptr,
+                                void* ws, const CombineJob& job, int d, cudaStream_t stream, cudaError_t* result, const void* q_ahead = nullptr,
                                 const float* proj_ahead = nullptr, int uq_ahead = -1);
 bool query_ahead_supported(const Problem& p);
 // True when select_with_combine_launch has a kernel for this shape's select.

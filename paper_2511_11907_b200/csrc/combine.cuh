@@ -5,37 +5,52 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "common.cuh"
+
 namespace kvswap {
 
 constexpr int kMaxSplits = 256;
 
-// D threads (c = 0..D-1) merge row `row` of partial [rows, splits, D + 2] = (m, l, acc[D]) into
-// out[row, :] and lse[row].  Every load of the row is issued before anything is computed (one
+// Partials [rows, slots, D + 2] = (m, l, acc[D]) of a gather whose lists (heads_per_list rows each) were dealt to
+// warps_per_list consecutive warps, 8 to a CTA: of a row's slots as many are filled as CTAs took part in its list.
+struct CombineJob {
+  const float* partial;
+  float* out;              // [rows, D]
+  float* lse;              // NULL or [rows]
+  int rows, slots, heads_per_list, warps_per_list;
+};
+
+inline CombineJob combine_job(const Problem& p, const Workspace& w, const float* partial, float* out, float* lse) {
+  return CombineJob{partial, out, lse, p.B * p.Hq, w.splits, w.heads_per_cta, w.warps_per_list};
+}
+
+// D threads (c = 0..D-1) merge row `row` of `job`.  Every load of the row is issued before anything is computed (one
 // memory round trip); the split weights are formed once by the first warp of the D threads and
 // shared through w_s [kMaxSplits] and norm_s [2].  The D threads meet at named barrier `barrier`
-// (0 = the CTA-wide one: then the CTA has exactly D threads).  `live` false: the threads only keep
+// (0 = the CTA-wide one: then the CTA has exactly D threads).  Without a row (row >= job.rows) the threads only keep
 // the barrier company.
 template <int D>
-__device__ __forceinline__ void combine_row(const float* __restrict__ partial, float* __restrict__ out,
-                                            float* __restrict__ lse, int splits, int64_t row, bool live, int c,
-                                            float* w_s, float* norm_s, int barrier) {
+__device__ __forceinline__ void combine_row(const CombineJob& job, int row, int c, float* w_s, float* norm_s, int barrier) {
   constexpr float kLn2 = 0.6931471805599453f;
   constexpr int kUnroll = 16;
-  const float* src = partial + row * splits * (D + 2);
+  const bool live = row < job.rows;
+  const int list = row / job.heads_per_list;
+  const int splits = ((list + 1) * job.warps_per_list - 1) / 8 - list * job.warps_per_list / 8 + 1;
+  const float* src = job.partial + int64_t(row) * job.slots * (D + 2);
   float a_first[kUnroll];
 #pragma unroll
-  for (int s = 0; s < kUnroll; ++s) a_first[s] = (live && s < splits) ? src[s * (D + 2) + 2 + c] : 0.f;
+  for (int s = 0; s < kUnroll; ++s) a_first[s] = (live && s < splits) ? __ldcg(src + s * (D + 2) + 2 + c) : 0.f;
   if (live && c < 32) {
     // weights: lane s handles splits s, s + 32, ...
     float mx = -INFINITY;
-    for (int s = c; s < splits; s += 32) mx = fmaxf(mx, src[s * (D + 2)]);
+    for (int s = c; s < splits; s += 32) mx = fmaxf(mx, __ldcg(src + s * (D + 2)));
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     float lsum = 0.f;
     for (int s = c; s < splits; s += 32) {
-      const float w = (mx > -INFINITY) ? exp2f(src[s * (D + 2)] - mx) : 0.f;
+      const float w = (mx > -INFINITY) ? exp2f(__ldcg(src + s * (D + 2)) - mx) : 0.f;
       w_s[s] = w;
-      lsum = fmaf(src[s * (D + 2) + 1], w, lsum);
+      lsum = fmaf(__ldcg(src + s * (D + 2) + 1), w, lsum);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
@@ -50,9 +65,9 @@ __device__ __forceinline__ void combine_row(const float* __restrict__ partial, f
   float a = 0.f;
 #pragma unroll
   for (int s = 0; s < kUnroll; ++s) if (s < splits) a = fmaf(a_first[s], w_s[s], a);
-  for (int s = kUnroll; s < splits; ++s) a = fmaf(src[s * (D + 2) + 2 + c], w_s[s], a);
-  out[row * D + c] = a * norm_s[0];
-  if (lse != nullptr && c == 0) lse[row] = norm_s[1];
+  for (int s = kUnroll; s < splits; ++s) a = fmaf(__ldcg(src + s * (D + 2) + 2 + c), w_s[s], a);
+  job.out[int64_t(row) * D + c] = a * norm_s[0];
+  if (job.lse != nullptr && c == 0) job.lse[row] = norm_s[1];
 }
 
 }  // namespace kvswap

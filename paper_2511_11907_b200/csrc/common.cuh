@@ -15,6 +15,7 @@ namespace kvswap {
 constexpr int kNumSMs = 148;  // B200: 2 dies x 74 SMs; grids are sized in multiples of this.
 
 // Shape with every "0 = dense" stride resolved and the derived sizes filled in.
+struct CombineJob;   // combine.cuh
 struct Problem {
   int B, N, Hq, Hkv, d, r, Hm, G, M;
   int kv_dtype, meta_dtype, q_dtype, scope;
@@ -52,10 +53,13 @@ struct Workspace {
   size_t off_softmax;  // float [B, Hq, r] per-head low-rank queries + [B, Hq, chunks, 2] softmax statistics (scorer variant)
   size_t off_adapter;  // bf16 or fp16 [H_kv, 3 r, d]  adapter split into three pieces of K's type (project_keys on tcgen05), then float [H_kv, r]: fp16, its scales
   size_t total;
-  int splits;          // split-K factor of sparse_decode for this shape
+  int splits;          // split-K partials of a row of sparse_decode for this shape, at most
+  int splits_static;   // ... of a plan in whole CTAs, two per SM: what the static scratch is checked with (no fewer than `splits`)
+  int warps_per_list;  // warps of the gather that share a list
   int splits_room;     // splits the partials are planned for: no fewer than `splits` of any context length and flags
   int heads_per_cta;   // query heads sharing one K/V pass in sparse_decode
   int depth;           // shared-memory stages per compute warp in sparse_decode
+  bool long_gather;    // the gather takes one CTA per SM and half of its registers: a decode step runs the next layer's select beside it
   bool beside;         // a decode step runs the gather beside the next layer's one-launch predictor (splits planned for what that leaves)
   bool merge_in_cluster;   // the splits of a list form a cluster that merges them (no combine pass; the same bits)
   bool merge_alone;    // ... also when sparse_decode is called on its own
@@ -64,6 +68,10 @@ struct Workspace {
 int resolve(const kvswap_shape* s, Problem* p);            // validation; returns kvswap_status
 void plan_workspace(const Problem& p, Workspace* w);
 void plan_sparse_decode(const Problem& p, Workspace* w);   // fills splits, heads_per_cta, depth
+// sparse_decode_long.cu: takes over the plan (and the launch) of a long gather.
+void plan_long_gather(const Problem& p, Workspace* w);
+cudaError_t launch_long_gather(const Problem& p, const Workspace& w, const void* q, const void* K, const void* V,
+                               const int32_t* group_idx, const int32_t* n_selected, float* partial, uint32_t* err, cudaStream_t st);
 
 // Kernel launchers (each returns a cudaError_t from the launch).
 // `scratch` is the workspace region at off_adapter (project_keys_umma_scratch_bytes, may be NULL).
@@ -136,16 +144,21 @@ cudaError_t launch_sparse_decode(const Problem& p, const Workspace& w, const voi
                                  const void* V, const int32_t* group_idx, const int32_t* n_selected,
                                  float* partial, float* out, float* lse, uint32_t* err, cudaStream_t st,
                                  bool combine = true);
-cudaError_t launch_combine_only(const Problem& p, const Workspace& w, const float* partial, float* out, float* lse,
-                                cudaStream_t st);
-// launch_topk_parts for problem `p` and, in the same launch, the merge of `n_rows` rows of split-K
-// partials [n_rows, splits, d + 2] (of whatever attention produced them) into out / lse.  With
+cudaError_t launch_combine(const Problem& p, const CombineJob& job, const CombineJob& job2, cudaStream_t st);
+// The TopK of one layer beside the gather of the layer before (topk_beside.cuh), with the merge of an earlier gather's
+// partials (job.rows = 0: none) and the queries of a later layer as in launch_combine_select.  Merge and queries do not wait:
+// partials, q_ahead and proj_ahead must have been complete before the kernel enqueued ahead of this one let it start.
+bool select_beside_supported(const Problem& p);
+cudaError_t launch_select_beside(const Problem& p, const float* scores, int32_t* group_idx, int32_t* n_selected,
+                                 const CombineJob& job, const void* q_ahead, const float* proj_ahead, float* uq_ahead,
+                                 cudaStream_t st);
+// launch_topk_parts for problem `p` and, in the same launch, the merge of the split-K partials of `job` (of whatever
+// attention produced them).  With
 // q_ahead != NULL the launch also builds the summed low-rank queries of another layer of the same shape
 // (its q and proj) into uq_ahead [B, Su, r], for a streaming scorer that is enqueued next: the bits are
 // those the scorer would build itself.  Only where score_stream_fuses_query(p).
 cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_t* top_hist, int32_t* group_idx,
-                                  int32_t* n_selected, const float* partial, float* out, float* lse, int splits,
-                                  int n_rows, int d, const void* q_ahead, const float* proj_ahead, float* uq_ahead,
+                                  int32_t* n_selected, const CombineJob& job, int d, const void* q_ahead, const float* proj_ahead, float* uq_ahead,
                                   cudaStream_t st);
 // Row sets of the streaming scorer for `p` (0 when it does not take the shape) and scope blocks per
 // (sequence, metadata head): the arguments of row_set() in lowrank_query.cuh.

@@ -82,10 +82,11 @@ __device__ __forceinline__ float query_entry(const float* upart, int row, int j,
 // 128-byte reads of A_g; at R = 16 a read covers two channels); it requests the adapter rows of its
 // items first, then the CTA sums the query heads into shared memory, so that both loads share one
 // round trip.  The partial products are added in a fixed order, whatever the number of warps.  Threads 0 ..
-// 32 NW - 1 of the CTA call (NW = 16: at most two items per warp, or 32: one, in half the registers), and
+// 32 NW - 1 of the CTA call (NW = 16: at most two items per warp, LEAN: one after the other, or NW = 32: one; both take half
+// the registers), and
 // meet at barrier BAR (0: the CTA has exactly that many threads).  qsum [kQuerySumFloats] and upart
 // [kQueryPartFloats] are shared-memory scratch, urow [8 * R] receives the result.
-template <int BAR, int R, int NW = kQueryWarps>
+template <int BAR, int R, int NW = kQueryWarps, bool LEAN = false>
 __device__ void build_queries(const Problem& p, const void* q, const float* __restrict__ proj, RowSet rs,
                               float* qsum, float* upart, float* urow) {
   auto sync = [] {
@@ -108,19 +109,16 @@ __device__ void build_queries(const Problem& p, const void* q, const float* __re
     const int it0 = warp, it1 = warp + NW;
 #pragma unroll 1
     for (int pass = 0; pass < kPasses; ++pass) {
-      float a0[kLoads], a1[NW == 16 ? kLoads : 1];
-      {
-        const int64_t at0 = int64_t(head0 + t0 + (it0 >> ch_shift)) * p.d + (it0 & (chunks - 1)) * 32 + ch0;
-        const int64_t at1 = int64_t(head0 + t0 + (it1 >> ch_shift)) * p.d + (it1 & (chunks - 1)) * 32 + ch0;
-        const float* P0 = proj + at0 * R + pass * 32 + col;
-        const float* P1 = proj + at1 * R + pass * 32 + col;
+      constexpr bool kSecond = NW == 16 && !LEAN;
+      float a0[kLoads], a1[kSecond ? kLoads : 1];
+      auto request = [&](int it, float* a) {
+        const int64_t at = int64_t(head0 + t0 + (it >> ch_shift)) * p.d + (it & (chunks - 1)) * 32 + ch0;
+        const float* P = proj + at * R + pass * 32 + col;
 #pragma unroll
-        for (int cc = 0; cc < kLoads; ++cc) a0[cc] = (it0 < n_items) ? P0[cc * step * R] : 0.f;
-        if constexpr (NW == 16) {
-#pragma unroll
-          for (int cc = 0; cc < kLoads; ++cc) a1[cc] = (it1 < n_items) ? P1[cc * step * R] : 0.f;
-        }
-      }
+        for (int cc = 0; cc < kLoads; ++cc) a[cc] = (it < n_items) ? P[cc * step * R] : 0.f;
+      };
+      request(it0, a0);
+      if constexpr (kSecond) request(it1, a1);
       if (pass == 0) {
         for (int i = tid; i < (nt << d_shift); i += 32 * NW) {
           const int tt = i >> d_shift, c = i & (p.d - 1);
@@ -138,7 +136,12 @@ __device__ void build_queries(const Problem& p, const void* q, const float* __re
         upart[it * 32 + lane] = acc;
       };
       multiply(it0, a0);
-      if constexpr (NW == 16) multiply(it1, a1);
+      if constexpr (kSecond) {
+        multiply(it1, a1);
+      } else if constexpr (NW == 16) {
+        request(it1, a0);
+        multiply(it1, a0);
+      }
       sync();
       if (tid < kQueryCols * 32) {
         const int row = tid >> 5, j = tid & 31, at = row * R + pass * 32 + j;

@@ -48,13 +48,20 @@ constexpr int kHistWords = kScoreCols * kKeyTopBins / 2;  // two 16-bit counters
 constexpr int kMaxSets = 4;                               // row sets one CTA may touch when it builds the queries itself
 constexpr int kMultiTiles = 8;                            // tiles whose scores a warp sums over the heads together
 
-template <int META, int R, int GS>
+// How a CTA works: kForms builds the low-rank queries and counts leading digits, kCounts finds the queries in memory, kDeep
+// finds them too, does not count and has a third stage in the counters' place (a decode step whose select does without:
+// topk_beside.cuh).  The flush of the counters alone took 3 us of a layer there, and with three stages a warp has nearly all
+// of its 3.5 tiles in flight before its dependency wait: 11.3 -> 6.5 us from the wait to the end at B = 4, N = 131072.
+enum ScoreMode { kForms, kCounts, kDeep };
+
+template <int META, int R, int GS, ScoreMode MODE>
 struct ScoreSmem {
-  unsigned char tiles[kScoreWarps * kScoreDepth * ScoreStage<META, R, GS>::kBytes];      // 128 KB of stages, or 96
-  uint32_t hist[kHistWords];                              // 64 KB
-  unsigned long long full[kScoreWarps * kScoreDepth];
-  float urow[kMaxSets][kScoreCols * R];                   // summed low-rank queries per row set of the CTA
-  static constexpr int kScratch = kQuerySumFloats + kQueryPartFloats;
+  static constexpr int kDepth = MODE == kDeep ? kScoreDepth + 1 : kScoreDepth;
+  unsigned char tiles[kScoreWarps * kDepth * ScoreStage<META, R, GS>::kBytes];           // 128 KB of stages, or 96; kDeep: 192 or 144
+  uint32_t hist[MODE == kDeep ? 4 : kHistWords];          // 64 KB
+  unsigned long long full[kScoreWarps * kDepth];
+  float urow[MODE == kForms ? kMaxSets : 1][MODE == kForms ? kScoreCols * R : 4];   // summed low-rank queries per row set of the CTA
+  static constexpr int kScratch = MODE == kForms ? kQuerySumFloats + kQueryPartFloats : 4;
   // scratch of build_queries (qsum, then upart), afterwards the warps' score buffers
   static constexpr int kBuffers = GS >= 0 ? 0 : kScoreWarps * kScoreCols * generic_pitch(ScoreStage<META, R, GS>::kRows);
   float sc[kBuffers > kScratch ? kBuffers : kScratch];
@@ -75,15 +82,18 @@ struct StreamArgs {
   uint32_t* err;
 };
 
-template <int META, int R, int GS, bool FUSED>       // GS = log2(G), 0..5, or -1
+template <int META, int R, int GS, ScoreMode MODE>   // GS = log2(G), 0..5, or -1
 __global__ void __launch_bounds__(kScoreThreads, 1)
 score_stream_kernel(Problem p, StreamArgs a) {
   constexpr uint32_t kFull = 0xffffffffu;
+  constexpr bool FUSED = MODE == kForms;
+  using Smem = ScoreSmem<META, R, GS, MODE>;
   constexpr int kRowBytes = MetaRows<META, R>::kRowBytes, kElem = MetaRows<META, R>::kElem;
   constexpr int kStageBytes = ScoreStage<META, R, GS>::kBytes, kStageRows = ScoreStage<META, R, GS>::kRows;
-  constexpr int kDepth = kScoreDepth, kWarps = kScoreWarps, kThreads = kScoreThreads, kCols = kScoreCols;
+  constexpr int kDepth = Smem::kDepth, kWarps = kScoreWarps, kThreads = kScoreThreads, kCols = kScoreCols;
   extern __shared__ __align__(128) unsigned char dyn[];
-  auto* sm = reinterpret_cast<ScoreSmem<META, R, GS>*>(dyn);
+  auto* sm = reinterpret_cast<Smem*>(dyn);
+  const bool counts = MODE != kDeep && a.top_hist != nullptr;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rq = lane >> 2, qt = lane & 3;
@@ -91,7 +101,7 @@ score_stream_kernel(Problem p, StreamArgs a) {
     for (int s = 0; s < kDepth; ++s) mbar_init(smem_addr(&sm->full[warp * kDepth + s]), 1);
     mbar_init_fence();
   }
-  if (a.top_hist != nullptr) {
+  if (counts) {
     uint4* H = reinterpret_cast<uint4*>(sm->hist);
     for (int i = threadIdx.x; i < kHistWords / 4; i += kThreads) H[i] = make_uint4(0u, 0u, 0u, 0u);
   }
@@ -191,7 +201,7 @@ score_stream_kernel(Problem p, StreamArgs a) {
   auto publish = [&](float* dst, float x) {
     x += 0.f;                                       // -0 becomes +0: the TopK that follows relies on it
     *dst = x;
-    if (a.top_hist != nullptr) {
+    if (counts) {
       const uint32_t bin = score_key_top(x);
       if (my_col >= 0) {
         atomicAdd(&sm->hist[(my_col * kKeyTopBins + int(bin)) >> 1], 1u << ((bin & 1u) << 4));
@@ -235,7 +245,7 @@ score_stream_kernel(Problem p, StreamArgs a) {
         scope_ok = rq < ns_cur;
         const int64_t prob = int64_t(rs.b) * p.S + s0 + (scope_ok ? rq : 0);
         my_row = a.scores + prob * p.score_pitch;
-        if (a.top_hist != nullptr) {
+        if (counts) {
           my_hist = a.top_hist + prob * (kKeyTopBins / 2);
           const int col = (c.rest - rest0) * ns_cols + (multi ? 0 : rq);
           my_col = ((scope_ok || multi) && col < kCols) ? col : -1;
@@ -285,7 +295,7 @@ score_stream_kernel(Problem p, StreamArgs a) {
   }
 
   // ---- the CTA's counts join the global histograms --------------------------------------------------------
-  if (a.top_hist != nullptr) {
+  if (counts) {
     __syncthreads();
     for (int i = threadIdx.x; i < kHistWords / 4; i += kThreads) {
       const uint4 v = reinterpret_cast<const uint4*>(sm->hist)[i];
@@ -321,14 +331,17 @@ template <> cudaError_t launch_score_stream_rows<KVSWAP_F32, 64>(const Problem&,
 
 template <int META, int R, int GS>
 cudaError_t launch_score_stream_gs(const Problem& p, const StreamArgs& a, bool fused, int ctas, cudaStream_t st) {
-  const size_t smem = sizeof(ScoreSmem<META, R, GS>) + 128;
-  static_assert(sizeof(ScoreSmem<META, R, GS>) + 128 <= 227 * 1024, "shared memory of one CTA");
-  auto go = [&](auto kern) -> cudaError_t {
+  auto go = [&](auto kern, auto mode) -> cudaError_t {
+    using Smem = ScoreSmem<META, R, GS, decltype(mode)::value>;
+    static_assert(sizeof(Smem) + 128 <= 227 * 1024, "shared memory of one CTA");
+    const size_t smem = sizeof(Smem) + 128;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     return launch_pdl(kern, dim3(ctas), dim3(kScoreThreads), smem, st, p, a);
   };
-  return fused ? go(score_stream_kernel<META, R, GS, true>) : go(score_stream_kernel<META, R, GS, false>);
+  return fused                   ? go(score_stream_kernel<META, R, GS, kForms>, std::integral_constant<ScoreMode, kForms>())
+         : a.top_hist != nullptr ? go(score_stream_kernel<META, R, GS, kCounts>, std::integral_constant<ScoreMode, kCounts>())
+                                 : go(score_stream_kernel<META, R, GS, kDeep>, std::integral_constant<ScoreMode, kDeep>());
 }
 
 #define KVSWAP_SCORE_STREAM_ROWS(META, R)                                                                            \

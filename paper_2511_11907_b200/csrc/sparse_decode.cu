@@ -29,6 +29,7 @@
 #include "cluster.cuh"
 #include "combine.cuh"
 #include "common.cuh"
+#include "gather.cuh"
 
 namespace kvswap {
 namespace {
@@ -38,7 +39,6 @@ constexpr int kWarps = 8;                       // warps per CTA
 constexpr int kThreads = kWarps * 32;
 constexpr int kMaxDepth = 4;                    // stages per warp, at most
 constexpr int kMaxStages = kWarps * kMaxDepth;
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
 // Control block at the start of dynamic shared memory.
@@ -49,28 +49,8 @@ struct Control {
 };
 constexpr int kControlBytes = (sizeof(Control) + 255) & ~255;
 
-// Byte offset inside a stage half of byte `col` of row `r` (rows of ROWB bytes, pieces of 16).
-template <uint32_t ROWB>
-__device__ __forceinline__ uint32_t swz(uint32_t r, uint32_t col) {
-  return r * ROWB + ((((col >> 4) ^ (r & 7u)) << 4) | (col & 15u));
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
-  // src_bytes = 16 copies, 0 writes zeros without touching global memory
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 template <typename Q_T>
 __device__ __forceinline__ float q_to_float(Q_T v) { return float(v); }
-
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // DPL consecutive channels of one staged row, widened to fp32.
 template <typename KV_T, int DPL>
@@ -264,51 +244,6 @@ struct AluEngine {
 // Q, K and V enter unrounded (they are stored in the operand type); the scale 1/sqrt(d) is
 // applied to the fp32 logits.
 // ------------------------------------------------------------------------------------------
-template <typename KV_T>
-__device__ __forceinline__ void mma_k16(float (&d)[4], uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
-  // rows 8..15 of A (a1, a3) are zero
-  if constexpr (std::is_same<KV_T, __nv_bfloat16>::value) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
-  } else {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1));
-  }
-}
-template <typename KV_T>
-__device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
-  if constexpr (std::is_same<KV_T, __nv_bfloat16>::value) {
-    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
-  } else {
-    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(b0));
-  }
-}
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-// Two fp32 values -> packed 16-bit pair (x in the low half) and the packed remainders.
-template <typename KV_T>
-__device__ __forceinline__ void split_pair(float x, float y, uint32_t& hi, uint32_t& lo) {
-  if constexpr (std::is_same<KV_T, __nv_bfloat16>::value) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-    const float2 hf = __bfloat1622float2(h);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(x - hf.x, y - hf.y);
-    hi = *reinterpret_cast<const uint32_t*>(&h); lo = *reinterpret_cast<const uint32_t*>(&l);
-  } else {
-    const __half2 h = __floats2half2_rn(x, y);
-    const float2 hf = __half22float2(h);
-    const __half2 l = __floats2half2_rn(x - hf.x, y - hf.y);
-    hi = *reinterpret_cast<const uint32_t*>(&h); lo = *reinterpret_cast<const uint32_t*>(&l);
-  }
-}
-
 template <typename KV_T, typename Q_T, int D, int RH>
 struct MmaEngine {
   static_assert(sizeof(KV_T) == 2 && std::is_same<KV_T, Q_T>::value, "16-bit K/V and q of one type");
@@ -633,17 +568,18 @@ sparse_decode_splitk_kernel(Problem p, const Q_T* __restrict__ q, const KV_T* __
   if (wait_late) pdl_wait();
 }
 
-// K5: merge the split partials of one (sequence, head): one CTA of D threads per row (combine.cuh).
+// K5: merge the split partials of one attention, or of two, a CTA of D threads per (sequence, head) (combine.cuh).
 template <int D>
 __global__ void __launch_bounds__(D)
-combine_kernel(const float* __restrict__ partial, float* __restrict__ out, float* __restrict__ lse, int splits) {
+combine_kernel(CombineJob job, CombineJob job2) {
   __shared__ float w_s[kMaxSplits];
   __shared__ float norm_s[2];                  // 1 / sum of weights (or 0), lse
   // The next kernel of the stream may start its own prologue at once; this one needs the
   // partials of the gather kernel before it.
   pdl_trigger();
   pdl_wait();
-  combine_row<D>(partial, out, lse, splits, blockIdx.x, true, threadIdx.x, w_s, norm_s, 0);
+  const bool second = int(blockIdx.x) >= job.rows;
+  combine_row<D>(second ? job2 : job, int(blockIdx.x) - (second ? job.rows : 0), threadIdx.x, w_s, norm_s, 0);
 }
 
 template <typename KV_T, int D>
@@ -683,8 +619,7 @@ cudaError_t launch_one(const Problem& p, const Workspace& w, const void* q, cons
   e = launch_pdl(kern, grid, dim3(kThreads), smem, st, p, qt, Kt, Vt, group_idx, n_selected, partial, out, lse, w.splits,
                  depth, g_shift, err);
   if (e != cudaSuccess || !combine) return e;
-  return launch_pdl(combine_kernel<D>, dim3(p.B * p.Hq), dim3(D), 0, st, static_cast<const float*>(partial), out,
-                    lse, w.splits);
+  return launch_combine(p, combine_job(p, w, partial, out, lse), CombineJob{}, st);
 }
 
 template <typename KV_T, typename Q_T, int D>
@@ -802,20 +737,26 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
   // fp32 layer 16.2 us against 18.6); clusters of more than 8 take longer than gather and combine even so
   // (B = 1, N = 16384, 8 heads, 2048 tokens attended: 8.3 us against 6.5).
   w->merge_alone = w->merge_in_cluster && best <= 8;
-  w->splits = int(best);
+  w->splits = w->splits_static = int(best);
+  w->warps_per_list = int(best) * kWarps;
+  w->long_gather = false;
+  if (!w->merge_in_cluster && !w->beside) plan_long_gather(p, w);
 }
 
-// The combine pass alone, for a gather that was enqueued with combine = false.
-cudaError_t launch_combine_only(const Problem& p, const Workspace& w, const float* partial, float* out, float* lse,
-                                cudaStream_t st) {
-  if (p.d == 128)
-    return launch_pdl(combine_kernel<128>, dim3(p.B * p.Hq), dim3(128), 0, st, partial, out, lse, w.splits);
-  return launch_pdl(combine_kernel<64>, dim3(p.B * p.Hq), dim3(64), 0, st, partial, out, lse, w.splits);
+// The combine pass alone, for gathers that were enqueued with combine = false.
+cudaError_t launch_combine(const Problem& p, const CombineJob& job, const CombineJob& job2, cudaStream_t st) {
+  const dim3 grid(job.rows + job2.rows), block(p.d);
+  return p.d == 128 ? launch_pdl(combine_kernel<128>, grid, block, 0, st, job, job2)
+                    : launch_pdl(combine_kernel<64>, grid, block, 0, st, job, job2);
 }
 
 cudaError_t launch_sparse_decode(const Problem& p, const Workspace& w, const void* q, const void* K, const void* V,
                                  const int32_t* group_idx, const int32_t* n_selected, float* partial, float* out,
                                  float* lse, uint32_t* err, cudaStream_t st, bool combine) {
+  if (w.long_gather) {
+    const cudaError_t e = launch_long_gather(p, w, q, K, V, group_idx, n_selected, partial, err, st);
+    return e != cudaSuccess || !combine ? e : launch_combine(p, combine_job(p, w, partial, out, lse), CombineJob{}, st);
+  }
   switch (p.kv_dtype) {
     case KVSWAP_F32: return launch_q<float>(p, w, q, K, V, group_idx, n_selected, partial, out, lse, err, combine, st);
     case KVSWAP_BF16: return launch_q<__nv_bfloat16>(p, w, q, K, V, group_idx, n_selected, partial, out, lse, err, combine, st);

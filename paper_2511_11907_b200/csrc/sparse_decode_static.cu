@@ -64,7 +64,7 @@ extern "C" int kvswap_sparse_decode_static(const kvswap_shape* shape, const void
   Workspace w;
   plan_workspace(p, &w);
   // The first 256 bytes hold the device status word, the partials follow.
-  const size_t need = 256 + sizeof(float) * size_t(p.B) * p.Hq * w.splits * (p.d + 2);
+  const size_t need = 256 + sizeof(float) * size_t(p.B) * p.Hq * w.splits_static * (p.d + 2);
   if (need > size_t(KVSWAP_STATIC_SCRATCH_BYTES)) return KVSWAP_ERR_STATIC_SCRATCH;
   if (q == nullptr || K == nullptr || V == nullptr || group_idx == nullptr || n_selected == nullptr ||
       out == nullptr)

@@ -241,12 +241,12 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
       p_two_back.flags |= kFlagInputsTwoBack;
       const bool merged = next && merges &&
                           select_with_combine_launch(p_two_back, w, group_idx + size_t(l + 1) * idx_elems,
-                                                     n_selected + size_t(l + 1) * nsel_elems, ws, partial, out_l, lse_l,
-                                                     w.splits, p.B * p.Hq, p.d, stream, &e, q_ahead,
+                                                     n_selected + size_t(l + 1) * nsel_elems, ws,
+                                                     combine_job(p, w, partial, out_l, lse_l), p.d, stream, &e, q_ahead,
                                                      form ? layers->proj[l + 2] : nullptr, (l + 2) & 1);
       if (merged && form && e == cudaSuccess) formed_for = l + 2;
       if (!merged) {
-        e = launch_combine_only(p, w, partial, out_l, lse_l, stream);
+        e = launch_combine(p, combine_job(p, w, partial, out_l, lse_l), CombineJob{}, stream);
       }
       if (probed(l)) ev(probe_opt->ev_end);
       if (e != cudaSuccess) return KVSWAP_ERR_CUDA;
@@ -288,6 +288,66 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
         if (e != cudaSuccess) status = KVSWAP_ERR_CUDA;
       }
       return status;
+    }
+    // Long gathers: the select of a layer runs beside the gather of the layer before, which takes one CTA per SM and half of its
+    // registers, instead of behind it:
+    //   score(0) select(0) | score(1) select(1) attention(0) | score(2) select(2) attention(1) | ...
+    // The launch of select(l + 1) also merges the partials of attention(l - 1) and forms the queries of layer l + 2, beside
+    // score(l + 1); the scorer does not count leading digits.
+    // What each kernel waits for: score(l + 1) for attention(l - 1) and all before it, and lets select(l + 1) start only then;
+    // select(l + 1) lets attention(l) start when its own CTAs have, so the selection of layer l is complete by then; it
+    // waits for score(l + 1); attention(l) waits for select(l + 1), with one buffer of partials before it writes them, as the
+    // merge may still read those of layer l - 1, with two (layers take turns) at its end.
+    // 12 layers of B = 4, N = 131072, M = 1024: 517 -> 458 us; eight tokens over 12 layers of B = 8, N = 32760: 3239 -> 2900.
+    if (w.long_gather) {
+      const bool two = 2 * w.splits <= w.splits_room;
+      auto partial_of = [&](int l) { return two && (l & 1) ? partial + size_t(p.B) * p.Hq * w.splits * (p.d + 2) : partial; };
+      Problem p_late = p_settled;
+      p_late.flags |= kFlagWaitLate;
+      CombineJob pending = {};                      // gathered, not merged
+      cudaError_t e = cudaSuccess;
+      auto predict = [&](int l) {
+        const void* ql = static_cast<const char*>(q) + size_t(l) * q_bytes;
+        if (probed(l)) ev(probe_opt->ev_begin);
+        e = score_launch(p_settled, w, ql, layers->proj[l], layers->meta[l], nullptr, ws, stream, formed_for == l ? (l & 1) : -1,
+                         /*beside=*/true);
+        const bool form = ahead && l + 1 < L;
+        if (e == cudaSuccess)
+          e = select_beside_launch(p_settled, w, group_idx + size_t(l) * idx_elems, n_selected + size_t(l) * nsel_elems, ws, pending,
+                                   stream, form ? static_cast<const char*>(ql) + q_bytes : nullptr,
+                                   form ? layers->proj[l + 1] : nullptr, (l + 1) & 1);
+        if (form) formed_for = l + 1;
+        pending = CombineJob{};
+        if (probed(l)) ev(probe_opt->ev_mid);
+      };
+      int status = score(0);
+      if (status == KVSWAP_OK) status = select(0);
+      if (status != KVSWAP_OK) return status;
+      for (int l = 0; l < L && e == cudaSuccess; ++l) {
+        const bool last = l + 1 == L;
+        if (!last) predict(l + 1);
+        if (last && pending.rows > 0 && !two && e == cudaSuccess) {
+          e = launch_combine(p, pending, CombineJob{}, stream);
+          pending = CombineJob{};
+        }
+        // (the last layer's attention follows an attention, or its own selection)
+        float* out_l = out + size_t(l) * out_elems;
+        float* lse_l = lse_opt ? lse_opt + size_t(l) * p.B * p.Hq : nullptr;
+        if (e == cudaSuccess)
+          e = launch_sparse_decode(last ? p_wait : two ? p_late : p_settled, w, static_cast<const char*>(q) + size_t(l) * q_bytes,
+                                   layers->K[l], layers->V[l], group_idx + size_t(l) * idx_elems,
+                                   n_selected + size_t(l) * nsel_elems, partial_of(l), out_l, lse_l, static_cast<uint32_t*>(ws), stream,
+                                   /*combine=*/false);
+        const CombineJob job = combine_job(p, w, partial_of(l), out_l, lse_l);
+        if (last || probed(l)) {
+          if (e == cudaSuccess) e = launch_combine(p, pending, job, stream);
+          pending = CombineJob{};
+          if (probed(l)) ev(probe_opt->ev_end);
+        } else {
+          pending = job;
+        }
+      }
+      return e == cudaSuccess ? KVSWAP_OK : KVSWAP_ERR_CUDA;
     }
     int status = score(0);
     if (status == KVSWAP_OK) status = select(0);

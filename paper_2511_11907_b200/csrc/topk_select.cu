@@ -306,8 +306,7 @@ template <int P, int D>
 __global__ void __launch_bounds__(kPartThreads)
 combine_select_kernel(Problem p, const float* __restrict__ scores, uint32_t* __restrict__ top_hist,
                       int32_t* __restrict__ group_idx, int32_t* __restrict__ n_selected, int n_probs,
-                      const float* __restrict__ partial, float* __restrict__ out, float* __restrict__ lse, int splits,
-                      int n_rows, int n_comb, const void* __restrict__ q_ahead, const float* __restrict__ proj_ahead,
+                      CombineJob job, int n_comb, const void* __restrict__ q_ahead, const float* __restrict__ proj_ahead,
                       float* __restrict__ uq_ahead, int n_rests, int n_sub) {
   constexpr int kRows = kCombineRows<D>;             // rows of partials merged per CTA
   if (int(blockIdx.x) >= n_comb) {
@@ -338,8 +337,7 @@ combine_select_kernel(Problem p, const float* __restrict__ scores, uint32_t* __r
   pdl_wait();
   const int slot = int(threadIdx.x) / D;
   if (slot >= kRows) return;
-  const int64_t row = int64_t(blockIdx.x) * kRows + slot;
-  combine_row<D>(partial, out, lse, splits, row, row < n_rows, int(threadIdx.x) % D, w_s[slot], norm_s[slot], 1 + slot);
+  combine_row<D>(job, int(blockIdx.x) * kRows + slot, int(threadIdx.x) % D, w_s[slot], norm_s[slot], 1 + slot);
 }
 
 }  // namespace
@@ -359,11 +357,10 @@ cudaError_t launch_topk_parts(const Problem& p, const float* scores, uint32_t* t
 }
 
 cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_t* top_hist, int32_t* group_idx,
-                                  int32_t* n_selected, const float* partial, float* out, float* lse, int splits,
-                                  int n_rows, int d, const void* q_ahead, const float* proj_ahead, float* uq_ahead,
+                                  int32_t* n_selected, const CombineJob& job, int d, const void* q_ahead, const float* proj_ahead, float* uq_ahead,
                                   cudaStream_t st) {
   const int P = plan_topk_parts(p);
-  if (P == 0 || (d != 64 && d != 128) || splits > kMaxSplits) return cudaErrorInvalidValue;
+  if (P == 0 || (d != 64 && d != 128) || job.slots > kMaxSplits) return cudaErrorInvalidValue;
   // Query sets of the launch: the scorer's row sets, except that the KV heads of per-head metadata are taken eight at a
   // time like the scopes of joint metadata (a row's sum is the same; one head at a time used 4 of the CTA's 32 warps:
   // 20.6 us per launch at B = 4, 8 heads).  With fewer combine CTAs than sets, CTAs for queries alone are added.
@@ -380,11 +377,10 @@ cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_
   }
   const int n_probs = p.B * p.S;
   const int rows_per_cta = (d == 128) ? kCombineRows<128> : kCombineRows<64>;
-  const int n_comb = std::max((n_rows + rows_per_cta - 1) / rows_per_cta, std::min(n_rests, 32));
+  const int n_comb = std::max((job.rows + rows_per_cta - 1) / rows_per_cta, std::min(n_rests, 32));
   const dim3 grid(n_comb + P * n_probs), block(kPartThreads);
   auto go = [&](auto kern) {
-    return launch_pdl(kern, grid, block, 0, st, pq, scores, top_hist, group_idx, n_selected, n_probs, partial, out, lse,
-                      splits, n_rows, n_comb, q_ahead, proj_ahead, uq_ahead, n_rests, n_sub);
+    return launch_pdl(kern, grid, block, 0, st, pq, scores, top_hist, group_idx, n_selected, n_probs, job, n_comb, q_ahead, proj_ahead, uq_ahead, n_rests, n_sub);
   };
   auto by_parts = [&](auto d_tag) {
     constexpr int D = decltype(d_tag)::value;

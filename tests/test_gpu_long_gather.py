@@ -1,0 +1,100 @@
+"""Decode steps whose gather runs beside the next layer's select: bit for bit the per-layer calls, whose selection comes from
+another kernel (topk_parts_kernel), over the shapes the gather takes and over scores that are awkward to select from."""
+import dataclasses
+
+import pytest
+import torch
+
+from paper_2511_11907_b200 import binding as kv
+from paper_2511_11907_b200 import device_workload as DW
+from paper_2511_11907_b200 import runtime as rt
+from paper_2511_11907_b200 import workloads as W
+from launches import launched
+from test_gpu_decode_step import _run_case, _step_buffers
+
+pytestmark = pytest.mark.gpu
+
+KV, ALL = W.SCOPE_KV_HEAD, W.SCOPE_ALL_HEADS
+
+
+def _wl(**kw):
+    base = dict(layers=3, batch=4, n_ctx=20011, top_k=400, calib_rows=1024)
+    base.update(kw)
+    return dataclasses.replace(W.CONFIGS[5], name="long", walk_steps=1, **base)
+
+
+def _route(wl, meta_heads, scope, flags=0):
+    dw = DW.build(wl, 1 if meta_heads == "joint" else wl.n_kv_heads, scope, walk_steps=1, reserve_bytes=1 << 30)
+    shape = dw.shape.with_flags(flags)
+    ws = rt.alloc_workspace(shape)
+    for m in dw.meta:
+        m.zero_()
+    out, lse, idx, nsel = _step_buffers(dw)
+    layers = dw.layer_tables()
+    return launched(lambda: kv.kvswap_decode_step(shape, layers, dw.q_walk[0], out, lse, idx, nsel, ws))
+
+
+# head counts that leave one to eight query heads per row, heads of 64 channels, groups whose rows do not fill blocks of
+# eight, open groups of every length of a stage, one to four layers, a list per sequence, lists shared by whole and by broken CTAs
+@pytest.mark.parametrize("meta_heads,scope,kw", [
+    ("joint", KV, dict()),
+    ("joint", KV, dict(layers=1)),
+    ("joint", KV, dict(layers=2, n_ctx=20015)),
+    ("joint", KV, dict(layers=4, n_q_heads=24, batch=3, top_k=300, group_size=16, n_ctx=33000 + 15)),
+    ("joint", KV, dict(kv_dtype=W.F16, q_dtype=W.F16, n_q_heads=64, n_ctx=20008)),
+    ("joint", KV, dict(n_q_heads=8, top_k=333, n_ctx=20009)),
+    ("joint", KV, dict(head_dim=64, top_k=800)),
+    ("joint", KV, dict(group_size=4, top_k=800, n_ctx=20002)),
+    ("joint", KV, dict(group_size=12, top_k=270, n_ctx=20011)),
+    ("joint", KV, dict(group_size=1, top_k=3000, n_ctx=20011)),
+    ("joint", KV, dict(rank=64, batch=5)),
+    ("per_head", KV, dict(batch=3, top_k=450)),
+    ("joint", ALL, dict(batch=6)),
+    ("joint", KV, dict(batch=16, n_ctx=9003, top_k=200)),
+])
+def test_step_with_a_long_gather(meta_heads, scope, kw):
+    wl = _wl(**kw)
+    names = set(_route(wl, meta_heads, scope))
+    assert "sparse_decode_long_kernel" in names and "sparse_decode_splitk_kernel" not in names
+    assert ("select_beside_kernel" in names) == (wl.layers > 1)
+    _run_case(wl, meta_heads, scope)
+
+
+def test_step_with_a_long_gather_and_the_softmax_scorer():
+    wl = _wl()
+    assert "select_beside_kernel" in _route(wl, "joint", KV, kv.KVSWAP_SCORE_SOFTMAX)
+    _run_case(wl, "joint", KV, flags=kv.KVSWAP_SCORE_SOFTMAX)
+
+
+# Scores that the sampled bound, the list or its intervals do not fit: all equal, a few values (long ties at the threshold),
+# rising with the position, a run of large ones, infinities, and lists too long to be sampled for.
+@pytest.mark.parametrize("n_ctx,top_k", [(20011, 400), (70003, 512), (20011, 1500)])
+@pytest.mark.parametrize("kind", ["equal", "few", "ramp", "run", "inf"])
+def test_select_beside_on_awkward_scores(kind, n_ctx, top_k):
+    wl = _wl(layers=2, n_ctx=n_ctx, top_k=top_k, batch=4 if n_ctx < 50000 else 3)
+    dw = DW.build(wl, 1, KV, walk_steps=1, reserve_bytes=1 << 30)
+    shape, q, ws = dw.shape, dw.q_walk[0], rt.alloc_workspace(dw.shape)
+    for l in range(wl.layers):
+        kv.kvswap_project_keys(shape, dw.K[l], dw.proj[l], dw.meta[l], 0, wl.n_ctx, ws)
+        m = dw.meta[l]
+        pos = torch.arange(wl.n_ctx, device="cuda", dtype=torch.float32)[None, None, :, None]
+        if kind == "equal":
+            m.copy_(m[:, :, :1].clone().expand_as(m))
+        elif kind == "few":
+            m.copy_(m[:, :, :1].clone().float() * (1 + (pos * 0.618).frac().mul(5).floor()))
+        elif kind == "ramp":
+            m.copy_(m[:, :, :1].clone().float() * (1 + pos / wl.n_ctx))
+        elif kind == "run":
+            m[:, :, 4096:4096 + 8 * top_k] *= 30
+        else:
+            m[:, :, ::97] = float("inf")
+    out_a, lse_a, idx_a, nsel_a = _step_buffers(dw)
+    for l in range(wl.layers):
+        kv.kvswap_score_select(shape, q[l], dw.proj[l], dw.meta[l], idx_a[l], nsel_a[l], None, ws)
+        kv.kvswap_sparse_decode(shape, q[l], dw.K[l], dw.V[l], idx_a[l], nsel_a[l], out_a[l], lse_a[l], ws)
+    out_b, lse_b, idx_b, nsel_b = _step_buffers(dw)
+    kv.kvswap_decode_step(shape, dw.layer_tables(), q, out_b, lse_b, idx_b, nsel_b, ws)
+    torch.cuda.synchronize()
+    assert kv.kvswap_read_device_status(ws) == 0
+    assert torch.equal(nsel_a, nsel_b) and torch.equal(idx_a, idx_b)
+    assert torch.equal(out_a, out_b) and torch.equal(lse_a, lse_b)
