@@ -25,6 +25,7 @@ constexpr int kRows = 128;                                 // tokens per tile
 constexpr int kThreads = 256;
 constexpr int kIssuer = 128;                               // thread that requests K and issues the MMAs (warp 4)
 constexpr int kMaxHeads = 4;                               // heads (or pairs) per CTA
+constexpr int kMaxCluster = 8;
 constexpr size_t kMaxSmem = 220 * 1024;
 __host__ __device__ constexpr int short_ctas_per_sm(int r) { return r <= 32 ? 3 : 2; }      // by registers
 
@@ -83,6 +84,7 @@ project_keys_short_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, 
     mbar_init_fence();
   }
   pdl_wait();                                                          // K and the adapter may be the previous kernel's output
+  pdl_trigger();                                                       // the next layer's launch waits there in turn
   if (tid == kIssuer) {
     for (int s = 0; s < hpc; ++s) {
       const uint32_t dst = stage0 + uint32_t(s) * C::kHeadBytes, bar = smem_addr(&full[s]);
@@ -210,16 +212,17 @@ project_keys_short_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, 
   if (n_ctas > 1) { cluster_arrive(); cluster_wait(); }                // every CTA's sums are in place
 
   // ---- this CTA's share of the rows: sum over the cluster in rank order, one rounding ------------------------------------------
-  // (No trigger: a scorer whose inputs are settled requests metadata tiles ahead of its own wait.)
   const int share = kRows / n_ctas, r0 = rank * share;
   for (int e = tid; e < share * (R / 4); e += kThreads) {
     const int row = r0 + e / (R / 4), c4 = e % (R / 4);
     const uint32_t at = stage0 + uint32_t(row * kPitch + 4 * c4) * 4u;
-    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int r = 0; r < n_ctas; ++r) {
-      const float4 x = cluster_load4(cluster_map(at, uint32_t(r)));
-      sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
-    }
+    float4 x[kMaxCluster], sum = make_float4(0.f, 0.f, 0.f, 0.f);      // all loads out at once: one trip, not one per CTA
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r)
+      if (r < n_ctas) x[r] = cluster_load4(cluster_map(at, uint32_t(r)));
+#pragma unroll
+    for (int r = 0; r < kMaxCluster; ++r)
+      if (r < n_ctas) { sum.x += x[r].x; sum.y += x[r].y; sum.z += x[r].z; sum.w += x[r].w; }
     const int n = n0 + row;
     if (n < n_end)
       store_meta4(p, meta, int64_t(b) * p.meta_sb + int64_t(hm) * p.meta_sh + int64_t(n) * p.meta_sn + 4 * c4, sum);
@@ -256,7 +259,7 @@ bool plan_project_keys_short(const Problem& p, int n_begin, int n_end, ShortPlan
   // that allows.  8 heads of 128, r = 32: B = 1, N = 1500 5.7 us against 10.3 of the persistent kernel and its adapter
   // launch, N = 5003 (three CTAs per SM) 8.9 against 10.3; at N = 9000, where a second wave would start, 20 against
   // 10.4.  Two tiles per CTA, sharing the split adapter, took 17 us there, and operands from an adapter launch 10.3.
-  for (int cluster = 8; cluster >= 1; cluster /= 2) {
+  for (int cluster = kMaxCluster; cluster >= 1; cluster /= 2) {
     const int hpc = heads / cluster;
     const size_t smem = hpc * head_bytes + 2048;
     if (heads % cluster != 0 || hpc > kMaxHeads || hpc * stride > 512 || smem > kMaxSmem) continue;
