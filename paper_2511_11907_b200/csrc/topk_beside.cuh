@@ -252,19 +252,23 @@ __device__ __forceinline__ void topk_beside_body(const Problem& p, const float* 
   if (!exact) {
     // ---- intervals of the list's keys, until few keys share the M'-th key's ------------------------------------------------
     const int n = sm.n_list;
-    uint32_t low = bound;
-    int want = Mp, shift = max(0, 22 - __clz(int((sm.key_max - bound) | 1u)));    // 1024 intervals of 2^shift from `low`
+    // `span` intervals of 2^shift keys from `low`, first over the whole list, then over the one interval found: the keys
+    // above that are among the Mp - want that are selected already, and counted again they would raise the threshold.
+    uint32_t low = bound, span = kDigit;
+    int want = Mp, shift = max(0, 22 - __clz(int((sm.key_max - bound) | 1u)));
     while (true) {
       for (int j = tid; j < n; j += kBesideThreads) {
         const uint32_t k = sm.list_key[j];
         const uint32_t at = (k - low) >> shift;
-        if (k >= low && at < uint32_t(kDigit)) atomicAdd(&sm.hist[at], 1u);
+        if (k >= low && at < span) atomicAdd(&sm.hist[at], 1u);
       }
       find_digit(want);
       low += uint32_t(sm.bin) << shift;
       want = sm.want;
       if (sm.cnt == want || sm.cnt <= kBesideFew || shift == 0) break;
-      shift = max(0, shift - 10);
+      const int finer = max(0, shift - 10);
+      span = 1u << (shift - finer);
+      shift = finer;
       clear_digit();
     }
     const int cnt = sm.cnt;

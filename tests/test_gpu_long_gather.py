@@ -98,3 +98,75 @@ def test_select_beside_on_awkward_scores(kind, n_ctx, top_k):
     assert kv.kvswap_read_device_status(ws) == 0
     assert torch.equal(nsel_a, nsel_b) and torch.equal(idx_a, idx_b)
     assert torch.equal(out_a, out_b) and torch.equal(lse_a, lse_b)
+
+
+def _near_rows(kind, problems, groups, top_k, gen):
+    """Rows of group scores [problems, groups] whose threshold lies among many equal or nearly equal scores."""
+    def normal(*size):
+        return torch.randn(size, generator=gen, dtype=torch.float64)
+
+    def ulps(base, steps):
+        return (torch.tensor(base, dtype=torch.float32).view(torch.int32) + steps.int()).view(torch.float32)
+
+    if kind == "offset":                        # a common offset and a few outliers
+        x = 1000 + (0.3 if groups > 8192 else 0.1) * normal(problems, groups)
+        x[:, :20] += 5
+    elif kind.startswith("ties"):               # so many equal scores across the threshold, among others spread widely
+        n = int(kind[4:])
+        x = (30 * normal(problems, groups)).float().sort(descending=True).values
+        x[:, top_k - n // 2:top_k - n // 2 + n] = x[:, top_k:top_k + 1].clone()
+    elif kind == "plateau":                     # more equal scores than the list has room for
+        x = normal(problems, groups).float().sort(descending=True).values
+        x[:, top_k - 100:top_k + 3000] = x[:, top_k:top_k + 1].clone()
+    elif kind == "consecutive":                 # a hundred floats in a row, each many times
+        x = ulps(1.0, torch.randint(0, 100, (problems, groups), generator=gen))
+    else:                                       # "near": ties, with others up to 800 units in the last place above them
+        x = torch.rand((problems, groups), generator=gen) * 0.5
+        x[:, :top_k // 2] = 1.0
+        x[:, top_k // 2:top_k + top_k // 2] = ulps(1.0, torch.randint(1, 800, (problems, 2 * (top_k // 2)), generator=gen)[:, :top_k])
+        x[:, top_k:top_k + top_k // 2] = 1.0
+    x = x.float()
+    return x.gather(1, torch.rand(x.shape, generator=gen).argsort(1))
+
+
+# 24 to 40 rows per case, of whole and sampled lists; the selection is compared with the per-layer calls' and with a stable
+# sort of the scores in float64.
+@pytest.mark.parametrize("kind", ["offset", "ties33", "ties48", "ties128", "plateau", "consecutive", "near"])
+@pytest.mark.parametrize("n_ctx,batch,top_k", [(131072 + 3, 3, 1024), (32768 + 5, 5, 400), (16000 + 5, 5, 400), (32768 + 5, 5, 1400)])
+def test_select_beside_among_nearly_equal_scores(kind, n_ctx, batch, top_k):
+    wl = _wl(layers=2, n_ctx=n_ctx, top_k=top_k, batch=batch)
+    groups, S = n_ctx // 8, wl.n_kv_heads
+    if kind == "plateau" and groups < top_k + 3000:
+        pytest.skip("no room for the plateau")
+    dw = DW.build(wl, 1, KV, walk_steps=1, reserve_bytes=1 << 30)
+    shape, q, ws = dw.shape, dw.q_walk[0], rt.alloc_workspace(dw.shape)
+    # Columns s, s + 8 and s + 16 of the compact cache hold the scores of scope s in three fp16 pieces, 2^11 apart: its low-rank
+    # query has 1, 2^-11 and 2^-22 there.
+    q[..., 0] = 1 / wl.rho
+    gen = torch.Generator().manual_seed(n_ctx + top_k)
+    for l in range(wl.layers):
+        dw.proj[l].zero_()
+        dw.meta[l].zero_()
+        x = _near_rows(kind, wl.batch * S, groups, top_k, gen).view(wl.batch, S, groups).cuda()
+        for k in range(3):
+            dw.proj[l][torch.arange(S), 0, torch.arange(S) + S * k] = 2.0 ** (-11 * k)
+            piece = (x * 2.0 ** (11 * k)).half()
+            x = x - piece.float() * 2.0 ** (-11 * k)
+            dw.meta[l][:, 0, :groups * 8, S * k:S * (k + 1)] = piece.transpose(1, 2).repeat_interleave(8, 1)
+    step = _step_buffers(dw)
+    layers = dw.layer_tables()
+    call = lambda: kv.kvswap_decode_step(shape, layers, q, *step, ws)
+    names = launched(call)
+    assert "select_beside_kernel" in names
+    for buf in step:
+        buf.fill_(-7)
+    call()
+    out, lse, idx, nsel = _step_buffers(dw)
+    scores = torch.empty((wl.batch, S, groups), device="cuda")
+    for l in range(wl.layers):
+        kv.kvswap_score_select(shape, q[l], dw.proj[l], dw.meta[l], idx[l], nsel[l], scores, ws)
+        kv.kvswap_sparse_decode(shape, q[l], dw.K[l], dw.V[l], idx[l], nsel[l], out[l], lse[l], ws)
+        want = scores.double().sort(dim=-1, descending=True, stable=True).indices[..., :top_k].sort(-1).values
+        assert torch.equal(idx[l].long(), want) and torch.equal(step[2][l].long(), want)
+    assert kv.kvswap_read_device_status(ws) == 0
+    assert torch.equal(step[3], nsel) and torch.equal(step[0], out) and torch.equal(step[1], lse)
