@@ -34,6 +34,7 @@ def _route(wl, meta_heads, scope, flags=0):
     return launched(lambda: kv.kvswap_decode_step(shape, layers, dw.q_walk[0], out, lse, idx, nsel, ws))
 
 
+# (A gather is long from 40 MB on, and from 3300 bytes per group of the context.)
 # head counts that leave one to eight query heads per row, heads of 64 channels, groups whose rows do not fill blocks of
 # eight, open groups of every length of a stage, one to four layers, a list per sequence, lists shared by whole and by broken CTAs
 @pytest.mark.parametrize("meta_heads,scope,kw", [
@@ -46,11 +47,11 @@ def _route(wl, meta_heads, scope, flags=0):
     ("joint", KV, dict(head_dim=64, top_k=800)),
     ("joint", KV, dict(group_size=4, top_k=800, n_ctx=20002)),
     ("joint", KV, dict(group_size=12, top_k=270, n_ctx=20011)),
-    ("joint", KV, dict(group_size=1, top_k=3000, n_ctx=20011)),
+    ("joint", KV, dict(group_size=1, top_k=3000, n_ctx=12011)),
     ("joint", KV, dict(rank=64, batch=5)),
     ("per_head", KV, dict(batch=3, top_k=450)),
     ("joint", ALL, dict(batch=6)),
-    ("joint", KV, dict(batch=16, n_ctx=9003, top_k=200)),
+    ("joint", KV, dict(batch=16, n_ctx=20003, top_k=200)),
 ])
 def test_step_with_a_long_gather(meta_heads, scope, kw):
     wl = _wl(**kw)
