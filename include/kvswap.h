@@ -271,9 +271,10 @@ int kvswap_sparse_decode_static(const kvswap_shape* shape, const void* q, const 
  * HOST array of L DEVICE pointers: K[l], V[l] are [B, H_kv, N, d]; meta[l] is [B, H_m, N, r];
  * proj[l] is [H_kv, d, r] fp32.  max_lookahead bounds how many layers the predictor may run ahead of the
  * attention: 1 = layer l is predicted while layer l-1 is attended (what a model allows, whose layer-l
- * prediction needs the input of layer l-1); 0 = no limit.  Both steps predict exactly one layer ahead,
- * which satisfies every bound.  (Layer l is scored once the K/V of layer l-2 have been attended; where gathers are
- * long, the split partials of that attention are merged while layer l is scored.)
+ * prediction needs the input of layer l-1): it is scored once the outputs of layer l-2 are complete.  0 = no
+ * limit.  Both steps predict one layer ahead; without a limit, or with one above 1, a step whose gathers are
+ * long merges the split partials of layer l-2 while layer l is scored.  (The queries of all layers are given
+ * at the call, and a layer's may be taken through its proj before the layer's turn, whatever the bound.)
  * Negative values are KVSWAP_ERR_SHAPE.
  */
 typedef struct {

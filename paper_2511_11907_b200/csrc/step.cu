@@ -292,14 +292,17 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
     // Long gathers: the select of a layer runs beside the gather of the layer before, which takes one CTA per SM and half of its
     // registers, instead of behind it:
     //   score(0) select(0) | score(1) select(1) attention(0) | score(2) select(2) attention(1) | ...
-    // The launch of select(l + 1) also merges the partials of attention(l - 1) and forms the queries of layer l + 2, beside
-    // score(l + 1); the scorer does not count leading digits.
-    // What each kernel waits for: score(l + 1) for attention(l - 1) and all before it, and lets select(l + 1) start only then;
-    // select(l + 1) lets attention(l) start when its own CTAs have, so the selection of layer l is complete by then; it
-    // waits for score(l + 1); attention(l) waits for select(l + 1), with one buffer of partials before it writes them, as the
-    // merge may still read those of layer l - 1, with two (layers take turns) at its end.
-    // 12 layers of B = 4, N = 131072, M = 1024: 517 -> 458 us; eight tokens over 12 layers of B = 8, N = 32760: 3239 -> 2900.
+    // The launch of select(l + 1) also forms the queries of layer l + 2, beside score(l + 1); the scorer does not count leading
+    // digits.  With a lookahead of one layer a combine follows each gather, and score(l + 1) waits for that of layer l - 1, whose
+    // outputs the input of layer l + 1 is made from.  Otherwise the launch of select(l + 1) merges the partials of
+    // attention(l - 1) too, beside score(l + 1).
+    // What each kernel waits for: score(l + 1) for attention(l - 1) or its combine and all before it, and lets select(l + 1)
+    // start only then; select(l + 1) lets attention(l) start when its own CTAs have, so the selection of layer l is complete by
+    // then; it waits for score(l + 1); attention(l) waits for select(l + 1): with one buffer of partials before it writes them,
+    // as the merge may still read those of layer l - 1, with two (layers take turns) at its end.  So up to three kernels are in
+    // flight: a scorer's successor starts only when all before the scorer is complete, and every kernel waits before it ends.
     if (w.long_gather) {
+      const bool merge_first = layers->max_lookahead == 1;
       const bool two = 2 * w.splits <= w.splits_room;
       auto partial_of = [&](int l) { return two && (l & 1) ? partial + size_t(p.B) * p.Hq * w.splits * (p.d + 2) : partial; };
       Problem p_late = p_settled;
@@ -339,7 +342,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
                                    n_selected + size_t(l) * nsel_elems, partial_of(l), out_l, lse_l, static_cast<uint32_t*>(ws), stream,
                                    /*combine=*/false);
         const CombineJob job = combine_job(p, w, partial_of(l), out_l, lse_l);
-        if (last || probed(l)) {
+        if (last || merge_first || probed(l)) {
           if (e == cudaSuccess) e = launch_combine(p, pending, job, stream);
           pending = CombineJob{};
           if (probed(l)) ev(probe_opt->ev_end);

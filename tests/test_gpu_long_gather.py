@@ -23,14 +23,14 @@ def _wl(**kw):
     return dataclasses.replace(W.CONFIGS[5], name="long", walk_steps=1, **base)
 
 
-def _route(wl, meta_heads, scope, flags=0):
+def _route(wl, meta_heads, scope, flags=0, lookahead=0):
     dw = DW.build(wl, 1 if meta_heads == "joint" else wl.n_kv_heads, scope, walk_steps=1, reserve_bytes=1 << 30)
     shape = dw.shape.with_flags(flags)
     ws = rt.alloc_workspace(shape)
     for m in dw.meta:
         m.zero_()
     out, lse, idx, nsel = _step_buffers(dw)
-    layers = dw.layer_tables()
+    layers = dw.layer_tables(lookahead)
     return launched(lambda: kv.kvswap_decode_step(shape, layers, dw.q_walk[0], out, lse, idx, nsel, ws))
 
 
@@ -59,6 +59,41 @@ def test_step_with_a_long_gather(meta_heads, scope, kw):
     assert "sparse_decode_long_kernel" in names and "sparse_decode_splitk_kernel" not in names
     assert ("select_beside_kernel" in names) == (wl.layers > 1)
     _run_case(wl, meta_heads, scope)
+
+
+# four query heads per list, and one: eleven lists per KV head, whose partials have one buffer
+@pytest.mark.parametrize("q_heads", [32, 88])
+@pytest.mark.parametrize("lookahead", [0, 1, 2])
+def test_lookahead_of_one_layer_merges_a_layer_before_the_next_but_one_is_scored(q_heads, lookahead):
+    """... and another bound beside that, or ahead of the last gather where there is one buffer of partials."""
+    wl = _wl(layers=4, n_q_heads=q_heads)
+    predict, attend = ["score_stream_kernel", "select_beside_kernel"], ["sparse_decode_long_kernel"]
+    if lookahead == 1:
+        want = 3 * (predict + attend + ["combine_kernel"]) + attend + ["combine_kernel"]
+    else:
+        want = 3 * (predict + attend) + ["combine_kernel"] * (q_heads == 88) + attend + ["combine_kernel"]
+    assert _route(wl, "joint", KV, lookahead=lookahead) == ["score_stream_kernel", "topk_parts_kernel"] + want
+    _run_case(wl, "joint", KV, lookahead)
+
+
+@pytest.mark.parametrize("layer", [0, 1, 2, 3])
+@pytest.mark.parametrize("lookahead", [0, 1])
+def test_probed_step_with_a_long_gather(layer, lookahead):
+    wl = _wl(layers=4)
+    dw = DW.build(wl, 1, KV, walk_steps=1, reserve_bytes=1 << 30)
+    shape, q, ws = dw.shape, dw.q_walk[0], rt.alloc_workspace(dw.shape)
+    for l in range(wl.layers):
+        kv.kvswap_project_keys(shape, dw.K[l], dw.proj[l], dw.meta[l], 0, wl.n_ctx, ws)
+    layers, plain, probed = dw.layer_tables(lookahead), _step_buffers(dw), _step_buffers(dw)
+    kv.kvswap_decode_step(shape, layers, q, *plain, ws)
+    events = [torch.cuda.Event(enable_timing=True) for _ in range(3)]
+    for e in events:
+        e.record()                                           # (created on first use)
+    kv.kvswap_decode_step(shape, layers, q, *probed, ws, kv.make_probe(layer, *events))
+    torch.cuda.synchronize()
+    assert events[0].elapsed_time(events[1]) > 0 and events[1].elapsed_time(events[2]) > 0
+    assert all(torch.equal(a, b) for a, b in zip(plain, probed))
+    assert kv.kvswap_read_device_status(ws) == 0
 
 
 def test_step_with_a_long_gather_and_the_softmax_scorer():
