@@ -42,7 +42,7 @@ select_beside_kernel(Problem p, const float* __restrict__ scores, int32_t* __res
   pdl_trigger();
   const int slot = int(threadIdx.x) / D;
   for (int row = blockIdx.x * kMergeRows<D>; row < job.rows; row += n_first * kMergeRows<D>) {
-    combine_row<D>(job, row + slot, int(threadIdx.x) % D, sm.ahead.w[slot], sm.ahead.norm[slot], 1 + slot);
+    combine_row<D, false>(job, row + slot, int(threadIdx.x) % D, sm.ahead.w[slot], sm.ahead.norm[slot], 1 + slot);
     __syncthreads();                                    // the weights are free for the next rows
   }
   if (a.q != nullptr) {

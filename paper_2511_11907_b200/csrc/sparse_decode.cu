@@ -35,7 +35,7 @@ namespace kvswap {
 namespace {
 
 constexpr int kTok = 8;                         // tokens per stage
-constexpr int kWarps = 8;                       // warps per CTA
+constexpr int kWarps = kGatherWarps;            // warps per CTA
 constexpr int kThreads = kWarps * 32;
 constexpr int kMaxDepth = 4;                    // stages per warp, at most
 constexpr int kMaxStages = kWarps * kMaxDepth;
@@ -569,7 +569,7 @@ sparse_decode_splitk_kernel(Problem p, const Q_T* __restrict__ q, const KV_T* __
 }
 
 // K5: merge the split partials of one attention, or of two, a CTA of D threads per (sequence, head) (combine.cuh).
-template <int D>
+template <int D, bool WHOLE, bool TWO>
 __global__ void __launch_bounds__(D)
 combine_kernel(CombineJob job, CombineJob job2) {
   __shared__ float w_s[kMaxSplits];
@@ -578,8 +578,9 @@ combine_kernel(CombineJob job, CombineJob job2) {
   // partials of the gather kernel before it.
   pdl_trigger();
   pdl_wait();
-  const bool second = int(blockIdx.x) >= job.rows;
-  combine_row<D>(second ? job2 : job, int(blockIdx.x) - (second ? job.rows : 0), threadIdx.x, w_s, norm_s, 0);
+  const int row = blockIdx.x;
+  if (!TWO || row < job.rows) combine_row<D, WHOLE>(job, row, threadIdx.x, w_s, norm_s, 0);
+  else combine_row<D, WHOLE>(job2, row - job.rows, threadIdx.x, w_s, norm_s, 0);
 }
 
 template <typename KV_T, int D>
@@ -743,11 +744,16 @@ void plan_sparse_decode(const Problem& p, Workspace* w) {
   if (!w->merge_in_cluster && !w->beside) plan_long_gather(p, w);
 }
 
-// The combine pass alone, for gathers that were enqueued with combine = false.
+// The combine pass alone, for one or two gathers that were enqueued with combine = false.
 cudaError_t launch_combine(const Problem& p, const CombineJob& job, const CombineJob& job2, cudaStream_t st) {
   const dim3 grid(job.rows + job2.rows), block(p.d);
-  return p.d == 128 ? launch_pdl(combine_kernel<128>, grid, block, 0, st, job, job2)
-                    : launch_pdl(combine_kernel<64>, grid, block, 0, st, job, job2);
+  auto go = [&](auto kern) { return launch_pdl(kern, grid, block, 0, st, job, job2); };
+  auto by_kind = [&](auto d_tag) {
+    constexpr int D = decltype(d_tag)::value;
+    if (job2.rows > 0) return go(combine_kernel<D, false, true>);
+    return job.whole() ? go(combine_kernel<D, true, false>) : go(combine_kernel<D, false, false>);
+  };
+  return p.d == 128 ? by_kind(std::integral_constant<int, 128>()) : by_kind(std::integral_constant<int, 64>());
 }
 
 cudaError_t launch_sparse_decode(const Problem& p, const Workspace& w, const void* q, const void* K, const void* V,

@@ -18,7 +18,7 @@ namespace kvswap {
 namespace {
 
 constexpr int kTok = 16;                        // tokens per stage
-constexpr int kWarps = 8;                       // warps per CTA
+constexpr int kWarps = kGatherWarps;            // warps per CTA
 constexpr int kThreads = kWarps * 32;
 constexpr int kMaxDepth = 8;                    // stages per warp, at most
 

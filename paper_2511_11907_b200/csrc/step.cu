@@ -343,7 +343,7 @@ static int decode_step_impl(const kvswap_shape* shape, const kvswap_layers* laye
                                    /*combine=*/false);
         const CombineJob job = combine_job(p, w, partial_of(l), out_l, lse_l);
         if (last || merge_first || probed(l)) {
-          if (e == cudaSuccess) e = launch_combine(p, pending, job, stream);
+          if (e == cudaSuccess) e = launch_combine(p, job, pending, stream);
           pending = CombineJob{};
           if (probed(l)) ev(probe_opt->ev_end);
         } else {

@@ -337,7 +337,7 @@ combine_select_kernel(Problem p, const float* __restrict__ scores, uint32_t* __r
   pdl_wait();
   const int slot = int(threadIdx.x) / D;
   if (slot >= kRows) return;
-  combine_row<D>(job, int(blockIdx.x) * kRows + slot, int(threadIdx.x) % D, w_s[slot], norm_s[slot], 1 + slot);
+  combine_row<D, true>(job, int(blockIdx.x) * kRows + slot, int(threadIdx.x) % D, w_s[slot], norm_s[slot], 1 + slot);
 }
 
 }  // namespace
@@ -360,7 +360,7 @@ cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_
                                   int32_t* n_selected, const CombineJob& job, int d, const void* q_ahead, const float* proj_ahead, float* uq_ahead,
                                   cudaStream_t st) {
   const int P = plan_topk_parts(p);
-  if (P == 0 || (d != 64 && d != 128) || job.slots > kMaxSplits) return cudaErrorInvalidValue;
+  if (P == 0 || (d != 64 && d != 128) || job.slots > kMaxSplits || !job.whole()) return cudaErrorInvalidValue;
   // Query sets of the launch: the scorer's row sets, except that the KV heads of per-head metadata are taken eight at a
   // time like the scopes of joint metadata (a row's sum is the same; one head at a time used 4 of the CTA's 32 warps:
   // 20.6 us per launch at B = 4, 8 heads).  With fewer combine CTAs than sets, CTAs for queries alone are added.
