@@ -146,7 +146,7 @@ cudaError_t score_launch(const Problem& p_in, const Workspace& w, const void* q,
   p.score_pitch = group_scores_opt ? p.NG : workspace_score_pitch(p);     // a caller's buffer is dense [B, S, NG]
   if (p.flags & KVSWAP_SCORE_SOFTMAX) {
     float* u_heads = reinterpret_cast<float*>(base + w.off_softmax);
-    uint32_t* top_hist = counts_top_digit(p) && !beside ? reinterpret_cast<uint32_t*>(base + w.off_hist) : nullptr;
+    uint32_t* top_hist = counts_top_digit(p) ? reinterpret_cast<uint32_t*>(base + w.off_hist) : nullptr;
     return launch_score_softmax(p, q, proj, meta, u_heads, u_heads + size_t(p.B) * p.Hq * p.r, scores, top_hist,
                                 static_cast<uint32_t*>(ws), stream);
   }

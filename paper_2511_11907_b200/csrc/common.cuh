@@ -122,6 +122,7 @@ cudaError_t launch_score_pool(const Problem& p, const float* uq, const void* met
 bool score_stream_rows(const Problem& p);        // metadata type and rank are among the scorer's
 bool score_stream_supported(const Problem& p);
 bool score_stream_fuses_query(const Problem& p);
+int score_stream_light_ctas(const Problem& p);
 bool score_stream_counts_top_digit(const Problem& p);
 cudaError_t launch_score_stream(const Problem& p, const void* q, const float* proj, const float* uq,
                                 const void* meta, float* scores, uint32_t* top_hist, uint32_t* err,

@@ -74,6 +74,15 @@ bool score_stream_rows(const Problem& p) {
 bool score_stream_supported(const Problem& p) { Plan pl; return plan(p, &pl); }
 bool score_stream_fuses_query(const Problem& p) { Plan pl; return plan(p, &pl) && pl.fused; }
 bool score_stream_counts_top_digit(const Problem& p) { Plan pl; return plan(p, &pl) && pl.counts; }
+// CTAs of the scorer that neither forms queries nor counts (kDeep, queries found in memory), where it leaves half of an SM's
+// registers: 512 threads of 47 to 60 for fp16 rows of 16 or 32 and groups of 2 to 32, 52 to 60 for 8-bit rows and groups
+// of 8 to 32 (fp16 rows of 64, fp32 rows, groups of one or of other lengths: 67 to 127).  Else 0.
+int score_stream_light_ctas(const Problem& p) {
+  Plan pl;
+  if (!plan(p, &pl) || !pl.fused) return 0;
+  const bool light = p.meta_dtype == KVSWAP_F16 ? p.r <= 32 && pl.g_shift >= 1 : p.meta_dtype == KVSWAP_E4M3 && pl.g_shift >= 3;
+  return light ? pl.ctas : 0;
+}
 void score_stream_row_sets(const Problem& p, int* n_rests, int* n_sub) {
   Plan pl;
   const bool ok = plan(p, &pl);

@@ -404,15 +404,19 @@ void plan_long_gather(const Problem& p, Workspace* w) {
   const int64_t tokens = int64_t(p.M) * p.G + (p.N - int64_t(p.NG) * p.G);
   const size_t row = size_t(p.d) * 2;
   // A long gather of the tensor-core engine deals the warps of the whole GPU to the lists, not whole CTAs, with stages of 16
-  // tokens and one CTA per SM: as fast as two CTAs of half the stages (29.6 and 29.4 us at B = 4, 8 x 8192 tokens attended), it
-  // leaves half of the registers to the next layer's select, which a decode step then runs beside it (step.cu).  That takes
-  // 8 us there and 15 for 16384 groups, and the scorer behind waits for both: not where the gather is over long before.
-  // (B = 2, 8 heads, N = 50003, 3200 tokens, 26 MB: 210 against 203 us for 8 layers; B = 3, 8 heads, N = 98301, 4800 tokens, 59 MB: 275
-  // against 309 for 12.)
+  // tokens and one CTA per SM: it leaves half of the registers to the next layer's select, which a decode step then runs
+  // beside it (step.cu), and takes as long as two CTAs of half the stages or a little longer (a score_select and a
+  // sparse_decode of 92 MB, 4 sequences, 8 heads: 42.6 against 42.0 us; 8 sequences, heads of 64 channels 44.0 against 45.1).
+  // The select takes 8 us there, 15 for 16384 groups, and the scorer behind waits for both: not where the gather is over long
+  // before.  us a layer with the other plan / with this one and no bound on the lookahead / bounded to one layer:
+  //   4 sequences,  32768 tokens   50 MB 24.1 / 20.9 / 22.5    80 MB 28.6 / 26.7 / 28.4    110 MB 33.7 / 32.2 / 33.7
+  //   4 sequences,  65536 tokens   50 MB 25.6 / 23.3 / 25.3    80 MB 30.1 / 27.7 / 30.0    110 MB 35.1 / 32.4 / 34.5
+  //   8 sequences,  65536 tokens   50 MB 31.3 / 27.7 / 30.1    80 MB 36.2 / 32.0 / 35.0    110 MB 40.8 / 36.2 / 39.3
+  //   4 sequences, 131072 tokens   60 MB 32.5 / 30.5 / 32.8    80 MB 35.7 / 34.1 / 37.1    110 MB 40.7 / 38.2 / 41.5
+  // (groups of 8; 2 sequences of 50003 tokens, 26 MB: 25.4 / 26.2 unbounded).  134 MB of the last row gain again, 43.1 / 38.5 / 41.5.
   const int64_t bytes = problems * tokens * int64_t(2 * row);
-  // With more lists than SMs a second select on an SM would keep the gather off it.
-  w->long_gather = p.kv_dtype != KVSWAP_F32 && p.q_dtype == p.kv_dtype && select_beside_supported(p) && p.B * p.S < kNumSMs &&
-                   bytes >= std::max<int64_t>(40 << 20, int64_t(p.NG) * 3300);
+  w->long_gather = p.kv_dtype != KVSWAP_F32 && p.q_dtype == p.kv_dtype && select_beside_supported(p) &&
+                   bytes >= std::max<int64_t>(47 << 20, int64_t(p.NG) * 5000);
   if (!w->long_gather) return;
   const int64_t n_stages = (tokens + kTok - 1) / kTok;
   auto slots_of = [&](int64_t per_list) {                        // CTAs that a list is spread over, at most

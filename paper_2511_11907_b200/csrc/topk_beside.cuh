@@ -34,6 +34,22 @@ constexpr int kListKeys = 2048;              // room of the list
 constexpr int kDigit = 1024;                 // bins of the second and third digit
 constexpr int kBesideFew = 32;                 // candidates that one warp ranks directly instead of by another digit
 
+// Even sample of a row: one key of every NG / 2^bits, and the rank in it that the M'-th key's share falls behind.
+struct BesideSample {
+  int bits, rank;
+  // Whether the list has room for the keys that reach a sampled key of that rank, 3.5 deviations allowed for.
+  __host__ __device__ __forceinline__ bool list_has_room(int at_rank, int NG) const {
+    return (float(at_rank) + 3.5f * sqrtf(float(at_rank))) * float(NG) <= float(kListKeys << bits);
+  }
+};
+__host__ __device__ __forceinline__ BesideSample beside_sample(int NG, int Mp) {
+  BesideSample s;
+  s.bits = NG > 8192 ? 11 : 10;
+  const float share = float(Mp) * float(1 << s.bits) / float(NG);
+  s.rank = int(share + 3.5f * sqrtf(share)) + 4;
+  return s;
+}
+
 struct BesideSmem {
   uint32_t sel[4 * kBesideParts];               // selected keys: word 4 v + e, bit lane: key 128 v + 4 lane + e
   uint32_t hist[kKeyTopBins / 2];            // leading digit: two 16-bit counters a word; kDigit words otherwise; at last the
@@ -161,14 +177,11 @@ __device__ __forceinline__ void topk_beside_body(const Problem& p, const float* 
   };
 
   // ---- the first round of keys, and a bound ------------------------------------------------------------------------
-  // even sample: one key of every NG / 2^bits; the rank that the M'-th key's share of it falls behind
   constexpr int kSample = P == 4 ? 4 : 2;      // keys per thread, at most
-  const int bits = P == 4 && NG > kBesidePart * kBesideWarps * P ? 11 : 10;
-  const float share = float(Mp) * float(1 << bits) / float(NG);
-  const int rank = int(share + 3.5f * sqrtf(share)) + 4;
-  // (count over the whole row at once where the list would not have room for what is to be expected)
-  bool exact = NG > kListKeys && (float(rank) + 3.5f * sqrtf(float(rank))) * float(NG) > float(kListKeys << bits);
-  const bool sampled = NG > kListKeys && !exact;
+  const BesideSample even = beside_sample(NG, Mp);
+  const int bits = even.bits, rank = even.rank;
+  const bool sampled = NG > kListKeys;
+  bool exact = false;                          // the digits of the whole row are counted instead
   float sample[kSample];
 #pragma unroll
   for (int k = 0; k < kSample; ++k)
@@ -187,7 +200,7 @@ __device__ __forceinline__ void topk_beside_body(const Problem& p, const float* 
     const int want = sm.want, reach = rank - want + sm.cnt;    // samples that reach the bin
     clear_digit();
     bound = top << 20;
-    if ((float(reach) + 3.5f * sqrtf(float(reach))) * float(NG) > float(kListKeys << bits)) {   // too coarse
+    if (!even.list_has_room(reach, NG)) {                      // too coarse
 #pragma unroll
       for (int k = 0; k < kSample; ++k) {
         const uint32_t key = score_key(sample[k]);
@@ -396,9 +409,13 @@ __device__ __forceinline__ void topk_beside_body(const Problem& p, const float* 
   }
 }
 
-// Parts per warp and round (1, 2 or 4); 0 when the row is too long for this select (or empty).
+// Parts per warp and round (1, 2 or 4); 0 when the row is too long for this select (or empty), or when so many are to be
+// selected that the list has no room for what a sample lets through: counting the row's digits instead is exact, but
+// slow (4 sequences, 16384 groups, M = 1400: 42.5 us a layer against 36.3 with the select behind the gather).
 inline int plan_topk_beside(const Problem& p) {
-  if (p.NG < 1 || p.NG > kBesideParts * kBesidePart ) return 0;
+  if (p.NG < 1 || p.NG > kBesideParts * kBesidePart) return 0;
+  const BesideSample s = beside_sample(p.NG, p.Mp);
+  if (p.NG > kListKeys && !s.list_has_room(s.rank, p.NG)) return 0;
   const int need = (p.NG + kBesidePart * kBesideWarps - 1) / (kBesidePart * kBesideWarps);
   return need <= 1 ? 1 : need <= 2 ? 2 : 4;
 }

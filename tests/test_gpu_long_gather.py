@@ -34,31 +34,59 @@ def _route(wl, meta_heads, scope, flags=0, lookahead=0):
     return launched(lambda: kv.kvswap_decode_step(shape, layers, dw.q_walk[0], out, lse, idx, nsel, ws))
 
 
-# (A gather is long from 40 MB on, and from 3300 bytes per group of the context.)
-# head counts that leave one to eight query heads per row, heads of 64 channels, groups whose rows do not fill blocks of
-# eight, open groups of every length of a stage, one to four layers, a list per sequence, lists shared by whole and by broken CTAs
-@pytest.mark.parametrize("meta_heads,scope,kw", [
-    ("joint", KV, dict()),
-    ("joint", KV, dict(layers=1)),
-    ("joint", KV, dict(layers=2, n_ctx=20015)),
-    ("joint", KV, dict(layers=4, n_q_heads=24, batch=3, top_k=300, group_size=16, n_ctx=33000 + 15)),
-    ("joint", KV, dict(kv_dtype=W.F16, q_dtype=W.F16, n_q_heads=64, n_ctx=20008)),
-    ("joint", KV, dict(n_q_heads=8, top_k=333, n_ctx=20009)),
-    ("joint", KV, dict(head_dim=64, top_k=800)),
-    ("joint", KV, dict(group_size=4, top_k=800, n_ctx=20002)),
-    ("joint", KV, dict(group_size=12, top_k=270, n_ctx=20011)),
-    ("joint", KV, dict(group_size=1, top_k=3000, n_ctx=12011)),
-    ("joint", KV, dict(rank=64, batch=5)),
-    ("per_head", KV, dict(batch=3, top_k=450)),
-    ("joint", ALL, dict(batch=6)),
-    ("joint", KV, dict(batch=16, n_ctx=20003, top_k=200)),
+# A gather is long from 47 MiB on, and from 5000 bytes per group of the context; and only where the select has room beside the
+# scorer (select_beside_supported).  Head counts that leave one to eight query heads per row, heads of 64 channels, groups whose rows
+# do not fill blocks of eight, open groups of every length of a stage, one to four layers, lists shared by whole and by broken
+# CTAs and by one warp each, both stored types and ranks.
+@pytest.mark.parametrize("kw", [
+    dict(),
+    dict(layers=1),
+    dict(layers=2, n_ctx=20015),
+    dict(layers=4, n_q_heads=24, batch=3, top_k=300, group_size=16, n_ctx=33000 + 15),
+    dict(kv_dtype=W.F16, q_dtype=W.F16, n_q_heads=64, n_ctx=20008),
+    dict(n_q_heads=8, n_ctx=20009),
+    dict(n_q_heads=88, n_ctx=20010),
+    dict(head_dim=64, top_k=800),
+    dict(group_size=4, top_k=800, n_ctx=20002),
+    dict(group_size=2, batch=5, top_k=1400, n_ctx=20003),
+    dict(group_size=32, top_k=100, n_ctx=20012),
+    dict(rank=16, batch=5),
+    dict(meta_dtype=W.E4M3, batch=5),
+    dict(batch=8, top_k=200),
 ])
-def test_step_with_a_long_gather(meta_heads, scope, kw):
+def test_step_with_a_long_gather(kw):
     wl = _wl(**kw)
-    names = set(_route(wl, meta_heads, scope))
+    names = set(_route(wl, "joint", KV))
     assert "sparse_decode_long_kernel" in names and "sparse_decode_splitk_kernel" not in names
     assert ("select_beside_kernel" in names) == (wl.layers > 1)
+    _run_case(wl, "joint", KV)
+
+
+# Gathers as long whose select has no such room, or nothing to gain: the schedule of shorter ones
+@pytest.mark.parametrize("meta_heads,scope,kw", [
+    ("joint", KV, dict(rank=64, batch=5)),
+    ("joint", KV, dict(rank=128)),
+    ("joint", KV, dict(meta_dtype=W.F32)),
+    ("joint", KV, dict(group_size=12, top_k=270)),
+    ("joint", KV, dict(group_size=1, top_k=3200, n_ctx=10011)),
+    ("joint", KV, dict(top_k=1900)),
+    ("joint", KV, dict(batch=16, n_ctx=20003, top_k=200)),
+    ("joint", KV, dict(batch=8, n_ctx=16005, top_k=200)),
+    ("per_head", KV, dict(batch=3, top_k=550)),
+    ("joint", ALL, dict(batch=6)),
+    ("per_head", ALL, dict(batch=3, n_q_heads=32, n_kv_heads=16, top_k=300)),
+])
+def test_step_with_a_gather_as_long_and_no_room_beside_it(meta_heads, scope, kw):
+    wl = _wl(**kw)
+    names = set(_route(wl, meta_heads, scope))
+    assert "sparse_decode_splitk_kernel" in names and not names & {"sparse_decode_long_kernel", "select_beside_kernel"}
     _run_case(wl, meta_heads, scope)
+
+
+def test_step_with_a_gather_as_long_behind_the_softmax_scorer():
+    wl = _wl()
+    assert "sparse_decode_long_kernel" not in _route(wl, "joint", KV, kv.KVSWAP_SCORE_SOFTMAX)
+    _run_case(wl, "joint", KV, flags=kv.KVSWAP_SCORE_SOFTMAX)
 
 
 # four query heads per list, and one: eleven lists per KV head, whose partials have one buffer
@@ -96,14 +124,8 @@ def test_probed_step_with_a_long_gather(layer, lookahead):
     assert kv.kvswap_read_device_status(ws) == 0
 
 
-def test_step_with_a_long_gather_and_the_softmax_scorer():
-    wl = _wl()
-    assert "select_beside_kernel" in _route(wl, "joint", KV, kv.KVSWAP_SCORE_SOFTMAX)
-    _run_case(wl, "joint", KV, flags=kv.KVSWAP_SCORE_SOFTMAX)
-
-
 # Scores that the sampled bound, the list or its intervals do not fit: all equal, a few values (long ties at the threshold),
-# rising with the position, a run of large ones, infinities, and lists too long to be sampled for.
+# rising with the position, a run of large ones, infinities; few, many and most groups selected.
 @pytest.mark.parametrize("n_ctx,top_k", [(20011, 400), (70003, 512), (20011, 1500)])
 @pytest.mark.parametrize("kind", ["equal", "few", "ramp", "run", "inf"])
 def test_select_beside_on_awkward_scores(kind, n_ctx, top_k):
@@ -129,7 +151,11 @@ def test_select_beside_on_awkward_scores(kind, n_ctx, top_k):
         kv.kvswap_score_select(shape, q[l], dw.proj[l], dw.meta[l], idx_a[l], nsel_a[l], None, ws)
         kv.kvswap_sparse_decode(shape, q[l], dw.K[l], dw.V[l], idx_a[l], nsel_a[l], out_a[l], lse_a[l], ws)
     out_b, lse_b, idx_b, nsel_b = _step_buffers(dw)
-    kv.kvswap_decode_step(shape, dw.layer_tables(), q, out_b, lse_b, idx_b, nsel_b, ws)
+    layers = dw.layer_tables()
+    assert "select_beside_kernel" in launched(lambda: kv.kvswap_decode_step(shape, layers, q, out_b, lse_b, idx_b, nsel_b, ws))
+    for buf in (out_b, lse_b, idx_b, nsel_b):
+        buf.fill_(-7)
+    kv.kvswap_decode_step(shape, layers, q, out_b, lse_b, idx_b, nsel_b, ws)
     torch.cuda.synchronize()
     assert kv.kvswap_read_device_status(ws) == 0
     assert torch.equal(nsel_a, nsel_b) and torch.equal(idx_a, idx_b)
