@@ -163,7 +163,7 @@ project_keys_umma_kernel(Problem p, const __grid_constant__ CUtensorMap map_k, c
 
   // The kernel before this one splits the adapter, and let this one start once everything before it was
   // complete: K may be fetched at once, the pieces and their scales only after the wait.  No early trigger
-  // here: a scorer whose inputs are settled requests metadata tiles ahead of its own wait.
+  // here: the stages leave little of an SM's shared memory, so what follows would find no room before the end.
   if (warp == 0) {
     // ================================ producer ==============================================
     if (lane == 0) {

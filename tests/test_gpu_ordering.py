@@ -161,3 +161,40 @@ def test_step_whose_inputs_are_settled_still_orders_its_own_kernels(layers_n, N,
         bad += (~torch.isfinite(out)).any() | (out != want[i % 2][0]).any() | (idx != want[i % 2][1]).any()
     torch.cuda.synchronize()
     assert int(bad) == 0 and kv.kvswap_read_device_status(ws) == 0
+
+
+# the short kernel, which lets its successor start early, the general one, and the tensor-core one of long prompts
+@pytest.mark.parametrize("N,per_head,r", [(1500, False, 32), (3001, True, 32), (1500, False, 128), (70000, False, 32)])
+@pytest.mark.parametrize("kind", ["call", "step"])
+def test_scorer_behind_the_projection_of_its_metadata(N, per_head, r, kind):
+    H, d, M = 8, 128, 64
+    hm = H if per_head else 1
+    shape = kv.make_shape(batch=1, n_ctx=N, n_q_heads=4 * H, n_kv_heads=H, head_dim=d, rank=r, meta_heads=hm, group_size=8,
+                          top_k=M, kv_dtype=kv.KVSWAP_BF16, meta_dtype=kv.KVSWAP_F16, q_dtype=kv.KVSWAP_BF16)
+    q, K = _randn(1, 1, 4 * H, d, dtype=torch.bfloat16, seed=90), _randn(1, H, N, d, dtype=torch.bfloat16, seed=91)
+    proj = _randn(H, d, r, seed=92) * 0.1
+    meta, ws = torch.empty((1, hm, N, r), dtype=torch.float16, device="cuda"), rt.alloc_workspace(shape)
+    out = torch.empty((1, 1, 4 * H, d), device="cuda")
+    idx, nsel = torch.empty((1, 1, H, M), dtype=torch.int32, device="cuda"), torch.empty((1, 1, H), dtype=torch.int32, device="cuda")
+    layers = kv.make_layers([K], [K], [meta], [proj], 0)
+
+    def consume():
+        if kind == "call":
+            kv.kvswap_score_select(shape, q[0], proj, meta, idx[0], nsel[0], None, ws)
+        else:
+            kv.kvswap_decode_step(shape, layers, q, out, None, idx, nsel, ws)
+
+    kv.kvswap_project_keys(shape, K, proj, meta, 0, N, ws)
+    torch.cuda.synchronize()
+    consume()
+    torch.cuda.synchronize()
+    want = idx.clone()
+    for _ in range(10):
+        meta.zero_()
+        idx.fill_(-7)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(100000)                           # both calls are queued before the first one starts
+        kv.kvswap_project_keys(shape, K, proj, meta, 0, N, ws)
+        consume()
+        torch.cuda.synchronize()
+        assert torch.equal(idx, want)
