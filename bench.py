@@ -43,7 +43,7 @@ UNIT = "steps/s"
 # kernel from one ncu capture at the workload's full shapes on three layers (the traffic of a launch
 # does not depend on the layer count).  None for workloads that were not captured, or whose kernel
 # has changed since.  Key: (config, metadata layout, scope).
-NCU_TRAFFIC = {(5, "joint", "kv_head"): 134451029 + 3957163, (5, "per_head", "kv_head"): 134451029 + 3957163}
+NCU_TRAFFIC = {(5, "joint", "kv_head"): 134455296 + 3414528, (5, "per_head", "kv_head"): 134451029 + 3957163}
 
 
 def esz_of(dtype: int) -> int:
@@ -235,6 +235,19 @@ def cpu_baseline(wl, dw, meta_heads, scope_name, rt):
 # GPU arm
 # --------------------------------------------------------------------------------------------
 MIN_CALLS = 2000          # launches of a call timed per figure, whatever --steps says
+
+
+def kernels_of(torch, call):
+    """Kernels that call() launches, counted in a stream capture of it."""
+    from cuda.bindings import driver as cu
+    graph, side = torch.cuda.CUDAGraph(keep_graph=True), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        call()
+    raw = cu.CUgraph(graph.raw_cuda_graph())
+    _, _, n = cu.cuGraphGetNodes(raw)
+    _, nodes, n = cu.cuGraphGetNodes(raw, n)
+    return sum(cu.cuGraphNodeGetType(x)[1] == cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL for x in nodes[:n])
 
 
 def graph_call_us(torch, fns, min_calls=None):
@@ -569,7 +582,8 @@ def run_ours(args, wl):
         "keys_scored_per_sec": value * keys_per_step,
         "keys_scored_per_sec_k2k3": roof_sel["keys_scored_per_sec_k2k3"],
         "schedule": {"predictor_lookahead_layers": 1,
-                     "order": "score(l+1), attention(l), [combine(l) + top-k(l+1)] on one stream; programmatic dependent launches",
+                     "order": "score(l+1), attention(l), combine(l) on one stream, top-k(l+1) beside a long attention or "
+                              "with the combine behind it; programmatic dependent launches",
                      "step_bytes_per_sec_gbs": (decode_bytes + select_bytes) * L / (ms_per_step * 1e-3) / 1e9},
         "growing_context": {"value": world * 1e3 * grow_steps / grow_ms, "unit": UNIT, "steps": grow_steps,
                             "n_ctx": [N - grow_steps, N], "ms_per_step": grow_ms / grow_steps,
@@ -578,7 +592,7 @@ def run_ours(args, wl):
         "reuse_buffer": reuse,
         "e2e": {"value": world * 1e3 * e2e_steps / e2e_ms, "unit": UNIT, "h2d_bytes_per_step": q_bytes,
                 "d2h_bytes_per_step": out_bytes, "steps": e2e_steps},
-        "gpu_launches": (3 * L + 1) * steps,
+        "gpu_launches": kernels_of(torch, lambda: step(0)) * steps,
         "roofline": roof,
         "roofline_score_select": roof_sel,
         "secondary": secondary,
