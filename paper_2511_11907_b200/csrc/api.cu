@@ -195,8 +195,8 @@ cudaError_t select_launch(const Problem& p_in, const Workspace& w, int32_t* grou
 // (launch_sparse_decode with combine = false, any shape) has been enqueued before: one launch.  False
 // when the select of this shape has no such kernel (the caller then launches the two separately).
 bool select_with_combine_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected,
-                                void* ws, const CombineJob& job, int d, cudaStream_t stream, cudaError_t* result, const void* q_ahead,
-                                const float* proj_ahead, int uq_ahead) {
+                                void* ws, const CombineJob& job, int d, cudaStream_t stream, cudaError_t* result,
+                                const void* q_ahead, const float* proj_ahead, int uq_ahead) {
   Problem p = p_in;
   p.score_pitch = workspace_score_pitch(p);
   if (!select_merges_with_combine(p)) return false;
@@ -204,7 +204,8 @@ bool select_with_combine_launch(const Problem& p_in, const Workspace& w, int32_t
   float* uq = reinterpret_cast<float*>(base + w.off_uq + (uq_ahead > 0 ? w.uq_bytes : 0));
   const bool ahead = q_ahead != nullptr && uq_ahead >= 0 && score_stream_fuses_query(p);
   *result = launch_combine_select(p, reinterpret_cast<float*>(base + w.off_scores),
-                                  reinterpret_cast<uint32_t*>(base + w.off_hist), group_idx, n_selected, job, d, ahead ? q_ahead : nullptr, proj_ahead, uq, stream);
+                                  reinterpret_cast<uint32_t*>(base + w.off_hist), group_idx, n_selected, job, d,
+                                  ahead ? q_ahead : nullptr, proj_ahead, uq, stream);
   return true;
 }
 

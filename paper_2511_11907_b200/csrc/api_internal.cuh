@@ -31,8 +31,8 @@ cudaError_t select_launch(const Problem& p_in, const Workspace& w, int32_t* grou
 // low-rank queries of the layer with that q and proj_ahead into query buffer uq_ahead (0 or 1) of the
 // workspace, where this shape's scorer can take them from (query_ahead_supported).
 bool select_with_combine_launch(const Problem& p_in, const Workspace& w, int32_t* group_idx, int32_t* n_selected,
-                                void* ws, const CombineJob& job, int d, cudaStream_t stream, cudaError_t* result, const void* q_ahead = nullptr,
-                                const float* proj_ahead = nullptr, int uq_ahead = -1);
+                                void* ws, const CombineJob& job, int d, cudaStream_t stream, cudaError_t* result,
+                                const void* q_ahead = nullptr, const float* proj_ahead = nullptr, int uq_ahead = -1);
 bool query_ahead_supported(const Problem& p);
 // True when select_with_combine_launch has a kernel for this shape's select.
 bool select_merges_with_combine(const Problem& p);

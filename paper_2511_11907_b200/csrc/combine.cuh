@@ -32,14 +32,14 @@ inline CombineJob combine_job(const Problem& p, const Workspace& w, const float*
   return CombineJob{partial, out, lse, p.B * p.Hq, w.splits, w.heads_per_cta, w.warps_per_list};
 }
 
-// D threads (c = 0..D-1) merge row `row` of `job`.  Every load of the row's first splits is issued before anything is computed
-// (one memory round trip; the loads bypass L1, as the partials need not be those of the kernel waited for); the split weights are
-// formed once by the first warp of the D threads and
-// shared through w_s [kMaxSplits] and norm_s [2].  The D threads meet at named barrier `barrier`
-// (0 = the CTA-wide one: then the CTA has exactly D threads).  Without a row (row >= job.rows) the threads only keep
-// the barrier company.  WHOLE: every slot is filled (job.whole()).  The kernels that only meet such jobs are built without the
-// division, whose instructions alone took 0.9 us of a call with a separate combine (45.1 -> 44.2 us for a score_select and a
-// sparse_decode of 92 MB, 4 sequences).
+// D threads (c = 0..D-1) merge row `row` of `job`.  Every load of the row's first splits is issued before anything is
+// computed (one memory round trip; the loads bypass L1, as the partials need not be those of the kernel waited for); the
+// split weights are formed once by the first warp of the D threads and shared through w_s [kMaxSplits] and norm_s [2].  The
+// D threads meet at named barrier `barrier` (0 = the CTA-wide one: then the CTA has exactly D threads).  Without a row
+// (row >= job.rows) the threads only keep the barrier company.
+// WHOLE: every slot is filled (job.whole()).  The kernels that only meet such jobs are built without the division, whose
+// instructions alone took 0.9 us of a call with a separate combine (45.1 -> 44.2 us for a score_select and a sparse_decode
+// of 92 MB, 4 sequences).
 template <int D, bool WHOLE>
 __device__ __forceinline__ void combine_row(const CombineJob& job, int row, int c, float* w_s, float* norm_s, int barrier) {
   constexpr float kLn2 = 0.6931471805599453f;

@@ -59,7 +59,7 @@ struct Workspace {
   int splits_room;     // splits the partials are planned for: no fewer than `splits` of any context length and flags
   int heads_per_cta;   // query heads sharing one K/V pass in sparse_decode
   int depth;           // shared-memory stages per compute warp in sparse_decode
-  bool long_gather;    // the gather takes one CTA per SM and half of its registers: a decode step runs the next layer's select beside it
+  bool long_gather;    // the gather takes one CTA per SM and half of its registers: a step runs the next layer's select beside it
   bool beside;         // a decode step runs the gather beside the next layer's one-launch predictor (splits planned for what that leaves)
   bool merge_in_cluster;   // the splits of a list form a cluster that merges them (no combine pass; the same bits)
   bool merge_alone;    // ... also when sparse_decode is called on its own
@@ -159,8 +159,8 @@ cudaError_t launch_select_beside(const Problem& p, const float* scores, int32_t*
 // (its q and proj) into uq_ahead [B, Su, r], for a streaming scorer that is enqueued next: the bits are
 // those the scorer would build itself.  Only where score_stream_fuses_query(p).
 cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_t* top_hist, int32_t* group_idx,
-                                  int32_t* n_selected, const CombineJob& job, int d, const void* q_ahead, const float* proj_ahead, float* uq_ahead,
-                                  cudaStream_t st);
+                                  int32_t* n_selected, const CombineJob& job, int d, const void* q_ahead,
+                                  const float* proj_ahead, float* uq_ahead, cudaStream_t st);
 // Row sets of the streaming scorer for `p` (0 when it does not take the shape) and scope blocks per
 // (sequence, metadata head): the arguments of row_set() in lowrank_query.cuh.
 void score_stream_row_sets(const Problem& p, int* n_rests, int* n_sub);

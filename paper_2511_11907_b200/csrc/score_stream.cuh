@@ -50,14 +50,14 @@ constexpr int kMultiTiles = 8;                            // tiles whose scores 
 
 // How a CTA works: kForms builds the low-rank queries and counts leading digits, kCounts finds the queries in memory, kDeep
 // finds them too, does not count and has a third stage in the counters' place (a decode step whose select does without:
-// topk_beside.cuh).  The flush of the counters alone took 3 us of a layer there, and with three stages a warp has nearly all
-// of its 3.5 tiles in flight before its dependency wait: 11.3 -> 6.5 us from the wait to the end at B = 4, N = 131072.
+// topk_beside.cuh).  It flushes nothing, and with three stages a warp has nearly all of its 3.5 tiles in flight before its
+// dependency wait: 14.7 -> 11.8 us as a launch of its own at B = 4, N = 131072.
 enum ScoreMode { kForms, kCounts, kDeep };
 
 template <int META, int R, int GS, ScoreMode MODE>
 struct ScoreSmem {
   static constexpr int kDepth = MODE == kDeep ? kScoreDepth + 1 : kScoreDepth;
-  unsigned char tiles[kScoreWarps * kDepth * ScoreStage<META, R, GS>::kBytes];           // 128 KB of stages, or 96; kDeep: 192 or 144
+  unsigned char tiles[kScoreWarps * kDepth * ScoreStage<META, R, GS>::kBytes];   // 128 KB of stages, or 96; kDeep: 192 or 144
   uint32_t hist[MODE == kDeep ? 4 : kHistWords];          // 64 KB
   unsigned long long full[kScoreWarps * kDepth];
   float urow[MODE == kForms ? kMaxSets : 1][MODE == kForms ? kScoreCols * R : 4];   // summed low-rank queries per row set of the CTA

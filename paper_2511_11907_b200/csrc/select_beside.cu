@@ -109,7 +109,8 @@ cudaError_t launch_select_beside(const Problem& p, const float* scores, int32_t*
                                          n_selected, job, n_first, a);
   };
   const int P = plan_topk_beside(p);
-  if (p.d == 128) return P == 1 ? go(select_beside_kernel<1, 128>) : P == 2 ? go(select_beside_kernel<2, 128>) : go(select_beside_kernel<4, 128>);
+  if (p.d == 128)
+    return P == 1 ? go(select_beside_kernel<1, 128>) : P == 2 ? go(select_beside_kernel<2, 128>) : go(select_beside_kernel<4, 128>);
   return P == 1 ? go(select_beside_kernel<1, 64>) : P == 2 ? go(select_beside_kernel<2, 64>) : go(select_beside_kernel<4, 64>);
 }
 

@@ -2,10 +2,10 @@
 // file's head first) with the warps of the whole GPU dealt to the lists instead of whole CTAs, stages of 16 tokens and one CTA
 // per SM, in half of an SM's registers, so that a decode step runs the next layer's select beside it (topk_beside.cuh, step.cu).
 //
-// Bound by HBM: 22.5 us for 134 MB (B = 4, 8 KV heads, 8192 tokens attended) on SMs without a select, 26.4 on those with one.
-// What made eight warps keep up with sixteen: 16 tokens per stage (half the softmax bookkeeping, P.V with k = 16), two chains of
+// Bound by HBM: 134 MB (B = 4, 8 KV heads, 8192 tokens attended) in 28.1 us as a launch of its own, as the sixteen warps per SM
+// of sparse_decode.cu.  What made eight warps keep up: 16 tokens per stage (half the softmax bookkeeping, P.V with k = 16), two chains of
 // products per block of logits, the sum of the weights left to the lanes until the end, one address per block of eight rows where
-// G is a multiple of 8.  (Stages of 8 tokens with eight warps: 32 us.)
+// G is a multiple of 8.
 #include <algorithm>
 #include <cstdint>
 
@@ -156,8 +156,8 @@ template <typename KV_T, int D, int RH>
 __global__ void __launch_bounds__(kThreads, 2)           // (two: no more than 128 registers)
 sparse_decode_long_kernel(Problem p, const KV_T* __restrict__ q, const KV_T* __restrict__ K,
                             const KV_T* __restrict__ V, const int32_t* __restrict__ group_idx,
-                            const int32_t* __restrict__ n_selected, float* __restrict__ partial, SplitGrid sg, int depth, int g_shift,
-                            uint32_t* __restrict__ err) {
+                            const int32_t* __restrict__ n_selected, float* __restrict__ partial, SplitGrid sg, int depth,
+                            int g_shift, uint32_t* __restrict__ err) {
   constexpr uint32_t ROWB = D * sizeof(KV_T);                  // bytes of one K or V row
   constexpr uint32_t HALFB = kTok * ROWB;                      // K (or V) part of a stage
   constexpr uint32_t kPieces = ROWB / 16;                      // 16-byte pieces per row
@@ -407,13 +407,14 @@ void plan_long_gather(const Problem& p, Workspace* w) {
   // tokens and one CTA per SM: it leaves half of the registers to the next layer's select, which a decode step then runs
   // beside it (step.cu), and takes as long as two CTAs of half the stages or a little longer (a score_select and a
   // sparse_decode of 92 MB, 4 sequences, 8 heads: 42.6 against 42.0 us; 8 sequences, heads of 64 channels 44.0 against 45.1).
-  // The select takes 8 us there, 15 for 16384 groups, and the scorer behind waits for both: not where the gather is over long
-  // before.  us a layer with the other plan / with this one and no bound on the lookahead / bounded to one layer:
+  // The select takes longer the more groups there are, and the scorer behind waits for both: not where the gather is over
+  // long before.  us a layer with the other plan / with this one and no bound on the lookahead / bounded to one layer:
   //   4 sequences,  32768 tokens   50 MB 24.1 / 20.9 / 22.5    80 MB 28.6 / 26.7 / 28.4    110 MB 33.7 / 32.2 / 33.7
   //   4 sequences,  65536 tokens   50 MB 25.6 / 23.3 / 25.3    80 MB 30.1 / 27.7 / 30.0    110 MB 35.1 / 32.4 / 34.5
   //   8 sequences,  65536 tokens   50 MB 31.3 / 27.7 / 30.1    80 MB 36.2 / 32.0 / 35.0    110 MB 40.8 / 36.2 / 39.3
   //   4 sequences, 131072 tokens   60 MB 32.5 / 30.5 / 32.8    80 MB 35.7 / 34.1 / 37.1    110 MB 40.7 / 38.2 / 41.5
-  // (groups of 8; 2 sequences of 50003 tokens, 26 MB: 25.4 / 26.2 unbounded).  134 MB of the last row gain again, 43.1 / 38.5 / 41.5.
+  // (groups of 8; 2 sequences of 50003 tokens, 26 MB: 25.4 / 26.2 unbounded).  134 MB of the last row gain again,
+  // 43.2 / 38.8 / 41.9.
   const int64_t bytes = problems * tokens * int64_t(2 * row);
   w->long_gather = p.kv_dtype != KVSWAP_F32 && p.q_dtype == p.kv_dtype && select_beside_supported(p) &&
                    bytes >= std::max<int64_t>(47 << 20, int64_t(p.NG) * 5000);
@@ -425,7 +426,7 @@ void plan_long_gather(const Problem& p, Workspace* w) {
       most = std::max(most, ((l + 1) * per_list - 1) / kWarps - l * per_list / kWarps + 1);
     return most;
   };
-  auto cost = [&](int64_t per_list) {                            // in half stages of the slowest warp; 4 for what a CTA costs by itself
+  auto cost = [&](int64_t per_list) {                // in half stages of the slowest warp; 4 for what a CTA costs by itself
     const int64_t ctas = (problems * per_list + kWarps - 1) / kWarps;
     return (ctas + kNumSMs - 1) / kNumSMs * ((n_stages + per_list - 1) / per_list * 2 + 4);
   };
@@ -436,7 +437,8 @@ void plan_long_gather(const Problem& p, Workspace* w) {
     if (k < 1) continue;
     const int64_t each = (n_stages + k - 1) / k;
     k = (n_stages + each - 1) / each;
-    if (slots_of(k) > best) k = k >= kWarps ? k / kWarps * kWarps : k >= 4 ? 4 : k >= 2 ? 2 : 1;   // (never more than `best` CTAs: see splits_room)
+    // (never more than `best` CTAs: see splits_room)
+    if (slots_of(k) > best) k = k >= kWarps ? k / kWarps * kWarps : k >= 4 ? 4 : k >= 2 ? 2 : 1;
     if (slots_of(k) <= best && cost(k) < cost(per_list)) per_list = k;
   }
   w->depth = int(std::min<size_t>(kMaxDepth, (192u << 10) / (kWarps * 2 * kTok * row)));

@@ -13,7 +13,7 @@ namespace kvswap {
 //      some 3.5 deviations below the M'-th key's share.
 //   2. The keys that reach the bound (all keys of a short row) are listed: some 1.5 M' of them.
 //   3. A histogram of the list over 1024 equal intervals of the keys finds the interval of the M'-th key; the few keys in
-//      that are ranked by one warp (while they are many, it is cut into 1024 in turn).
+//      that are ranked by one warp (while they are many, it is cut in turn, down to single keys).
 //   4. The selected ones are bits of a map, four keys per lane of a part of 128, from which the positions follow: population
 //      counts, one scan over the parts.
 // Where the list does not come out as expected (more than its room, or fewer than M': scores that run with the position of
@@ -21,10 +21,10 @@ namespace kvswap {
 //
 // It runs beside the gather of the layer before, in what that leaves of an SM: half of the registers and some 30 KB of
 // shared memory.  Unlike topk_parts.cuh it needs no counts of the scorer, whose flush would lie between the two gathers,
-// and one CTA does with a row.  A histogram of all keys in place of the sample kept the SM's shared memory
-// busy (many keys share a bin) and the gather beside it took 29.5 us, not 22.7 (B = 4, 8 heads, 16384 groups).  Bound by
-// latency, and by the gather's share of the issue slots: loads, sample, list, histogram, ranking, scan, writes take 6 us for
-// 4096 groups on an SM of its own, 8 to 9 beside a gather, 15 for 16384.
+// and one CTA does with a row.  A histogram of all keys in place of the sample kept the SM's shared memory busy (many keys
+// share a bin) and held up the gather beside it.  Bound by latency, and by the gather's share of the issue slots: loads,
+// sample, list, histogram, ranking, scan, writes; 13.2 us for 16384 groups as a launch of its own (B = 4, 8 heads), where the
+// kernel that starts from the scorer's counts takes 9.4 with four CTAs per row.
 // ------------------------------------------------------------------------------------------
 constexpr int kBesideThreads = 512;
 constexpr int kBesideWarps = kBesideThreads / 32;

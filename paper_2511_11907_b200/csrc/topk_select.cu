@@ -357,8 +357,8 @@ cudaError_t launch_topk_parts(const Problem& p, const float* scores, uint32_t* t
 }
 
 cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_t* top_hist, int32_t* group_idx,
-                                  int32_t* n_selected, const CombineJob& job, int d, const void* q_ahead, const float* proj_ahead, float* uq_ahead,
-                                  cudaStream_t st) {
+                                  int32_t* n_selected, const CombineJob& job, int d, const void* q_ahead,
+                                  const float* proj_ahead, float* uq_ahead, cudaStream_t st) {
   const int P = plan_topk_parts(p);
   if (P == 0 || (d != 64 && d != 128) || job.slots > kMaxSplits || !job.whole()) return cudaErrorInvalidValue;
   // Query sets of the launch: the scorer's row sets, except that the KV heads of per-head metadata are taken eight at a
@@ -380,7 +380,8 @@ cudaError_t launch_combine_select(const Problem& p, const float* scores, uint32_
   const int n_comb = std::max((job.rows + rows_per_cta - 1) / rows_per_cta, std::min(n_rests, 32));
   const dim3 grid(n_comb + P * n_probs), block(kPartThreads);
   auto go = [&](auto kern) {
-    return launch_pdl(kern, grid, block, 0, st, pq, scores, top_hist, group_idx, n_selected, n_probs, job, n_comb, q_ahead, proj_ahead, uq_ahead, n_rests, n_sub);
+    return launch_pdl(kern, grid, block, 0, st, pq, scores, top_hist, group_idx, n_selected, n_probs, job, n_comb, q_ahead,
+                      proj_ahead, uq_ahead, n_rests, n_sub);
   };
   auto by_parts = [&](auto d_tag) {
     constexpr int D = decltype(d_tag)::value;

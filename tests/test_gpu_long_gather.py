@@ -35,9 +35,9 @@ def _route(wl, meta_heads, scope, flags=0, lookahead=0):
 
 
 # A gather is long from 47 MiB on, and from 5000 bytes per group of the context; and only where the select has room beside the
-# scorer (select_beside_supported).  Head counts that leave one to eight query heads per row, heads of 64 channels, groups whose rows
-# do not fill blocks of eight, open groups of every length of a stage, one to four layers, lists shared by whole and by broken
-# CTAs and by one warp each, both stored types and ranks.
+# scorer (select_beside_supported).  Head counts that leave one to eight query heads per row, heads of 64 channels, groups whose
+# rows do not fill blocks of eight, open groups of several lengths, one to four layers, lists of whole and of broken CTAs, both
+# stored types and ranks.
 @pytest.mark.parametrize("kw", [
     dict(),
     dict(layers=1),
@@ -185,7 +185,7 @@ def _near_rows(kind, problems, groups, top_k, gen):
     else:                                       # "near": ties, with others up to 800 units in the last place above them
         x = torch.rand((problems, groups), generator=gen) * 0.5
         x[:, :top_k // 2] = 1.0
-        x[:, top_k // 2:top_k + top_k // 2] = ulps(1.0, torch.randint(1, 800, (problems, 2 * (top_k // 2)), generator=gen)[:, :top_k])
+        x[:, top_k // 2:top_k + top_k // 2] = ulps(1.0, torch.randint(1, 800, (problems, top_k), generator=gen))
         x[:, top_k:top_k + top_k // 2] = 1.0
     x = x.float()
     return x.gather(1, torch.rand(x.shape, generator=gen).argsort(1))
@@ -194,7 +194,8 @@ def _near_rows(kind, problems, groups, top_k, gen):
 # 24 to 40 rows per case, of whole and sampled lists; the selection is compared with the per-layer calls' and with a stable
 # sort of the scores in float64.
 @pytest.mark.parametrize("kind", ["offset", "ties33", "ties48", "ties128", "plateau", "consecutive", "near"])
-@pytest.mark.parametrize("n_ctx,batch,top_k", [(131072 + 3, 3, 1024), (32768 + 5, 5, 400), (16000 + 5, 5, 400), (32768 + 5, 5, 1400)])
+@pytest.mark.parametrize("n_ctx,batch,top_k",
+                         [(131072 + 3, 3, 1024), (32768 + 5, 5, 400), (16000 + 5, 5, 400), (32768 + 5, 5, 1400)])
 def test_select_beside_among_nearly_equal_scores(kind, n_ctx, batch, top_k):
     wl = _wl(layers=2, n_ctx=n_ctx, top_k=top_k, batch=batch)
     groups, S = n_ctx // 8, wl.n_kv_heads

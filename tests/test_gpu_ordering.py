@@ -175,7 +175,8 @@ def test_scorer_behind_the_projection_of_its_metadata(N, per_head, r, kind):
     proj = _randn(H, d, r, seed=92) * 0.1
     meta, ws = torch.empty((1, hm, N, r), dtype=torch.float16, device="cuda"), rt.alloc_workspace(shape)
     out = torch.empty((1, 1, 4 * H, d), device="cuda")
-    idx, nsel = torch.empty((1, 1, H, M), dtype=torch.int32, device="cuda"), torch.empty((1, 1, H), dtype=torch.int32, device="cuda")
+    idx = torch.empty((1, 1, H, M), dtype=torch.int32, device="cuda")
+    nsel = torch.empty((1, 1, H), dtype=torch.int32, device="cuda")
     layers = kv.make_layers([K], [K], [meta], [proj], 0)
 
     def consume():
